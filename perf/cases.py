@@ -48,7 +48,7 @@ def listed():
         # a whole steady state: Newton from the perturbed conduction state, 32^3 uniform
         dict(name="newton_fp64_32", kind="newton", prec=64, nx=32, ny=32, nz=32, stretch=0.0, Gr=1.0e5),
         # a whole eigen-solve: the four leading eigenvalues about a smooth flow
-        dict(name="eigen_fp64_24", kind="eigen", prec=64, nx=24, ny=24, nz=24, stretch=0.0, Gr=1.0e4),
+        dict(name="eigen_fp64_16", kind="eigen", prec=64, nx=16, ny=16, nz=16, stretch=0.0, Gr=1.0e5),
     ]
 
 
@@ -260,7 +260,7 @@ def prepare(case, seed):
         s["opts"] = o
     if kind == "eigen":
         o = fv.fv_arnoldi_default_opts()
-        o.tol = 1e-10
+        o.tol, o.max_degree = 1e-10, 100
         s["opts"] = o
     return s
 
