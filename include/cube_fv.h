@@ -191,7 +191,7 @@ int fv_jvp_project_batch(fv_grid g, int prec, double Gr, double sigma, const voi
                          void* W, int flags);
 
 /* The block stencil's z-chunk picked by the autotuner (0 = not tuned: the
- * built-in 32 planes) and the block size it was timed on. */
+ * built-in rule) and the block size it was timed on. */
 int fv_get_tuning(fv_grid g, int* pair_zchunk, int* tuned_nvec);
 
 /* Several problems (e.g. continuation points at different Gr on grids of

@@ -521,7 +521,11 @@ int fv_grid_create(const fv_grid_desc* desc, void* stream, fv_grid* out) {
   g->Pr = desc->Pr;
   g->stream = (cudaStream_t)stream;
   AxisHost ax[3];
-  int st = FV_OK;
+  int st = FV_OK, dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+    g->sms = sms;
+  else
+    cudaGetLastError();
   for (int d = 0; d < 3 && st == FV_OK; ++d) {
     if (given[d]) {
       g->xf[d].assign(given[d], given[d] + n[d] + 1);

@@ -103,6 +103,7 @@ struct fv_grid_s {
   fv::FdmDev<double> cd64, fd64;
   fv::FdmDev<float> cd32, fd32;
   fv::Workspace ws;
+  int sms = 152;              // multiprocessors of the device
   long long wait_spins = -1;  // polls of a device-side wait before it gives up; < 0: the default
   double sigma_default;
   double min_width[3];
@@ -129,6 +130,15 @@ namespace fv {
 // seconds on every GPU this library targets, far above any legitimate wait).
 constexpr long long kDefaultWaitSpins = 1LL << 22;
 inline long long wait_spins(const fv_grid_s* g) { return g->wait_spins < 0 ? kDefaultWaitSpins : g->wait_spins; }
+
+// Planes marched by one CTA of a z-marching stencil over `tiles` (x, y) tiles of nvec states: the chunk with
+// the smallest makespan of the busiest multiprocessor, ceil(CTAs / SMs) CTAs of chunk + 1 plane times each (the
+// extra one stands for a CTA's two halo planes and its pipeline fill).  The stencils are bound by their
+// arithmetic (FP64: two operations per clock and SM; FP32: issue slots), so what counts is how evenly the
+// planes spread over the SMs.  Fixed chunks of 32 planes gave a 32^3 grid 4 CTAs (FP64 J.v 629 us; with this
+// rule 128 CTAs, 26 us), a 64^3 grid 16 (FP32 39.5 -> 8.4 us), and left 100^3 FP64 at 64 planes on the busiest
+// SM where 35 suffice (849 -> 470 us).
+int stencil_chunk(const fv_grid_s* g, int tiles, int nvec);
 
 // ------------------------------------------------------------------ error reporting
 void set_error(const std::string& msg);

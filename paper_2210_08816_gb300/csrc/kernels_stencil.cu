@@ -193,15 +193,15 @@ __global__ void __launch_bounds__(256) k_stencil(Geo<R> g, int N, R Gr, R invPr,
 }
 
 // ------------------------------------------------------------------------------------------------
-// z-marching variant.  A block owns a 32 x 8 (x, y) tile of cells and marches over a chunk of kZChunk
-// planes.  For every input array it keeps the planes k-1, k, k+1 of the tile plus a one-cell x/y halo in
+// z-marching variant.  A block owns a 32 x 8 (x, y) tile of cells and marches over a chunk of zc planes
+// (stencil_chunk).  For every input array it keeps the planes k-1, k, k+1 of the tile plus a one-cell x/y halo in
 // a 4-slot shared-memory ring (slot = plane mod 4); cp.async copies of plane k+2 fly while plane k is
 // computed.  Each input element is read from global memory ~1.3 times (halo) instead of ~7 times
 // through L1 as in the one-thread-per-cell kernel.
 // Plane tile of one array in shared memory: kHY rows of kPW elements; the cell (tx, ty) sits at row ty + 1,
 // column tx + kX0 (columns kX0 - 1 .. kX0 + kTX hold the x halo; the TMA box starts 4 columns left of the
 // tile so that its x coordinate stays on a 16-byte boundary).
-constexpr int kTX = 32, kTY = 8, kHY = kTY + 2, kPW = 40, kX0 = 4, kPL = kHY * kPW, kZChunk = 32;
+constexpr int kTX = 32, kTY = 8, kHY = kTY + 2, kPW = 40, kX0 = 4, kPL = kHY * kPW;
 
 template <typename R, int NA>
 struct Ring {
@@ -391,7 +391,7 @@ template <typename R, int MODE>
 __global__ void __launch_bounds__(kTX * kTY, sizeof(R) == 4 ? 3 : 2)
     k_stencil_z(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmv, int use_tma,
                 int* err, long long spins, Geo<R> g, int N, R Gr, R invPr, R sigma, const R* __restrict__ q, const R* __restrict__ v,
-                R* __restrict__ out, int nch) {
+                R* __restrict__ out, int zc, int nch) {
   constexpr int NA = (MODE == 0) ? 4 : 8;
   constexpr int AB = (MODE == 0) ? 0 : 4;
   constexpr int NWARP = kTX * kTY / 32;
@@ -405,11 +405,11 @@ __global__ void __launch_bounds__(kTX * kTY, sizeof(R) == 4 ? 3 : 2)
   // blockIdx.z = z-chunk + nch * vector: vector `vec` of a block of states stored one after another in v and
   // out (4N elements each); its fields are fields 4 vec .. 4 vec + 3 of the tensor map tmv
   const int vec = (int)blockIdx.z / nch;
-  const int i0 = blockIdx.x * kTX, j0 = blockIdx.y * kTY, k0 = ((int)blockIdx.z - vec * nch) * kZChunk;
+  const int i0 = blockIdx.x * kTX, j0 = blockIdx.y * kTY, k0 = ((int)blockIdx.z - vec * nch) * zc;
   v += (size_t)vec * 4 * N;
   out += (size_t)vec * 4 * N;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-  const int kend = min(k0 + kZChunk, nz);
+  const int kend = min(k0 + zc, nz);
   if (use_tma && tid == 0) {
     for (int s = 0; s < kRing; ++s)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar[s])) : "memory");
@@ -827,6 +827,20 @@ inline void cell_grid(const fv_grid_s* g, dim3& grid, dim3& block) {
 
 }  // namespace
 
+int stencil_chunk(const fv_grid_s* g, int tiles, int nvec) {
+  int best = 1;
+  long long best_cost = -1;
+  for (int nch = 1; nch <= g->nz; ++nch) {
+    const int zc = (g->nz + nch - 1) / nch;
+    const long long ctas = (long long)tiles * ((g->nz + zc - 1) / zc) * nvec;
+    if (ctas > 1LL << 20 || (long long)((g->nz + zc - 1) / zc) * nvec > 65535) break;
+    const long long cost = ((ctas + g->sms - 1) / g->sms) * (zc + 1);
+    if (best_cost < 0 || cost < best_cost) best = zc, best_cost = cost;
+  }
+  if (best_cost < 0) best = g->nz;
+  return best;
+}
+
 // 4D tensor map of one state (x, y, z, field) with boxes of kPW x kHY x 1 x 4 elements
 template <typename R>
 int state_map(const fv_grid_s* g, const R* ptr, CUtensorMap* m, int nvec = 1) {
@@ -854,15 +868,16 @@ int launch_stencil_z(const fv_grid_s* g, double Gr, double sigma, const R* q, co
   int use_tma = ((g->nx * sizeof(R)) % 16 == 0 && g->nx >= 64 && g->ny >= 16 && ((uintptr_t)q % 16) == 0 &&
                  ((uintptr_t)v % 16) == 0) ? 1 : 0;
   if (use_tma && (state_map<R>(g, q, &tq) != FV_OK || state_map<R>(g, v, &tv, nvec) != FV_OK)) use_tma = 0;
-  const int nch = (g->nz + kZChunk - 1) / kZChunk;
+  const int gx = (g->nx + kTX - 1) / kTX, gy = (g->ny + kTY - 1) / kTY;
+  const int zc = stencil_chunk(g, gx * gy, nvec), nch = (g->nz + zc - 1) / zc;
   if (nvec < 1 || (long long)nch * nvec > 65535) {
     set_error("launch_stencil_z: too many vectors in one block");
     return FV_EINVAL;
   }
-  dim3 grid((g->nx + kTX - 1) / kTX, (g->ny + kTY - 1) / kTY, nch * nvec);
+  dim3 grid(gx, gy, nch * nvec);
   ProfScope ps(g, PROF_STENCIL);
   k_stencil_z<R, MODE><<<grid, kTX * kTY, smem, g->stream>>>(tq, tv, use_tma, g->ws.err, wait_spins(g), geo_of<R>(g), (int)g->N,
-                                                             (R)Gr, (R)(1.0 / g->Pr), (R)sigma, q, v, out, nch);
+                                                             (R)Gr, (R)(1.0 / g->Pr), (R)sigma, q, v, out, zc, nch);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }

@@ -5,7 +5,7 @@
 // shared memory filled by 4D TMA boxes, but a thread computes the cells (x, y) and (x + 1, y), x even.
 // The two cells share most of their x-neighbours, so the ring is read with 8-byte loads (pairs at even
 // offsets) plus scalars (odd offsets): about half the shared-memory loads per cell, the instruction
-// stream that bounded the one-cell form.  Block: 64 x 8 cells (256 threads), z-chunks of 32 planes.
+// stream that bounded the one-cell form.  Block: 64 x 8 cells (256 threads), z-chunks by stencil_chunk.
 // Wall cases without branches as in the one-cell J.v form: the face-normal wall slot holds zero, the
 // halo outside the domain arrives zero-filled, and the metric arrays hold the wall values; only T's
 // zero-flux walls (y, z) are selects.
@@ -20,7 +20,7 @@ constexpr int kPX = 64, kPY = 8, kPHY = kPY + 2;
 constexpr int kPW2 = 72;            // ring row: x from i0 - 4 to i0 + 67 (TMA x start on a 16-byte boundary)
 constexpr int kPX0 = 4;             // column of the tile's first cell
 constexpr int kPL2 = kPHY * kPW2;   // one array's plane tile
-constexpr int kPZChunk = 32, kPRing = 4, kPNA = 8;  // default z-chunk (planes marched by one CTA)
+constexpr int kPRing = 4, kPNA = 8;
 constexpr long long kPWaitLimit = 1LL << 22;
 
 // ---------------------------------------------------------------- pair arithmetic
@@ -246,8 +246,8 @@ __global__ void __launch_bounds__(kPX / 2 * kPY, 2)
   const int tid = threadIdx.x;
   const int tx = tid % (kPX / 2), ty = tid / (kPX / 2);
   // BLOCK: blockIdx.z = z-chunk + nch * vector, vector `vec` of the block is fields 4 vec .. 4 vec + 3 of
-  // tmv; otherwise one vector in chunks of kPZChunk planes
-  if (!BLOCK) zc = kPZChunk, nch = gridDim.z;
+  // tmv; otherwise one vector in chunks of zc planes
+  if (!BLOCK) nch = gridDim.z;
   const int vec = BLOCK ? (int)blockIdx.z / nch : 0;
   const int i0 = blockIdx.x * kPX, j0 = blockIdx.y * kPY, k0 = ((int)blockIdx.z - vec * nch) * zc;
   if (BLOCK) out += (size_t)vec * 4 * N;
@@ -365,8 +365,9 @@ int launch_stencil_pair(const fv_grid_s* g, double Gr, double sigma, const float
     FV_CUDA(cudaFuncSetAttribute(k_stencil_pair<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     attr_set = true;
   }
-  // blocks of vectors march the z-chunk the autotuner picked (if it ran); single vectors the default
-  const int zc = (nvec > 1 && g->tune.pair_zc > 0) ? g->tune.pair_zc : kPZChunk;
+  // blocks of vectors march the z-chunk the autotuner picked, if it ran; otherwise stencil_chunk's
+  const int zc = (nvec > 1 && g->tune.pair_zc > 0) ? g->tune.pair_zc
+                                                   : stencil_chunk(g, g->nx / kPX * ((g->ny + kPY - 1) / kPY), nvec);
   const int nch = (g->nz + zc - 1) / zc;
   if (nvec < 1 || (long long)nch * nvec > 65535) {
     set_error("launch_stencil_pair: too many vectors in one block for this z-chunk");
