@@ -78,58 +78,65 @@ struct DevBuf {
   }
 };
 
+// Metrics and 1D decompositions of one precision in one device buffer: the half-size operators if `half` is
+// given, else the dense ones.
 template <typename R>
-static int upload_axes(fv_grid_s* g, const AxisHost* ax, int which, Geo<R>& geo, FdmDev<R>& fdm, FdmDev<R>& cd,
-                       FdmDev<R>& fd) {
-  size_t total = 0;
-  for (int d = 0; d < 3; ++d) total += 4 * (size_t)(ax[d].n + 1) + 3 * ((size_t)ax[d].n + 2 * (size_t)ax[d].n * ax[d].n);
-  std::vector<R> h(total);
+static int upload_axes(fv_grid_s* g, const AxisHost* ax, const HalfOpHost (*half)[3], int which, Geo<R>& geo,
+                       FdmDev<R>& fdm, FdmDev<R>& cd, FdmDev<R>& fd, HalfDev<R> (&hd)[3][3]) {
+  std::vector<R> h;
   std::vector<size_t> off;
-  size_t o = 0;
   auto put = [&](const std::vector<double>& v) {
-    off.push_back(o);
-    for (double x : v) h[o++] = (R)x;
+    off.push_back(h.size());
+    h.insert(h.end(), v.begin(), v.end());
+    h.resize((h.size() + 15) & ~(size_t)15, R(0));  // every array on a 64-byte boundary
   };
   for (int d = 0; d < 3; ++d) {
-    put(ax[d].idx);
-    put(ax[d].idc);
-    put(ax[d].wl);
-    put(ax[d].wr);
-    put(ax[d].lam);
-    put(ax[d].Einv);
-    put(ax[d].E);
-    put(ax[d].cd_lam);
-    put(ax[d].cd_Einv);
-    put(ax[d].cd_E);
-    put(ax[d].fd_lam);
-    put(ax[d].fd_Einv);
-    put(ax[d].fd_E);
+    const AxisHost& a = ax[d];
+    for (const auto* v : {&a.idx, &a.idc, &a.wl, &a.wr}) put(*v);
+    if (half)
+      for (int kind = 0; kind < 3; ++kind) {
+        const HalfOpHost& o = half[d][kind];
+        for (const auto* v : {&o.lam, &o.F[0], &o.F[1], &o.E[0], &o.E[1]}) put(*v);
+      }
+    else
+      for (const auto* v : {&a.lam, &a.Einv, &a.E, &a.cd_lam, &a.cd_Einv, &a.cd_E, &a.fd_lam, &a.fd_Einv, &a.fd_E})
+        put(*v);
   }
   void* buf = nullptr;
-  cudaError_t e = cudaMalloc(&buf, total * sizeof(R));
+  cudaError_t e = cudaMalloc(&buf, h.size() * sizeof(R));
   if (e != cudaSuccess) {
     set_error(std::string("cudaMalloc metrics: ") + cudaGetErrorString(e));
     return FV_ENOMEM;
   }
   g->metric_buf[which] = buf;
-  FV_CUDA(cudaMemcpy(buf, h.data(), total * sizeof(R), cudaMemcpyHostToDevice));
+  FV_CUDA(cudaMemcpy(buf, h.data(), h.size() * sizeof(R), cudaMemcpyHostToDevice));
   const R* base = (const R*)buf;
+  size_t c = 0;
+  auto next = [&]() { return base + off[c++]; };
   for (int d = 0; d < 3; ++d) {
     geo.n[d] = ax[d].n;
-    const size_t* od = off.data() + 13 * d;
-    geo.idx[d] = base + od[0];
-    geo.idc[d] = base + od[1];
-    geo.wl[d] = base + od[2];
-    geo.wr[d] = base + od[3];
-    fdm.lam[d] = base + od[4];
-    fdm.Einv[d] = base + od[5];
-    fdm.E[d] = base + od[6];
-    cd.lam[d] = base + od[7];
-    cd.Einv[d] = base + od[8];
-    cd.E[d] = base + od[9];
-    fd.lam[d] = base + od[10];
-    fd.Einv[d] = base + od[11];
-    fd.E[d] = base + od[12];
+    geo.idx[d] = next();
+    geo.idc[d] = next();
+    geo.wl[d] = next();
+    geo.wr[d] = next();
+    if (half) {
+      for (int kind = 0; kind < 3; ++kind) {
+        HalfDev<R>& o = hd[d][kind];
+        o.lam = next();
+        o.F[0] = next();
+        o.F[1] = next();
+        o.E[0] = next();
+        o.E[1] = next();
+        o.k0 = half[d][kind].k0;
+        o.S = half[d][kind].S;
+      }
+      continue;
+    }
+    for (FdmDev<R>* f : {&fdm, &cd, &fd}) {
+      f->lam[d] = next();
+      f->Einv[d] = next();
+      f->E[d] = next();
+    }
   }
   return FV_OK;
 }
@@ -261,10 +268,7 @@ struct Vec {
 template <typename R>
 static int diffusion_solve(fv_grid_s* g, const R* in, R* out, double s = 0.0) {
   FV_TRY(ensure_ws<R>(g));
-  R* tmp = (R*)g->ws.t0[prec_index<R>()];
-  for (int f = 0; f < 4; ++f)
-    FV_TRY(launch_field_solve<R>(g, f, in + (size_t)f * g->N, out + (size_t)f * g->N, tmp, s));
-  return FV_OK;
+  return launch_diffusion_solve<R>(g, in, out, (R*)g->ws.Y[prec_index<R>()], s);
 }
 
 // Right preconditioner M^-1 = P L^-1 (the diffusion part of J inverted, then projected): it removes
@@ -533,15 +537,36 @@ int fv_grid_create(const fv_grid_desc* desc, void* stream, fv_grid* out) {
     } else {
       g->xf[d] = tanh_faces(n[d], desc->stretch);
     }
-    if (st == FV_OK) st = build_axis(g->xf[d], ax[d]);
+    if (st == FV_OK) st = build_axis(g->xf[d], ax[d], true);
     if (st == FV_OK) {
       double mw = 1.0;
       for (int i = 0; i < n[d]; ++i) mw = std::min(mw, g->xf[d][i + 1] - g->xf[d][i]);
       g->min_width[d] = mw;
     }
   }
-  if (st == FV_OK) st = upload_axes<double>(g, ax, 0, g->geo64, g->fdm64, g->cd64, g->fd64);
-  if (st == FV_OK) st = upload_axes<float>(g, ax, 1, g->geo32, g->fdm32, g->cd32, g->fd32);
+  // mirror-symmetric grids (the built-in ones always): half-size decompositions; others: dense ones
+  HalfOpHost half[3][3];
+  if (st == FV_OK) g->half_ready = mirror_symmetric(g->xf[0]) && mirror_symmetric(g->xf[1]) && mirror_symmetric(g->xf[2]);
+  for (int d = 0; d < 3 && st == FV_OK; ++d) {
+    int same = -1;
+    for (int b = 0; b < d && same < 0; ++b)
+      if (g->xf[b] == g->xf[d]) same = b;
+    if (g->half_ready) {
+      for (int kind = 0; kind < 3 && st == FV_OK; ++kind) {
+        if (same >= 0)
+          half[d][kind] = half[same][kind];
+        else
+          st = build_half_op(ax[d], kind, half[d][kind]);
+      }
+    } else if (same >= 0) {
+      ax[d] = ax[same];
+    } else {
+      st = build_axis(g->xf[d], ax[d]);
+    }
+  }
+  const HalfOpHost(*hp)[3] = g->half_ready ? half : nullptr;
+  if (st == FV_OK) st = upload_axes<double>(g, ax, hp, 0, g->geo64, g->fdm64, g->cd64, g->fd64, g->half64);
+  if (st == FV_OK) st = upload_axes<float>(g, ax, hp, 1, g->geo32, g->fdm32, g->cd32, g->fd32, g->half32);
   if (st == FV_OK && tc_eligible(g)) {
     std::vector<double> idx[3] = {ax[0].idx, ax[1].idx, ax[2].idx}, idc[3] = {ax[0].idc, ax[1].idc, ax[2].idc};
     if (tc_setup(g, idx, idc) != FV_OK) {  // keep the SIMT passes

@@ -37,6 +37,15 @@ struct FdmDev {
   const R* lam[3];
 };
 
+// Half-size decomposition of one 1D operator of a mirror-symmetric axis (HalfOpHost on the device).
+template <typename R>
+struct HalfDev {
+  const R* F[2] = {nullptr, nullptr};
+  const R* E[2] = {nullptr, nullptr};
+  const R* lam = nullptr;
+  int k0 = 0, S = 0;
+};
+
 struct Workspace {
   // per precision (0 = FP64, 1 = FP32): J.v output (4N), two transform buffers (N each), potential (N)
   void* Y[2] = {nullptr, nullptr};
@@ -102,6 +111,11 @@ struct fv_grid_s {
   // Dirichlet diffusion operators (cell-centred, face-centred) of the Newton preconditioner
   fv::FdmDev<double> cd64, fd64;
   fv::FdmDev<float> cd32, fd32;
+  // the same operators as half-size problems, [axis][kind], when every axis is mirror-symmetric; the dense
+  // matrices above are then not built
+  bool half_ready = false;
+  fv::HalfDev<double> half64[3][3];
+  fv::HalfDev<float> half32[3][3];
   fv::Workspace ws;
   int sms = 152;              // multiprocessors of the device
   long long wait_spins = -1;  // polls of a device-side wait before it gives up; < 0: the default
@@ -217,11 +231,12 @@ int launch_poisson(const fv_grid_s* g, const R* rhs, R* phi, R* tmp);
 // The same solve for nvec fields stored one after another (N elements each) in rhs, phi and tmp.
 template <typename R>
 int launch_poisson_block(const fv_grid_s* g, const R* rhs, R* phi, R* tmp, int nvec);
-// out = L_f^-1 in for one field f (0..2 velocity with no-slip walls, 3 temperature with Eqs. 4-6 homogeneous
-// and the 1/Pr factor): the diffusion operator of J, inverted by fast diagonalisation (6 passes).
-// s != 0: (L_f - s I)^-1 (the shifted operator of a pseudo-time step 1/s).
+// out = L^-1 in for the four fields of a state (fields 0..2 velocity with no-slip walls, 3 temperature with
+// Eqs. 4-6 homogeneous and the 1/Pr factor): the diffusion operator of J, inverted by fast diagonalisation
+// (6 passes).  s != 0: (L - s I)^-1 (the shifted operator of a pseudo-time step 1/s).  tmp: 4N elements, no
+// alias of in or out; in and out may alias.
 template <typename R>
-int launch_field_solve(const fv_grid_s* g, int field, const R* in, R* out, R* tmp, double s = 0.0);
+int launch_diffusion_solve(const fv_grid_s* g, const R* in, R* out, R* tmp, double s = 0.0);
 
 // BLAS-1 and reductions (kernels_blas.cu).  Results land in g->ws.scalars[slot...].
 template <typename R>
@@ -310,11 +325,26 @@ struct AxisHost {
 // Faces 0 .. n of the tanh-stretched grid with stretching s (s = 0: uniform), mirrored about 1/2.
 std::vector<double> tanh_faces(int n, double s);
 // Metrics and 1D decompositions of the axis with faces xf (strictly increasing); FV_EINVAL otherwise.
-int build_axis(const std::vector<double>& xf, AxisHost& a);
+// metrics_only: without the decompositions.
+int build_axis(const std::vector<double>& xf, AxisHost& a, bool metrics_only = false);
 // True if the faces are their own mirror image about 1/2 (x_f[n-i] = 1 - x_f[i] to 4 units of round-off):
 // the tensor-core passes split each 1D eigenproblem into symmetric and antisymmetric halves, which holds
 // only on such axes.
 bool mirror_symmetric(const std::vector<double>& xf);
+// The 1D operators of a mirror-symmetric axis as two half-size problems (symmetric and antisymmetric vectors).
+// Kinds: the Neumann operator of the pressure solve, the cell-centred and the face-centred Dirichlet diffusion
+// operators.  Unknown k0 + i pairs with S - k0 - i (i < h = ceil(n / 2)); the modes are in the order
+// [h symmetric | floor(n / 2) antisymmetric], each by decreasing eigenvalue.  A face operator's n - 1 modes
+// leave one slot over, the last of the shorter kind: its rows are zero and its eigenvalue is -1.
+//   forward:  mode c (part 0: symmetric, 1: antisymmetric) = sum_i F[part][c][i] (r[k0+i] +- r[S-k0-i])
+//   backward: r[k0+i], r[S-k0-i] = sum_c E[0][i][c] sym[c] +- sum_c E[1][i][c] anti[c]
+// F and E are h x h, row-major, zero where a part is shorter.
+enum { HALF_NEUMANN = 0, HALF_CELL = 1, HALF_FACE = 2 };
+struct HalfOpHost {
+  int n, k0, S;
+  std::vector<double> lam, F[2], E[2];
+};
+int build_half_op(const AxisHost& a, int kind, HalfOpHost& o);
 
 // ------------------------------------------------------------------ Chebyshev filter ellipses (host_cheb.cpp)
 struct Ritz {

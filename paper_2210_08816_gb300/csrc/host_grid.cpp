@@ -98,7 +98,84 @@ static int build_dirichlet_ops(AxisHost& a) {
   return tridiag_operator(mf, fd, fo, FW, n, 1, a.fd_lam, a.fd_Einv, a.fd_E);
 }
 
-int build_axis(const std::vector<double>& xf, AxisHost& a) {
+// Half-size problems of a centro-symmetric tridiagonal matrix (m unknowns, diagonal d, off-diagonal e): the
+// restriction to vectors with y[i] = +-y[m-1-i] is the leading block with the coupling across the midpoint
+// folded into its last diagonal entry (m even), or, for m odd, the symmetric block keeps the midpoint with its
+// coupling scaled by sqrt 2 (the basis vector of a pair is (e_i + e_mirror) / sqrt 2) and the antisymmetric
+// block drops it.  Y: columns by decreasing eigenvalue.
+static int half_eig(int m, const std::vector<double>& d, const std::vector<double>& e, bool anti,
+                    std::vector<double>& lam, std::vector<double>& Y) {
+  const int hm = m / 2, sz = anti ? hm : (m + 1) / 2;
+  lam.assign(sz, 0.0);
+  Y.assign((size_t)sz * sz, 0.0);
+  if (sz == 0) return FV_OK;
+  std::vector<double> dd(d.begin(), d.begin() + sz), ee(std::max(sz - 1, 1), 0.0), Q;
+  for (int i = 0; i + 1 < sz; ++i) ee[i] = e[i];
+  if (m % 2 == 0)
+    dd[sz - 1] += (anti ? -1.0 : 1.0) * e[hm - 1];
+  else if (!anti && sz >= 2)
+    ee[sz - 2] *= std::sqrt(2.0);
+  if (!tridiag_eig(sz, dd, ee, Q)) return invalid("tridiagonal eigensolver did not converge");
+  std::vector<int> ord(sz);
+  std::iota(ord.begin(), ord.end(), 0);
+  std::sort(ord.begin(), ord.end(), [&](int a, int b) { return dd[a] > dd[b]; });
+  for (int c = 0; c < sz; ++c) {
+    lam[c] = dd[ord[c]];
+    for (int i = 0; i < sz; ++i) Y[(size_t)i * sz + c] = Q[(size_t)i * sz + ord[c]];
+  }
+  return FV_OK;
+}
+
+int build_half_op(const AxisHost& a, int kind, HalfOpHost& o) {
+  const int n = a.n, h = (n + 1) / 2, k0 = kind == HALF_FACE ? 1 : 0, m = n - k0;
+  o.n = n;
+  o.k0 = k0;
+  o.S = kind == HALF_FACE ? n : n - 1;
+  // the two halves of the axis agree to round-off of the faces; their mean keeps the operator symmetric and
+  // half the difference away from either
+  std::vector<double> idx(n), idc(n + 1), d(m), e(std::max(m - 1, 1), 0.0), W(m);
+  for (int i = 0; i < n; ++i) idx[i] = 0.5 * (a.idx[i] + a.idx[n - 1 - i]);
+  for (int f = 0; f <= n; ++f) idc[f] = 0.5 * (a.idc[f] + a.idc[n - f]);
+  for (int i = 0; i < m; ++i) {
+    if (kind == HALF_FACE) {
+      const int p = i + 1;
+      W[i] = 1.0 / idc[p];
+      d[i] = -(idx[p] + idx[p - 1]) / W[i];
+    } else {
+      double s = 0.0;
+      if (i >= 1 || kind == HALF_CELL) s -= idc[i];
+      if (i + 1 <= n - 1 || kind == HALF_CELL) s -= idc[i + 1];
+      W[i] = 1.0 / idx[i];
+      d[i] = s / W[i];
+    }
+  }
+  for (int i = 0; i + 1 < m; ++i)
+    e[i] = (kind == HALF_FACE ? idx[i + 1] : idc[i + 1]) / std::sqrt(W[i] * W[i + 1]);
+  o.lam.assign(n, -1.0);  // -1: the dummy mode of the wall slot of a face operator (its rows are zero)
+  const size_t hh = (size_t)h * h;
+  for (int part = 0; part < 2; ++part) {
+    std::vector<double>&F = o.F[part], &E = o.E[part], lam, Y;
+    F.assign(hh, 0.0);
+    E.assign(hh, 0.0);
+    FV_TRY(half_eig(m, d, e, part == 1, lam, Y));
+    const int sz = (int)lam.size();
+    if (kind == HALF_NEUMANN && part == 0) lam[0] = 0.0;  // the constant vector: an exact null vector
+    for (int c = 0; c < sz; ++c) {
+      o.lam[(part ? h : 0) + c] = lam[c];
+      for (int i = 0; i < sz; ++i) {
+        // a pair: the unit vector's share of each of its two cells is 1 / sqrt 2; the midpoint stands alone and
+        // its forward entry is halved because the pass feeds it the sum r + r
+        const bool mid = (m % 2 == 1) && i == sz - 1 && part == 0;
+        const double y = Y[(size_t)i * sz + c] * (mid ? 1.0 : std::sqrt(0.5));
+        F[(size_t)c * h + i] = y * std::sqrt(W[i]) * (mid ? 0.5 : 1.0);
+        E[(size_t)i * h + c] = y / std::sqrt(W[i]);
+      }
+    }
+  }
+  return FV_OK;
+}
+
+int build_axis(const std::vector<double>& xf, AxisHost& a, bool metrics_only) {
   const int n = (int)xf.size() - 1;
   a.n = n;
   std::vector<double> dx(n), xc(n);
@@ -119,6 +196,7 @@ int build_axis(const std::vector<double>& xf, AxisHost& a) {
     a.wl[f] = dx[f] / (dx[f - 1] + dx[f]);
     a.wr[f] = dx[f - 1] / (dx[f - 1] + dx[f]);
   }
+  if (metrics_only) return FV_OK;
   // 1D Neumann operator A = W^-1 S; symmetric form B = W^-1/2 S W^-1/2 (tridiagonal)
   std::vector<double> d(n), e(std::max(n - 1, 1), 0.0);
   for (int i = 0; i < n; ++i) {

@@ -13,6 +13,8 @@
 // all six are one GEMM shape, C[p][m] = sum_k A[p][k] B[m][k] with both operands k-contiguous, stored
 // transposed (out[m][p]).  Tiles BM (p) x BN (m), slabs of BK; thread (tx, ty) owns p = tx + 16 i and
 // m = ty + 16 j, so each store instruction writes 16 consecutive p.
+#include <type_traits>
+
 #include "fv_internal.h"
 
 namespace fv {
@@ -104,6 +106,202 @@ __global__ void __launch_bounds__(256) k_transform(PassArgs t, const R* __restri
   }
 }
 
+// The passes of a mirror-symmetric grid on the CUDA cores: every 1D operator splits into a symmetric and an
+// antisymmetric half (see HalfOpHost), so that a pass contracts the sums and differences of mirrored inputs
+// with two h x h matrices, half the multiplications of the dense form.
+//
+// A CTA owns 32 rows p (one per lane: the rotated store writes 32 consecutive p) and 4 U mode or cell pairs;
+// warp w holds the accumulators of pairs U w .. U w + U - 1, symmetric and antisymmetric.  Slabs of 32 inputs
+// pairs are staged k-major (padded rows: no bank conflicts), the matrix slabs beside them are read as
+// broadcasts.  The FP64 form is bound by the FP64 pipe (two operations per clock and SM: 8 warps cover it), so
+// what matters is that the CTAs spread over all SMs: U falls from 4 to 1 until the launch has two CTAs per SM.
+// blockIdx.z: field of a block of fields stored one after another; with op_mask 3 field f uses operator f (the
+// diffusion solve), with 0 all use operator 0.
+constexpr int kHalfK = 32;
+
+template <typename R>
+struct HalfArgs {
+  const R* M[2][4];    // symmetric / antisymmetric matrix per operator
+  const R* lam[3][4];  // scaled pass: eigenvalues of the three axes per operator
+  R fac[4], shift[4];  // scaled pass: fac / (lam_z + lam_y + lam_x - shift)
+  int k0[4], S[4];
+  int P, n, nb, op_mask, scale, zero_mode;
+};
+
+template <typename R, bool BWD, int U>
+__global__ void __launch_bounds__(128) k_half(const __grid_constant__ HalfArgs<R> t, const R* __restrict__ in,
+                                               R* __restrict__ out) {
+  constexpr int UB = 4 * U, V = 16 / sizeof(R);
+  using Vec = typename std::conditional<sizeof(R) == 4, float4, double2>::type;
+  __shared__ R As[2][kHalfK][33];
+  __shared__ __align__(16) R Bs[2][UB][kHalfK];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n = t.n, P = t.P, h = (n + 1) / 2, ha = n / 2;
+  const int op = (int)blockIdx.z & t.op_mask;
+  const int p0 = blockIdx.x * 32, j0 = blockIdx.y * UB;
+  const int k0 = t.k0[op], S = t.S[op];
+  const R* __restrict__ Ms = t.M[0][op];
+  const R* __restrict__ Ma = t.M[1][op];
+  in += (size_t)blockIdx.z * P * n;
+  out += (size_t)blockIdx.z * P * n;
+  R acc[2][U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) acc[0][u] = acc[1][u] = R(0);
+  for (int kc = 0; kc < h; kc += kHalfK) {
+    const int k = kc + lane;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int row = warp + 4 * r, p = p0 + row;
+      R s = R(0), a = R(0);
+      if (p < P && k < h) {
+        const R* src = in + (size_t)p * n;
+        if (BWD) {
+          s = src[k];
+          a = k < ha ? src[h + k] : R(0);
+        } else {
+          const R x = src[k0 + k], y = src[S - k0 - k];
+          s = x + y;
+          a = x - y;
+        }
+      }
+      As[0][lane][row] = s;
+      As[1][lane][row] = a;
+    }
+#pragma unroll
+    for (int u = warp; u < UB; u += 4) {
+      const bool in_m = j0 + u < h && k < h;
+      Bs[0][u][lane] = in_m ? Ms[(size_t)(j0 + u) * h + k] : R(0);
+      Bs[1][u][lane] = in_m ? Ma[(size_t)(j0 + u) * h + k] : R(0);
+    }
+    __syncthreads();
+    const int kn = min(kHalfK, (h - kc + V - 1) / V * V);  // the slab is zero-filled beyond h
+    for (int kk = 0; kk < kn; kk += V) {
+      R a0[V], a1[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        a0[v] = As[0][kk + v][lane];
+        a1[v] = As[1][kk + v][lane];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const Vec b0 = *reinterpret_cast<const Vec*>(&Bs[0][warp * U + u][kk]);
+        const Vec b1 = *reinterpret_cast<const Vec*>(&Bs[1][warp * U + u][kk]);
+        const R* e0 = reinterpret_cast<const R*>(&b0);
+        const R* e1 = reinterpret_cast<const R*>(&b1);
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          acc[0][u] = fma(a0[v], e0[v], acc[0][u]);
+          acc[1][u] = fma(a1[v], e1[v], acc[1][u]);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  const int p = p0 + lane;
+  if (p >= P) return;
+  R l01 = R(0);
+  bool null_row = false;
+  if (!BWD && t.scale) {
+    const int a = p / t.nb, b = p - a * t.nb;
+    l01 = t.lam[1][op][a] + t.lam[0][op][b] - t.shift[op];
+    null_row = t.zero_mode && p == 0;
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int j = j0 + warp * U + u;
+    if (j >= h) break;
+    R s = acc[0][u], a = acc[1][u];
+    if (BWD) {
+      const int i1 = k0 + j, i2 = S - i1;
+      if (i1 <= i2) {  // (an odd face axis has one pair less than h)
+        out[(size_t)i1 * P + p] = s + a;
+        out[(size_t)i2 * P + p] = s - a;
+      }
+      if (k0 == 1 && j == 0) out[p] = R(0);  // the wall slot
+    } else {
+      if (t.scale) {
+        const R* lz = t.lam[2][op];
+        s = (null_row && j == 0) ? R(0) : t.fac[op] * s / (lz[j] + l01);
+        if (j < ha) a = t.fac[op] * a / (lz[h + j] + l01);
+      }
+      out[(size_t)j * P + p] = s;
+      if (j < ha) out[(size_t)(h + j) * P + p] = a;
+    }
+  }
+}
+
+template <typename R>
+const HalfDev<R> (&half_of(const fv_grid_s* g))[3][3];
+template <>
+const HalfDev<double> (&half_of<double>(const fv_grid_s* g))[3][3] { return g->half64; }
+template <>
+const HalfDev<float> (&half_of<float>(const fv_grid_s* g))[3][3] { return g->half32; }
+
+// One pass along `axis` over nf fields of a (na x nb) x n block, kinds[op][axis] = the operators (one, or four
+// with per_field): in[a][b][k] -> out[m][a][b] with the modes in the half order.
+template <typename R>
+int half_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int (*kinds)[3], bool per_field,
+              const double* sfac, const double* shift, const R* in, R* out, bool scale, bool zero_mode, int nf) {
+  const auto& H = half_of<R>(g);
+  HalfArgs<R> t{};
+  t.n = axis == 0 ? g->nx : axis == 1 ? g->ny : g->nz;
+  t.P = na * nb;
+  t.nb = nb;
+  t.op_mask = per_field ? 3 : 0;
+  t.scale = scale ? 1 : 0;
+  t.zero_mode = zero_mode ? 1 : 0;
+  for (int op = 0; op < (per_field ? 4 : 1); ++op) {
+    const HalfDev<R>& d = H[axis][kinds[op][axis]];
+    for (int part = 0; part < 2; ++part) t.M[part][op] = bwd ? d.E[part] : d.F[part];
+    for (int x = 0; x < 3; ++x) t.lam[x][op] = H[x][kinds[op][x]].lam;
+    t.fac[op] = (R)sfac[op];
+    t.shift[op] = (R)shift[op];
+    t.k0[op] = d.k0;
+    t.S[op] = d.S;
+  }
+  const int h = (t.n + 1) / 2;
+  const long long rows = (long long)((t.P + 31) / 32) * nf;
+  const int U = rows * ((h + 15) / 16) >= 2 * g->sms ? 4 : rows * ((h + 7) / 8) >= 2 * g->sms ? 2 : 1;
+  const dim3 grid((t.P + 31) / 32, (h + 4 * U - 1) / (4 * U), nf);
+  ProfScope ps(g, PROF_TRANSFORM);
+  if (bwd) {
+    if (U == 4) k_half<R, true, 4><<<grid, 128, 0, g->stream>>>(t, in, out);
+    else if (U == 2) k_half<R, true, 2><<<grid, 128, 0, g->stream>>>(t, in, out);
+    else k_half<R, true, 1><<<grid, 128, 0, g->stream>>>(t, in, out);
+  } else {
+    if (U == 4) k_half<R, false, 4><<<grid, 128, 0, g->stream>>>(t, in, out);
+    else if (U == 2) k_half<R, false, 2><<<grid, 128, 0, g->stream>>>(t, in, out);
+    else k_half<R, false, 1><<<grid, 128, 0, g->stream>>>(t, in, out);
+  }
+  FV_CUDA(cudaGetLastError());
+  return FV_OK;
+}
+
+// the six passes over nf fields: in -> out, tmp of the same size (out may alias in)
+template <typename R>
+int half_solve(const fv_grid_s* g, const int (*kinds)[3], bool per_field, const double* sfac, const double* shift,
+               bool zero_mode, const R* in, R* out, R* tmp, int nf) {
+  const int nx = g->nx, ny = g->ny, nz = g->nz;
+  if (nf < 1 || nf > 65535) {
+    set_error("half_solve: number of fields out of range");
+    return FV_EINVAL;
+  }
+  // forward: (z,y,x) -> (mx,z,y) -> (my,mx,z) -> (mz,my,mx) / Lambda; backward the same way round
+  FV_TRY(half_pass<R>(g, 0, false, nz, ny, kinds, per_field, sfac, shift, in, tmp, false, zero_mode, nf));
+  FV_TRY(half_pass<R>(g, 1, false, nx, nz, kinds, per_field, sfac, shift, tmp, out, false, zero_mode, nf));
+  FV_TRY(half_pass<R>(g, 2, false, ny, nx, kinds, per_field, sfac, shift, out, tmp, true, zero_mode, nf));
+  FV_TRY(half_pass<R>(g, 0, true, nz, ny, kinds, per_field, sfac, shift, tmp, out, false, zero_mode, nf));
+  FV_TRY(half_pass<R>(g, 1, true, nx, nz, kinds, per_field, sfac, shift, out, tmp, false, zero_mode, nf));
+  return half_pass<R>(g, 2, true, ny, nx, kinds, per_field, sfac, shift, tmp, out, false, zero_mode, nf);
+}
+
+constexpr int kPoissonKinds[1][3] = {{HALF_NEUMANN, HALF_NEUMANN, HALF_NEUMANN}};
+// fields u, v, w: face-centred along the own axis, cell-centred Dirichlet across; T: Dirichlet in x only
+constexpr int kDiffusionKinds[4][3] = {{HALF_FACE, HALF_CELL, HALF_CELL},
+                                       {HALF_CELL, HALF_FACE, HALF_CELL},
+                                       {HALF_CELL, HALF_CELL, HALF_FACE},
+                                       {HALF_CELL, HALF_NEUMANN, HALF_NEUMANN}};
+
 template <typename R>
 const FdmDev<R>& fdm_of(const fv_grid_s* g);
 template <>
@@ -154,44 +352,6 @@ const FdmDev<float>& fd_of<float>(const fv_grid_s* g) { return g->fd32; }
 }  // namespace
 
 template <typename R>
-int launch_poisson(const fv_grid_s* g, const R* rhs, R* phi, R* tmp) {
-  const FdmDev<R>& f = fdm_of<R>(g);
-  const int nx = g->nx, ny = g->ny, nz = g->nz;
-  // forward: (z,y,x) -> (mx,z,y) -> (my,mx,z) -> (mz,my,mx) / Lambda
-  FV_TRY(pass<R>(g, f.Einv[0], nz, ny, nx, rhs, tmp, false));
-  FV_TRY(pass<R>(g, f.Einv[1], nx, nz, ny, tmp, phi, false));
-  FV_TRY(pass<R>(g, f.Einv[2], ny, nx, nz, phi, tmp, true));
-  // backward: (mz,my,mx) -> (x,mz,my) -> (y,x,mz) -> (z,y,x)
-  FV_TRY(pass<R>(g, f.E[0], nz, ny, nx, tmp, phi, false));
-  FV_TRY(pass<R>(g, f.E[1], nx, nz, ny, phi, tmp, false));
-  FV_TRY(pass<R>(g, f.E[2], ny, nx, nz, tmp, phi, false));
-  return FV_OK;
-}
-
-template <>
-int launch_poisson<float>(const fv_grid_s* g, const float* rhs, float* phi, float* tmp) {
-  const int nx = g->nx, ny = g->ny, nz = g->nz;
-  if (g->tc.ready) {  // the same six passes on the tensor cores (3 x TF32 split, FP32 accuracy; modes in
-                      // the symmetric / antisymmetric order of the mirror-symmetric grid)
-    FV_TRY(tc_pass(g, 0, false, nz, ny, rhs, tmp, false));
-    FV_TRY(tc_pass(g, 1, false, nx, nz, tmp, phi, false));
-    FV_TRY(tc_pass(g, 2, false, ny, nx, phi, tmp, true));
-    FV_TRY(tc_pass(g, 0, true, nz, ny, tmp, phi, false));
-    FV_TRY(tc_pass(g, 1, true, nx, nz, phi, tmp, false));
-    FV_TRY(tc_pass(g, 2, true, ny, nx, tmp, phi, false));
-    return FV_OK;
-  }
-  const FdmDev<float>& f = fdm_of<float>(g);
-  FV_TRY(pass<float>(g, f.Einv[0], nz, ny, nx, rhs, tmp, false));
-  FV_TRY(pass<float>(g, f.Einv[1], nx, nz, ny, tmp, phi, false));
-  FV_TRY(pass<float>(g, f.Einv[2], ny, nx, nz, phi, tmp, true));
-  FV_TRY(pass<float>(g, f.E[0], nz, ny, nx, tmp, phi, false));
-  FV_TRY(pass<float>(g, f.E[1], nx, nz, ny, phi, tmp, false));
-  FV_TRY(pass<float>(g, f.E[2], ny, nx, nz, tmp, phi, false));
-  return FV_OK;
-}
-
-template <typename R>
 int launch_poisson_block(const fv_grid_s* g, const R* rhs, R* phi, R* tmp, int nvec) {
   const int nx = g->nx, ny = g->ny, nz = g->nz;
   if (nvec < 1 || nvec > 65535) {
@@ -199,7 +359,7 @@ int launch_poisson_block(const fv_grid_s* g, const R* rhs, R* phi, R* tmp, int n
     return FV_EINVAL;
   }
   if constexpr (sizeof(R) == 4) {
-    if (g->tc.ready && g->tc.sms > 0) {  // the tensor-core passes over the stacked fields, one launch each
+    if (g->tc.ready) {  // the tensor-core passes over the stacked fields (3 x TF32 split, FP32 accuracy)
       FV_TRY(tc_pass(g, 0, false, nz, ny, rhs, tmp, false, nvec));
       FV_TRY(tc_pass(g, 1, false, nx, nz, tmp, phi, false, nvec));
       FV_TRY(tc_pass(g, 2, false, ny, nx, phi, tmp, true, nvec));
@@ -209,16 +369,28 @@ int launch_poisson_block(const fv_grid_s* g, const R* rhs, R* phi, R* tmp, int n
       return FV_OK;
     }
   }
+  if (g->half_ready) {
+    const double one = 1.0, zero = 0.0;
+    return half_solve<R>(g, kPoissonKinds, false, &one, &zero, true, rhs, phi, tmp, nvec);
+  }
+  // dense passes, forward: (z,y,x) -> (mx,z,y) -> (my,mx,z) -> (mz,my,mx) / Lambda
   const FdmDev<R>& f = fdm_of<R>(g);
   FV_TRY(pass<R>(g, f.Einv[0], nz, ny, nx, rhs, tmp, false, nvec));
   FV_TRY(pass<R>(g, f.Einv[1], nx, nz, ny, tmp, phi, false, nvec));
   FV_TRY(pass<R>(g, f.Einv[2], ny, nx, nz, phi, tmp, true, nvec));
+  // backward: (mz,my,mx) -> (x,mz,my) -> (y,x,mz) -> (z,y,x)
   FV_TRY(pass<R>(g, f.E[0], nz, ny, nx, tmp, phi, false, nvec));
   FV_TRY(pass<R>(g, f.E[1], nx, nz, ny, phi, tmp, false, nvec));
   FV_TRY(pass<R>(g, f.E[2], ny, nx, nz, tmp, phi, false, nvec));
   return FV_OK;
 }
 
+template <typename R>
+int launch_poisson(const fv_grid_s* g, const R* rhs, R* phi, R* tmp) {
+  return launch_poisson_block<R>(g, rhs, phi, tmp, 1);
+}
+
+template int launch_poisson<float>(const fv_grid_s*, const float*, float*, float*);
 template int launch_poisson<double>(const fv_grid_s*, const double*, double*, double*);
 template int launch_poisson_block<double>(const fv_grid_s*, const double*, double*, double*, int);
 template int launch_poisson_block<float>(const fv_grid_s*, const float*, float*, float*, int);
@@ -227,30 +399,38 @@ template int launch_poisson_block<float>(const fv_grid_s*, const float*, float*,
 // velocity component c uses the face-centred Dirichlet operator along its own axis and the cell-centred
 // Dirichlet operator across (no-slip walls half a cell away); temperature uses cell-centred Dirichlet in
 // x (Eq. 4, homogeneous) and the Neumann operator in y and z (Eqs. 5-6), with s_T = 1/Pr.  No zero mode.
-// in and out may alias; tmp may not.
 // s != 0: (L_f - s I)^-1 instead (the eigenvalues of L_f are (lam_x + lam_y + lam_z) / s_f).
+// On mirror-symmetric grids the four fields go through each pass together (6 launches instead of 24).
 template <typename R>
-int launch_field_solve(const fv_grid_s* g, int field, const R* in, R* out, R* tmp, double s) {
-  const FdmDev<R>* op[3];
-  for (int d = 0; d < 3; ++d) {
-    if (field < 3)
-      op[d] = (d == field) ? &fd_of<R>(g) : &cd_of<R>(g);
-    else
-      op[d] = (d == 0) ? &cd_of<R>(g) : &fdm_of<R>(g);
-  }
-  const R* lam[3] = {op[0]->lam[0], op[1]->lam[1], op[2]->lam[2]};
-  const double sfac = (field == 3) ? g->Pr : 1.0;
+int launch_diffusion_solve(const fv_grid_s* g, const R* in, R* out, R* tmp, double s) {
   const int nx = g->nx, ny = g->ny, nz = g->nz;
-  FV_TRY(pass_ops<R>(g, op[0]->Einv[0], nz, ny, nx, in, tmp, false, lam, false, 1.0));
-  FV_TRY(pass_ops<R>(g, op[1]->Einv[1], nx, nz, ny, tmp, out, false, lam, false, 1.0));
-  FV_TRY(pass_ops<R>(g, op[2]->Einv[2], ny, nx, nz, out, tmp, true, lam, false, sfac, 1, s * sfac));
-  FV_TRY(pass_ops<R>(g, op[0]->E[0], nz, ny, nx, tmp, out, false, lam, false, 1.0));
-  FV_TRY(pass_ops<R>(g, op[1]->E[1], nx, nz, ny, out, tmp, false, lam, false, 1.0));
-  FV_TRY(pass_ops<R>(g, op[2]->E[2], ny, nx, nz, tmp, out, false, lam, false, 1.0));
+  if (g->half_ready) {
+    const double sfac[4] = {1.0, 1.0, 1.0, g->Pr}, shift[4] = {s, s, s, s * g->Pr};
+    return half_solve<R>(g, kDiffusionKinds, true, sfac, shift, false, in, out, tmp, 4);
+  }
+  for (int f = 0; f < 4; ++f) {
+    const FdmDev<R>* op[3];
+    for (int d = 0; d < 3; ++d) {
+      if (f < 3)
+        op[d] = (d == f) ? &fd_of<R>(g) : &cd_of<R>(g);
+      else
+        op[d] = (d == 0) ? &cd_of<R>(g) : &fdm_of<R>(g);
+    }
+    const R* lam[3] = {op[0]->lam[0], op[1]->lam[1], op[2]->lam[2]};
+    const double sfac = (f == 3) ? g->Pr : 1.0;
+    const R* fi = in + (size_t)f * g->N;
+    R* fo = out + (size_t)f * g->N;
+    FV_TRY(pass_ops<R>(g, op[0]->Einv[0], nz, ny, nx, fi, tmp, false, lam, false, 1.0));
+    FV_TRY(pass_ops<R>(g, op[1]->Einv[1], nx, nz, ny, tmp, fo, false, lam, false, 1.0));
+    FV_TRY(pass_ops<R>(g, op[2]->Einv[2], ny, nx, nz, fo, tmp, true, lam, false, sfac, 1, s * sfac));
+    FV_TRY(pass_ops<R>(g, op[0]->E[0], nz, ny, nx, tmp, fo, false, lam, false, 1.0));
+    FV_TRY(pass_ops<R>(g, op[1]->E[1], nx, nz, ny, fo, tmp, false, lam, false, 1.0));
+    FV_TRY(pass_ops<R>(g, op[2]->E[2], ny, nx, nz, tmp, fo, false, lam, false, 1.0));
+  }
   return FV_OK;
 }
 
-template int launch_field_solve<double>(const fv_grid_s*, int, const double*, double*, double*, double);
-template int launch_field_solve<float>(const fv_grid_s*, int, const float*, float*, float*, double);
+template int launch_diffusion_solve<double>(const fv_grid_s*, const double*, double*, double*, double);
+template int launch_diffusion_solve<float>(const fv_grid_s*, const float*, float*, float*, double);
 
 }  // namespace fv
