@@ -17,8 +17,8 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIBDIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(LIBDIR, "libcubefv.so")
-SOURCES = ["kernels_stencil.cu", "kernels_stencil2.cu", "kernels_fdm.cu", "kernels_tc.cu", "kernels_blas.cu", "host_linalg.cpp",
-           "host_cheb.cpp", "host_grid.cpp", "host_tc.cpp", "fv_api.cpp", "noalloc.cu", "kernels_prolong.cu", "kernels_diag.cu"]
+SOURCES = ["kernels_stencil.cu", "kernels_stencil2.cu", "kernels_fdm.cu", "kernels_tc.cu", "kernels_digit.cu", "kernels_blas.cu", "host_linalg.cpp",
+           "host_cheb.cpp", "host_grid.cpp", "host_tc.cpp", "host_digits.cpp", "fv_api.cpp", "noalloc.cu", "kernels_prolong.cu", "kernels_diag.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -30,7 +30,7 @@ def _nvcc() -> str:
 
 
 def _headers():
-    return [os.path.join(CSRC, "fv_internal.h"), os.path.join(ROOT, "include", "cube_fv.h")]
+    return [os.path.join(CSRC, "fv_internal.h"), os.path.join(CSRC, "tcgen05.cuh"), os.path.join(ROOT, "include", "cube_fv.h")]
 
 
 def _stale(obj: str, deps) -> bool:

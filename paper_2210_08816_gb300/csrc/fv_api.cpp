@@ -141,6 +141,61 @@ static int upload_axes(fv_grid_s* g, const AxisHost* ax, const HalfOpHost (*half
   return FV_OK;
 }
 
+// The half-size operators as digits for the tensor-core passes, both precisions, in one device buffer; axes with
+// the same faces share theirs.
+static int upload_digits(fv_grid_s* g, const HalfOpHost (*half)[3]) {
+  struct Item {
+    size_t dig, exp;
+  };
+  std::vector<unsigned char> buf, blocks;
+  std::vector<int> exps;
+  Item items[3][3][2][2];  // [axis][kind][precision][direction]
+  auto put = [&](const void* p, size_t bytes) {
+    const size_t at = buf.size();
+    buf.resize((at + bytes + 255) & ~(size_t)255, 0);
+    std::memcpy(buf.data() + at, p, bytes);
+    return at;
+  };
+  for (int d = 0; d < 3; ++d) {
+    int same = -1;
+    for (int b = 0; b < d && same < 0; ++b)
+      if (g->xf[b] == g->xf[d]) same = b;
+    for (int kind = 0; kind < 3; ++kind)
+      for (int prec = 0; prec < 2; ++prec)
+        for (int dir = 0; dir < 2; ++dir) {
+          Item& it = items[d][kind][prec][dir];
+          if (same >= 0) {
+            it = items[same][kind][prec][dir];
+            continue;
+          }
+          const HalfOpHost& o = half[d][kind];
+          build_digits(dir ? o.E : o.F, (o.n + 1) / 2, prec ? kDigits32 : kDigits64, prec ? kDigitCols32 : kDigitCols64,
+                       blocks, exps);
+          it.dig = put(blocks.data(), blocks.size());
+          it.exp = put(exps.data(), exps.size() * sizeof(int));
+        }
+  }
+  if (cudaMalloc(&g->digit_buf, buf.size()) != cudaSuccess) {
+    g->digit_buf = nullptr;
+    cudaGetLastError();
+    set_error("digit operand allocation failed");
+    return FV_ENOMEM;
+  }
+  FV_CUDA(cudaMemcpy(g->digit_buf, buf.data(), buf.size(), cudaMemcpyHostToDevice));
+  const unsigned char* base = (const unsigned char*)g->digit_buf;
+  for (int d = 0; d < 3; ++d)
+    for (int kind = 0; kind < 3; ++kind)
+      for (int dir = 0; dir < 2; ++dir) {
+        g->half64[d][kind].dig[dir] = base + items[d][kind][0][dir].dig;
+        g->half64[d][kind].dexp[dir] = (const int*)(base + items[d][kind][0][dir].exp);
+        g->half32[d][kind].dig[dir] = base + items[d][kind][1][dir].dig;
+        g->half32[d][kind].dexp[dir] = (const int*)(base + items[d][kind][1][dir].exp);
+      }
+  FV_TRY(digit_setup());
+  g->digit_ready = true;
+  return FV_OK;
+}
+
 template <typename R>
 static constexpr int prec_index() {
   return sizeof(R) == 8 ? 0 : 1;
@@ -567,6 +622,7 @@ int fv_grid_create(const fv_grid_desc* desc, void* stream, fv_grid* out) {
   const HalfOpHost(*hp)[3] = g->half_ready ? half : nullptr;
   if (st == FV_OK) st = upload_axes<double>(g, ax, hp, 0, g->geo64, g->fdm64, g->cd64, g->fd64, g->half64);
   if (st == FV_OK) st = upload_axes<float>(g, ax, hp, 1, g->geo32, g->fdm32, g->cd32, g->fd32, g->half32);
+  if (st == FV_OK && g->half_ready && (std::max({n[0], n[1], n[2]}) + 1) / 2 <= kDigitMaxH) st = upload_digits(g, half);
   if (st == FV_OK && tc_eligible(g)) {
     std::vector<double> idx[3] = {ax[0].idx, ax[1].idx, ax[2].idx}, idc[3] = {ax[0].idc, ax[1].idc, ax[2].idc};
     if (tc_setup(g, idx, idc) != FV_OK) {  // keep the SIMT passes
@@ -611,6 +667,7 @@ int fv_grid_destroy(fv_grid g) {
   if (g->ws.host_scalars) cudaFreeHost(g->ws.host_scalars);
   for (cudaEvent_t e : g->prof.pool) cudaEventDestroy(e);
   if (g->tc.buf) cudaFree(g->tc.buf);
+  if (g->digit_buf) cudaFree(g->digit_buf);
   if (g->ws.err) cudaFree(g->ws.err);
   if (g->batch_exec) cudaGraphExecDestroy(g->batch_exec);
   if (g->capture_stream) cudaStreamDestroy(g->capture_stream);

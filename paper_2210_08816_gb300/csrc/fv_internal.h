@@ -44,6 +44,9 @@ struct HalfDev {
   const R* E[2] = {nullptr, nullptr};
   const R* lam = nullptr;
   int k0 = 0, S = 0;
+  // the matrices as digits (build_digits) and their rows' exponents, forward and backward
+  const unsigned char* dig[2] = {nullptr, nullptr};
+  const int* dexp[2] = {nullptr, nullptr};
 };
 
 struct Workspace {
@@ -114,6 +117,8 @@ struct fv_grid_s {
   // the same operators as half-size problems, [axis][kind], when every axis is mirror-symmetric; the dense
   // matrices above are then not built
   bool half_ready = false;
+  bool digit_ready = false;  // ... and as digits for the tensor cores (h <= kDigitMaxH on every axis)
+  void* digit_buf = nullptr;
   fv::HalfDev<double> half64[3][3];
   fv::HalfDev<float> half32[3][3];
   fv::Workspace ws;
@@ -238,6 +243,13 @@ int launch_poisson_block(const fv_grid_s* g, const R* rhs, R* phi, R* tmp, int n
 template <typename R>
 int launch_diffusion_solve(const fv_grid_s* g, const R* in, R* out, R* tmp, double s = 0.0);
 
+// One pass along `axis` over nf fields by exact digit products on the tensor cores (kernels_digit.cu): in[a][b][k]
+// -> out[m][a][b]; kinds[op][axis] = the operators, one, or four with per_field (field f uses operator f).
+template <typename R>
+int digit_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int (*kinds)[3], bool per_field,
+               const double* sfac, const double* shift, const R* in, R* out, bool scale, bool zero_mode, int nf);
+int digit_setup();
+
 // BLAS-1 and reductions (kernels_blas.cu).  Results land in g->ws.scalars[slot...].
 template <typename R>
 int launch_dot(const fv_grid_s* g, const R* a, const R* b, size_t n, int slot);
@@ -345,6 +357,15 @@ struct HalfOpHost {
   std::vector<double> lam, F[2], E[2];
 };
 int build_half_op(const AxisHost& a, int kind, HalfOpHost& o);
+
+// ------------------------------------------------------------------ digits (host_digits.cpp)
+// Digits per value, outputs per unit of work, and the longest half axis (order sums stay below 2^24).
+constexpr int kDigits64 = 7, kDigitCols64 = 32, kDigits32 = 4, kDigitCols32 = 64, kDigitMaxH = 128;
+// The two h x h matrices as D balanced base-256 digits (FP16), row j on the common exponent exps[j] of both parts:
+// M[part][j][k] = 2^exps[j] sum_i digit_i 256^(D-1-i).  Blocks [part][group of NC rows][slab of 32 columns], each
+// D NC rows (digit i, output j % NC at row i NC + j % NC) of 64 bytes, 64-byte swizzled.
+void build_digits(const std::vector<double> (&M)[2], int h, int D, int NC, std::vector<unsigned char>& blocks,
+                  std::vector<int>& exps);
 
 // ------------------------------------------------------------------ Chebyshev filter ellipses (host_cheb.cpp)
 struct Ritz {

@@ -1,0 +1,613 @@
+// Fast-diagonalisation passes on the tensor cores by exact digit products (FP64 fields, and FP32 fields of any
+// size and operator): the error-free splitting of Ozaki, Ogita, Oishi & Rump (Numer. Algorithms 59, 2012) with
+// fixed-point rows, on tcgen05.mma kind::f16.
+//
+// A pass contracts the sums and differences of mirrored inputs with two h x h matrices (see HalfOpHost).  Each row
+// of inputs is written on a common exponent as an integer of D balanced base-256 digits, x = 2^e sum_i x_i
+// 256^(D-1-i), |x_i| <= 128, and so is each row of a matrix (on the host, build_digits).  Digits are exact in
+// FP16, a product of two is at most 2^14, and the sum over K <= 128 inputs of the at most 7 products of one order
+// i + j is an integer below 2^24: FP32 accumulators hold it exactly.  Orders 0 .. D-1 are kept:
+//   FP64: D = 7 (56 bits), 28 products; the first dropped order lies 2^-56 below the largest product of the row.
+//   FP32: D = 4 (32 bits), 10 products.
+// The epilogue joins the D accumulators as a 64-bit integer, so the only roundings are the digits' quantisation,
+// the dropped orders and the conversion of the result: below those of the FP64 fused multiply-add chain (errors
+// against 64 bits: 256^3 Chebyshev step 3.3e-14 by the CUDA-core passes).
+//
+// Why: GB300 issues two FP64 operations per clock and SM (1.23 TFLOP/s measured in k_half); the 28 FP16 products
+// cost 155 GFLOP per 256^3 pass where the FP16 tensor rate is 1.9 PFLOP/s.
+//
+// Layout.  Stacking the matrix digits j = 0 .. D-1-i of NC outputs as rows of one B operand makes all products of
+// input digit i ONE instruction: N = (D - i) NC columns, accumulated at column i NC, where block d of NC columns
+// holds order d.  A unit of work is 128 rows x NC pairs, both parts; TMEM columns 0 and 256 hold the symmetric and
+// the antisymmetric accumulators.  A CTA walks a contiguous range of units (the groups of NC pairs of a tile follow
+// each other, so its rows stay in L2 and their exponents are found once).  Warps:
+//   0      bulk copies of the B digits (pre-swizzled blocks) into the slots of a ring
+//   1      TMEM allocation, MMA issue
+//   2-17   workers: row exponents, then per slab of 32 inputs the sum and difference digits into two slots; the
+//          epilogue of unit u (four warps per TMEM lane quadrant) between the first and the second slab of unit
+//          u + 1, so that the MMAs find digits waiting when the accumulators are free
+// Barriers per slot: full (B landed), conv (all workers), empty (commit); per unit accf (commit) and acce.
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <type_traits>
+#include <utility>
+
+#include "fv_internal.h"
+#include "tcgen05.cuh"
+
+namespace fv {
+namespace {
+
+constexpr int kDgRows = 128;
+constexpr int kDgSlots = 3;
+constexpr int kDgWarps = 16;  // workers
+constexpr int kDgIts = kDgRows / (2 * kDgWarps);  // row pairs of a worker warp per slab
+constexpr int kDgThreads = 32 * (2 + kDgWarps);
+constexpr int kDgE = 2;  // outputs of a row read from TMEM at a time
+constexpr int kDgDigitBytes = kDgRows * 64;  // one digit of a 128 x 32 slab (64-byte swizzled rows)
+
+template <typename R>
+struct Dg;
+template <>
+struct Dg<double> {
+  static constexpr int D = kDigits64, NC = kDigitCols64;
+  using Int = long long;
+};
+template <>
+struct Dg<float> {
+  static constexpr int D = kDigits32, NC = kDigitCols32;
+  using Int = int;
+};
+
+template <typename R>
+struct DgArgs {
+  const unsigned char* B[4];  // per operator: digit blocks [part][group][slab] of this direction
+  const int* eM[4];           // per operator: exponent of every output pair
+  const R* lam[3][4];         // scaled pass: eigenvalues of the three axes per operator
+  R fac[4], shift[4];         // scaled pass: fac / (lam_z + lam_y + lam_x - shift)
+  int k0[4], S[4];
+  int P, n, nb, op_mask, scale, zero_mode;
+  int tiles, groups, nslab, units, vec;
+  int* err;
+  long long spins;
+};
+
+__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
+          tmem_d),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t (&r)[2]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(taddr));
+}
+
+// x on the row's exponent E as an integer, truncated: FP64 |I| < 2^53 with value I 2^(E - 1075), FP32 |I| < 2^29
+// with value I 2^(E - 155).  E >= 64 (FP32: 32) and shifts clamp, so that zeros and subnormals shift out.  (FP64:
+// the dropped bits lie below 2^-52 of the row's largest input, a quarter of what the roundings of an FMA chain over
+// 128 inputs add up to.)
+__device__ __forceinline__ long long to_fixed(double x, int E) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  unsigned long long m = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | lo;
+  asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(E - (int)(((unsigned)hi & 0x7fffffffu) >> 20)));
+  const long long sg = (long long)(hi >> 31);
+  return ((long long)m ^ sg) - sg;
+}
+__device__ __forceinline__ int to_fixed(float x, int E) {
+  const int b = __float_as_int(x);
+  unsigned m = (((unsigned)b & 0x7fffffu) | 0x800000u) << 5;
+  asm("shr.u32 %0, %0, %1;" : "+r"(m) : "r"(E - (int)(((unsigned)b & 0x7fffffffu) >> 23)));
+  const int sg = b >> 31;
+  return ((int)m ^ sg) - sg;
+}
+
+// The D balanced digits of two neighbouring inputs as FP16 pairs, digit i at dst + i * kDgDigitBytes.  Adding 128 to
+// every digit makes them the bytes of an unsigned integer; 0x6400 | byte is the FP16 number 1024 + byte.
+__device__ __forceinline__ void put_pair(unsigned char* dst, uint32_t h) {
+  const __half2 r = __hadd2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(0xE480)));  // - 1152
+  *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(&r);
+}
+// digits lo and lo - 1 of both inputs from the low (sel 0x5410) or high (0x7632) halves of their words
+__device__ __forceinline__ void put_two(unsigned char* dst, int lo, uint32_t a, uint32_t b, uint32_t sel) {
+  const uint32_t w = __byte_perm(a, b, sel);
+  put_pair(dst + lo * kDgDigitBytes, __byte_perm(w, 0x64646464u, 0x4240));
+  put_pair(dst + (lo - 1) * kDgDigitBytes, __byte_perm(w, 0x64646464u, 0x4341));
+}
+__device__ __forceinline__ void put_digits(unsigned char* dst, long long I0, long long I1) {
+  constexpr unsigned long long kBias = 0x80808080808080ull;
+  const unsigned long long u0 = (unsigned long long)I0 + kBias, u1 = (unsigned long long)I1 + kBias;
+  const uint32_t a0 = (uint32_t)u0, a1 = (uint32_t)(u0 >> 32), b0 = (uint32_t)u1, b1 = (uint32_t)(u1 >> 32);
+  put_two(dst, 6, a0, b0, 0x5410);
+  put_two(dst, 4, a0, b0, 0x7632);
+  put_two(dst, 2, a1, b1, 0x5410);
+  put_pair(dst, __byte_perm(a1, b1, 0x7632) | 0x64006400u);
+}
+__device__ __forceinline__ void put_digits(unsigned char* dst, int I0, int I1) {
+  const uint32_t a = (uint32_t)I0 + 0x80808080u, b = (uint32_t)I1 + 0x80808080u;
+  put_two(dst, 3, a, b, 0x5410);
+  put_two(dst, 1, a, b, 0x7632);
+}
+
+// Two neighbouring values: one vector load when `vec` (the pair is aligned), else two scalar ones; the second only
+// if `two`.
+template <typename R>
+__device__ __forceinline__ void load_two(const R* __restrict__ p, bool vec, bool two, R& a, R& b) {
+  if (vec) {
+    using V2 = typename std::conditional<sizeof(R) == 8, double2, float2>::type;
+    const V2 v = __ldg(reinterpret_cast<const V2*>(p));
+    a = v.x;
+    b = v.y;
+  } else {
+    a = __ldg(p);
+    b = two ? __ldg(p + 1) : R(0);
+  }
+}
+
+// The D order sums of one output joined.  FP64: an integer V = 2^-8 sum_d A_d 256^(6-d) (value V 2^(E + eM -
+// 1019)), |V| < 2^62 so that S +- A fits.
+__device__ __forceinline__ long long join_orders(const uint32_t (&r)[7][kDgE], int j) {
+  auto A = [&](int d) { return __float2int_rn(__uint_as_float(r[d][j])); };
+  const long long hi = (long long)(A(1) * 256 + A(2)) * 16777216 + ((long long)A(0) << 40);
+  return hi + (long long)A(3) * 65536 + (long long)A(4) * 256 + (A(5) + (A(6) >> 8));
+}
+// FP32: the number sum_d A_d 256^(3-d) (value V 2^(E + eM - 131)) to one rounding of each half and of their sum
+__device__ __forceinline__ float join_orders(const uint32_t (&r)[4][kDgE], int j) {
+  auto A = [&](int d) { return __float2int_rn(__uint_as_float(r[d][j])); };
+  return fmaf((float)(A(0) * 256 + A(1)), 65536.0f, (float)(A(2) * 256 + A(3)));
+}
+
+// v 2^e rounded to nearest; integer arithmetic only (an FP64 operation per output would cost as much as the MMAs).
+// fast: |e| is small enough that the result is normal whatever v is (or zero).
+__device__ __forceinline__ double from_fixed(long long v, int e, bool fast) {
+  const long long sg = v >> 63;
+  unsigned long long u = (unsigned long long)((v ^ sg) - sg);  // <= 2^62
+  if (u == 0) return 0.0;
+  const int lz = __clzll((long long)u) - 1;
+  u = ((u << lz) + 512) >> 10;          // 53 bits, the leading one at bit 52 (or 53 after rounding up)
+  const int be = e + 62 - lz + 1023;    // biased exponent
+  unsigned long long b = u + ((unsigned long long)(unsigned)(be - 1) << 52);
+  if (!fast) b = be >= 2047 ? 0x7ff0000000000000ull : be < 1 ? 0ull : b;
+  return __longlong_as_double((long long)(b | ((unsigned long long)sg << 63)));
+}
+__device__ __forceinline__ float from_fixed(float v, int e, bool fast) {
+  return fast ? v * __uint_as_float((unsigned)(e + 127) << 23) : ldexpf(v, e);
+}
+
+template <typename R>
+__device__ __forceinline__ R quiet_nan();
+template <>
+__device__ __forceinline__ double quiet_nan<double>() { return __longlong_as_double(0x7ff8000000000000LL); }
+template <>
+__device__ __forceinline__ float quiet_nan<float>() { return __uint_as_float(0x7fc00000u); }
+
+// A unit of work (field, tile of rows, group of outputs), stepped without divisions: every warp keeps its own, and
+// the integer divisions of a fresh decomposition per slab cost the workers as much as a slab's conversion.
+template <typename R>
+struct DgUnit {
+  int group, tile, field;
+  __device__ __forceinline__ DgUnit(const DgArgs<R>& t, int u) {
+    const int ft = u / t.groups;
+    group = u - ft * t.groups;
+    field = ft / t.tiles;
+    tile = ft - field * t.tiles;
+  }
+  __device__ __forceinline__ void step(const DgArgs<R>& t) {
+    if (++group == t.groups) {
+      group = 0;
+      if (++tile == t.tiles) tile = 0, ++field;
+    }
+  }
+};
+
+template <typename R, bool BWD>
+__global__ void __launch_bounds__(kDgThreads, 1)
+    k_digit_pass(const __grid_constant__ DgArgs<R> t, const R* __restrict__ in, R* __restrict__ out) {
+  constexpr int D = Dg<R>::D, NC = Dg<R>::NC;
+  constexpr bool F64 = sizeof(R) == 8;
+  constexpr int kExpShift = F64 ? 20 : 23, kExpMax = F64 ? 2047 : 255, kExpMin = F64 ? 64 : 32;
+  constexpr uint32_t kABytes = D * kDgDigitBytes, kBBytes = D * NC * 64, kSlotBytes = kABytes + kBBytes;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t bar_full[kDgSlots], bar_conv[kDgSlots], bar_empty[kDgSlots];
+  __shared__ __align__(8) uint64_t bar_accf, bar_acce, bar_drain;
+  __shared__ uint32_t tmem_slot;
+  // exponents of the rows, four tiles deep: a warp can find those of tile T + 1 while another still reads T - 1's in
+  // an epilogue (tile T + 2 has to wait for that epilogue's MMAs)
+  __shared__ int row_exp[4][kDgRows];
+  __shared__ int out_exp[4][kDigitMaxH];  // exponents of the matrix rows per operator
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const uint32_t base = smem_u32(smem);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int n = t.n, P = t.P, h = (n + 1) / 2, ha = n / 2;
+  const int u0 = (int)((long long)t.units * blockIdx.x / gridDim.x);
+  const int u1 = (int)((long long)t.units * (blockIdx.x + 1) / gridDim.x);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kDgSlots; ++s) {
+      mbar_init(smem_u32(&bar_full[s]), 1);
+      mbar_init(smem_u32(&bar_conv[s]), 32 * kDgWarps);
+      mbar_init(smem_u32(&bar_empty[s]), 1);
+    }
+    mbar_init(smem_u32(&bar_accf), 1);
+    mbar_init(smem_u32(&bar_acce), kDgWarps);
+    mbar_init(smem_u32(&bar_drain), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int i = threadIdx.x; i < (t.op_mask + 1) * h; i += kDgThreads) out_exp[i / h][i % h] = t.eM[i / h][i % h];
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int gi = 0, issued = 0;
+      bool ok = true;
+      DgUnit<R> un(t, u0), nx = un;
+      for (int u = u0; u < u1 && ok; ++u) {
+        const int group = un.group, op = un.field & t.op_mask;
+        // the rows of the next tile into L2, while this one is worked on
+        if (u == u0 || group == 0) {
+          int v = u;
+          do nx.step(t), ++v;
+          while (nx.group != 0);
+          if (v < u1) {
+            const R* src = in + ((size_t)nx.field * P + (size_t)nx.tile * kDgRows) * n;
+            const uint32_t bytes = (uint32_t)(min(kDgRows, P - nx.tile * kDgRows) * n * sizeof(R)) & ~15u;
+            if ((uintptr_t)src % 16 == 0 && bytes)
+              asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+          }
+        }
+        for (int j = 0; j < t.nslab && ok; ++j)
+          for (int part = 0; part < 2; ++part, ++gi) {
+            const int st = gi % kDgSlots;
+            if (gi >= kDgSlots &&
+                !mbar_wait(smem_u32(&bar_empty[st]), ((gi / kDgSlots) - 1) & 1, t.err, 31, t.spins)) {
+              ok = false;
+              break;
+            }
+            const uint32_t fb = smem_u32(&bar_full[st]);
+            mbar_expect_tx(fb, kBBytes);
+            bulk_load(base + st * kSlotBytes + kABytes,
+                      t.B[op] + ((size_t)(part * t.groups + group) * t.nslab + j) * kBBytes, kBBytes, fb);
+            ++issued;
+          }
+        un.step(t);
+      }
+      // every issued copy has landed before the block may exit
+      for (int g2 = (issued > kDgSlots ? issued - kDgSlots : 0); g2 < issued; ++g2)
+        mbar_wait(smem_u32(&bar_full[g2 % kDgSlots]), (g2 / kDgSlots) & 1, t.err, 32, kWaitLimit);
+    }
+  } else if (warp == 1) {
+    // descriptors differ from the first slot's by constants: one addition per MMA (building each from its address in
+    // one lane cost 140 clocks per MMA, more than the MMA itself: 64 on average)
+    const uint64_t desc0 = smem_desc(base);
+    int gi = 0;
+    bool ok = true;
+    for (int u = u0; u < u1 && ok; ++u) {
+      if (u > u0 && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_acce), (u - u0 - 1) & 1, t.err, 33, t.spins))) {
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      for (int j = 0; j < t.nslab && ok; ++j)
+        for (int part = 0; part < 2; ++part, ++gi) {
+          const int st = gi % kDgSlots;
+          const uint32_t ph = (gi / kDgSlots) & 1;
+          if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_full[st]), ph, t.err, 34, t.spins) &&
+                                           mbar_wait(smem_u32(&bar_conv[st]), ph, t.err, 35, t.spins))) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t da = desc0 + (uint64_t)((st * kSlotBytes) >> 4), db = da + (kABytes >> 4);
+          const uint32_t acc = tmem + part * 256;
+          if (elect_one()) {
+#pragma unroll
+            for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+              for (int i = 0; i < D; ++i) {
+                // M = 128, N = (D - i) NC, FP16 operands, FP32 accumulators
+                constexpr uint32_t kId = (1u << 4) | ((kDgRows / 16u) << 24);
+                mma_f16(acc + i * NC, da + ((i * kDgDigitBytes + kk * 32) >> 4), db + (kk * 32 >> 4),
+                        kId | ((uint32_t)((D - i) * NC / 8) << 17), (kk > 0 || i > 0) ? 1u : (uint32_t)(j > 0));
+              }
+            mma_commit(smem_u32(&bar_empty[st]));
+            // (the last slab's second part: arrives once every MMA of the unit has completed)
+            if (part == 1 && j == t.nslab - 1) mma_commit(smem_u32(&bar_accf));
+          }
+          __syncwarp();
+        }
+    }
+    // give-up path: wait (full limit) for every MMA issued so far before the accumulators are freed
+    if (!ok) {
+      if (elect_one()) mma_commit(smem_u32(&bar_drain));
+      mbar_wait(smem_u32(&bar_drain), 0, t.err, 36, kWaitLimit);
+    }
+  } else {
+    // a worker warp converts rows 2 (kDgWarps it + cw), + 1 (half a warp each; a lane takes two neighbouring input
+    // pairs) and reads TMEM lanes 32 (warp % 4) .. + 31 in the epilogue (one row per thread)
+    const int cw = warp - 2, rh = lane >> 4, kl = (lane & 15) * 2;
+    const bool vec = t.vec != 0;
+    const int erow = (warp % 4) * 32 + lane;
+    const uint32_t lane_base = tmem + ((uint32_t)((warp % 4) * 32) << 16);
+    const int total = (u1 - u0) * t.nslab;
+    int item = 0, tc = 0;  // slabs done; count of tiles (row_exp)
+    bool ok = true;
+    DgUnit<R> un(t, u0), nx = un, pv = un;  // this unit, the next slab's, the one before
+    // inputs of row pair `it` for the slab of an item; those of the next slab are requested as soon as this one's
+    // are converted
+    R x0[kDgIts], x1[kDgIts], y0[kDgIts], y1[kDgIts];
+    auto load_row = [&](int it, const R* __restrict__ src, int rows, int k, int k0, int S) {
+      const int row = 2 * (kDgWarps * it + cw) + rh;
+      const bool two = k + 1 < h;
+      x0[it] = x1[it] = y0[it] = y1[it] = R(0);
+      if (k < h && row < rows) {
+        const R* p = src + (size_t)row * n;
+        if (BWD) {
+          load_two<R>(p + k, vec, two, x0[it], x1[it]);
+          if (k < ha) load_two<R>(p + h + k, vec, k + 1 < ha, y0[it], y1[it]);
+        } else if (vec && two) {
+          load_two<R>(p + k0 + k, true, true, x0[it], x1[it]);
+          load_two<R>(p + S - k0 - k - 1, true, true, y1[it], y0[it]);
+        } else {
+          load_two<R>(p + k0 + k, false, two, x0[it], x1[it]);
+          y0[it] = __ldg(p + S - k0 - k);
+          y1[it] = two ? __ldg(p + S - k0 - k - 1) : R(0);
+        }
+      }
+    };
+    // slabs j of unit u0 + du; one turn more for the epilogue of the last unit
+    for (int du = 0, j = 0; ok; ++item) {
+      if (item < total) {
+        const int op = un.field & t.op_mask;
+        const int k0 = t.k0[op], S = t.S[op];
+        const R* __restrict__ src = in + ((size_t)un.field * P + (size_t)un.tile * kDgRows) * n;
+        const int rows = min(kDgRows, P - un.tile * kDgRows);
+        if (j == 0 && (du == 0 || un.group == 0)) {
+          ++tc;
+          // largest magnitude of each of the warp's rows (FP64: by the high words), 16 loads in flight; a face
+          // axis' wall slot holds no input
+          constexpr int kRows = 2 * kDgIts, kStep = sizeof(R) / 4;
+          unsigned m[kRows];
+#pragma unroll
+          for (int r = 0; r < kRows; ++r) m[r] = 0;
+          const unsigned* __restrict__ w0 = reinterpret_cast<const unsigned*>(src) + (kStep - 1);
+#pragma unroll 1
+          for (int k = (BWD ? 0 : k0) + lane; k - lane < n; k += 64) {
+            unsigned v[2][kRows];
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+              for (int r = 0; r < kRows; ++r) {
+                const int row = min(2 * (kDgWarps * (r >> 1) + cw) + (r & 1), rows - 1);
+                v[q][r] = __ldg(w0 + ((size_t)row * n + min(k + 32 * q, n - 1)) * kStep);
+              }
+#pragma unroll
+            for (int r = 0; r < kRows; ++r) m[r] = max(m[r], max(v[0][r] & 0x7fffffffu, v[1][r] & 0x7fffffffu));
+          }
+#pragma unroll
+          for (int r = 0; r < kRows; ++r) {
+            const unsigned top = __reduce_max_sync(0xffffffffu, m[r]);
+            if (lane == 0)
+              row_exp[tc & 3][2 * (kDgWarps * (r >> 1) + cw) + (r & 1)] = max((int)(top >> kExpShift), kExpMin);
+          }
+          __syncwarp();
+        }
+        const int* __restrict__ re = row_exp[tc & 3];
+        const int gi = 2 * item, s0 = gi % kDgSlots, s1 = (gi + 1) % kDgSlots;
+        if (item == 0) {
+#pragma unroll
+          for (int it = 0; it < kDgIts; ++it) load_row(it, src, rows, kl, k0, S);
+        }
+        // the next item: this unit's next slab, or the first of the next unit
+        if (j + 1 == t.nslab) nx.step(t);
+        const R* __restrict__ nsrc = in + ((size_t)nx.field * P + (size_t)nx.tile * kDgRows) * n;
+        const int nrows = item + 1 < total ? min(kDgRows, P - nx.tile * kDgRows) : 0;
+        const int nk = (j + 1 == t.nslab ? 0 : (j + 1) * 32) + kl;
+        const int nk0 = t.k0[nx.field & t.op_mask], nS = t.S[nx.field & t.op_mask];
+        using I = typename Dg<R>::Int;
+        I i0[kDgIts], i1[kDgIts], j0[kDgIts], j1[kDgIts];
+#pragma unroll
+        for (int it = 0; it < kDgIts; ++it) {
+          const int E = re[2 * (kDgWarps * it + cw) + rh];
+          i0[it] = to_fixed(x0[it], E);
+          i1[it] = to_fixed(x1[it], E);
+          j0[it] = to_fixed(y0[it], E);
+          j1[it] = to_fixed(y1[it], E);
+          load_row(it, nsrc, nrows, nk, nk0, nS);
+        }
+        // each slot is filled as soon as it is free: with three slots, the MMAs of the slab before run meanwhile
+        constexpr int kRow = 2 * kDgWarps * 64;
+        const int off = (2 * cw + rh) * 64 + (((kl >> 3) ^ (cw & 3)) << 4) + (kl & 7) * 2;  // row >> 1 = cw mod 4
+        if (gi >= kDgSlots && !mbar_wait(smem_u32(&bar_empty[s0]), ((gi / kDgSlots) - 1) & 1, t.err, 37, t.spins)) {
+          ok = false;
+          break;
+        }
+        unsigned char* dst = smem + s0 * kSlotBytes + off;
+#pragma unroll
+        for (int it = 0; it < kDgIts; ++it)
+          put_digits(dst + it * kRow, BWD ? i0[it] : i0[it] + j0[it], BWD ? i1[it] : i1[it] + j1[it]);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_arrive(smem_u32(&bar_conv[s0]));
+        if (gi + 1 >= kDgSlots &&
+            !mbar_wait(smem_u32(&bar_empty[s1]), (((gi + 1) / kDgSlots) - 1) & 1, t.err, 38, t.spins)) {
+          ok = false;
+          break;
+        }
+        dst = smem + s1 * kSlotBytes + off;
+#pragma unroll
+        for (int it = 0; it < kDgIts; ++it)
+          put_digits(dst + it * kRow, BWD ? j0[it] : i0[it] - j0[it], BWD ? j1[it] : i1[it] - j1[it]);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_arrive(smem_u32(&bar_conv[s1]));
+      }
+      if (j == 0 && du > 0) {  // epilogue of the previous unit
+        const int group = pv.group, op = pv.field & t.op_mask, p = pv.tile * kDgRows + erow;
+        const bool newer = item < total && un.group == 0;  // tile tc is already the next one
+        const bool live = p < P;
+        const int k0 = t.k0[op], S = t.S[op];
+        R* __restrict__ o = out + (size_t)pv.field * P * n + p;
+        R l01 = R(0);
+        if (!BWD && t.scale && live) {
+          const int a = p / t.nb, b = p - a * t.nb;
+          l01 = t.lam[1][op][a] + t.lam[0][op][b] - t.shift[op];
+        }
+        ok = mbar_wait(smem_u32(&bar_accf), (du - 1) & 1, t.err, 39, t.spins);
+        if (!__all_sync(0xffffffffu, ok)) {
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int E = row_exp[(newer ? tc - 1 : tc) & 3][erow];
+        const bool bad = E == kExpMax;  // an Inf or NaN among the row's inputs
+        const int c1 = min(NC, h - group * NC);
+#pragma unroll 1
+        for (int c0 = (cw >> 2) * kDgE; c0 < c1; c0 += (kDgWarps / 4) * kDgE) {
+          decltype(join_orders(std::declval<const uint32_t(&)[D][kDgE]>(), 0)) vs[kDgE], va[kDgE];
+          uint32_t rs[D][kDgE], ra[D][kDgE];
+#pragma unroll
+          for (int d = 0; d < D; ++d) tmem_ld2(lane_base + d * NC + c0, rs[d]);
+#pragma unroll
+          for (int d = 0; d < D; ++d) tmem_ld2(lane_base + 256 + d * NC + c0, ra[d]);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int q = 0; q < kDgE; ++q) vs[q] = join_orders(rs, q), va[q] = join_orders(ra, q);
+          if (live) {
+#pragma unroll
+            for (int q = 0; q < kDgE; ++q) {
+              const int jj = group * NC + c0 + q;
+              if (jj >= h) break;
+              const int e = E + out_exp[op][jj] - (F64 ? 1019 : 131);
+              // (FP32 fast: the factor 2^e is normal and |v| < 2^48 cannot overflow)
+              const bool fast = F64 ? (e > -1000 && e < 900) : (e > -120 && e < 70);
+              R s = from_fixed(BWD ? vs[q] + va[q] : vs[q], e, fast);
+              R a = from_fixed(BWD ? vs[q] - va[q] : va[q], e, fast);
+              if (bad) s = a = quiet_nan<R>();
+              if (BWD) {
+                const int i1 = k0 + jj, i2 = S - i1;
+                if (i1 <= i2) {  // (an odd face axis has one pair less than h)
+                  o[(size_t)i1 * P] = s;
+                  o[(size_t)i2 * P] = a;
+                }
+                if (k0 == 1 && jj == 0) o[0] = R(0);  // the wall slot
+              } else {
+                if (t.scale) {
+                  const R* lz = t.lam[2][op];
+                  s = (t.zero_mode && p == 0 && jj == 0) ? R(0) : t.fac[op] * s / (lz[jj] + l01);
+                  if (jj < ha) a = t.fac[op] * a / (lz[h + jj] + l01);
+                }
+                o[(size_t)jj * P] = s;
+                if (jj < ha) o[(size_t)(h + jj) * P] = a;
+              }
+            }
+          }
+        }
+        // the accumulators' values are in registers (tcgen05.wait::ld): the MMAs may reuse them
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bar_acce));
+      }
+      if (item == total) break;
+      if (++j == t.nslab) {
+        j = 0;
+        ++du;
+        pv = un;
+        un.step(t);
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
+template <typename R>
+constexpr size_t digit_smem() {
+  return (size_t)kDgSlots * (Dg<R>::D * kDgDigitBytes + Dg<R>::D * Dg<R>::NC * 64) + 1024;
+}
+
+template <typename R>
+const HalfDev<R> (&half_of(const fv_grid_s* g))[3][3];
+template <>
+const HalfDev<double> (&half_of<double>(const fv_grid_s* g))[3][3] { return g->half64; }
+template <>
+const HalfDev<float> (&half_of<float>(const fv_grid_s* g))[3][3] { return g->half32; }
+
+}  // namespace
+
+int digit_setup() {
+  static_assert(digit_smem<double>() <= 227 * 1024 && digit_smem<float>() <= 227 * 1024, "ring fits shared memory");
+  FV_CUDA(cudaFuncSetAttribute(k_digit_pass<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)digit_smem<double>()));
+  FV_CUDA(cudaFuncSetAttribute(k_digit_pass<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)digit_smem<double>()));
+  FV_CUDA(cudaFuncSetAttribute(k_digit_pass<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)digit_smem<float>()));
+  FV_CUDA(cudaFuncSetAttribute(k_digit_pass<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)digit_smem<float>()));
+  return FV_OK;
+}
+
+template <typename R>
+int digit_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int (*kinds)[3], bool per_field,
+               const double* sfac, const double* shift, const R* in, R* out, bool scale, bool zero_mode, int nf) {
+  const auto& H = half_of<R>(g);
+  DgArgs<R> t{};
+  t.n = axis == 0 ? g->nx : axis == 1 ? g->ny : g->nz;
+  t.P = na * nb;
+  t.nb = nb;
+  t.op_mask = per_field ? 3 : 0;
+  t.scale = scale ? 1 : 0;
+  t.zero_mode = zero_mode ? 1 : 0;
+  const int h = (t.n + 1) / 2;
+  bool cells = true;
+  for (int op = 0; op < (per_field ? 4 : 1); ++op) {
+    const HalfDev<R>& d = H[axis][kinds[op][axis]];
+    t.B[op] = d.dig[bwd ? 1 : 0];
+    t.eM[op] = d.dexp[bwd ? 1 : 0];
+    for (int x = 0; x < 3; ++x) t.lam[x][op] = H[x][kinds[op][x]].lam;
+    t.fac[op] = (R)sfac[op];
+    t.shift[op] = (R)shift[op];
+    t.k0[op] = d.k0;
+    t.S[op] = d.S;
+    cells = cells && d.k0 == 0;
+  }
+  // pairs of neighbours by one load: rows of an even length from an aligned base, pairs at even offsets
+  t.vec = t.n % 2 == 0 && (bwd ? h % 2 == 0 : cells) && (uintptr_t)in % (2 * sizeof(R)) == 0;
+  t.tiles = (t.P + kDgRows - 1) / kDgRows;
+  t.groups = (h + Dg<R>::NC - 1) / Dg<R>::NC;
+  t.nslab = (h + 31) / 32;
+  const long long units = (long long)t.tiles * t.groups * nf;
+  if (units > (1LL << 30)) {
+    set_error("digit_pass: too many fields in one block");
+    return FV_EINVAL;
+  }
+  t.units = (int)units;
+  t.err = g->ws.err;
+  t.spins = wait_spins(g);
+  const unsigned grid = (unsigned)std::min<long long>(units, g->sms);
+  ProfScope ps(g, PROF_TRANSFORM_TC);
+  if (bwd)
+    k_digit_pass<R, true><<<grid, kDgThreads, digit_smem<R>(), g->stream>>>(t, in, out);
+  else
+    k_digit_pass<R, false><<<grid, kDgThreads, digit_smem<R>(), g->stream>>>(t, in, out);
+  FV_CUDA(cudaGetLastError());
+  return FV_OK;
+}
+
+template int digit_pass<double>(const fv_grid_s*, int, bool, int, int, const int (*)[3], bool, const double*,
+                                const double*, const double*, double*, bool, bool, int);
+template int digit_pass<float>(const fv_grid_s*, int, bool, int, int, const int (*)[3], bool, const double*,
+                               const double*, const float*, float*, bool, bool, int);
+
+}  // namespace fv

@@ -237,11 +237,25 @@ const HalfDev<double> (&half_of<double>(const fv_grid_s* g))[3][3] { return g->h
 template <>
 const HalfDev<float> (&half_of<float>(const fv_grid_s* g))[3][3] { return g->half32; }
 
+// Digit products on the tensor cores (kernels_digit.cu) instead of the CUDA-core form, by the multiplications of a
+// half-size pass.  A digit pass costs ~16 us before its length shows (one unit of work: exponents, digits, MMAs,
+// epilogue one after another), a CUDA-core pass ~8.  FP64 (pass, us, CUDA cores / digits): 32^3 9.7 / 16,
+// 56^3 19.2 / 19.4, 64^3 25.6 / 19.8, 100^3 130 / 36, 160^3 589 / 78, four fields of 40^3 26 / 21.  FP32, whose
+// CUDA-core rate is 64 times higher: 112^3 18.4 / 18.7, 150^3 40.9 / 40.6, 200^3 109 / 75, four fields of 100^3
+// 38.7 / 40.4, of 112^3 48.9 / 42.1, of 250^3 875 / 433.
+template <typename R>
+bool digit_wins(int n, long long rows) {
+  return (double)rows * n * ((n + 1) / 2) >= (sizeof(R) == 8 ? 4.5e6 : 2.6e8);
+}
+
 // One pass along `axis` over nf fields of a (na x nb) x n block, kinds[op][axis] = the operators (one, or four
 // with per_field): in[a][b][k] -> out[m][a][b] with the modes in the half order.
 template <typename R>
 int half_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int (*kinds)[3], bool per_field,
               const double* sfac, const double* shift, const R* in, R* out, bool scale, bool zero_mode, int nf) {
+  const int len = axis == 0 ? g->nx : axis == 1 ? g->ny : g->nz;
+  if (g->digit_ready && digit_wins<R>(len, (long long)na * nb * nf))
+    return digit_pass<R>(g, axis, bwd, na, nb, kinds, per_field, sfac, shift, in, out, scale, zero_mode, nf);
   const auto& H = half_of<R>(g);
   HalfArgs<R> t{};
   t.n = axis == 0 ? g->nx : axis == 1 ? g->ny : g->nz;

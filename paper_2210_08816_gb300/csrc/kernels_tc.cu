@@ -37,6 +37,7 @@
 #include <vector>
 
 #include "fv_internal.h"
+#include "tcgen05.cuh"
 
 namespace fv {
 namespace {
@@ -47,42 +48,6 @@ constexpr int kTcRowBytes = kTcBK * 4;
 constexpr int kTcABytes = kTcBM * kTcRowBytes;  // one A slab tile (8 KB)
 constexpr int kTcStages = 3;
 constexpr int kTcThreads = 192;
-constexpr long long kWaitLimit = 1LL << 22;  // bounded spin on every mbarrier (seconds at most)
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// bounded wait (at most `spins` polls); on expiry records `code` in *err and returns false
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err, int code,
-                                          long long spins = kWaitLimit) {
-  for (long long i = 0; i < spins; ++i)
-    if (mbar_try(bar, parity)) return true;
-  atomicCAS(err, 0, code);
-  return false;
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
   asm volatile(
@@ -92,44 +57,12 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
-// Plain bulk copy global -> shared (contiguous bytes, 16-byte aligned ends), completing on an mbarrier.
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar)
-               : "memory");
-}
-
-// Shared-memory matrix descriptor: K-major operand, 64-byte swizzle, 8-row groups 512 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFF) >> 4);        // start address
-  d |= (uint64_t)1 << 16;                         // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)((8 * kTcRowBytes) >> 4) << 32;  // stride byte offset: next 8-row group
-  d |= (uint64_t)1 << 46;                         // descriptor version (sm_100 family)
-  d |= (uint64_t)4 << 61;                         // 64-byte swizzle
-  return d;
-}
-
 __device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(
           tmem_d),
       "l"(a), "l"(b), "r"(idesc), "r"(acc)
       : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
-      "[%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
 // Converter helpers.  A 64-byte swizzled row r keeps its 16-byte chunk c at physical chunk c ^ ((r >> 1) & 3).
@@ -443,55 +376,56 @@ __global__ void __launch_bounds__(kTcpThreads, 1)
         mbar_wait(smem_u32(&bar_full[gi % kTcpStages]), (gi / kTcpStages) & 1, err, 12, kWaitLimit);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc =
-          (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(h >> 3) << 17) | ((uint32_t)(kTcBM >> 4) << 24);
-      bool ok = true;
-      int last = -1;  // last tile whose accumulator commit was issued
-      for (int ti = 0; ti < my_tiles && ok; ++ti) {
-        const int b = ti & 1;
-        if (ti >= 2 && !mbar_wait(smem_u32(&bar_acce[b]), ((ti / 2) - 1) & 1, err, 13, spins)) {
+    // descriptors differ from the first stage's by multiples of 16 bytes: additions only (building each from its
+    // address in one lane cost 140 clocks per MMA, more than the MMA's own 64)
+    const uint64_t desc0 = smem_desc(base);
+    const uint32_t idesc =
+        (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(h >> 3) << 17) | ((uint32_t)(kTcBM >> 4) << 24);
+    bool ok = true;
+    for (int ti = 0; ti < my_tiles && ok; ++ti) {
+      const int b = ti & 1;
+      if (ti >= 2 &&
+          !__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_acce[b]), ((ti / 2) - 1) & 1, err, 13, spins))) {
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t dacc = tmem + (uint32_t)(b * 256);
+      for (int j = 0; j < nst; ++j) {
+        const int gi = ti * nst + j, st = gi % kTcpStages;
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_conv[st]), (gi / kTcpStages) & 1, err, 14, spins))) {
           ok = false;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t dacc = tmem + (uint32_t)(b * 256);
-        for (int j = 0; j < nst; ++j) {
-          const int gi = ti * nst + j, st = gi % kTcpStages;
-          if (!mbar_wait(smem_u32(&bar_conv[st]), (gi / kTcpStages) & 1, err, 14, spins)) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t sb = base + st * stage_bytes;
-          const uint32_t lb = lo_base + (uint32_t)(gi % kTcpLoSlots) * (2u * kTcABytes);
+        const uint64_t ds = desc0 + (uint64_t)((st * stage_bytes) >> 4);
+        const uint64_t dl = desc0 + (uint64_t)((kTcpStages * stage_bytes + (gi % kTcpLoSlots) * (2u * kTcABytes)) >> 4);
+        if (elect_one()) {
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
-            const uint32_t a_hi = sb + half * kTcABytes, a_lo = lb + half * kTcABytes;
-            const uint32_t b_hi = sb + 2u * kTcABytes + (2 * half) * b_bytes, b_lo = b_hi + b_bytes;
+            const uint64_t a_hi = ds + (half * kTcABytes >> 4), a_lo = dl + (half * kTcABytes >> 4);
+            const uint64_t b_hi = ds + ((2u * kTcABytes) >> 4) + (uint64_t)(2 * half) * (b_bytes >> 4);
+            const uint64_t b_lo = b_hi + (b_bytes >> 4);
             const uint32_t d = dacc + (uint32_t)(half * h);
 #pragma unroll
             for (int kk = 0; kk < kTcBK / 8; ++kk) {
-              const uint64_t ahi = smem_desc(a_hi + kk * 32), alo = smem_desc(a_lo + kk * 32);
-              const uint64_t bhi = smem_desc(b_hi + kk * 32), blo = smem_desc(b_lo + kk * 32);
-              mma_tf32(d, ahi, bhi, idesc, (j > 0 || kk > 0) ? 1u : 0u);
-              mma_tf32(d, ahi, blo, idesc, 1u);
-              mma_tf32(d, alo, bhi, idesc, 1u);
+              mma_tf32(d, a_hi + 2 * kk, b_hi + 2 * kk, idesc, kk > 0 ? 1u : (uint32_t)(j > 0));
+              mma_tf32(d, a_hi + 2 * kk, b_lo + 2 * kk, idesc, 1u);
+              mma_tf32(d, a_lo + 2 * kk, b_hi + 2 * kk, idesc, 1u);
             }
           }
           mma_commit(smem_u32(&bar_empty[st]));
           mma_commit(smem_u32(&bar_lofree[gi % kTcpLoSlots]));  // the remainder slot is free again
+          if (j == nst - 1) mma_commit(smem_u32(&bar_accf[b]));  // arrives once every MMA issued so far has completed
         }
-        mma_commit(smem_u32(&bar_accf[b]));  // arrives once every MMA issued so far has completed
-        last = ti;
+        __syncwarp();
       }
-      // give-up path: a commit after every MMA issued so far (including those of a tile left half done)
-      // arrives once they have all completed; wait for it (full limit) before the accumulators are freed
-      (void)last;
-      if (!ok) {
-        mma_commit(smem_u32(&bar_drain));
-        mbar_wait(smem_u32(&bar_drain), 0, err, 16, kWaitLimit);
-      }
+    }
+    // give-up path: a commit after every MMA issued so far (including those of a tile left half done) arrives once
+    // they have all completed; wait for it (full limit) before the accumulators are freed
+    if (!ok) {
+      if (elect_one()) mma_commit(smem_u32(&bar_drain));
+      mbar_wait(smem_u32(&bar_drain), 0, err, 16, kWaitLimit);
     }
   } else if (warp < 6) {
     // converters: thread t owns row t of every stage's A tiles and of every remainder slot

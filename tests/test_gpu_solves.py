@@ -17,7 +17,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 PR = 0.71
 SIZES = [(2, 3, 5), (4, 2, 3), (16, 16, 16), (31, 33, 32), (64, 65, 31), (100, 63, 36), (129, 40, 50), (17, 130, 66),
-         (33, 20, 255), (256, 34, 48)]
+         (33, 20, 255), (256, 34, 48), (255, 130, 131)]
 
 
 @pytest.fixture(scope="module")
@@ -158,4 +158,38 @@ def test_direct_solves_match_dense_decompositions(fv, shape, prec):
         fv.fv_jvp_project(g, prec, 1e3, -2.0, q, V[i * g.n:(i + 1) * g.n].clone(), one)
         assert float((W[i * g.n:(i + 1) * g.n] - one).norm()) <= (1e-13 if prec == 0 else 1e-5) * float(one.norm())
     assert fv.fv_sync(g) == fv.FV_OK
+    g.close()
+
+
+def test_digit_pass_gives_up_and_recovers(fv):
+    """With a wait limit of 0 the tensor-core passes of an FP64 solve stop and report it; the handle stays usable."""
+    og = D.Grid(64, 66, 65, stretch=1.0, Pr=PR)
+    g = fv.Grid(64, 66, 65, stretch=1.0, Pr=PR)
+    b = _fields(og, 9, np.float64)
+    x = torch.tensor(np.stack(b), dtype=torch.float64, device="cuda").view(-1)
+    out, again = torch.empty_like(x), torch.empty_like(x)
+    fv.fv_diffusion_solve(g, 0, x, out)
+    assert fv.fv_sync(g) == fv.FV_OK
+    fv.fv_set_wait_limit(g, 0)
+    fv.fv_diffusion_solve(g, 0, x, again)
+    assert fv.fv_sync(g) == fv.FV_ETIMEOUT
+    fv.fv_set_wait_limit(g, -1)
+    fv.fv_diffusion_solve(g, 0, x, again)
+    assert fv.fv_sync(g) == fv.FV_OK and torch.equal(out, again)
+    g.close()
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_digit_pass_keeps_non_finite_inputs_visible(fv, bad):
+    og = D.Grid(64, 64, 64, stretch=1.0, Pr=PR)
+    g = fv.Grid(64, 64, 64, stretch=1.0, Pr=PR)
+    x = torch.tensor(np.stack(_fields(og, 9, np.float64)), dtype=torch.float64, device="cuda").view(-1)
+    x[3 * og.nx ** 3 + 777] = bad
+    out = torch.zeros_like(x)
+    fv.fv_diffusion_solve(g, 0, x, out)
+    T = out.view(4, -1)
+    assert not bool(torch.isfinite(T[3]).any()) and bool(torch.isfinite(T[:3]).all())
+    x.zero_()
+    fv.fv_diffusion_solve(g, 0, x, out)
+    assert not bool(out.any())
     g.close()
