@@ -66,6 +66,10 @@ struct Workspace {
   int bcap[2] = {0, 0};
   unsigned bgen = 0;  // bumped whenever the block buffers are reallocated (captured graphs refer to them)
 };
+// Tile (cells) and z-chunk of the flux stencil for blocks of nvec vectors (0: not chosen yet).
+struct FluxPlan {
+  int nvec = 0, tx = 0, ty = 0, zc = 0;
+};
 // Launch shapes picked by the autotuner (0 = the built-in default).
 struct Tune {
   int pair_zc = 0;        // z-planes marched by one CTA of the two-cell J.v stencil
@@ -129,6 +133,7 @@ struct fv_grid_s {
   mutable fv::Profiler prof;
   fv::TcState tc;
   fv::Tune tune;
+  mutable fv::FluxPlan flux[2];  // tiles of the flux stencil: single vectors, blocks
   // batched J.v + projection: the captured launch sequence of the last argument set, replayed while the
   // arguments stay the same, and the private stream it is captured on
   cudaStream_t capture_stream = nullptr;
@@ -150,13 +155,11 @@ namespace fv {
 constexpr long long kDefaultWaitSpins = 1LL << 22;
 inline long long wait_spins(const fv_grid_s* g) { return g->wait_spins < 0 ? kDefaultWaitSpins : g->wait_spins; }
 
-// Planes marched by one CTA of a z-marching stencil over `tiles` (x, y) tiles of nvec states: the chunk with
+// Planes marched by one CTA of an FP32 z-marching stencil over `tiles` (x, y) tiles of nvec states: the chunk with
 // the smallest makespan of the busiest multiprocessor, ceil(CTAs / SMs) CTAs of chunk + 1 plane times each (the
-// extra one stands for a CTA's two halo planes and its pipeline fill).  The stencils are bound by their
-// arithmetic (FP64: two operations per clock and SM; FP32: issue slots), so what counts is how evenly the
-// planes spread over the SMs.  Fixed chunks of 32 planes gave a 32^3 grid 4 CTAs (FP64 J.v 629 us; with this
-// rule 128 CTAs, 26 us), a 64^3 grid 16 (FP32 39.5 -> 8.4 us), and left 100^3 FP64 at 64 planes on the busiest
-// SM where 35 suffice (849 -> 470 us).
+// extra one stands for a CTA's two halo planes and its pipeline fill).  The stencils are bound by issue slots and
+// shared-memory loads, so what counts is how evenly the planes spread over the SMs.  Fixed chunks of 32 planes gave a
+// 64^3 grid 16 CTAs (39.5 us; with this rule 10.7) and a 100^3 grid 208 (41 -> 33 us); 16 vectors of 64^3 66 -> 61.
 int stencil_chunk(const fv_grid_s* g, int tiles, int nvec);
 
 // ------------------------------------------------------------------ error reporting
@@ -213,6 +216,12 @@ int launch_correct(const fv_grid_s* g, const R* Y, const R* phi, double alpha, c
 // v may be null.  No norm.
 template <typename R>
 int launch_correct_block(const fv_grid_s* g, const R* Y, const R* phi, const R* v, double beta, R* out, int nvec);
+
+// FP64 F (MODE 0) and J.v (MODE 1) with every flux computed once (kernels_flux.cu), nvec states one after another in
+// v and out.
+template <int MODE>
+int launch_flux(const fv_grid_s* g, double Gr, double sigma, const double* q, const double* v, double* out,
+                int nvec = 1);
 
 // FP32 J.v with two x-adjacent cells per thread (kernels_stencil2.cu): nx a multiple of 64, ny >= 16,
 // 16-byte aligned q and v (TMA plane ring).

@@ -1,11 +1,6 @@
-// Stencil kernels of the staggered finite-volume discretisation (Section 2, Eqs. 1-6):
-//   residual F(q; Gr), Jacobian-vector product J(q) v, divergence D, and the fused
-//   gradient correction of the projection.
-//
-// One thread per cell (i, j, k) produces the four outputs that live in that cell's slots: the
-// x-face u at x_f[i], the y-face v at y_f[j], the z-face w at z_f[k] and T at the centre.
-// Wall slots (i == 0 for u, ...) are written as zero.  Inputs are read through the read-only
-// path; the neighbour re-reads of a block are served by L1/L2, so DRAM sees each field ~once.
+// Stencil kernels of the staggered finite-volume discretisation (Section 2, Eqs. 1-6): the FP32 Jacobian-vector
+// product J(q) v of any grid (kernels_stencil2.cu has the two-cell form of wide grids, kernels_flux.cu the FP64 F and
+// J.v), divergence D, and the fused gradient correction of the projection.
 #include <cstring>
 
 #include "fv_internal.h"
@@ -26,109 +21,6 @@ __device__ __forceinline__ R ld(const R* __restrict__ a, int o) {
   return __ldg(a + o);
 }
 
-// Momentum component C at the C-face slot p[C] (1 <= p[C] <= n[C]-1).
-//   conv = S(a, b) = div(a b) + div(b a)  (symmetrised convective bilinear form)
-//   lap  = Lap b  (no-slip walls)
-// For d == C the fluxes sit at the cell centres p-1 and p bounding the C-control volume:
-//   (mean a)(mean b) + (mean b)(mean a) = 2 (mean a)(mean b), differenced over the centre spacing.
-// For d != C the fluxes sit on the d-faces p[d] and p[d]+1: the d-velocity interpolated along C to the
-// C-face times the C-velocity interpolated along d to the d-face; zero through a wall.
-template <typename R, int C>
-__device__ __forceinline__ void momentum_terms(const Geo<R>& g, const R* __restrict__ a, const R* __restrict__ b,
-                                               int N, const Cell<R>& c, R& conv, R& lap) {
-  const R* aC = a + C * N;
-  const R* bC = b + C * N;
-  const int pc = c.p[C], nc = g.n[C];
-  const int o = c.o, sC = c.s[C];
-  const R aH = ld(aC, o), bH = ld(bC, o);
-  const R aM = (pc >= 2) ? ld(aC, o - sC) : R(0);
-  const R bM = (pc >= 2) ? ld(bC, o - sC) : R(0);
-  const R aP = (pc + 1 < nc) ? ld(aC, o + sC) : R(0);
-  const R bP = (pc + 1 < nc) ? ld(bC, o + sC) : R(0);
-  const R idcC = g.idc[C][pc];
-  const R aE = R(0.5) * (aH + aP), bE = R(0.5) * (bH + bP);
-  const R aW = R(0.5) * (aM + aH), bW = R(0.5) * (bM + bH);
-  conv = R(2) * (aE * bE - aW * bW) * idcC;
-  lap = ((bP - bH) * g.idx[C][pc] - (bH - bM) * g.idx[C][pc - 1]) * idcC;
-  const R wlC = g.wl[C][pc], wrC = g.wr[C][pc];
-#pragma unroll
-  for (int t = 1; t <= 2; ++t) {
-    const int D = (C + t) % 3;
-    const R* aD = a + D * N;
-    const R* bD = b + D * N;
-    const int pd = c.p[D], nd = g.n[D];
-    const int sD = c.s[D];
-    R fLo = R(0), fHi = R(0), gLo, gHi;
-    if (pd >= 1) {  // lower d-face is interior
-      const R aDc = wlC * ld(aD, o - sC) + wrC * ld(aD, o);
-      const R bDc = wlC * ld(bD, o - sC) + wrC * ld(bD, o);
-      const R bCm = ld(bC, o - sD), aCm = ld(aC, o - sD);
-      const R aCd = g.wl[D][pd] * aCm + g.wr[D][pd] * aH;
-      const R bCd = g.wl[D][pd] * bCm + g.wr[D][pd] * bH;
-      fLo = aDc * bCd + bDc * aCd;
-      gLo = (bH - bCm) * g.idc[D][pd];
-    } else {
-      gLo = bH * g.idc[D][0];
-    }
-    if (pd + 1 <= nd - 1) {  // upper d-face is interior
-      const int oU = o + sD;
-      const R aDc = wlC * ld(aD, oU - sC) + wrC * ld(aD, oU);
-      const R bDc = wlC * ld(bD, oU - sC) + wrC * ld(bD, oU);
-      const R bCp = ld(bC, oU), aCp = ld(aC, oU);
-      const R aCd = g.wl[D][pd + 1] * aH + g.wr[D][pd + 1] * aCp;
-      const R bCd = g.wl[D][pd + 1] * bH + g.wr[D][pd + 1] * bCp;
-      fHi = aDc * bCd + bDc * aCd;
-      gHi = (bCp - bH) * g.idc[D][pd + 1];
-    } else {
-      gHi = -bH * g.idc[D][nd];
-    }
-    const R ixD = g.idx[D][pd];
-    conv += (fHi - fLo) * ixD;
-    lap += (gHi - gLo) * ixD;
-  }
-}
-
-// Temperature at the cell: conv = div(a_vel T_b) + div(b_vel T_a); lap = Lap T_b with T = T_hot at
-// x = 0 and 0 at x = 1 (Eq. 4), zero flux through the y and z walls (Eqs. 5-6).
-template <typename R>
-__device__ __forceinline__ void temperature_terms(const Geo<R>& g, const R* __restrict__ a, const R* __restrict__ b,
-                                                  int N, const Cell<R>& c, R T_hot, R& conv, R& lap) {
-  const R* Ta = a + 3 * N;
-  const R* Tb = b + 3 * N;
-  const int o = c.o;
-  const R TaH = ld(Ta, o), TbH = ld(Tb, o);
-  conv = R(0);
-  lap = R(0);
-#pragma unroll
-  for (int D = 0; D < 3; ++D) {
-    const R* aD = a + D * N;
-    const R* bD = b + D * N;
-    const int pd = c.p[D], nd = g.n[D];
-    const int sD = c.s[D];
-    R fLo = R(0), fHi = R(0), gLo = R(0), gHi = R(0);
-    if (pd >= 1) {
-      const R Tam = ld(Ta, o - sD), Tbm = ld(Tb, o - sD);
-      const R wl = g.wl[D][pd], wr = g.wr[D][pd];
-      fLo = ld(aD, o) * (wl * Tbm + wr * TbH) + ld(bD, o) * (wl * Tam + wr * TaH);
-      gLo = (TbH - Tbm) * g.idc[D][pd];
-    } else if (D == 0) {
-      gLo = (TbH - T_hot) * g.idc[0][0];
-    }
-    if (pd + 1 <= nd - 1) {
-      const int oU = o + sD;
-      const R Tap = ld(Ta, oU), Tbp = ld(Tb, oU);
-      const R wl = g.wl[D][pd + 1], wr = g.wr[D][pd + 1];
-      fHi = ld(aD, oU) * (wl * TbH + wr * Tbp) + ld(bD, oU) * (wl * TaH + wr * Tap);
-      gHi = (Tbp - TbH) * g.idc[D][pd + 1];
-    } else if (D == 0) {
-      gHi = -TbH * g.idc[0][nd];
-    }
-    const R ixD = g.idx[D][pd];
-    conv += (fHi - fLo) * ixD;
-    lap += (gHi - gLo) * ixD;
-  }
-}
-
 template <typename R>
 __device__ __forceinline__ bool cell_of_thread(const Geo<R>& g, Cell<R>& c) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -145,55 +37,8 @@ __device__ __forceinline__ bool cell_of_thread(const Geo<R>& g, Cell<R>& c) {
   return true;
 }
 
-// mode 0: residual  out = -S(q,q)/2 + Lap q (+ Dirichlet data) + Gr T_q e_z
-// mode 1: J.v       out = -S(q,v) + Lap v + Gr T_v e_z - sigma v
-template <typename R, int MODE>
-__global__ void __launch_bounds__(256) k_stencil(Geo<R> g, int N, R Gr, R invPr, R sigma,
-                                                  const R* __restrict__ q, const R* __restrict__ v,
-                                                  R* __restrict__ out) {
-  Cell<R> c;
-  if (!cell_of_thread(g, c)) return;
-  const R* b = (MODE == 0) ? q : v;
-  const R half = (MODE == 0) ? R(0.5) : R(1);
-  R conv, lap;
-  // u
-  if (c.p[0] >= 1) {
-    momentum_terms<R, 0>(g, q, b, N, c, conv, lap);
-    R r = lap - half * conv;
-    if (MODE == 1) r -= sigma * ld(v, c.o);
-    out[c.o] = r;
-  } else {
-    out[c.o] = R(0);
-  }
-  // v
-  if (c.p[1] >= 1) {
-    momentum_terms<R, 1>(g, q, b, N, c, conv, lap);
-    R r = lap - half * conv;
-    if (MODE == 1) r -= sigma * ld(v, N + c.o);
-    out[N + c.o] = r;
-  } else {
-    out[N + c.o] = R(0);
-  }
-  // w (+ buoyancy Gr T interpolated to the z-face)
-  if (c.p[2] >= 1) {
-    momentum_terms<R, 2>(g, q, b, N, c, conv, lap);
-    const R* Tb = b + 3 * N;
-    const R Tf = g.wl[2][c.p[2]] * ld(Tb, c.o - c.s[2]) + g.wr[2][c.p[2]] * ld(Tb, c.o);
-    R r = lap - half * conv + Gr * Tf;
-    if (MODE == 1) r -= sigma * ld(v, 2 * N + c.o);
-    out[2 * N + c.o] = r;
-  } else {
-    out[2 * N + c.o] = R(0);
-  }
-  // T
-  temperature_terms<R>(g, q, b, N, c, (MODE == 0) ? R(1) : R(0), conv, lap);
-  R r = lap * invPr - half * conv;
-  if (MODE == 1) r -= sigma * ld(v, 3 * N + c.o);
-  out[3 * N + c.o] = r;
-}
-
 // ------------------------------------------------------------------------------------------------
-// z-marching variant.  A block owns a 32 x 8 (x, y) tile of cells and marches over a chunk of zc planes
+// z-marching J.v.  A block owns a 32 x 8 (x, y) tile of cells and marches over a chunk of zc planes
 // (stencil_chunk).  For every input array it keeps the planes k-1, k, k+1 of the tile plus a one-cell x/y halo in
 // a 4-slot shared-memory ring (slot = plane mod 4); cp.async copies of plane k+2 fly while plane k is
 // computed.  Each input element is read from global memory ~1.3 times (halo) instead of ~7 times
@@ -247,23 +92,20 @@ __device__ __forceinline__ const AxM<R>& axm(const AxM<R>& x, const AxM<R>& y, c
   return D == 0 ? x : (D == 1 ? y : z);
 }
 
-// Same mathematics as momentum_terms / temperature_terms, reading neighbours from the ring.
-// Arrays 0..3 are the advecting state a, arrays AB..AB+3 the advected field b (AB = 0 for F, 4 for J.v).
-// GHOST (J.v, homogeneous wall data): the wall cases need no branches, because the general formulas give
-// them when they read zeros there: the face-normal wall slot 0 holds zero, everything outside the domain
-// arrives zero-filled in the ring, and the metric arrays hold the wall values (idc[0] = 2 / dx_0,
-// idc[n] = 2 / dx_{n-1}, wl = wr = 0 on the wall faces).  Only T's zero-flux walls (y, z) keep theirs.
-template <typename R, int C, int NA, int AB, bool GHOST>
-__device__ __forceinline__ void momentum_ring(const Geo<R>& g, const Ring<R, NA>& S, const int p[3], const AxM<R>& mx,
-                                              const AxM<R>& my, const AxM<R>& mz, R& conv, R& lap) {
+// Momentum component C: conv = S(q, v) = div(q v) + div(v q) (symmetrised convective form), lap = Lap v; temperature
+// likewise.  Arrays 0..3 are the advecting state a = q, arrays AB..AB+3 the advected field b = v.  The wall cases
+// need no branches, because the general formulas give them when they read zeros there: the face-normal wall slot 0
+// holds zero, everything outside the domain arrives zero-filled in the ring, and the metric arrays hold the wall
+// values (idc[0] = 2 / dx_0, idc[n] = 2 / dx_{n-1}, wl = wr = 0 on the wall faces).  Only T's zero-flux walls (y, z)
+// keep theirs.
+template <typename R, int C, int NA, int AB>
+__device__ __forceinline__ void momentum_ring(const Ring<R, NA>& S, const AxM<R>& mx, const AxM<R>& my,
+                                              const AxM<R>& mz, R& conv, R& lap) {
   constexpr int cx = unit(C, 0), cy = unit(C, 1), cz = unit(C, 2);
   const AxM<R>& MC = axm<C>(mx, my, mz);
-  const int pc = p[C], nc = g.n[C];
   const R aH = S.at(C, 0, 0, 0), bH = S.at(AB + C, 0, 0, 0);
-  const R aM = (GHOST || pc >= 2) ? S.at(C, -cx, -cy, -cz) : R(0);
-  const R bM = (GHOST || pc >= 2) ? S.at(AB + C, -cx, -cy, -cz) : R(0);
-  const R aP = (GHOST || pc + 1 < nc) ? S.at(C, cx, cy, cz) : R(0);
-  const R bP = (GHOST || pc + 1 < nc) ? S.at(AB + C, cx, cy, cz) : R(0);
+  const R aM = S.at(C, -cx, -cy, -cz), bM = S.at(AB + C, -cx, -cy, -cz);
+  const R aP = S.at(C, cx, cy, cz), bP = S.at(AB + C, cx, cy, cz);
   const R aE = R(0.5) * (aH + aP), bE = R(0.5) * (bH + bP);
   const R aW = R(0.5) * (aM + aH), bW = R(0.5) * (bM + bH);
   conv = R(2) * (aE * bE - aW * bW) * MC.ic;
@@ -274,9 +116,8 @@ __device__ __forceinline__ void momentum_ring(const Geo<R>& g, const Ring<R, NA>
     const int D = (C + t) % 3;
     const AxM<R>& MD = (D == 0) ? mx : (D == 1 ? my : mz);
     const int dx = unit(D, 0), dy = unit(D, 1), dz = unit(D, 2);
-    const int pd = p[D], nd = g.n[D];
-    R fLo = R(0), fHi = R(0), gLo, gHi;
-    if (GHOST || pd >= 1) {
+    R fLo, fHi, gLo, gHi;
+    {
       const R aDc = wlC * S.at(D, -cx, -cy, -cz) + wrC * S.at(D, 0, 0, 0);
       const R bDc = wlC * S.at(AB + D, -cx, -cy, -cz) + wrC * S.at(AB + D, 0, 0, 0);
       const R bCm = S.at(AB + C, -dx, -dy, -dz), aCm = S.at(C, -dx, -dy, -dz);
@@ -284,10 +125,8 @@ __device__ __forceinline__ void momentum_ring(const Geo<R>& g, const Ring<R, NA>
       const R bCd = MD.wl * bCm + MD.wr * bH;
       fLo = aDc * bCd + bDc * aCd;
       gLo = (bH - bCm) * MD.ic;
-    } else {
-      gLo = bH * MD.ic0;
     }
-    if (GHOST || pd + 1 <= nd - 1) {
+    {
       const R aDc = wlC * S.at(D, dx - cx, dy - cy, dz - cz) + wrC * S.at(D, dx, dy, dz);
       const R bDc = wlC * S.at(AB + D, dx - cx, dy - cy, dz - cz) + wrC * S.at(AB + D, dx, dy, dz);
       const R bCp = S.at(AB + C, dx, dy, dz), aCp = S.at(C, dx, dy, dz);
@@ -295,18 +134,16 @@ __device__ __forceinline__ void momentum_ring(const Geo<R>& g, const Ring<R, NA>
       const R bCd = MD.wlp * bH + MD.wrp * bCp;
       fHi = aDc * bCd + bDc * aCd;
       gHi = (bCp - bH) * MD.icp;
-    } else {
-      gHi = -bH * MD.icn;
     }
     conv += (fHi - fLo) * MD.ix;
     lap += (gHi - gLo) * MD.ix;
   }
 }
 
-template <typename R, int NA, int AB, bool GHOST>
+template <typename R, int NA, int AB>
 __device__ __forceinline__ void temperature_ring(const Geo<R>& g, const Ring<R, NA>& S, const int p[3],
-                                                 const AxM<R>& mx, const AxM<R>& my, const AxM<R>& mz, R T_hot,
-                                                 R& conv, R& lap) {
+                                                 const AxM<R>& mx, const AxM<R>& my, const AxM<R>& mz, R& conv,
+                                                 R& lap) {
   const R TaH = S.at(3, 0, 0, 0), TbH = S.at(AB + 3, 0, 0, 0);
   conv = R(0);
   lap = R(0);
@@ -315,32 +152,14 @@ __device__ __forceinline__ void temperature_ring(const Geo<R>& g, const Ring<R, 
     const AxM<R>& MD = (D == 0) ? mx : (D == 1 ? my : mz);
     const int dx = unit(D, 0), dy = unit(D, 1), dz = unit(D, 2);
     const int pd = p[D], nd = g.n[D];
-    R fLo = R(0), fHi = R(0), gLo = R(0), gHi = R(0);
-    if constexpr (GHOST) {  // one basic block: x Dirichlet T = 0 by the ghost zero, y / z zero flux by a select
-      const R Tam = S.at(3, -dx, -dy, -dz), Tbm = S.at(AB + 3, -dx, -dy, -dz);
-      fLo = S.at(D, 0, 0, 0) * (MD.wl * Tbm + MD.wr * TbH) + S.at(AB + D, 0, 0, 0) * (MD.wl * Tam + MD.wr * TaH);
-      gLo = (D == 0 || pd >= 1) ? (TbH - Tbm) * MD.ic : R(0);
-      const R Tap = S.at(3, dx, dy, dz), Tbp = S.at(AB + 3, dx, dy, dz);
-      fHi = S.at(D, dx, dy, dz) * (MD.wlp * TbH + MD.wrp * Tbp) +
-            S.at(AB + D, dx, dy, dz) * (MD.wlp * TaH + MD.wrp * Tap);
-      gHi = (D == 0 || pd + 1 <= nd - 1) ? (Tbp - TbH) * MD.icp : R(0);
-    } else if (pd >= 1) {
-      const R Tam = S.at(3, -dx, -dy, -dz), Tbm = S.at(AB + 3, -dx, -dy, -dz);
-      fLo = S.at(D, 0, 0, 0) * (MD.wl * Tbm + MD.wr * TbH) + S.at(AB + D, 0, 0, 0) * (MD.wl * Tam + MD.wr * TaH);
-      gLo = (TbH - Tbm) * MD.ic;
-    } else if (D == 0) {
-      gLo = (TbH - T_hot) * MD.ic0;
-    }
-    if constexpr (!GHOST) {
-      if (pd + 1 <= nd - 1) {
-        const R Tap = S.at(3, dx, dy, dz), Tbp = S.at(AB + 3, dx, dy, dz);
-        fHi = S.at(D, dx, dy, dz) * (MD.wlp * TbH + MD.wrp * Tbp) +
-              S.at(AB + D, dx, dy, dz) * (MD.wlp * TaH + MD.wrp * Tap);
-        gHi = (Tbp - TbH) * MD.icp;
-      } else if (D == 0) {
-        gHi = -TbH * MD.icn;
-      }
-    }
+    // x Dirichlet T = 0 by the ghost zero, y / z zero flux by a select
+    const R Tam = S.at(3, -dx, -dy, -dz), Tbm = S.at(AB + 3, -dx, -dy, -dz);
+    const R fLo = S.at(D, 0, 0, 0) * (MD.wl * Tbm + MD.wr * TbH) + S.at(AB + D, 0, 0, 0) * (MD.wl * Tam + MD.wr * TaH);
+    const R gLo = (D == 0 || pd >= 1) ? (TbH - Tbm) * MD.ic : R(0);
+    const R Tap = S.at(3, dx, dy, dz), Tbp = S.at(AB + 3, dx, dy, dz);
+    const R fHi = S.at(D, dx, dy, dz) * (MD.wlp * TbH + MD.wrp * Tbp) +
+                  S.at(AB + D, dx, dy, dz) * (MD.wlp * TaH + MD.wrp * Tap);
+    const R gHi = (D == 0 || pd + 1 <= nd - 1) ? (Tbp - TbH) * MD.icp : R(0);
     conv += (fHi - fLo) * MD.ix;
     lap += (gHi - gLo) * MD.ix;
   }
@@ -385,15 +204,14 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, int* err
   return false;
 }
 
-// MODE 0: residual (arrays: q), MODE 1: J.v (arrays: q then v).  use_tma: plane tiles arrive by one 4D TMA
-// box per state (x, y, z, field) with zero fill outside the domain; otherwise by per-element cp.async.
-template <typename R, int MODE>
-__global__ void __launch_bounds__(kTX * kTY, sizeof(R) == 4 ? 3 : 2)
+// Arrays: q then v.  use_tma: plane tiles arrive by one 4D TMA box per state (x, y, z, field) with zero fill outside
+// the domain; otherwise by per-element cp.async.
+template <typename R>
+__global__ void __launch_bounds__(kTX * kTY, 3)
     k_stencil_z(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmv, int use_tma,
                 int* err, long long spins, Geo<R> g, int N, R Gr, R invPr, R sigma, const R* __restrict__ q, const R* __restrict__ v,
                 R* __restrict__ out, int zc, int nch) {
-  constexpr int NA = (MODE == 0) ? 4 : 8;
-  constexpr int AB = (MODE == 0) ? 0 : 4;
+  constexpr int NA = 8, AB = 4;
   constexpr int NWARP = kTX * kTY / 32;
   constexpr uint32_t kBox = 4u * kPL * sizeof(R);  // one state's box: 4 fields x kHY x kPW
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -431,8 +249,7 @@ __global__ void __launch_bounds__(kTX * kTY, sizeof(R) == 4 ? 3 : 2)
               "%5, %6}], [%2];" ::"r"(smem_addr(slot)),
               "l"(reinterpret_cast<uint64_t>(&tmq)), "r"(b), "r"(i0 - kX0), "r"(j0 - 1), "r"(kk), "r"(0)
               : "memory");
-          if (NA == 8)
-            asm volatile(
+          asm volatile(
                 "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, "
                 "%4, %5, %6}], [%2];" ::"r"(smem_addr(slot + 4 * kPL)),
                 "l"(reinterpret_cast<uint64_t>(&tmv)), "r"(b), "r"(i0 - kX0), "r"(j0 - 1), "r"(kk), "r"(4 * vec)
@@ -477,7 +294,6 @@ __global__ void __launch_bounds__(kTX * kTY, sizeof(R) == 4 ? 3 : 2)
   ok = __syncthreads_and(ok);  // one decision for the whole CTA
   const int i = i0 + tx, j = j0 + ty;
   const bool active = (i < nx && j < ny);
-  const R half = (MODE == 0) ? R(0.5) : R(1);
   const AxM<R> mx = load_axm(g, 0, active ? i : 0), my = load_axm(g, 1, active ? j : 0);
   for (int k = k0; k < kend && ok; ++k) {
     if (k + 2 <= kend) {  // plane k+2 feeds the output plane k+1
@@ -494,53 +310,21 @@ __global__ void __launch_bounds__(kTX * kTY, sizeof(R) == 4 ? 3 : 2)
       const int p[3] = {i, j, k};
       const int o = (k * ny + j) * nx + i;
       R conv, lap;
-      if constexpr (MODE == 1) {
-        // J.v: all four equations in one basic block (the wall outputs by selects), so that the compiler
-        // can share the ring loads between them
-        momentum_ring<R, 0, NA, AB, true>(g, S, p, mx, my, mz, conv, lap);
-        const R r0 = lap - conv - sigma * S.at(AB + 0, 0, 0, 0);
-        momentum_ring<R, 1, NA, AB, true>(g, S, p, mx, my, mz, conv, lap);
-        const R r1 = lap - conv - sigma * S.at(AB + 1, 0, 0, 0);
-        momentum_ring<R, 2, NA, AB, true>(g, S, p, mx, my, mz, conv, lap);
-        const R Tf = mz.wl * S.at(AB + 3, 0, 0, -1) + mz.wr * S.at(AB + 3, 0, 0, 0);
-        const R r2 = lap - conv + Gr * Tf - sigma * S.at(AB + 2, 0, 0, 0);
-        temperature_ring<R, NA, AB, true>(g, S, p, mx, my, mz, R(0), conv, lap);
-        const R r3 = lap * invPr - conv - sigma * S.at(AB + 3, 0, 0, 0);
-        out[o] = (i >= 1) ? r0 : R(0);
-        out[N + o] = (j >= 1) ? r1 : R(0);
-        out[2 * N + o] = (k >= 1) ? r2 : R(0);
-        out[3 * N + o] = r3;
-      } else {
-        if (i >= 1) {
-          momentum_ring<R, 0, NA, AB, MODE == 1>(g, S, p, mx, my, mz, conv, lap);
-          R r = lap - half * conv;
-          if (MODE == 1) r -= sigma * S.at(AB + 0, 0, 0, 0);
-          out[o] = r;
-        } else {
-          out[o] = R(0);
-        }
-        if (j >= 1) {
-          momentum_ring<R, 1, NA, AB, MODE == 1>(g, S, p, mx, my, mz, conv, lap);
-          R r = lap - half * conv;
-          if (MODE == 1) r -= sigma * S.at(AB + 1, 0, 0, 0);
-          out[N + o] = r;
-        } else {
-          out[N + o] = R(0);
-        }
-        if (k >= 1) {
-          momentum_ring<R, 2, NA, AB, MODE == 1>(g, S, p, mx, my, mz, conv, lap);
-          const R Tf = mz.wl * S.at(AB + 3, 0, 0, -1) + mz.wr * S.at(AB + 3, 0, 0, 0);
-          R r = lap - half * conv + Gr * Tf;
-          if (MODE == 1) r -= sigma * S.at(AB + 2, 0, 0, 0);
-          out[2 * N + o] = r;
-        } else {
-          out[2 * N + o] = R(0);
-        }
-        temperature_ring<R, NA, AB, MODE == 1>(g, S, p, mx, my, mz, (MODE == 0) ? R(1) : R(0), conv, lap);
-        R r = lap * invPr - half * conv;
-        if (MODE == 1) r -= sigma * S.at(AB + 3, 0, 0, 0);
-        out[3 * N + o] = r;
-      }
+      // all four equations in one basic block (the wall outputs by selects), so that the compiler can share the
+      // ring loads between them
+      momentum_ring<R, 0, NA, AB>(S, mx, my, mz, conv, lap);
+      const R r0 = lap - conv - sigma * S.at(AB + 0, 0, 0, 0);
+      momentum_ring<R, 1, NA, AB>(S, mx, my, mz, conv, lap);
+      const R r1 = lap - conv - sigma * S.at(AB + 1, 0, 0, 0);
+      momentum_ring<R, 2, NA, AB>(S, mx, my, mz, conv, lap);
+      const R Tf = mz.wl * S.at(AB + 3, 0, 0, -1) + mz.wr * S.at(AB + 3, 0, 0, 0);
+      const R r2 = lap - conv + Gr * Tf - sigma * S.at(AB + 2, 0, 0, 0);
+      temperature_ring<R, NA, AB>(g, S, p, mx, my, mz, conv, lap);
+      const R r3 = lap * invPr - conv - sigma * S.at(AB + 3, 0, 0, 0);
+      out[o] = (i >= 1) ? r0 : R(0);
+      out[N + o] = (j >= 1) ? r1 : R(0);
+      out[2 * N + o] = (k >= 1) ? r2 : R(0);
+      out[3 * N + o] = r3;
     }
     if (!use_tma) cp_async_wait_all();  // plane k+2 has landed
     ok = __syncthreads_and(ready);      // nobody reads the slot of plane k-1 any more; stop together
@@ -852,13 +636,13 @@ int state_map(const fv_grid_s* g, const R* ptr, CUtensorMap* m, int nvec = 1) {
                            ptr, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
-template <typename R, int MODE>
+template <typename R>
 int launch_stencil_z(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out, int nvec = 1) {
-  constexpr int NA = (MODE == 0) ? 4 : 8;
+  constexpr int NA = 8;
   const size_t smem = (size_t)NA * kRing * kPL * sizeof(R);
   static bool attr_set = false;
   if (!attr_set) {
-    FV_CUDA(cudaFuncSetAttribute(k_stencil_z<R, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    FV_CUDA(cudaFuncSetAttribute(k_stencil_z<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     attr_set = true;
   }
   // TMA needs 16-byte aligned rows and base addresses; small grids take the cp.async path
@@ -876,20 +660,25 @@ int launch_stencil_z(const fv_grid_s* g, double Gr, double sigma, const R* q, co
   }
   dim3 grid(gx, gy, nch * nvec);
   ProfScope ps(g, PROF_STENCIL);
-  k_stencil_z<R, MODE><<<grid, kTX * kTY, smem, g->stream>>>(tq, tv, use_tma, g->ws.err, wait_spins(g), geo_of<R>(g), (int)g->N,
+  k_stencil_z<R><<<grid, kTX * kTY, smem, g->stream>>>(tq, tv, use_tma, g->ws.err, wait_spins(g), geo_of<R>(g), (int)g->N,
                                                              (R)Gr, (R)(1.0 / g->Pr), (R)sigma, q, v, out, zc, nch);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }
 
+// FP64 by the flux form (kernels_flux.cu), whose operation count bounds it; FP32 by the forms below it measured
+// against: 256^3 two cells per thread 206 us, flux form 334; 100^3 one cell 33, flux 46; 64^3 10.8 / 16.6
 template <typename R>
 int launch_residual(const fv_grid_s* g, double Gr, const R* q, R* F) {
-  return launch_stencil_z<R, 0>(g, Gr, 0.0, q, q, F);
+  return launch_flux<0>(g, Gr, 0.0, q, q, F);
 }
 
 template <typename R>
 int launch_jvp_block(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out, int nvec) {
-  return launch_stencil_z<R, 1>(g, Gr, sigma, q, v, out, nvec);
+  if constexpr (sizeof(R) == 8)
+    return launch_flux<1>(g, Gr, sigma, q, v, out, nvec);
+  else
+    return launch_stencil_z<R>(g, Gr, sigma, q, v, out, nvec);
 }
 
 template <typename R>
@@ -897,7 +686,7 @@ int launch_jvp(const fv_grid_s* g, double Gr, double sigma, const R* q, const R*
   if constexpr (sizeof(R) == 4) {  // two cells per thread (kernels_stencil2.cu) where its tiles fit
     if (stencil_pair_eligible(g, q, v)) return launch_stencil_pair(g, Gr, sigma, q, v, out);
   }
-  return launch_stencil_z<R, 1>(g, Gr, sigma, q, v, out);
+  return launch_jvp_block<R>(g, Gr, sigma, q, v, out, 1);
 }
 
 template <typename R>
