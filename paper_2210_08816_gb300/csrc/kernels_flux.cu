@@ -403,9 +403,8 @@ int launch_flux(const fv_grid_s* g, double Gr, double sigma, const double* q, co
   t.pw = tile_width(pl.tx);
   t.err = g->ws.err;
   t.spins = wait_spins(g);
-  // TMA: rows and bases on 16-byte boundaries, boxes no larger than the grid
-  t.use_tma = (g->nx * sizeof(R)) % 16 == 0 && t.pw <= g->nx && t.ty + 2 <= g->ny && (uintptr_t)q % 16 == 0 &&
-              (uintptr_t)v % 16 == 0;
+  // TMA: rows and bases on 16-byte boundaries
+  t.use_tma = (g->nx * sizeof(R)) % 16 == 0 && (uintptr_t)q % 16 == 0 && (uintptr_t)v % 16 == 0;
   t.pl = (pl.ty + 2) * t.pw;
   CUtensorMap tq, tv;
   std::memset(&tq, 0, sizeof(tq));
