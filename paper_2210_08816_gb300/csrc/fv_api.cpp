@@ -1030,8 +1030,7 @@ int fv_batch_plan_destroy(fv_batch_plan plan) {
 
 int fv_diagnostics(fv_grid g, const double* q, double* ekin, double* nu) {
   if (!g || !q) return invalid("null argument");
-  FV_TRY(launch_ekin(g, q, 0));
-  FV_TRY(launch_nusselt(g, q, 1));
+  FV_TRY(launch_diagnostics(g, q, 0));
   double v[2];
   FV_TRY(read_scalars(g, 0, 2, v));
   if (ekin) *ekin = v[0];
@@ -1049,8 +1048,7 @@ int fv_time_step(fv_grid g, double Gr, double dt, int nsteps, double* q, double*
   Vec<double> V{g, n};
   auto record = [&](int i) -> int {
     if (!ekin && !nu) return FV_OK;
-    FV_TRY(launch_ekin(g, q, 0));
-    FV_TRY(launch_nusselt(g, q, 1));
+    FV_TRY(launch_diagnostics(g, q, 0));
     double v[2];
     FV_TRY(read_scalars(g, 0, 2, v));
     if (ekin) ekin[i] = v[0];

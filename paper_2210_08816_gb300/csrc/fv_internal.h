@@ -234,10 +234,9 @@ int launch_stencil_pair(const fv_grid_s* g, double Gr, double sigma, const float
 // of Eqs. 4-6 (kernels_prolong.cu); runs on gf's stream.  Not projected.
 int launch_prolong(const fv_grid_s* gc, const double* qc, const fv_grid_s* gf, double* qf);
 
-// Diagnostics of Section 4.2.3 (kernels_diag.cu), FP64 state q: E_kin (Eq. 12) and the hot-wall Nusselt
-// number (Eq. 13) into g->ws.scalars[slot].
-int launch_ekin(const fv_grid_s* g, const double* q, int slot);
-int launch_nusselt(const fv_grid_s* g, const double* q, int slot);
+// Diagnostics of Section 4.2.3 (kernels_diag.cu), FP64 state q: E_kin (Eq. 12) into g->ws.scalars[slot] and the
+// hot-wall Nusselt number (Eq. 13) into g->ws.scalars[slot + 1].
+int launch_diagnostics(const fv_grid_s* g, const double* q, int slot);
 
 // Fast-diagonalisation Poisson solve (kernels_fdm.cu): phi = (DG)^+ rhs; rhs and phi may alias.
 template <typename R>

@@ -8,6 +8,8 @@
 // Both use the metric arrays of the handle (idc[d][f] = 1 / centre spacing, idc[d][0] = 2 / dx_0,
 // idx[d][c] = 1 / width) and the library's deterministic two-pass reduction (fixed block partials, then
 // their sum in a fixed order).  The wall slot of a face-normal velocity holds 0 and adds nothing.
+#include <algorithm>
+
 #include "fv_internal.h"
 
 namespace fv {
@@ -35,66 +37,69 @@ __device__ __forceinline__ double block_sum(double v) {
   return r;
 }
 
-// partial sums of u_f^2 V_f over the three velocity fields (3 N elements), one chunk per block
-__global__ void __launch_bounds__(kThreads) k_ekin_partial(Geo<double> g, const double* __restrict__ q,
+// Blocks 0 .. be - 1: partial sums of u_f^2 V_f / 2 over the x-rows of the three velocity fields, a warp per row.  The
+// two x-factors of the control volumes (centre spacings and widths: one over the metrics) are formed once per block,
+// the factors across once per row, so that a face costs two FP64 operations; with a division and four products per
+// face the sum was bound by the FP64 pipe.  The other blocks: partial sums of the hot-wall flux over the ny * nz wall
+// cells.  (64^3, both diagnostics with their sums: four launches, 77 us of kernels; now two.)
+__global__ void __launch_bounds__(kThreads) k_diag_partial(Geo<double> g, const double* __restrict__ q, int be,
                                                             double* __restrict__ part) {
-  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-  const long long N = (long long)nx * ny * nz, n3 = 3 * N;
-  const long long L = (n3 + gridDim.x - 1) / gridDim.x;
-  const long long s = (long long)blockIdx.x * L, e = s + L < n3 ? s + L : n3;
+  __shared__ double vol[2][kMaxN];
+  const int nx = g.n[0], ny = g.n[1], rows = g.n[1] * g.n[2];
   double acc = 0.0;
-  for (long long t = s + threadIdx.x; t < e; t += kThreads) {
-    const int c = (int)(t / N);
-    const long long o = t - (long long)c * N;
-    const int i = (int)(o % nx), j = (int)((o / nx) % ny), k = (int)(o / ((long long)nx * ny));
-    const int p[3] = {i, j, k};
-    // control volume: centre spacing along the own axis (face p), widths across
-    double inv = g.idc[c][p[c]];
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-      if (d != c) inv *= g.idx[d][p[d]];
-    const double u = q[t];
-    acc += 0.5 * u * u / inv;
+  if ((int)blockIdx.x < be) {
+    for (int x = threadIdx.x; x < nx; x += kThreads) {
+      vol[0][x] = 1.0 / g.idc[0][x];
+      vol[1][x] = 1.0 / g.idx[0][x];
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int r = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); r < 3 * rows; r += be * (kThreads / 32)) {
+      const int c = r / rows, jk = r - c * rows, k = jk / ny, j = jk - k * ny;
+      const double* __restrict__ f = q + (size_t)r * nx;
+      const double* v = vol[c == 0 ? 0 : 1];
+      double sum = 0.0;
+      for (int x = lane; x < nx; x += 32) {
+        const double u = f[x];
+        sum = fma(u * u, v[x], sum);
+      }
+      acc += 0.5 * sum / ((c == 1 ? g.idc[1][j] : g.idx[1][j]) * (c == 2 ? g.idc[2][k] : g.idx[2][k]));
+    }
+  } else {
+    const double* T = q + 3 * (size_t)rows * nx;
+    const int bn = gridDim.x - be;
+    for (int t = (blockIdx.x - be) * kThreads + threadIdx.x; t < rows; t += bn * kThreads) {
+      const int k = t / ny, j = t - k * ny;
+      const double grad = (T[(size_t)t * nx] - 1.0) * g.idc[0][0];  // over the half cell dx_0 / 2
+      acc += grad / (g.idx[1][j] * g.idx[2][k]);
+    }
   }
   const double r = block_sum(acc);
   if (threadIdx.x == 0) part[blockIdx.x] = r;
 }
 
-// partial sums of the hot-wall flux over the ny * nz wall cells
-__global__ void __launch_bounds__(kThreads) k_nusselt_partial(Geo<double> g, const double* __restrict__ q,
-                                                               double* __restrict__ part) {
-  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-  const long long N = (long long)nx * ny * nz, nw = (long long)ny * nz;
-  const long long L = (nw + gridDim.x - 1) / gridDim.x;
-  const long long s = (long long)blockIdx.x * L, e = s + L < nw ? s + L : nw;
-  const double* T = q + 3 * N;
-  double acc = 0.0;
-  for (long long t = s + threadIdx.x; t < e; t += kThreads) {
-    const int j = (int)(t % ny), k = (int)(t / ny);
-    const double grad = (T[((long long)k * ny + j) * nx] - 1.0) * g.idc[0][0];  // over the half cell dx_0 / 2
-    acc += grad / (g.idx[1][j] * g.idx[2][k]);
-  }
-  const double r = block_sum(acc);
-  if (threadIdx.x == 0) part[blockIdx.x] = r;
+// out[0] = sum of part[0 .. be), out[1] = sum of part[be .. be + bn), in a fixed order
+__global__ void __launch_bounds__(kThreads) k_diag_finish(const double* __restrict__ part, int be, int bn,
+                                                           double* __restrict__ out) {
+  const double* p = part + (blockIdx.x == 0 ? 0 : be);
+  const int n = blockIdx.x == 0 ? be : bn;
+  double v = 0.0;
+  for (int t = threadIdx.x; t < n; t += kThreads) v += p[t];
+  const double r = block_sum(v);
+  if (threadIdx.x == 0) out[blockIdx.x] = r;
 }
 
 }  // namespace
 
-int launch_ekin(const fv_grid_s* g, const double* q, int slot) {
+// E_kin into scalars[slot], Nu into scalars[slot + 1]: one launch for the partials of both, one for the sums
+int launch_diagnostics(const fv_grid_s* g, const double* q, int slot) {
   ProfScope ps(g, PROF_REDUCE);
-  k_ekin_partial<<<kReduceBlocks, kThreads, 0, g->stream>>>(g->geo64, q, g->ws.partials);
+  const int be = std::min(kReduceBlocks, (3 * g->ny * g->nz + 31) / 32);  // four rows per warp
+  const int bn = std::min(kReduceBlocks, (g->ny * g->nz + kThreads - 1) / kThreads);
+  k_diag_partial<<<be + bn, kThreads, 0, g->stream>>>(g->geo64, q, be, g->ws.partials);
   FV_CUDA(cudaGetLastError());
-  FV_TRY(launch_sum_partials(g, kReduceBlocks, slot));
-  return FV_OK;
-}
-
-int launch_nusselt(const fv_grid_s* g, const double* q, int slot) {
-  ProfScope ps(g, PROF_REDUCE);
-  const long long nw = (long long)g->ny * g->nz;
-  const int blocks = (int)std::min<long long>(kReduceBlocks, (nw + kThreads - 1) / kThreads);
-  k_nusselt_partial<<<blocks, kThreads, 0, g->stream>>>(g->geo64, q, g->ws.partials);
+  k_diag_finish<<<2, kThreads, 0, g->stream>>>(g->ws.partials, be, bn, g->ws.scalars + slot);
   FV_CUDA(cudaGetLastError());
-  FV_TRY(launch_sum_partials(g, blocks, slot));
   return FV_OK;
 }
 
