@@ -169,8 +169,10 @@ static int upload_digits(fv_grid_s* g, const HalfOpHost (*half)[3]) {
             continue;
           }
           const HalfOpHost& o = half[d][kind];
-          build_digits(dir ? o.E : o.F, (o.n + 1) / 2, prec ? kDigits32 : kDigits64, prec ? kDigitCols32 : kDigitCols64,
-                       blocks, exps);
+          if (prec)
+            build_halves(dir ? o.E : o.F, (o.n + 1) / 2, kDigitCols32, blocks, exps);
+          else
+            build_digits(dir ? o.E : o.F, (o.n + 1) / 2, kDigits64, kDigitCols64, blocks, exps);
           it.dig = put(blocks.data(), blocks.size());
           it.exp = put(exps.data(), exps.size() * sizeof(int));
         }

@@ -89,17 +89,14 @@ struct Profiler {
   std::vector<cudaEvent_t> pool;
   size_t used = 0;
 };
-// Tensor-core (tcgen05) pressure-solve operands: per axis [fwd_hi, fwd_lo, bwd_hi, bwd_lo] tensor maps.
+// Operands of the tensor-core (tcgen05) pressure-solve passes.
 struct TcState {
   bool ready = false;
   void* buf = nullptr;
-  // per axis: [fwd_s_hi, fwd_s_lo, fwd_a_hi, fwd_a_lo, bwd_s_hi, bwd_s_lo, bwd_a_hi, bwd_a_lo]
-  CUtensorMap B[3][8];
   const float* lam[3] = {nullptr, nullptr, nullptr};  // eigenvalues in the tensor-core mode order
   // per axis and direction (0 forward, 1 backward): the four B matrices of every K step laid out as the
   // shared-memory stage holds them (64-byte swizzled rows), one contiguous block per step
   const unsigned char* Bsw[3][2] = {{nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}};
-  int sms = 0;  // multiprocessors of the device (grid of the persistent passes)
 };
 }  // namespace fv
 
@@ -367,12 +364,16 @@ struct HalfOpHost {
 int build_half_op(const AxisHost& a, int kind, HalfOpHost& o);
 
 // ------------------------------------------------------------------ digits (host_digits.cpp)
-// Digits per value, outputs per unit of work, and the longest half axis (order sums stay below 2^24).
-constexpr int kDigits64 = 7, kDigitCols64 = 32, kDigits32 = 4, kDigitCols32 = 64, kDigitMaxH = 128;
+// Parts per value and outputs per unit of work of the digit passes, and their longest half axis (the FP64 order sums
+// stay within 2^24).
+constexpr int kDigits64 = 7, kDigitCols64 = 32, kDigits32 = 2, kDigitCols32 = 64, kDigitMaxH = 128;
 // The two h x h matrices as D balanced base-256 digits (FP16), row j on the common exponent exps[j] of both parts:
 // M[part][j][k] = 2^exps[j] sum_i digit_i 256^(D-1-i).  Blocks [part][group of NC rows][slab of 32 columns], each
 // D NC rows (digit i, output j % NC at row i NC + j % NC) of 64 bytes, 64-byte swizzled.
 void build_digits(const std::vector<double> (&M)[2], int h, int D, int NC, std::vector<unsigned char>& blocks,
+                  std::vector<int>& exps);
+// The same for FP32 fields: two FP16 parts of every entry, M[part][j][k] = 2^exps[j] (hi + lo), in the same blocks.
+void build_halves(const std::vector<double> (&M)[2], int h, int NC, std::vector<unsigned char>& blocks,
                   std::vector<int>& exps);
 
 // ------------------------------------------------------------------ Chebyshev filter ellipses (host_cheb.cpp)

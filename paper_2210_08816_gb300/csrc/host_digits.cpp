@@ -10,43 +10,93 @@
 
 namespace fv {
 
-// FP16 bits of an integer of magnitude <= 128 (exact)
-static uint16_t half_bits(int v) {
-  if (v == 0) return 0;
-  const unsigned m = (unsigned)std::abs(v);
-  int e = 0;
-  while ((m >> e) > 1) ++e;
-  return (uint16_t)((v < 0 ? 0x8000u : 0u) | ((unsigned)(e + 15) << 10) | ((m << (10 - e)) & 0x3ffu));
+// FP16 bits of the integers -128 .. 128 (exact)
+struct HalfTable {
+  uint16_t bits[257];
+  HalfTable() {
+    for (int v = -128; v <= 128; ++v) {
+      const unsigned m = (unsigned)std::abs(v);
+      int e = 0;
+      while ((m >> e) > 1) ++e;
+      bits[v + 128] = m == 0 ? 0
+                             : (uint16_t)((v < 0 ? 0x8000u : 0u) | ((unsigned)(e + 15) << 10) | ((m << (10 - e)) & 0x3ffu));
+    }
+  }
+};
+
+// Largest magnitude of row j of both parts as the exponent q with |entries| < 2^q
+static int row_exponent(const std::vector<double> (&M)[2], int h, int j) {
+  double top = 0.0;
+  for (int part = 0; part < 2; ++part)
+    for (int k = 0; k < h; ++k) top = std::max(top, std::fabs(M[part][(size_t)j * h + k]));
+  int q = 0;
+  if (top > 0.0) std::frexp(top, &q);
+  return q;
 }
+
+// Offset, in halves, of column k of row r of a block: 64-byte rows, 16-byte chunk c at c ^ ((r >> 1) & 3)
+static inline size_t swizzled(int r, int kk) { return (size_t)r * 32 + (((kk >> 3) ^ ((r >> 1) & 3)) << 3) + (kk & 7); }
 
 void build_digits(const std::vector<double> (&M)[2], int h, int D, int NC, std::vector<unsigned char>& blocks,
                   std::vector<int>& exps) {
+  static const HalfTable table;
   const int groups = (h + NC - 1) / NC, nslab = (h + 31) / 32;
-  const size_t block = (size_t)D * NC * 64;
+  const size_t block = (size_t)D * NC * 32;  // halves
+  blocks.assign(block * 2 * groups * nslab * 2, 0);
+  uint16_t* out = reinterpret_cast<uint16_t*>(blocks.data());
   exps.assign(h, 0);
   for (int j = 0; j < h; ++j) {
-    double top = 0.0;
+    exps[j] = row_exponent(M, h, j) - (8 * D - 1);  // integers of magnitude <= 2^(8 D - 1)
+    const double scale = std::ldexp(1.0, -exps[j]);
     for (int part = 0; part < 2; ++part)
-      for (int k = 0; k < h; ++k) top = std::max(top, std::fabs(M[part][(size_t)j * h + k]));
-    int q = 0;
-    if (top > 0.0) std::frexp(top, &q);  // top < 2^q
-    exps[j] = q - (8 * D - 1);           // integers of magnitude <= 2^(8 D - 1)
-  }
-  blocks.assign(block * 2 * groups * nslab, 0);
-  for (int part = 0; part < 2; ++part)
-    for (int j = 0; j < h; ++j)
       for (int k = 0; k < h; ++k) {
-        long long J = std::llrint(std::ldexp(M[part][(size_t)j * h + k], -exps[j]));
-        unsigned char* b = blocks.data() + ((size_t)(part * groups + j / NC) * nslab + k / 32) * block;
+        long long J = std::llrint(M[part][(size_t)j * h + k] * scale);
+        uint16_t* b = out + ((size_t)(part * groups + j / NC) * nslab + k / 32) * block;
         for (int i = D - 1; i >= 0; --i) {
           const int dgt = i == 0 ? (int)J : (int)(((J + 128) & 255) - 128);
           J = (J - dgt) >> 8;
-          // row r of the stacked operand, 64-byte swizzled: 16-byte chunk c at c ^ ((r >> 1) & 3)
-          const int r = i * NC + j % NC, kk = k % 32, c = (kk >> 3) ^ ((r >> 1) & 3);
-          const uint16_t v = half_bits(dgt);
-          std::memcpy(b + (size_t)r * 64 + c * 16 + (kk & 7) * 2, &v, 2);
+          b[swizzled(i * NC + j % NC, k % 32)] = table.bits[dgt + 128];
         }
       }
+  }
+}
+
+// FP16 rounding of |v| < 65520 (nearest even, subnormals included): the value and its bits
+static double round_half(double v, uint16_t& bits) {
+  uint64_t u;
+  std::memcpy(&u, &v, 8);
+  const int e = std::max((int)((u >> 52) & 0x7ff) - 1023, -14);
+  uint64_t unit = (uint64_t)(e - 10 + 1023) << 52, inverse = (uint64_t)(10 - e + 1023) << 52;
+  double un, in;
+  std::memcpy(&un, &unit, 8);
+  std::memcpy(&in, &inverse, 8);
+  const long long m = std::llrint(std::fabs(v) * in);  // in units of 2^(e - 10)
+  // m = 2048 carries into the exponent field, m < 1024 is subnormal
+  bits = (uint16_t)((v < 0 ? 0x8000u : 0u) | (m == 0 ? 0u : ((unsigned)(e + 14) << 10) + (unsigned)m));
+  const double r = (double)m * un;
+  return v < 0 ? -r : r;
+}
+
+void build_halves(const std::vector<double> (&M)[2], int h, int NC, std::vector<unsigned char>& blocks,
+                  std::vector<int>& exps) {
+  const int groups = (h + NC - 1) / NC, nslab = (h + 31) / 32;
+  const size_t block = (size_t)2 * NC * 32;  // halves
+  exps.assign(h, 0);
+  blocks.assign(block * 2 * groups * nslab * 2, 0);
+  uint16_t* out = reinterpret_cast<uint16_t*>(blocks.data());
+  for (int j = 0; j < h; ++j) {
+    exps[j] = row_exponent(M, h, j) - 14;  // scaled below 2^14
+    const double scale = std::ldexp(1.0, -exps[j]);
+    for (int part = 0; part < 2; ++part)
+      for (int k = 0; k < h; ++k) {
+        const double x = M[part][(size_t)j * h + k] * scale;
+        uint16_t v[2];
+        const double hi = round_half(x, v[0]);
+        round_half(x - hi, v[1]);
+        uint16_t* b = out + ((size_t)(part * groups + j / NC) * nslab + k / 32) * block;
+        for (int i = 0; i < 2; ++i) b[swizzled(i * NC + j % NC, k % 32)] = v[i];
+      }
+  }
 }
 
 }  // namespace fv

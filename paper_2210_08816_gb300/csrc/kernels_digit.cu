@@ -1,24 +1,30 @@
-// Fast-diagonalisation passes on the tensor cores by exact digit products (FP64 fields, and FP32 fields of any
-// size and operator): the error-free splitting of Ozaki, Ogita, Oishi & Rump (Numer. Algorithms 59, 2012) with
-// fixed-point rows, on tcgen05.mma kind::f16.
+// Fast-diagonalisation passes on the tensor cores by products of FP16 parts (tcgen05.mma kind::f16): FP64 fields, and
+// FP32 fields of any size and operator.
 //
-// A pass contracts the sums and differences of mirrored inputs with two h x h matrices (see HalfOpHost).  Each row
-// of inputs is written on a common exponent as an integer of D balanced base-256 digits, x = 2^e sum_i x_i
-// 256^(D-1-i), |x_i| <= 128, and so is each row of a matrix (on the host, build_digits).  Digits are exact in
-// FP16, a product of two is at most 2^14, and the sum over K <= 128 inputs of the at most 7 products of one order
-// i + j is an integer below 2^24: FP32 accumulators hold it exactly.  Orders 0 .. D-1 are kept:
-//   FP64: D = 7 (56 bits), 28 products; the first dropped order lies 2^-56 below the largest product of the row.
-//   FP32: D = 4 (32 bits), 10 products.
-// The epilogue joins the D accumulators as a 64-bit integer, so the only roundings are the digits' quantisation,
-// the dropped orders and the conversion of the result: below those of the FP64 fused multiply-add chain (errors
-// against 64 bits: 256^3 Chebyshev step 3.3e-14 by the CUDA-core passes).
+// A pass contracts the sums and differences of mirrored inputs with two h x h matrices (see HalfOpHost).
+//
+// FP64: exact digit products, the error-free splitting of Ozaki, Ogita, Oishi & Rump (Numer. Algorithms 59, 2012) with
+// fixed-point rows.  Each row of inputs is written on a common exponent as an integer of 7 balanced base-256 digits,
+// x = 2^e sum_i x_i 256^(6-i), |x_i| <= 128, and so is each row of a matrix (on the host, build_digits).  Digits are
+// exact in FP16, a product of two is at most 2^14, and the sum over K <= 128 inputs of the at most 7 products of one
+// order i + j is an integer of at most 2^24: FP32 accumulators hold it exactly.  Orders 0 .. 6 are kept (28 products;
+// the first dropped one lies 2^-56 below the row's largest product) and joined in the epilogue as a 64-bit integer,
+// so the only roundings are the digits' quantisation, the dropped orders and the conversion of the result.
+//
+// FP32: rows scaled by a power of two into FP16's range, every value as the sum of two FP16 numbers (23 bits), all four
+// products, with the leading one spread over two accumulators.  (Fixed-point digits as in FP64 would need 32 bits: with
+// 25 their error, absolute in a row, was up to 4 times that of FP32 arithmetic on stretched grids.)
 //
 // Why: GB300 issues two FP64 operations per clock and SM (1.23 TFLOP/s measured in k_half); the 28 FP16 products
-// cost 155 GFLOP per 256^3 pass where the FP16 tensor rate is 1.9 PFLOP/s.
+// cost 155 GFLOP per 256^3 pass where the FP16 tensor rate is 1.9 PFLOP/s.  Measured, six passes, CUDA cores / here:
+// FP64 256^3 21.9 / 1.94 ms, 100^3 794 / 217 us; FP32 100^3 98 / 76 us, 250^3 1360 / 450 us, four fields of 256^3
+// 5.2 / 1.65 ms.  Errors against 64 bits are at or below those of the CUDA-core passes (FP32 100^3 product 3.9e-7 ->
+// 2.4e-7, FP64 256^3 3.4e-14 as before).  What bounds a unit is the workers' instruction issue (FP64: digits and the
+// joining of the accumulators, 56 % of the integer pipe), not the MMAs (19 % of the tensor pipe).
 //
-// Layout.  Stacking the matrix digits j = 0 .. D-1-i of NC outputs as rows of one B operand makes all products of
+// Layout (FP64).  Stacking the matrix digits j = 0 .. D-1-i of NC outputs as rows of one B operand makes all products of
 // input digit i ONE instruction: N = (D - i) NC columns, accumulated at column i NC, where block d of NC columns
-// holds order d.  A unit of work is 128 rows x NC pairs, both parts; TMEM columns 0 and 256 hold the symmetric and
+// holds order d.  (FP32: blocks hi hi twice, then the rest.)  A unit of work is 128 rows x NC pairs, both parts; TMEM columns 0 and 256 hold the symmetric and
 // the antisymmetric accumulators.  A CTA walks a contiguous range of units (the groups of NC pairs of a tile follow
 // each other, so its rows stay in L2 and their exponents are found once).  Warps:
 //   0      bulk copies of the B digits (pre-swizzled blocks) into the slots of a ring
@@ -31,7 +37,6 @@
 
 #include <algorithm>
 #include <type_traits>
-#include <utility>
 
 #include "fv_internal.h"
 #include "tcgen05.cuh"
@@ -40,24 +45,24 @@ namespace fv {
 namespace {
 
 constexpr int kDgRows = 128;
-constexpr int kDgSlots = 3;
 constexpr int kDgWarps = 16;  // workers
 constexpr int kDgIts = kDgRows / (2 * kDgWarps);  // row pairs of a worker warp per slab
 constexpr int kDgThreads = 32 * (2 + kDgWarps);
-constexpr int kDgE = 2;  // outputs of a row read from TMEM at a time
 constexpr int kDgDigitBytes = kDgRows * 64;  // one digit of a 128 x 32 slab (64-byte swizzled rows)
 
+// D digits per value, NC outputs per unit, ACC accumulators per output, E outputs of a row read from TMEM at a time,
+// slots of the ring; the type a scaled input has and the type the joined accumulators have
 template <typename R>
 struct Dg;
 template <>
 struct Dg<double> {
-  static constexpr int D = kDigits64, NC = kDigitCols64;
-  using Int = long long;
+  static constexpr int D = kDigits64, NC = kDigitCols64, ACC = D, E = 2, kSlots = 3;
+  using Val = long long;
 };
 template <>
 struct Dg<float> {
-  static constexpr int D = kDigits32, NC = kDigitCols32;
-  using Int = int;
+  static constexpr int D = kDigits32, NC = kDigitCols32, ACC = 3, E = 4, kSlots = 6;
+  using Val = float;
 };
 
 template <typename R>
@@ -81,32 +86,35 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t a, uint64_t b,
       : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t (&r)[2]) {
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[2]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
 
-// x on the row's exponent E as an integer, truncated: FP64 |I| < 2^53 with value I 2^(E - 1075), FP32 |I| < 2^29
-// with value I 2^(E - 155).  E >= 64 (FP32: 32) and shifts clamp, so that zeros and subnormals shift out.  (FP64:
-// the dropped bits lie below 2^-52 of the row's largest input, a quarter of what the roundings of an FMA chain over
-// 128 inputs add up to.)
-__device__ __forceinline__ long long to_fixed(double x, int E) {
+__device__ __forceinline__ unsigned magnitude_bits(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned magnitude_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+
+// x on the row's exponent E.  FP64: an integer, truncated, |I| < 2^54 with value I 2^(E - 1076); E >= 64 and shifts
+// clamp, so that zeros and subnormals shift out (the dropped bits lie below 2^-53 of the row's largest input, a
+// fraction of what the roundings of an FMA chain over its inputs add up to).  FP32: scaled below 2^14, value
+// y 2^(E - 140).
+__device__ __forceinline__ long long scaled(double x, int E) {
   const int hi = __double2hiint(x);
   const unsigned lo = (unsigned)__double2loint(x);
-  unsigned long long m = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | lo;
+  unsigned long long m = (((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | lo) << 1;
   asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(E - (int)(((unsigned)hi & 0x7fffffffu) >> 20)));
   const long long sg = (long long)(hi >> 31);
   return ((long long)m ^ sg) - sg;
 }
-__device__ __forceinline__ int to_fixed(float x, int E) {
-  const int b = __float_as_int(x);
-  unsigned m = (((unsigned)b & 0x7fffffu) | 0x800000u) << 5;
-  asm("shr.u32 %0, %0, %1;" : "+r"(m) : "r"(E - (int)(((unsigned)b & 0x7fffffffu) >> 23)));
-  const int sg = b >> 31;
-  return ((int)m ^ sg) - sg;
-}
+__device__ __forceinline__ float scaled(float x, int E) { return x * __uint_as_float((unsigned)(267 - E) << 23); }
 
-// The D balanced digits of two neighbouring inputs as FP16 pairs, digit i at dst + i * kDgDigitBytes.  Adding 128 to
-// every digit makes them the bytes of an unsigned integer; 0x6400 | byte is the FP16 number 1024 + byte.
+// The D digits of two neighbouring inputs as FP16 pairs, digit i at dst + i * kDgDigitBytes.  FP64: balanced base-256
+// digits; adding 128 to each makes them the bytes of an unsigned integer; 0x6400 | byte is the FP16 number
+// 1024 + byte.
 __device__ __forceinline__ void put_pair(unsigned char* dst, uint32_t h) {
   const __half2 r = __hadd2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(0xE480)));  // - 1152
   *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(&r);
@@ -124,12 +132,15 @@ __device__ __forceinline__ void put_digits(unsigned char* dst, long long I0, lon
   put_two(dst, 6, a0, b0, 0x5410);
   put_two(dst, 4, a0, b0, 0x7632);
   put_two(dst, 2, a1, b1, 0x5410);
-  put_pair(dst, __byte_perm(a1, b1, 0x7632) | 0x64006400u);
+  put_pair(dst, __byte_perm(a1, b1, 0x7632) | 0x64006400u);  // the leading digit may be 256 - 128
 }
-__device__ __forceinline__ void put_digits(unsigned char* dst, int I0, int I1) {
-  const uint32_t a = (uint32_t)I0 + 0x80808080u, b = (uint32_t)I1 + 0x80808080u;
-  put_two(dst, 3, a, b, 0x5410);
-  put_two(dst, 1, a, b, 0x7632);
+// FP32: the value rounded to FP16 and the remainder rounded to FP16
+__device__ __forceinline__ void put_digits(unsigned char* dst, float y0, float y1) {
+  const __half2 h = __floats2half2_rn(y0, y1);
+  const float2 f = __half22float2(h);
+  const __half2 l = __floats2half2_rn(y0 - f.x, y1 - f.y);
+  *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(&h);
+  *reinterpret_cast<uint32_t*>(dst + kDgDigitBytes) = *reinterpret_cast<const uint32_t*>(&l);
 }
 
 // Two neighbouring values: one vector load when `vec` (the pair is aligned), else two scalar ones; the second only
@@ -148,16 +159,15 @@ __device__ __forceinline__ void load_two(const R* __restrict__ p, bool vec, bool
 }
 
 // The D order sums of one output joined.  FP64: an integer V = 2^-8 sum_d A_d 256^(6-d) (value V 2^(E + eM -
-// 1019)), |V| < 2^62 so that S +- A fits.
-__device__ __forceinline__ long long join_orders(const uint32_t (&r)[7][kDgE], int j) {
+// 1020)), |V| < 2^62 so that S +- A fits.
+__device__ __forceinline__ long long join_orders(const uint32_t (&r)[7][2], int j) {
   auto A = [&](int d) { return __float2int_rn(__uint_as_float(r[d][j])); };
   const long long hi = (long long)(A(1) * 256 + A(2)) * 16777216 + ((long long)A(0) << 40);
   return hi + (long long)A(3) * 65536 + (long long)A(4) * 256 + (A(5) + (A(6) >> 8));
 }
-// FP32: the number sum_d A_d 256^(3-d) (value V 2^(E + eM - 131)) to one rounding of each half and of their sum
-__device__ __forceinline__ float join_orders(const uint32_t (&r)[4][kDgE], int j) {
-  auto A = [&](int d) { return __float2int_rn(__uint_as_float(r[d][j])); };
-  return fmaf((float)(A(0) * 256 + A(1)), 65536.0f, (float)(A(2) * 256 + A(3)));
+// FP32: the sum of all (value V 2^(E + eM - 140))
+__device__ __forceinline__ float join_orders(const uint32_t (&r)[3][4], int j) {
+  return (__uint_as_float(r[0][j]) + __uint_as_float(r[1][j])) + __uint_as_float(r[2][j]);
 }
 
 // v 2^e rounded to nearest; integer arithmetic only (an FP64 operation per output would cost as much as the MMAs).
@@ -173,10 +183,6 @@ __device__ __forceinline__ double from_fixed(long long v, int e, bool fast) {
   if (!fast) b = be >= 2047 ? 0x7ff0000000000000ull : be < 1 ? 0ull : b;
   return __longlong_as_double((long long)(b | ((unsigned long long)sg << 63)));
 }
-__device__ __forceinline__ float from_fixed(float v, int e, bool fast) {
-  return fast ? v * __uint_as_float((unsigned)(e + 127) << 23) : ldexpf(v, e);
-}
-
 template <typename R>
 __device__ __forceinline__ R quiet_nan();
 template <>
@@ -206,18 +212,18 @@ struct DgUnit {
 template <typename R, bool BWD>
 __global__ void __launch_bounds__(kDgThreads, 1)
     k_digit_pass(const __grid_constant__ DgArgs<R> t, const R* __restrict__ in, R* __restrict__ out) {
-  constexpr int D = Dg<R>::D, NC = Dg<R>::NC;
+  constexpr int D = Dg<R>::D, NC = Dg<R>::NC, ACC = Dg<R>::ACC, E_ = Dg<R>::E, kSlots = Dg<R>::kSlots;
   constexpr bool F64 = sizeof(R) == 8;
   constexpr int kExpShift = F64 ? 20 : 23, kExpMax = F64 ? 2047 : 255, kExpMin = F64 ? 64 : 32;
   constexpr uint32_t kABytes = D * kDgDigitBytes, kBBytes = D * NC * 64, kSlotBytes = kABytes + kBBytes;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t bar_full[kDgSlots], bar_conv[kDgSlots], bar_empty[kDgSlots];
+  __shared__ __align__(8) uint64_t bar_full[kSlots], bar_conv[kSlots], bar_empty[kSlots];
   __shared__ __align__(8) uint64_t bar_accf, bar_acce, bar_drain;
   __shared__ uint32_t tmem_slot;
   // exponents of the rows, four tiles deep: a warp can find those of tile T + 1 while another still reads T - 1's in
   // an epilogue (tile T + 2 has to wait for that epilogue's MMAs)
   __shared__ int row_exp[4][kDgRows];
-  __shared__ int out_exp[4][kDigitMaxH];  // exponents of the matrix rows per operator
+  __shared__ int out_exp[4][kDigitMaxH];  // exponents of the matrix rows per operator (FP32: 2^exponent, as bits)
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t base = smem_u32(smem);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -226,7 +232,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
   const int u1 = (int)((long long)t.units * (blockIdx.x + 1) / gridDim.x);
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kDgSlots; ++s) {
+    for (int s = 0; s < kSlots; ++s) {
       mbar_init(smem_u32(&bar_full[s]), 1);
       mbar_init(smem_u32(&bar_conv[s]), 32 * kDgWarps);
       mbar_init(smem_u32(&bar_empty[s]), 1);
@@ -236,7 +242,8 @@ __global__ void __launch_bounds__(kDgThreads, 1)
     mbar_init(smem_u32(&bar_drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int i = threadIdx.x; i < (t.op_mask + 1) * h; i += kDgThreads) out_exp[i / h][i % h] = t.eM[i / h][i % h];
+  for (int i = threadIdx.x; i < (t.op_mask + 1) * h; i += kDgThreads) 
+    out_exp[i / h][i % h] = F64 ? t.eM[i / h][i % h] : (t.eM[i / h][i % h] + 127) << 23;  // FP32: the power of two
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                  "r"(512)
@@ -268,9 +275,9 @@ __global__ void __launch_bounds__(kDgThreads, 1)
         }
         for (int j = 0; j < t.nslab && ok; ++j)
           for (int part = 0; part < 2; ++part, ++gi) {
-            const int st = gi % kDgSlots;
-            if (gi >= kDgSlots &&
-                !mbar_wait(smem_u32(&bar_empty[st]), ((gi / kDgSlots) - 1) & 1, t.err, 31, t.spins)) {
+            const int st = gi % kSlots;
+            if (gi >= kSlots &&
+                !mbar_wait(smem_u32(&bar_empty[st]), ((gi / kSlots) - 1) & 1, t.err, 31, t.spins)) {
               ok = false;
               break;
             }
@@ -283,8 +290,8 @@ __global__ void __launch_bounds__(kDgThreads, 1)
         un.step(t);
       }
       // every issued copy has landed before the block may exit
-      for (int g2 = (issued > kDgSlots ? issued - kDgSlots : 0); g2 < issued; ++g2)
-        mbar_wait(smem_u32(&bar_full[g2 % kDgSlots]), (g2 / kDgSlots) & 1, t.err, 32, kWaitLimit);
+      for (int g2 = (issued > kSlots ? issued - kSlots : 0); g2 < issued; ++g2)
+        mbar_wait(smem_u32(&bar_full[g2 % kSlots]), (g2 / kSlots) & 1, t.err, 32, kWaitLimit);
     }
   } else if (warp == 1) {
     // descriptors differ from the first slot's by constants: one addition per MMA (building each from its address in
@@ -300,8 +307,8 @@ __global__ void __launch_bounds__(kDgThreads, 1)
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       for (int j = 0; j < t.nslab && ok; ++j)
         for (int part = 0; part < 2; ++part, ++gi) {
-          const int st = gi % kDgSlots;
-          const uint32_t ph = (gi / kDgSlots) & 1;
+          const int st = gi % kSlots;
+          const uint32_t ph = (gi / kSlots) & 1;
           if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_full[st]), ph, t.err, 34, t.spins) &&
                                            mbar_wait(smem_u32(&bar_conv[st]), ph, t.err, 35, t.spins))) {
             ok = false;
@@ -311,15 +318,29 @@ __global__ void __launch_bounds__(kDgThreads, 1)
           const uint64_t da = desc0 + (uint64_t)((st * kSlotBytes) >> 4), db = da + (kABytes >> 4);
           const uint32_t acc = tmem + part * 256;
           if (elect_one()) {
+            // M = 128, FP16 operands, FP32 accumulators
+            auto mma = [&](int col, int i, int row, int cols, int kk, bool acc_on) {  // input digit i, B rows from `row`
+              constexpr uint32_t kId = (1u << 4) | ((kDgRows / 16u) << 24);
+              mma_f16(acc + col, da + ((i * kDgDigitBytes + kk * 32) >> 4), db + ((row * 64 + kk * 32) >> 4),
+                      kId | ((uint32_t)(cols / 8) << 17), acc_on ? 1u : (uint32_t)(j > 0));
+            };
+            if constexpr (F64) {
 #pragma unroll
-            for (int kk = 0; kk < 2; ++kk)
+              for (int kk = 0; kk < 2; ++kk)
 #pragma unroll
-              for (int i = 0; i < D; ++i) {
-                // M = 128, N = (D - i) NC, FP16 operands, FP32 accumulators
-                constexpr uint32_t kId = (1u << 4) | ((kDgRows / 16u) << 24);
-                mma_f16(acc + i * NC, da + ((i * kDgDigitBytes + kk * 32) >> 4), db + (kk * 32 >> 4),
-                        kId | ((uint32_t)((D - i) * NC / 8) << 17), (kk > 0 || i > 0) ? 1u : (uint32_t)(j > 0));
-              }
+                for (int i = 0; i < D; ++i) mma(i * NC, i, 0, (D - i) * NC, kk, kk > 0 || i > 0);
+            } else {
+              // hi hi into two accumulators by turns (the tensor cores truncate their sums: half the steps, half the
+              // bias), the cross products and lo lo into the third
+              mma(0, 0, 0, NC, 0, false);
+              mma(2 * NC, 0, NC, NC, 0, false);
+              mma(2 * NC, 1, 0, NC, 0, true);
+              mma(2 * NC, 1, NC, NC, 0, true);
+              mma(NC, 0, 0, NC, 1, false);
+              mma(2 * NC, 0, NC, NC, 1, true);
+              mma(2 * NC, 1, 0, NC, 1, true);
+              mma(2 * NC, 1, NC, NC, 1, true);
+            }
             mma_commit(smem_u32(&bar_empty[st]));
             // (the last slab's second part: arrives once every MMA of the unit has completed)
             if (part == 1 && j == t.nslab - 1) mma_commit(smem_u32(&bar_accf));
@@ -372,9 +393,23 @@ __global__ void __launch_bounds__(kDgThreads, 1)
         const int k0 = t.k0[op], S = t.S[op];
         const R* __restrict__ src = in + ((size_t)un.field * P + (size_t)un.tile * kDgRows) * n;
         const int rows = min(kDgRows, P - un.tile * kDgRows);
-        if (j == 0 && (du == 0 || un.group == 0)) {
-          ++tc;
-          // largest magnitude of each of the warp's rows (FP64: by the high words), 16 loads in flight; a face
+        if (item == 0) {
+#pragma unroll
+          for (int it = 0; it < kDgIts; ++it) load_row(it, src, rows, kl, k0, S);
+        }
+        if (j == 0 && (du == 0 || un.group == 0)) ++tc;
+        if (j == 0 && (du == 0 || un.group == 0) && t.nslab == 1) {  // the rows are in the registers
+#pragma unroll
+          for (int it = 0; it < kDgIts; ++it) {
+            unsigned m = max(max(magnitude_bits(x0[it]), magnitude_bits(x1[it])),
+                             max(magnitude_bits(y0[it]), magnitude_bits(y1[it])));
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if ((lane & 15) == 0) row_exp[tc & 3][2 * (kDgWarps * it + cw) + rh] = max((int)(m >> kExpShift), kExpMin);
+          }
+          __syncwarp();
+        } else if (j == 0 && (du == 0 || un.group == 0)) {
+          // largest magnitude of each of the warp's rows (FP64: by the high words), 32 loads in flight; a face
           // axis' wall slot holds no input
           constexpr int kRows = 2 * kDgIts, kStep = sizeof(R) / 4;
           unsigned m[kRows];
@@ -382,17 +417,19 @@ __global__ void __launch_bounds__(kDgThreads, 1)
           for (int r = 0; r < kRows; ++r) m[r] = 0;
           const unsigned* __restrict__ w0 = reinterpret_cast<const unsigned*>(src) + (kStep - 1);
 #pragma unroll 1
-          for (int k = (BWD ? 0 : k0) + lane; k - lane < n; k += 64) {
-            unsigned v[2][kRows];
+          for (int k = (BWD ? 0 : k0) + lane; k - lane < n; k += 128) {
+            unsigned v[4][kRows];
 #pragma unroll
-            for (int q = 0; q < 2; ++q)
+            for (int q = 0; q < 4; ++q)
 #pragma unroll
               for (int r = 0; r < kRows; ++r) {
                 const int row = min(2 * (kDgWarps * (r >> 1) + cw) + (r & 1), rows - 1);
                 v[q][r] = __ldg(w0 + ((size_t)row * n + min(k + 32 * q, n - 1)) * kStep);
               }
 #pragma unroll
-            for (int r = 0; r < kRows; ++r) m[r] = max(m[r], max(v[0][r] & 0x7fffffffu, v[1][r] & 0x7fffffffu));
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+              for (int r = 0; r < kRows; ++r) m[r] = max(m[r], v[q][r] & 0x7fffffffu);
           }
 #pragma unroll
           for (int r = 0; r < kRows; ++r) {
@@ -403,32 +440,28 @@ __global__ void __launch_bounds__(kDgThreads, 1)
           __syncwarp();
         }
         const int* __restrict__ re = row_exp[tc & 3];
-        const int gi = 2 * item, s0 = gi % kDgSlots, s1 = (gi + 1) % kDgSlots;
-        if (item == 0) {
-#pragma unroll
-          for (int it = 0; it < kDgIts; ++it) load_row(it, src, rows, kl, k0, S);
-        }
+        const int gi = 2 * item, s0 = gi % kSlots, s1 = (gi + 1) % kSlots;
         // the next item: this unit's next slab, or the first of the next unit
         if (j + 1 == t.nslab) nx.step(t);
         const R* __restrict__ nsrc = in + ((size_t)nx.field * P + (size_t)nx.tile * kDgRows) * n;
         const int nrows = item + 1 < total ? min(kDgRows, P - nx.tile * kDgRows) : 0;
         const int nk = (j + 1 == t.nslab ? 0 : (j + 1) * 32) + kl;
         const int nk0 = t.k0[nx.field & t.op_mask], nS = t.S[nx.field & t.op_mask];
-        using I = typename Dg<R>::Int;
-        I i0[kDgIts], i1[kDgIts], j0[kDgIts], j1[kDgIts];
+        using Val = typename Dg<R>::Val;
+        Val i0[kDgIts], i1[kDgIts], j0[kDgIts], j1[kDgIts];
 #pragma unroll
         for (int it = 0; it < kDgIts; ++it) {
           const int E = re[2 * (kDgWarps * it + cw) + rh];
-          i0[it] = to_fixed(x0[it], E);
-          i1[it] = to_fixed(x1[it], E);
-          j0[it] = to_fixed(y0[it], E);
-          j1[it] = to_fixed(y1[it], E);
+          i0[it] = scaled(x0[it], E);
+          i1[it] = scaled(x1[it], E);
+          j0[it] = scaled(y0[it], E);
+          j1[it] = scaled(y1[it], E);
           load_row(it, nsrc, nrows, nk, nk0, nS);
         }
         // each slot is filled as soon as it is free: with three slots, the MMAs of the slab before run meanwhile
         constexpr int kRow = 2 * kDgWarps * 64;
         const int off = (2 * cw + rh) * 64 + (((kl >> 3) ^ (cw & 3)) << 4) + (kl & 7) * 2;  // row >> 1 = cw mod 4
-        if (gi >= kDgSlots && !mbar_wait(smem_u32(&bar_empty[s0]), ((gi / kDgSlots) - 1) & 1, t.err, 37, t.spins)) {
+        if (gi >= kSlots && !mbar_wait(smem_u32(&bar_empty[s0]), ((gi / kSlots) - 1) & 1, t.err, 37, t.spins)) {
           ok = false;
           break;
         }
@@ -438,8 +471,8 @@ __global__ void __launch_bounds__(kDgThreads, 1)
           put_digits(dst + it * kRow, BWD ? i0[it] : i0[it] + j0[it], BWD ? i1[it] : i1[it] + j1[it]);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive(smem_u32(&bar_conv[s0]));
-        if (gi + 1 >= kDgSlots &&
-            !mbar_wait(smem_u32(&bar_empty[s1]), (((gi + 1) / kDgSlots) - 1) & 1, t.err, 38, t.spins)) {
+        if (gi + 1 >= kSlots &&
+            !mbar_wait(smem_u32(&bar_empty[s1]), (((gi + 1) / kSlots) - 1) & 1, t.err, 38, t.spins)) {
           ok = false;
           break;
         }
@@ -469,45 +502,59 @@ __global__ void __launch_bounds__(kDgThreads, 1)
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const int E = row_exp[(newer ? tc - 1 : tc) & 3][erow];
         const bool bad = E == kExpMax;  // an Inf or NaN among the row's inputs
+        // FP32: 2^(E - 140), E in 32 .. 254
+        const float row_scale = __uint_as_float((unsigned)(min(E, 254) - 13) << 23);
         const int c1 = min(NC, h - group * NC);
 #pragma unroll 1
-        for (int c0 = (cw >> 2) * kDgE; c0 < c1; c0 += (kDgWarps / 4) * kDgE) {
-          decltype(join_orders(std::declval<const uint32_t(&)[D][kDgE]>(), 0)) vs[kDgE], va[kDgE];
-          uint32_t rs[D][kDgE], ra[D][kDgE];
+        for (int c0 = (cw >> 2) * E_; c0 < c1; c0 += (kDgWarps / 4) * E_) {
+          typename Dg<R>::Val vs[E_], va[E_];
+          uint32_t rs[ACC][E_], ra[ACC][E_];
 #pragma unroll
-          for (int d = 0; d < D; ++d) tmem_ld2(lane_base + d * NC + c0, rs[d]);
+          for (int d = 0; d < ACC; ++d) tmem_ld(lane_base + d * NC + c0, rs[d]);
 #pragma unroll
-          for (int d = 0; d < D; ++d) tmem_ld2(lane_base + 256 + d * NC + c0, ra[d]);
+          for (int d = 0; d < ACC; ++d) tmem_ld(lane_base + 256 + d * NC + c0, ra[d]);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-          for (int q = 0; q < kDgE; ++q) vs[q] = join_orders(rs, q), va[q] = join_orders(ra, q);
+          for (int q = 0; q < E_; ++q) vs[q] = join_orders(rs, q), va[q] = join_orders(ra, q);
           if (live) {
+            const int j0 = group * NC + c0;
+            // rows of the output: modes j and h + j, or cells k0 + j and S - k0 - j
+            R* __restrict__ o1 = o + (size_t)(BWD ? k0 + j0 : j0) * P;
+            R* __restrict__ o2 = o + (size_t)(BWD ? S - k0 - j0 : h + j0) * P;
 #pragma unroll
-            for (int q = 0; q < kDgE; ++q) {
-              const int jj = group * NC + c0 + q;
+            for (int q = 0; q < E_; ++q) {
+              const int jj = j0 + q;
               if (jj >= h) break;
-              const int e = E + out_exp[op][jj] - (F64 ? 1019 : 131);
-              // (FP32 fast: the factor 2^e is normal and |v| < 2^48 cannot overflow)
-              const bool fast = F64 ? (e > -1000 && e < 900) : (e > -120 && e < 70);
-              R s = from_fixed(BWD ? vs[q] + va[q] : vs[q], e, fast);
-              R a = from_fixed(BWD ? vs[q] - va[q] : va[q], e, fast);
+              R s, a;
+              if constexpr (F64) {
+                const int e = E + out_exp[op][jj] - 1020;
+                const bool fast = e > -1000 && e < 900;
+                s = from_fixed(BWD ? vs[q] + va[q] : vs[q], e, fast);
+                a = from_fixed(BWD ? vs[q] - va[q] : va[q], e, fast);
+              } else {  // both factors are powers of two
+                const float col = __int_as_float(out_exp[op][jj]);
+                s = (BWD ? vs[q] + va[q] : vs[q]) * col * row_scale;
+                a = (BWD ? vs[q] - va[q] : va[q]) * col * row_scale;
+              }
               if (bad) s = a = quiet_nan<R>();
               if (BWD) {
-                const int i1 = k0 + jj, i2 = S - i1;
-                if (i1 <= i2) {  // (an odd face axis has one pair less than h)
-                  o[(size_t)i1 * P] = s;
-                  o[(size_t)i2 * P] = a;
+                if (k0 + jj <= S - k0 - jj) {  // (an odd face axis has one pair less than h)
+                  *o1 = s;
+                  *o2 = a;
                 }
                 if (k0 == 1 && jj == 0) o[0] = R(0);  // the wall slot
+                o2 -= P;
               } else {
                 if (t.scale) {
                   const R* lz = t.lam[2][op];
                   s = (t.zero_mode && p == 0 && jj == 0) ? R(0) : t.fac[op] * s / (lz[jj] + l01);
                   if (jj < ha) a = t.fac[op] * a / (lz[h + jj] + l01);
                 }
-                o[(size_t)jj * P] = s;
-                if (jj < ha) o[(size_t)(h + jj) * P] = a;
+                *o1 = s;
+                if (jj < ha) *o2 = a;
+                o2 += P;
               }
+              o1 += P;
             }
           }
         }
@@ -533,7 +580,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
 
 template <typename R>
 constexpr size_t digit_smem() {
-  return (size_t)kDgSlots * (Dg<R>::D * kDgDigitBytes + Dg<R>::D * Dg<R>::NC * 64) + 1024;
+  return (size_t)Dg<R>::kSlots * (Dg<R>::D * kDgDigitBytes + Dg<R>::D * Dg<R>::NC * 64) + 1024;
 }
 
 template <typename R>

@@ -238,14 +238,13 @@ template <>
 const HalfDev<float> (&half_of<float>(const fv_grid_s* g))[3][3] { return g->half32; }
 
 // Digit products on the tensor cores (kernels_digit.cu) instead of the CUDA-core form, by the multiplications of a
-// half-size pass.  A digit pass costs ~16 us before its length shows (one unit of work: exponents, digits, MMAs,
-// epilogue one after another), a CUDA-core pass ~8.  FP64 (pass, us, CUDA cores / digits): 32^3 9.7 / 16,
-// 56^3 19.2 / 19.4, 64^3 25.6 / 19.8, 100^3 130 / 36, 160^3 589 / 78, four fields of 40^3 26 / 21.  FP32, whose
-// CUDA-core rate is 64 times higher: 112^3 18.4 / 18.7, 150^3 40.9 / 40.6, 200^3 109 / 75, four fields of 100^3
-// 38.7 / 40.4, of 112^3 48.9 / 42.1, of 250^3 875 / 433.
+// half-size pass: a digit pass has a floor of ~10 us (FP64 ~16) before its length shows.  Measured (us a pass, with
+// ~3 of event overhead, CUDA cores / digits): FP64 32^3 9.7 / 16, 56^3 19.2 / 19.4, 64^3 25.6 / 19.8, 100^3 130 / 36,
+// 160^3 589 / 78, four fields of 40^3 26 / 21; FP32 65^3 9.6 / 14, 100^3 16.1 / 12.7, 150^3 40.4 / 29.6, 200^3
+// 109 / 51, 250^3 227 / 75, four fields of 64^3 10.5 / 10.7, of 96^3 28.6 / 20.0, of 256^3 875 / 275.
 template <typename R>
 bool digit_wins(int n, long long rows) {
-  return (double)rows * n * ((n + 1) / 2) >= (sizeof(R) == 8 ? 4.5e6 : 2.6e8);
+  return (double)rows * n * ((n + 1) / 2) >= (sizeof(R) == 8 ? 4.5e6 : 3.5e7);
 }
 
 // One pass along `axis` over nf fields of a (na x nb) x n block, kinds[op][axis] = the operators (one, or four

@@ -19,14 +19,6 @@
 // A_lo B_lo and the TF32 rounding of the lo parts are ~2^-22 relative).  B_hi / B_lo are prepared on the
 // host; A is split in shared memory by the converter warps.
 //
-// One CTA = one 128-row tile of p and all n (<= 256) outputs; per stage two 16-wide K slabs of A (slab j
-// and its mirror n/16-1-j forward, slab j and j + n/32 backward) and the matching 16-wide slabs of the two
-// half-size B matrices, in a 3-stage ring:
-//   warp 0      TMA producer
-//   warp 1      TMEM allocation; one elected thread issues tcgen05.mma (M = 128, N = n/2, K = 8): per
-//               stage 2 k-steps x 3 products x 2 halves into two accumulators (TMEM columns 0 and n/2)
-//   warps 2..5  converters (sum / difference, hi / lo split), then the epilogue: tcgen05.ld -> out[m][p]
-// Every mbarrier wait is bounded; on expiry the kernel records an error code and drains.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -46,8 +38,6 @@ constexpr int kTcBM = 128;                 // rows per tile
 constexpr int kTcBK = 16;                  // fp32 elements per K slab (64 bytes: one 64-byte swizzle row)
 constexpr int kTcRowBytes = kTcBK * 4;
 constexpr int kTcABytes = kTcBM * kTcRowBytes;  // one A slab tile (8 KB)
-constexpr int kTcStages = 3;
-constexpr int kTcThreads = 192;
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
   asm volatile(
@@ -89,217 +79,22 @@ __device__ __forceinline__ void split4(const float4 x, float4& h, float4& l) {
   l.w = x.w - h.w;
 }
 
-template <bool SCALE, bool BWD>
-__global__ void __launch_bounds__(kTcThreads, 1)
-    k_transform_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB1hi,
-                   const __grid_constant__ CUtensorMap tmB1lo, const __grid_constant__ CUtensorMap tmB2hi,
-                   const __grid_constant__ CUtensorMap tmB2lo, float* __restrict__ out, int P, int n,
-                   const float* __restrict__ lx, const float* __restrict__ ly, const float* __restrict__ lz, int nb,
-                   int* err) {
-  extern __shared__ __align__(1024) unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t bar_full[kTcStages], bar_conv[kTcStages], bar_empty[kTcStages], bar_acc;
-  __shared__ uint32_t tmem_slot;
-  __shared__ float lz_s[256];  // eigenvalues of the contracted axis (scaled pass only)
-  const int h = n / 2;         // outputs per half, K per half
-  // 1024-byte aligned ring; per stage tiles T0..T7: A1, A2 (loaded), A1_lo, A2_lo (converted),
-  // B1_hi, B1_lo, B2_hi, B2_lo (loaded, h rows x 64 B each)
-  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t b_bytes = (uint32_t)h * kTcRowBytes;
-  const uint32_t stage_bytes = 4u * kTcABytes + 4u * b_bytes;
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int nst = n / (2 * kTcBK);  // stages per tile: pairs of slabs
-  const int p0 = blockIdx.x * kTcBM;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kTcStages; ++s) {
-      mbar_init(smem_u32(&bar_full[s]), 1);
-      mbar_init(smem_u32(&bar_conv[s]), 128);
-      mbar_init(smem_u32(&bar_empty[s]), 1);
-    }
-    mbar_init(smem_u32(&bar_acc), 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (SCALE)
-    for (int m = threadIdx.x; m < n; m += kTcThreads) lz_s[m] = lz[m];
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
-                 "r"(256)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_slot;
-
-  if (warp == 0) {
-    if (lane == 0) {
-      int issued = 0;
-      for (int j = 0; j < nst; ++j) {
-        const int st = j % kTcStages;
-        if (j >= kTcStages && !mbar_wait(smem_u32(&bar_empty[st]), ((j / kTcStages) - 1) & 1, err, 1)) break;
-        const uint32_t sb = base + st * stage_bytes;
-        const uint32_t fb = smem_u32(&bar_full[st]);
-        const int k1 = j * kTcBK;
-        const int k2 = BWD ? h + j * kTcBK : n - kTcBK - j * kTcBK;
-        mbar_expect_tx(fb, 2u * kTcABytes + 4u * b_bytes);
-        tma_load_2d(sb, &tmA, fb, k1, p0);
-        tma_load_2d(sb + kTcABytes, &tmA, fb, k2, p0);
-        tma_load_2d(sb + 4u * kTcABytes, &tmB1hi, fb, j * kTcBK, 0);
-        tma_load_2d(sb + 4u * kTcABytes + b_bytes, &tmB1lo, fb, j * kTcBK, 0);
-        tma_load_2d(sb + 4u * kTcABytes + 2u * b_bytes, &tmB2hi, fb, j * kTcBK, 0);
-        tma_load_2d(sb + 4u * kTcABytes + 3u * b_bytes, &tmB2lo, fb, j * kTcBK, 0);
-        ++issued;
-      }
-      // drain: every issued copy has landed before the block may exit
-      for (int j = (issued > kTcStages ? issued - kTcStages : 0); j < issued; ++j)
-        mbar_wait(smem_u32(&bar_full[j % kTcStages]), (j / kTcStages) & 1, err, 2);
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc =
-          (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(h >> 3) << 17) | ((uint32_t)(kTcBM >> 4) << 24);
-      bool ok = true;
-      for (int j = 0; j < nst && ok; ++j) {
-        const int st = j % kTcStages;
-        ok = mbar_wait(smem_u32(&bar_conv[st]), (j / kTcStages) & 1, err, 3);
-        if (!ok) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t sb = base + st * stage_bytes;
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          const uint32_t a_hi = sb + half * kTcABytes, a_lo = sb + (2 + half) * kTcABytes;
-          const uint32_t b_hi = sb + 4u * kTcABytes + (2 * half) * b_bytes, b_lo = b_hi + b_bytes;
-          const uint32_t d = tmem + (uint32_t)(half * h);
-#pragma unroll
-          for (int kk = 0; kk < kTcBK / 8; ++kk) {
-            const uint64_t ahi = smem_desc(a_hi + kk * 32), alo = smem_desc(a_lo + kk * 32);
-            const uint64_t bhi = smem_desc(b_hi + kk * 32), blo = smem_desc(b_lo + kk * 32);
-            mma_tf32(d, ahi, bhi, idesc, (j > 0 || kk > 0) ? 1u : 0u);
-            mma_tf32(d, ahi, blo, idesc, 1u);
-            mma_tf32(d, alo, bhi, idesc, 1u);
-          }
-        }
-        mma_commit(smem_u32(&bar_empty[st]));
-      }
-      mma_commit(smem_u32(&bar_acc));  // arrives once every MMA issued above has completed
-    }
-  } else {
-    // converters: thread t owns row t of the stage's A tiles
-    const int t = threadIdx.x - 64;
-    const int x = (t >> 1) & 3;  // swizzle pattern of this row
-    bool ok = true;
-    for (int j = 0; j < nst; ++j) {
-      const int st = j % kTcStages;
-      ok = mbar_wait(smem_u32(&bar_full[st]), (j / kTcStages) & 1, err, 4);
-      if (!ok) break;
-      unsigned char* sp = smem_raw + ((base + st * stage_bytes) - smem_u32(smem_raw)) + t * kTcRowBytes;
-      float4* a1 = reinterpret_cast<float4*>(sp);
-      float4* a2 = reinterpret_cast<float4*>(sp + kTcABytes);
-      float4* l1 = reinterpret_cast<float4*>(sp + 2 * kTcABytes);
-      float4* l2 = reinterpret_cast<float4*>(sp + 3 * kTcABytes);
-      if (BWD) {  // plain hi / lo split of both slabs, chunks visited in the swizzled order (no bank conflicts)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int pc = c ^ x;
-          float4 hh, ll;
-          split4(a1[pc], hh, ll);
-          a1[pc] = hh;
-          l1[pc] = ll;
-          split4(a2[pc], hh, ll);
-          a2[pc] = hh;
-          l2[pc] = ll;
-        }
-      } else {  // r[k] +- r[n-1-k]: logical chunk c of slab j pairs with logical chunk 3-c of the mirror slab,
-                // element e with element 3-e
-        float4 av[4], mv[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          av[c] = a1[c ^ x];
-          mv[c] = a2[(3 - c) ^ x];
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const float4 a = av[c], m = mv[c];
-          const float4 sum = make_float4(a.x + m.w, a.y + m.z, a.z + m.y, a.w + m.x);
-          const float4 dif = make_float4(a.x - m.w, a.y - m.z, a.z - m.y, a.w - m.x);
-          float4 hh, ll;
-          split4(sum, hh, ll);
-          a1[c ^ x] = hh;
-          l1[c ^ x] = ll;
-          split4(dif, hh, ll);
-          a2[c ^ x] = hh;
-          l2[c ^ x] = ll;
-        }
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      mbar_arrive(smem_u32(&bar_conv[st]));
-    }
-    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31, one row of the tile per thread; the
-    // tcgen05.ld below is warp-collective, so the go/no-go decision is made per warp
-    if (ok) ok = mbar_wait(smem_u32(&bar_acc), 0, err, 5);
-    if (__all_sync(0xffffffffu, ok)) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int q = warp % 4;
-      const int row = q * 32 + lane;
-      const int p = p0 + row;
-      float sa = 0.f, sb2 = 0.f;
-      int pa = 0, pb = 0;
-      if (SCALE && p < P) {
-        pa = p / nb;
-        pb = p - pa * nb;
-        sa = ly[pa];
-        sb2 = lx[pb];
-      }
-      const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16);
-      for (int c0 = 0; c0 < h; c0 += 16) {
-        uint32_t r1[16], r2[16];
-        tmem_ld16(lane_base + (uint32_t)c0, r1);
-        tmem_ld16(lane_base + (uint32_t)(h + c0), r2);
-        if (p < P) {
-#pragma unroll
-          for (int jj = 0; jj < 16; ++jj) {
-            const int m = c0 + jj;
-            const float v1 = __uint_as_float(r1[jj]), v2 = __uint_as_float(r2[jj]);
-            if (BWD) {  // cells m and n-1-m
-              out[(long long)m * P + p] = v1 + v2;
-              out[(long long)(n - 1 - m) * P + p] = v1 - v2;
-            } else if (SCALE) {  // symmetric mode m, antisymmetric mode h + m
-              const float s1 = (m == 0 && pa == 0 && pb == 0) ? 0.f : v1 * rcp_approx(lz_s[m] + sa + sb2);
-              out[(long long)m * P + p] = s1;
-              out[(long long)(h + m) * P + p] = v2 * rcp_approx(lz_s[h + m] + sa + sb2);
-            } else {
-              out[(long long)m * P + p] = v1;
-              out[(long long)(h + m) * P + p] = v2;
-            }
-          }
-        }
-      }
-    }
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (warp == 1) {
-    // if anything timed out, wait (bounded) for the MMAs issued so far before freeing their accumulator
-    if (*err != 0 && lane == 0) mbar_wait(smem_u32(&bar_acc), 0, err, 6);
-    __syncwarp();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256) : "memory");
-  }
-}
-
-// Persistent form of the same pass: one CTA per SM walks the tiles blockIdx.x, +gridDim.x, ...; the
+// One CTA per SM walks the 128-row tiles blockIdx.x, +gridDim.x, ... with all n outputs; per step two 16-wide K slabs
+// of A (slab j and its mirror n/16-1-j forward, slab j and j + n/32 backward) and the matching slabs of the two
+// half-size B matrices, 2 k-steps x 3 products x 2 halves of tcgen05.mma (M = 128, N = n/2, K = 8); the
 // shared-memory ring's phases run on across tiles (global stage counter), and two TMEM accumulators
 // (columns 0 and 256) let a separate epilogue warpgroup drain tile t while the MMAs of tile t + 1 run.
-// Warps: 0 TMA producer, 1 MMA issuer, 2-5 converters (row t of the A tiles), 6-9 epilogue.
+// Warps: 0 TMA producer, 1 MMA issuer, 2-9 converters (half a row of the A tiles each), 10-13 epilogue.
 // Barriers per step gi: full (TMA landed) -> conv (hi in place, lo in slot gi % 2) -> MMAs, whose commits
 // free the TMA stage (empty) and the remainder slot (lofree) for step gi + 4 and gi + 2.
-constexpr int kTcpThreads = 320;
+constexpr int kTcpConv = 256;  // converter threads
+constexpr int kTcpThreads = 64 + kTcpConv + 128;
 // Ring depths of the persistent pass: the TMA ring (A slabs by tensor copies, the step's B slabs by one
 // bulk copy of their pre-swizzled image) runs four stages deep; the converters' TF32 remainders of A live
 // in a separate two-slot ring, so the bytes in flight from DRAM per SM grow by a third within the same
 // shared memory.
 constexpr int kTcpStages = 4;
 constexpr int kTcpLoSlots = 2;
-constexpr bool kTcPersistent = true;  // the one-tile-per-CTA kernel above stays as the reference form
 
 template <bool SCALE, bool BWD>
 __global__ void __launch_bounds__(kTcpThreads, 1)
@@ -324,7 +119,7 @@ __global__ void __launch_bounds__(kTcpThreads, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < kTcpStages; ++s) {
       mbar_init(smem_u32(&bar_full[s]), 1);
-      mbar_init(smem_u32(&bar_conv[s]), 128);
+      mbar_init(smem_u32(&bar_conv[s]), kTcpConv);
       mbar_init(smem_u32(&bar_empty[s]), 1);
     }
     for (int s = 0; s < kTcpLoSlots; ++s) mbar_init(smem_u32(&bar_lofree[s]), 1);
@@ -427,9 +222,11 @@ __global__ void __launch_bounds__(kTcpThreads, 1)
       if (elect_one()) mma_commit(smem_u32(&bar_drain));
       mbar_wait(smem_u32(&bar_drain), 0, err, 16, kWaitLimit);
     }
-  } else if (warp < 6) {
-    // converters: thread t owns row t of every stage's A tiles and of every remainder slot
-    const int t = threadIdx.x - 64;
+  } else if (warp < 2 + kTcpConv / 32) {
+    // converters: threads t and t + 128 own row t of every stage's A tiles and of every remainder slot, one the
+    // 16-byte chunks 0 and 3, the other 1 and 2 (chunk c of a slab meets chunk 3 - c of its mirror, so neither reads
+    // what the other writes)
+    const int tt = threadIdx.x - 64, t = tt & 127, c0 = tt >> 7;
     const int x = (t >> 1) & 3;  // swizzle pattern of this row
     bool ok = true;
     for (int ti = 0; ti < my_tiles && ok; ++ti) {
@@ -452,38 +249,25 @@ __global__ void __launch_bounds__(kTcpThreads, 1)
         float4* a2 = reinterpret_cast<float4*>(sp + kTcABytes);
         float4* l1 = reinterpret_cast<float4*>(lp);
         float4* l2 = reinterpret_cast<float4*>(lp + kTcABytes);
-        if (BWD) {  // chunks in the swizzled order: no bank conflicts
+        const int pc[2] = {c0 ^ x, (3 - c0) ^ x};
+        const float4 av[2] = {a1[pc[0]], a1[pc[1]]}, mv[2] = {a2[pc[0]], a2[pc[1]]};
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const int pc = c ^ x;
-            float4 hh, ll;
-            split4(a1[pc], hh, ll);
-            a1[pc] = hh;
-            l1[pc] = ll;
-            split4(a2[pc], hh, ll);
-            a2[pc] = hh;
-            l2[pc] = ll;
+        for (int c = 0; c < 2; ++c) {
+          float4 hh, ll;
+          if (BWD) {
+            split4(av[c], hh, ll);
+            a1[pc[c]] = hh;
+            l1[pc[c]] = ll;
+            split4(mv[c], hh, ll);
+          } else {
+            const float4 a = av[c], m = mv[1 - c];
+            split4(make_float4(a.x + m.w, a.y + m.z, a.z + m.y, a.w + m.x), hh, ll);
+            a1[pc[c]] = hh;
+            l1[pc[c]] = ll;
+            split4(make_float4(a.x - m.w, a.y - m.z, a.z - m.y, a.w - m.x), hh, ll);
           }
-        } else {
-          float4 av[4], mv[4];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            av[c] = a1[c ^ x];
-            mv[c] = a2[(3 - c) ^ x];
-          }
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const float4 a = av[c], m = mv[c];
-            const float4 sum = make_float4(a.x + m.w, a.y + m.z, a.z + m.y, a.w + m.x);
-            const float4 dif = make_float4(a.x - m.w, a.y - m.z, a.z - m.y, a.w - m.x);
-            float4 hh, ll;
-            split4(sum, hh, ll);
-            a1[c ^ x] = hh;
-            l1[c ^ x] = ll;
-            split4(dif, hh, ll);
-            a2[c ^ x] = hh;
-            l2[c ^ x] = ll;
-          }
+          a2[pc[c]] = hh;
+          l2[pc[c]] = ll;
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive(smem_u32(&bar_conv[st]));
@@ -603,7 +387,6 @@ int encode_tensor_map(CUtensorMap* map, CUtensorMapDataType type, int rank, cons
 
 namespace {
 
-size_t tc_smem_bytes(int n) { return (size_t)kTcStages * (4 * kTcABytes + 4 * (size_t)(n / 2) * kTcRowBytes) + 1024; }
 size_t tcp_smem_bytes(int n) {
   return (size_t)kTcpStages * (2 * kTcABytes + 4 * (size_t)(n / 2) * kTcRowBytes) +
          (size_t)kTcpLoSlots * 2 * kTcABytes + 1024;
@@ -629,7 +412,6 @@ int tc_setup(fv_grid_s* g, const std::vector<double>* idx, const std::vector<dou
   FV_TRY(tc_host_operands(ns, idx, idc, op));
   const size_t total = op.buf.size();
   const std::vector<float>& hbuf = op.buf;
-  const auto& moff = op.moff;
   const auto& loff = op.loff;
   const auto& soff = op.soff;
   void* buf = nullptr;
@@ -641,25 +423,13 @@ int tc_setup(fv_grid_s* g, const std::vector<double>* idx, const std::vector<dou
   g->tc.buf = buf;
   FV_CUDA(cudaMemcpy(buf, hbuf.data(), total * sizeof(float), cudaMemcpyHostToDevice));
   for (int d = 0; d < 3; ++d) {
-    const int h = ns[d] / 2;
-    for (int j = 0; j < 8; ++j) FV_TRY(encode(&g->tc.B[d][j], (const float*)buf + moff[d][j], h, h, h));
     g->tc.lam[d] = (const float*)buf + loff[d];
     for (int dir = 0; dir < 2; ++dir) g->tc.Bsw[d][dir] = (const unsigned char*)((const float*)buf + soff[d][dir]);
   }
-  const int smem_max = (int)tc_smem_bytes(256);
-  FV_CUDA(cudaFuncSetAttribute(k_transform_tc<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
-  FV_CUDA(cudaFuncSetAttribute(k_transform_tc<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
-  FV_CUDA(cudaFuncSetAttribute(k_transform_tc<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
   const int smemp_max = (int)tcp_smem_bytes(256);
   FV_CUDA(cudaFuncSetAttribute(k_transform_tcp<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemp_max));
   FV_CUDA(cudaFuncSetAttribute(k_transform_tcp<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemp_max));
   FV_CUDA(cudaFuncSetAttribute(k_transform_tcp<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemp_max));
-  {
-    int dev = 0, sms = 0;
-    FV_CUDA(cudaGetDevice(&dev));
-    FV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    g->tc.sms = sms;
-  }
   g->tc.ready = true;
   return FV_OK;
 }
@@ -672,7 +442,7 @@ int tc_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const float*
             int nvec) {
   const int n = (axis == 0) ? g->nx : (axis == 1) ? g->ny : g->nz;
   const long long P = (long long)na * nb;
-  if (nvec < 1 || (nvec > 1 && !(kTcPersistent && g->tc.sms > 0)) || P * nvec > (1LL << 30)) {
+  if (nvec < 1 || P * nvec > (1LL << 30)) {
     set_error("tc_pass: batch of fields not supported here");
     return FV_EINVAL;
   }
@@ -680,14 +450,11 @@ int tc_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const float*
   CUtensorMap tmA;
   FV_TRY(encode(&tmA, in, Ptot, n, kTcBM));
   const long long ntiles = (Ptot + kTcBM - 1) / kTcBM;
-  const dim3 grid((unsigned)ntiles);
-  const size_t smem = tc_smem_bytes(n);
-  const CUtensorMap* B = g->tc.B[axis] + (bwd ? 4 : 0);
   ProfScope ps(g, PROF_TRANSFORM_TC);
-  if (kTcPersistent && g->tc.sms > 0) {
+  {
     const size_t smemp = tcp_smem_bytes(n);
     const unsigned char* bsw = g->tc.Bsw[axis][bwd ? 1 : 0];
-    const dim3 pgrid((unsigned)std::min<long long>(ntiles, g->tc.sms));
+    const dim3 pgrid((unsigned)std::min<long long>(ntiles, g->sms));
     if (bwd)
       k_transform_tcp<false, true><<<pgrid, kTcpThreads, smemp, g->stream>>>(
           tmA, bsw, out, (int)P, (int)Ptot, n, nullptr, nullptr, nullptr, nb, g->ws.err, wait_spins(g));
@@ -701,17 +468,6 @@ int tc_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const float*
     FV_CUDA(cudaGetLastError());
     return FV_OK;
   }
-  if (bwd)
-    k_transform_tc<false, true><<<grid, kTcThreads, smem, g->stream>>>(tmA, B[0], B[1], B[2], B[3], out, (int)P, n,
-                                                                       nullptr, nullptr, nullptr, nb, g->ws.err);
-  else if (scale)
-    k_transform_tc<true, false><<<grid, kTcThreads, smem, g->stream>>>(
-        tmA, B[0], B[1], B[2], B[3], out, (int)P, n, g->tc.lam[0], g->tc.lam[1], g->tc.lam[2], nb, g->ws.err);
-  else
-    k_transform_tc<false, false><<<grid, kTcThreads, smem, g->stream>>>(tmA, B[0], B[1], B[2], B[3], out, (int)P, n,
-                                                                        nullptr, nullptr, nullptr, nb, g->ws.err);
-  FV_CUDA(cudaGetLastError());
-  return FV_OK;
 }
 
 }  // namespace fv
