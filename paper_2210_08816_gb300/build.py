@@ -30,7 +30,7 @@ def _nvcc() -> str:
 
 
 def _headers():
-    return [os.path.join(CSRC, "fv_internal.h"), os.path.join(CSRC, "tcgen05.cuh"), os.path.join(ROOT, "include", "cube_fv.h")]
+    return [os.path.join(CSRC, "fv_internal.h"), os.path.join(CSRC, "tcgen05.cuh"), os.path.join(CSRC, "launch.cuh"), os.path.join(ROOT, "include", "cube_fv.h")]
 
 
 def _stale(obj: str, deps) -> bool:

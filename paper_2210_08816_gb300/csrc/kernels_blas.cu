@@ -12,6 +12,7 @@
 #include <string>
 
 #include "fv_internal.h"
+#include "launch.cuh"
 
 namespace fv {
 namespace {
@@ -94,6 +95,11 @@ __device__ __forceinline__ double dot_chunk<float>(const float* __restrict__ a, 
 template <typename R>
 __global__ void __launch_bounds__(kThreads) k_dot_partial(const R* __restrict__ a, const R* __restrict__ b, size_t n,
                                                            double* __restrict__ part) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  a += ready0;
+  b += ready0;
+  part += ready0;
   size_t s, e;
   chunk_of(n, s, e);
   double acc[1] = {dot_chunk<R>(a, b, s, e)};
@@ -104,6 +110,10 @@ __global__ void __launch_bounds__(kThreads) k_dot_partial(const R* __restrict__ 
 
 template <typename R>
 __global__ void __launch_bounds__(kThreads) k_maxabs_partial(const R* __restrict__ a, size_t n, double* __restrict__ part) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  a += ready0;
+  part += ready0;
   size_t s, e;
   chunk_of(n, s, e);
   R m = R(0);
@@ -125,6 +135,11 @@ template <typename R>
 __global__ void __launch_bounds__(kThreads) k_multidot_partial(const R* __restrict__ V, size_t ldv, int m,
                                                                 const R* __restrict__ w, size_t n,
                                                                 double* __restrict__ part) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  V += ready0;
+  if (w) w += ready0;
+  part += ready0;
   size_t s, e;
   chunk_of(n, s, e);
   const int i0 = blockIdx.y * 8;
@@ -159,6 +174,10 @@ __global__ void __launch_bounds__(kThreads) k_multidot_partial(const R* __restri
 // final pass: out[slot + blockIdx.x] = reduce(part[blockIdx.x * np .. + np])
 template <bool MAX>
 __global__ void __launch_bounds__(1024) k_finish(const double* __restrict__ part, int np, double* __restrict__ out) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  part += ready0;
+  out += ready0;
   __shared__ double sh[32];
   const double* p = part + (size_t)blockIdx.x * np;
   double v = 0.0;
@@ -178,6 +197,10 @@ __global__ void __launch_bounds__(1024) k_finish(const double* __restrict__ part
 // out[b] = sum of part[b * chunk .. min(np, (b + 1) * chunk)) in a fixed order
 __global__ void __launch_bounds__(1024) k_finish_chunks(const double* __restrict__ part, int np, int chunk,
                                                          double* __restrict__ out) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  part += ready0;
+  out += ready0;
   __shared__ double sh[32];
   const int s = blockIdx.x * chunk, e = min(np, s + chunk);
   double v = 0.0;
@@ -195,6 +218,13 @@ __global__ void __launch_bounds__(1024) k_finish_chunks(const double* __restrict
 template <typename R>
 __global__ void k_lincomb(size_t n, int nvec, R c0, R c1, R c2, R c3, const R* x0, const R* x1, const R* x2,
                           const R* x3, R* out) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  x0 += ready0;
+  x1 += ready0;
+  x2 += ready0;
+  x3 += ready0;
+  out += ready0;
   for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
     R r = c0 * x0[t];
     if (nvec > 1) r = fma(c1, x1[t], r);
@@ -207,6 +237,11 @@ __global__ void k_lincomb(size_t n, int nvec, R c0, R c1, R c2, R c3, const R* x
 template <typename R>
 __global__ void k_subtract_basis(const R* __restrict__ V, size_t ldv, int m, const double* __restrict__ h, R* w,
                                  size_t n) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  V += ready0;
+  h += ready0;
+  if (w) w += ready0;
   __shared__ R hs[256];
   for (int i = threadIdx.x; i < m; i += blockDim.x) hs[i] = (R)h[i];
   __syncthreads();
@@ -219,6 +254,10 @@ __global__ void k_subtract_basis(const R* __restrict__ V, size_t ldv, int m, con
 
 template <typename S, typename D>
 __global__ void k_convert(size_t n, const S* __restrict__ src, D* __restrict__ dst) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  src += ready0;
+  dst += ready0;
   for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x)
     dst[t] = (D)src[t];
 }
@@ -268,9 +307,9 @@ inline int stream_grid(size_t n) {
 template <typename R>
 int launch_dot(const fv_grid_s* g, const R* a, const R* b, size_t n, int slot) {
   ProfScope ps(g, PROF_REDUCE);
-  k_dot_partial<R><<<kReduceBlocks, kThreads, 0, g->stream>>>(a, b, n, g->ws.partials);
+  launch(k_dot_partial<R>, kReduceBlocks, kThreads, 0, g->stream, a, b, n, g->ws.partials);
   FV_CUDA(cudaGetLastError());
-  k_finish<false><<<1, 1024, 0, g->stream>>>(g->ws.partials, kReduceBlocks, g->ws.scalars + slot);
+  launch(k_finish<false>, 1, 1024, 0, g->stream, g->ws.partials, kReduceBlocks, g->ws.scalars + slot);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }
@@ -278,9 +317,9 @@ int launch_dot(const fv_grid_s* g, const R* a, const R* b, size_t n, int slot) {
 template <typename R>
 int launch_maxabs(const fv_grid_s* g, const R* a, size_t n, int slot) {
   ProfScope ps(g, PROF_REDUCE);
-  k_maxabs_partial<R><<<kReduceBlocks, kThreads, 0, g->stream>>>(a, n, g->ws.partials);
+  launch(k_maxabs_partial<R>, kReduceBlocks, kThreads, 0, g->stream, a, n, g->ws.partials);
   FV_CUDA(cudaGetLastError());
-  k_finish<true><<<1, 1024, 0, g->stream>>>(g->ws.partials, kReduceBlocks, g->ws.scalars + slot);
+  launch(k_finish<true>, 1, 1024, 0, g->stream, g->ws.partials, kReduceBlocks, g->ws.scalars + slot);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }
@@ -290,9 +329,9 @@ int launch_multidot(const fv_grid_s* g, const R* V, size_t ldv, int m, const R* 
   if (m <= 0) return FV_OK;
   dim3 grid(kReduceBlocks, (m + 7) / 8);
   ProfScope ps(g, PROF_REDUCE);
-  k_multidot_partial<R><<<grid, kThreads, 0, g->stream>>>(V, ldv, m, w, n, g->ws.partials);
+  launch(k_multidot_partial<R>, grid, kThreads, 0, g->stream, V, ldv, m, w, n, g->ws.partials);
   FV_CUDA(cudaGetLastError());
-  k_finish<false><<<m, 1024, 0, g->stream>>>(g->ws.partials, kReduceBlocks, g->ws.scalars + slot);
+  launch(k_finish<false>, m, 1024, 0, g->stream, g->ws.partials, kReduceBlocks, g->ws.scalars + slot);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }
@@ -300,7 +339,7 @@ int launch_multidot(const fv_grid_s* g, const R* V, size_t ldv, int m, const R* 
 template <typename R>
 int launch_lincomb(const fv_grid_s* g, size_t n, int nvec, const double* c, const R* const* x, R* out) {
   ProfScope ps(g, PROF_VECTOR);
-  k_lincomb<R><<<stream_grid(n), 256, 0, g->stream>>>(n, nvec, (R)c[0], (R)(nvec > 1 ? c[1] : 0.0),
+  launch(k_lincomb<R>, stream_grid(n), 256, 0, g->stream, n, nvec, (R)c[0], (R)(nvec > 1 ? c[1] : 0.0),
                                                        (R)(nvec > 2 ? c[2] : 0.0), (R)(nvec > 3 ? c[3] : 0.0),
                                                        x[0], nvec > 1 ? x[1] : x[0],
                                                        nvec > 2 ? x[2] : x[0], nvec > 3 ? x[3] : x[0], out);
@@ -313,20 +352,20 @@ int launch_subtract_basis(const fv_grid_s* g, const R* V, size_t ldv, int m, con
   if (m <= 0) return FV_OK;
   if (m > 256) return FV_EINVAL;
   ProfScope ps(g, PROF_VECTOR);
-  k_subtract_basis<R><<<stream_grid(n), 256, 0, g->stream>>>(V, ldv, m, h, w, n);
+  launch(k_subtract_basis<R>, stream_grid(n), 256, 0, g->stream, V, ldv, m, h, w, n);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }
 
 int launch_convert(const fv_grid_s* g, size_t n, const double* src, float* dst) {
   ProfScope ps(g, PROF_VECTOR);
-  k_convert<double, float><<<stream_grid(n), 256, 0, g->stream>>>(n, src, dst);
+  launch(k_convert<double, float>, stream_grid(n), 256, 0, g->stream, n, src, dst);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }
 int launch_convert(const fv_grid_s* g, size_t n, const float* src, double* dst) {
   ProfScope ps(g, PROF_VECTOR);
-  k_convert<float, double><<<stream_grid(n), 256, 0, g->stream>>>(n, src, dst);
+  launch(k_convert<float, double>, stream_grid(n), 256, 0, g->stream, n, src, dst);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }
@@ -343,11 +382,11 @@ int launch_sum_partials(const fv_grid_s* g, int np, int slot) {
   ProfScope ps(g, PROF_REDUCE);
   if (np > 4096) {  // two levels: 64 fixed chunks, then their sums (deterministic order)
     const int chunk = (np + 63) / 64;
-    k_finish_chunks<<<64, 1024, 0, g->stream>>>(g->ws.partials, np, chunk, g->ws.partials + kPartialSlots - 64);
+    launch(k_finish_chunks, 64, 1024, 0, g->stream, g->ws.partials, np, chunk, g->ws.partials + kPartialSlots - 64);
     FV_CUDA(cudaGetLastError());
-    k_finish<false><<<1, 1024, 0, g->stream>>>(g->ws.partials + kPartialSlots - 64, 64, g->ws.scalars + slot);
+    launch(k_finish<false>, 1, 1024, 0, g->stream, g->ws.partials + kPartialSlots - 64, 64, g->ws.scalars + slot);
   } else {
-    k_finish<false><<<1, 1024, 0, g->stream>>>(g->ws.partials, np, g->ws.scalars + slot);
+    launch(k_finish<false>, 1, 1024, 0, g->stream, g->ws.partials, np, g->ws.scalars + slot);
   }
   FV_CUDA(cudaGetLastError());
   return FV_OK;

@@ -11,6 +11,7 @@
 #include <algorithm>
 
 #include "fv_internal.h"
+#include "launch.cuh"
 
 namespace fv {
 namespace {
@@ -44,6 +45,10 @@ __device__ __forceinline__ double block_sum(double v) {
 // cells.  (64^3, both diagnostics with their sums: four launches, 77 us of kernels; now two.)
 __global__ void __launch_bounds__(kThreads) k_diag_partial(Geo<double> g, const double* __restrict__ q, int be,
                                                             double* __restrict__ part) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  q += ready0;
+  part += ready0;
   __shared__ double vol[2][kMaxN];
   const int nx = g.n[0], ny = g.n[1], rows = g.n[1] * g.n[2];
   double acc = 0.0;
@@ -81,6 +86,10 @@ __global__ void __launch_bounds__(kThreads) k_diag_partial(Geo<double> g, const 
 // out[0] = sum of part[0 .. be), out[1] = sum of part[be .. be + bn), in a fixed order
 __global__ void __launch_bounds__(kThreads) k_diag_finish(const double* __restrict__ part, int be, int bn,
                                                            double* __restrict__ out) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  part += ready0;
+  out += ready0;
   const double* p = part + (blockIdx.x == 0 ? 0 : be);
   const int n = blockIdx.x == 0 ? be : bn;
   double v = 0.0;
@@ -96,9 +105,9 @@ int launch_diagnostics(const fv_grid_s* g, const double* q, int slot) {
   ProfScope ps(g, PROF_REDUCE);
   const int be = std::min(kReduceBlocks, (3 * g->ny * g->nz + 31) / 32);  // four rows per warp
   const int bn = std::min(kReduceBlocks, (g->ny * g->nz + kThreads - 1) / kThreads);
-  k_diag_partial<<<be + bn, kThreads, 0, g->stream>>>(g->geo64, q, be, g->ws.partials);
+  launch(k_diag_partial, be + bn, kThreads, 0, g->stream, g->geo64, q, be, g->ws.partials);
   FV_CUDA(cudaGetLastError());
-  k_diag_finish<<<2, kThreads, 0, g->stream>>>(g->ws.partials, be, bn, g->ws.scalars + slot);
+  launch(k_diag_finish, 2, kThreads, 0, g->stream, g->ws.partials, be, bn, g->ws.scalars + slot);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }

@@ -39,6 +39,7 @@
 #include <type_traits>
 
 #include "fv_internal.h"
+#include "launch.cuh"
 #include "tcgen05.cuh"
 
 namespace fv {
@@ -228,6 +229,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
   const uint32_t base = smem_u32(smem);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int n = t.n, P = t.P, h = (n + 1) / 2, ha = n / 2;
+  pdl_begin();
   const int u0 = (int)((long long)t.units * blockIdx.x / gridDim.x);
   const int u1 = (int)((long long)t.units * (blockIdx.x + 1) / gridDim.x);
 
@@ -253,6 +255,9 @@ __global__ void __launch_bounds__(kDgThreads, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
+  const unsigned ready0 = pdl_wait();
+  in += ready0;
+  out += ready0;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -645,9 +650,9 @@ int digit_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int
   const unsigned grid = (unsigned)std::min<long long>(units, g->sms);
   ProfScope ps(g, PROF_TRANSFORM_TC);
   if (bwd)
-    k_digit_pass<R, true><<<grid, kDgThreads, digit_smem<R>(), g->stream>>>(t, in, out);
+    launch(k_digit_pass<R, true>, grid, kDgThreads, digit_smem<R>(), g->stream, t, in, out);
   else
-    k_digit_pass<R, false><<<grid, kDgThreads, digit_smem<R>(), g->stream>>>(t, in, out);
+    launch(k_digit_pass<R, false>, grid, kDgThreads, digit_smem<R>(), g->stream, t, in, out);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }

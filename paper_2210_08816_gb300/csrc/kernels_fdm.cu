@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "fv_internal.h"
+#include "launch.cuh"
 
 namespace fv {
 namespace {
@@ -45,6 +46,10 @@ __global__ void __launch_bounds__(256) k_transform(PassArgs t, const R* __restri
                                                     R* __restrict__ out, const R* __restrict__ lx,
                                                     const R* __restrict__ ly, const R* __restrict__ lz) {
   using T = TileCfg<R>;
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  in += ready0;
+  out += ready0;
   constexpr int BM = T::BM, BN = T::BN, BK = T::BK, TM = T::TM, TN = T::TN;
   __shared__ R As[BK][BM + 1];
   __shared__ R Bs[BK][BN + 1];
@@ -131,6 +136,10 @@ struct HalfArgs {
 template <typename R, bool BWD, int U>
 __global__ void __launch_bounds__(128) k_half(const __grid_constant__ HalfArgs<R> t, const R* __restrict__ in,
                                                R* __restrict__ out) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  in += ready0;
+  out += ready0;
   constexpr int UB = 4 * U, V = 16 / sizeof(R);
   using Vec = typename std::conditional<sizeof(R) == 4, float4, double2>::type;
   __shared__ R As[2][kHalfK][33];
@@ -277,15 +286,15 @@ int half_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int 
   const int U = rows * ((h + 15) / 16) >= 2 * g->sms ? 4 : rows * ((h + 7) / 8) >= 2 * g->sms ? 2 : 1;
   const dim3 grid((t.P + 31) / 32, (h + 4 * U - 1) / (4 * U), nf);
   ProfScope ps(g, PROF_TRANSFORM);
-  if (bwd) {
-    if (U == 4) k_half<R, true, 4><<<grid, 128, 0, g->stream>>>(t, in, out);
-    else if (U == 2) k_half<R, true, 2><<<grid, 128, 0, g->stream>>>(t, in, out);
-    else k_half<R, true, 1><<<grid, 128, 0, g->stream>>>(t, in, out);
-  } else {
-    if (U == 4) k_half<R, false, 4><<<grid, 128, 0, g->stream>>>(t, in, out);
-    else if (U == 2) k_half<R, false, 2><<<grid, 128, 0, g->stream>>>(t, in, out);
-    else k_half<R, false, 1><<<grid, 128, 0, g->stream>>>(t, in, out);
-  }
+  void (*k)(HalfArgs<R>, const R*, R*);
+  if (bwd)
+    k = U == 4 ? k_half<R, true, 4> : U == 2 ? k_half<R, true, 2> : k_half<R, true, 1>;
+  else
+    k = U == 4 ? k_half<R, false, 4> : U == 2 ? k_half<R, false, 2> : k_half<R, false, 1>;
+  if constexpr (sizeof(R) == 8)
+    launch_spread(k, grid, 128, 0, g->stream, t, in, out);
+  else
+    launch(k, grid, 128, 0, g->stream, t, in, out);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }
@@ -338,7 +347,7 @@ int pass_ops(const fv_grid_s* g, const R* M, int na, int nb, int K, const R* in,
   t.shift = shift;
   dim3 grid((t.P + T::BM - 1) / T::BM, (t.nm + T::BN - 1) / T::BN, nvec);
   ProfScope ps(g, PROF_TRANSFORM);
-  k_transform<R><<<grid, 256, 0, g->stream>>>(t, in, M, out, lam[0], lam[1], lam[2]);
+  launch_spread(k_transform<R>, grid, 256, 0, g->stream, t, in, M, out, lam[0], lam[1], lam[2]);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }

@@ -30,6 +30,7 @@
 #include <cstring>
 
 #include "fv_internal.h"
+#include "launch.cuh"
 #include "tcgen05.cuh"
 
 namespace fv {
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(kFxThreads, 1)
   const R* __restrict__ q = t.q;
   const R* __restrict__ v = t.v + (size_t)vec * 4 * N;
   R* __restrict__ out = t.out + (size_t)vec * 4 * N;
+  pdl_begin();
 
   // roles: cells; warp 8: the row past the tile's high y edge (y fluxes only); warp 9: the column past its high x
   // edge (x fluxes only)
@@ -123,6 +125,10 @@ __global__ void __launch_bounds__(kFxThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  const unsigned ready0 = pdl_wait();
+  q += ready0;
+  if (v) v += ready0;
+  out += ready0;
 
   // plane kk goes to slot (kk - k0 + 1) mod 3; planes outside the domain are not copied (they read as zero)
   auto issue = [&](int kk) {
@@ -428,7 +434,7 @@ int launch_flux(const fv_grid_s* g, double Gr, double sigma, const double* q, co
   }
   const dim3 grid((g->nx + pl.tx - 1) / pl.tx, (g->ny + pl.ty - 1) / pl.ty, t.nch * nvec);
   ProfScope ps(g, PROF_STENCIL);
-  k_flux<R, MODE><<<grid, kFxThreads, smem, g->stream>>>(tq, tv, t);
+  launch_spread(k_flux<R, MODE>, grid, kFxThreads, smem, g->stream, tq, tv, t);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }

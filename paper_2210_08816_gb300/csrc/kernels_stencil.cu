@@ -4,6 +4,7 @@
 #include <cstring>
 
 #include "fv_internal.h"
+#include "launch.cuh"
 
 namespace fv {
 namespace {
@@ -228,12 +229,17 @@ __global__ void __launch_bounds__(kTX * kTY, 3)
   out += (size_t)vec * 4 * N;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const int kend = min(k0 + zc, nz);
+  pdl_begin();
   if (use_tma && tid == 0) {
     for (int s = 0; s < kRing; ++s)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar[s])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  const unsigned ready0 = pdl_wait();
+  q += ready0;
+  if (v) v += ready0;
+  out += ready0;
   auto issue_plane = [&](int kk) {
     R* slot = sm + ((kk + kRing) % kRing) * NA * kPL;
     const bool kin = (kk >= 0 && kk < nz);
@@ -340,6 +346,10 @@ __global__ void __launch_bounds__(kTX * kTY, 3)
 template <typename R>
 __global__ void __launch_bounds__(256) k_divergence(Geo<R> g, int N, const R* __restrict__ vel,
                                                      R* __restrict__ rhs) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  vel += ready0;
+  rhs += ready0;
   Cell<R> c;
   if (!cell_of_thread(g, c)) return;
   R acc = R(0);
@@ -367,6 +377,13 @@ template <typename R>
 __global__ void __launch_bounds__(256) k_correct(Geo<R> g, int N, const R* Y, const R* __restrict__ phi,
                                                   R alpha, const R* v, R beta, const R* w, R gamma, R* out,
                                                   double* __restrict__ part) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  Y += ready0;
+  phi += ready0;
+  if (v) v += ready0;
+  if (w) w += ready0;
+  out += ready0;
   Cell<R> c;
   const bool act = cell_of_thread(g, c);
   float shi = 0.f, slo = 0.f;  // FP32 data
@@ -442,6 +459,10 @@ __device__ __forceinline__ float4 zero4() { return make_float4(0.f, 0.f, 0.f, 0.
 // blockIdx.z = z-block + nzc * vector (states of 4N, rhs fields of N, one after another)
 __global__ void __launch_bounds__(256) k_divergence4(Geo<float> g, int N, const float* __restrict__ vel,
                                                       float* __restrict__ rhs, int nzc) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  vel += ready0;
+  rhs += ready0;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2], pl = nx * ny;
   const int lane = threadIdx.x;
   const int vec = (int)blockIdx.z / nzc;
@@ -496,6 +517,13 @@ __device__ __forceinline__ void acc_sq(float& hi, float& lo, float r) {
 __global__ void __launch_bounds__(256) k_correct4(Geo<float> g, int N, const float* Y, const float* __restrict__ phi,
                                                    float alpha, const float* v, float beta, const float* w,
                                                    float gamma, float* out, double* __restrict__ part, int nzc) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  Y += ready0;
+  phi += ready0;
+  if (v) v += ready0;
+  if (w) w += ready0;
+  out += ready0;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2], pl = nx * ny;
   const int lane = threadIdx.x;
   // blockIdx.z = z-block + nzc * vector (Y, v, w, out: states of 4N; phi: fields of N, one after another)
@@ -660,7 +688,7 @@ int launch_stencil_z(const fv_grid_s* g, double Gr, double sigma, const R* q, co
   }
   dim3 grid(gx, gy, nch * nvec);
   ProfScope ps(g, PROF_STENCIL);
-  k_stencil_z<R><<<grid, kTX * kTY, smem, g->stream>>>(tq, tv, use_tma, g->ws.err, wait_spins(g), geo_of<R>(g), (int)g->N,
+  launch(k_stencil_z<R>, grid, kTX * kTY, smem, g->stream, tq, tv, use_tma, g->ws.err, wait_spins(g), geo_of<R>(g), (int)g->N,
                                                              (R)Gr, (R)(1.0 / g->Pr), (R)sigma, q, v, out, zc, nch);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
@@ -703,13 +731,13 @@ int launch_divergence(const fv_grid_s* g, const R* vel, R* rhs, int nvec) {
         return FV_EINVAL;
       }
       qg.z = nzc * nvec;
-      k_divergence4<<<qg, dim3(32, 8), 0, g->stream>>>(g->geo32, (int)g->N, vel, rhs, nzc);
+      launch(k_divergence4, qg, dim3(32, 8), 0, g->stream, g->geo32, (int)g->N, vel, rhs, nzc);
       FV_CUDA(cudaGetLastError());
       return FV_OK;
     }
   }
   for (int i = 0; i < nvec; ++i) {
-    k_divergence<R><<<grid, block, 0, g->stream>>>(geo_of<R>(g), (int)g->N, vel + (size_t)i * 4 * g->N,
+    launch(k_divergence<R>, grid, block, 0, g->stream, geo_of<R>(g), (int)g->N, vel + (size_t)i * 4 * g->N,
                                                    rhs + (size_t)i * g->N);
     FV_CUDA(cudaGetLastError());
   }
@@ -736,7 +764,7 @@ int launch_correct_block(const fv_grid_s* g, const R* Y, const R* phi, const R* 
     }
     qg.z = nzc * nvec;
     ProfScope ps(g, PROF_CORRECT);
-    k_correct4<<<qg, dim3(32, 8), 0, g->stream>>>(g->geo32, (int)g->N, Y, phi, 1.0f, v, (float)beta, nullptr, 0.0f,
+    launch(k_correct4, qg, dim3(32, 8), 0, g->stream, g->geo32, (int)g->N, Y, phi, 1.0f, v, (float)beta, nullptr, 0.0f,
                                                   out, nullptr, nzc);
     FV_CUDA(cudaGetLastError());
   }
@@ -757,12 +785,12 @@ int launch_correct(const fv_grid_s* g, const R* Y, const R* phi, double alpha, c
     ProfScope ps(g, PROF_CORRECT);
     if constexpr (sizeof(R) == 4) {
       if (quad)
-        k_correct4<<<grid, dim3(32, 8), 0, g->stream>>>(g->geo32, (int)g->N, Y, phi, (float)alpha, v, (float)beta, w,
+        launch(k_correct4, grid, dim3(32, 8), 0, g->stream, g->geo32, (int)g->N, Y, phi, (float)alpha, v, (float)beta, w,
                                                         (float)gamma, out, want ? g->ws.partials : nullptr,
                                                         (int)grid.z);
     }
     if (!quad)
-      k_correct<R><<<grid, block, 0, g->stream>>>(geo_of<R>(g), (int)g->N, Y, phi, (R)alpha, v, (R)beta, w,
+      launch(k_correct<R>, grid, block, 0, g->stream, geo_of<R>(g), (int)g->N, Y, phi, (R)alpha, v, (R)beta, w,
                                                   (R)gamma, out, want ? g->ws.partials : nullptr);
     FV_CUDA(cudaGetLastError());
   }

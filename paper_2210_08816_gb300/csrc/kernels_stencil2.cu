@@ -12,6 +12,7 @@
 #include <cstring>
 
 #include "fv_internal.h"
+#include "launch.cuh"
 
 namespace fv {
 namespace {
@@ -253,12 +254,15 @@ __global__ void __launch_bounds__(kPX / 2 * kPY, 2)
   if (BLOCK) out += (size_t)vec * 4 * N;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const int kend = min(k0 + zc, nz);
+  pdl_begin();
   if (tid == 0) {
     for (int s2 = 0; s2 < kPRing; ++s2)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr2(&bar[s2])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  const unsigned ready0 = pdl_wait();
+  out += ready0;
   auto issue_plane = [&](int kk) {
     float* slot = sm + ((kk + kPRing) % kPRing) * kPNA * kPL2;
     const uint32_t b = smem_addr2(&bar[(kk + kPRing) % kPRing]);
@@ -381,10 +385,10 @@ int launch_stencil_pair(const fv_grid_s* g, double Gr, double sigma, const float
   dim3 grid(g->nx / kPX, (g->ny + kPY - 1) / kPY, nch * nvec);
   ProfScope ps(g, PROF_STENCIL);
   if (nvec > 1)
-    k_stencil_pair<true><<<grid, kPX / 2 * kPY, smem, g->stream>>>(tq, tv, g->ws.err, wait_spins(g), g->geo32, (int)g->N, (float)Gr,
+    launch(k_stencil_pair<true>, grid, kPX / 2 * kPY, smem, g->stream, tq, tv, g->ws.err, wait_spins(g), g->geo32, (int)g->N, (float)Gr,
                                                                  (float)(1.0 / g->Pr), (float)sigma, out, zc, nch);
   else
-    k_stencil_pair<false><<<grid, kPX / 2 * kPY, smem, g->stream>>>(tq, tv, g->ws.err, wait_spins(g), g->geo32, (int)g->N, (float)Gr,
+    launch(k_stencil_pair<false>, grid, kPX / 2 * kPY, smem, g->stream, tq, tv, g->ws.err, wait_spins(g), g->geo32, (int)g->N, (float)Gr,
                                                                   (float)(1.0 / g->Pr), (float)sigma, out, zc, nch);
   FV_CUDA(cudaGetLastError());
   return FV_OK;

@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "fv_internal.h"
+#include "launch.cuh"
 #include "tcgen05.cuh"
 
 namespace fv {
@@ -114,6 +115,7 @@ __global__ void __launch_bounds__(kTcpThreads, 1)
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int nst = n / (2 * kTcBK);
   const int ntiles = (Ptot + kTcBM - 1) / kTcBM;
+  pdl_begin();
   const int my_tiles = (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
 
   if (threadIdx.x == 0) {
@@ -141,6 +143,8 @@ __global__ void __launch_bounds__(kTcpThreads, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
+  const unsigned ready0 = pdl_wait();
+  out += ready0;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -456,14 +460,14 @@ int tc_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const float*
     const unsigned char* bsw = g->tc.Bsw[axis][bwd ? 1 : 0];
     const dim3 pgrid((unsigned)std::min<long long>(ntiles, g->sms));
     if (bwd)
-      k_transform_tcp<false, true><<<pgrid, kTcpThreads, smemp, g->stream>>>(
+      launch(k_transform_tcp<false, true>, pgrid, kTcpThreads, smemp, g->stream, 
           tmA, bsw, out, (int)P, (int)Ptot, n, nullptr, nullptr, nullptr, nb, g->ws.err, wait_spins(g));
     else if (scale)
-      k_transform_tcp<true, false><<<pgrid, kTcpThreads, smemp, g->stream>>>(
+      launch(k_transform_tcp<true, false>, pgrid, kTcpThreads, smemp, g->stream, 
           tmA, bsw, out, (int)P, (int)Ptot, n, g->tc.lam[0], g->tc.lam[1], g->tc.lam[2], nb, g->ws.err,
           wait_spins(g));
     else
-      k_transform_tcp<false, false><<<pgrid, kTcpThreads, smemp, g->stream>>>(
+      launch(k_transform_tcp<false, false>, pgrid, kTcpThreads, smemp, g->stream, 
           tmA, bsw, out, (int)P, (int)Ptot, n, nullptr, nullptr, nullptr, nb, g->ws.err, wait_spins(g));
     FV_CUDA(cudaGetLastError());
     return FV_OK;

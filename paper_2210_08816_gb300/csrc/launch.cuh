@@ -1,0 +1,57 @@
+// Launches with programmatic stream serialisation: a kernel may start (block scheduling, barrier and tensor-memory
+// set-up, metrics) while its predecessor on the stream drains, and waits for the predecessor's results where it first
+// needs them.  Chains of short kernels are what this is for: a 64^3 J.v + projection is nine launches of 4-9 us.
+//
+// A kernel launched this way calls pdl_begin() first and pdl_wait() before its first access to anything a predecessor
+// writes or reads; every thread waits, so that a kernel never completes before its predecessor.  Read-only loads may
+// be moved by the compiler across a memory barrier, so pdl_wait() returns a zero that the compiler cannot know, to be
+// added to each pointer to such data: the addresses then depend on the wait.  (Passing the pointers themselves through
+// an asm statement loses their address space and __restrict__: 32^3 FP64 products 71 -> 101 us.)  Data written once at
+// grid creation (metrics, matrices) may be read before.
+#pragma once
+#include <cuda_runtime.h>
+
+namespace fv {
+
+__device__ __forceinline__ void pdl_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ unsigned pdl_wait() {
+  unsigned zero;
+  asm volatile("griddepcontrol.wait;\n mov.u32 %0, 0;" : "=r"(zero)::"memory");
+  return zero;
+}
+
+template <typename T>
+struct same_type {
+  using type = T;
+};
+
+template <typename... P>
+inline void launch(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                   typename same_type<P>::type... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = stream;
+  c.attrs = &at;
+  c.numAttrs = overlap ? 1 : 0;
+  cudaLaunchKernelEx(&c, kernel, args...);
+}
+template <typename... P>
+inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                   typename same_type<P>::type... args) {
+  launch(true, kernel, grid, block, smem, stream, args...);
+}
+// Without the overlap, for kernels bound by the FP64 pipe (two operations per clock and SM): blocks placed while the
+// predecessor still occupies most SMs pile up on the others, and the busiest SM sets the time (32^3 FP64 J.v +
+// projection 101 us with the overlap, 71 without).
+template <typename... P>
+inline void launch_spread(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                          typename same_type<P>::type... args) {
+  launch(false, kernel, grid, block, smem, stream, args...);
+}
+
+}  // namespace fv
