@@ -434,7 +434,7 @@ int launch_flux(const fv_grid_s* g, double Gr, double sigma, const double* q, co
   }
   const dim3 grid((g->nx + pl.tx - 1) / pl.tx, (g->ny + pl.ty - 1) / pl.ty, t.nch * nvec);
   ProfScope ps(g, PROF_STENCIL);
-  launch_spread(k_flux<R, MODE>, grid, kFxThreads, smem, g->stream, tq, tv, t);
+  launch(k_flux<R, MODE>, grid, kFxThreads, smem, g->stream, tq, tv, t);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }

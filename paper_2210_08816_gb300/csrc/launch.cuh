@@ -47,7 +47,8 @@ inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cud
 }
 // Without the overlap, for kernels bound by the FP64 pipe (two operations per clock and SM): blocks placed while the
 // predecessor still occupies most SMs pile up on the others, and the busiest SM sets the time (32^3 FP64 J.v +
-// projection 101 us with the overlap, 71 without).
+// projection 101 us with the overlap, 71 without).  A kernel whose registers or shared memory let one block on an SM
+// is spread evenly either way.
 template <typename... P>
 inline void launch_spread(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                           typename same_type<P>::type... args) {
