@@ -263,17 +263,20 @@ static int project_inplace(fv_grid_s* g, R* v, int max_it, double tol, int* iter
   const bool want = (div_rel != nullptr) || max_it > 1;
   double d0 = 0.0, dn = 0.0;
   int it = 0;
-  FV_TRY(launch_divergence<R>(g, v, phi));
+  FV_TRY(launch_divergence<R>(g, v, phi, 1, !want));
   if (want) {
     FV_TRY(launch_dot<R>(g, phi, phi, g->N, 0));
     FV_TRY(read_scalars(g, 0, 1, &d0));
     d0 = std::sqrt(d0);
   }
   for (it = 1; it <= std::max(1, max_it); ++it) {
+    if constexpr (sizeof(R) == 4) {
+      if (want && g->tc_ready) FV_TRY(launch_fieldmax(g, phi));
+    }
     FV_TRY(launch_poisson<R>(g, phi, phi, tmp));
     FV_TRY(launch_correct<R>(g, v, phi, 1.0, nullptr, 0.0, nullptr, 0.0, v));
     if (!want) break;
-    FV_TRY(launch_divergence<R>(g, v, phi));
+    FV_TRY(launch_divergence<R>(g, v, phi, 1, false));
     FV_TRY(launch_dot<R>(g, phi, phi, g->N, 0));
     FV_TRY(read_scalars(g, 0, 1, &dn));
     dn = std::sqrt(dn);
@@ -625,15 +628,14 @@ int fv_grid_create(const fv_grid_desc* desc, void* stream, fv_grid* out) {
   if (st == FV_OK) st = upload_axes<double>(g, ax, hp, 0, g->geo64, g->fdm64, g->cd64, g->fd64, g->half64);
   if (st == FV_OK) st = upload_axes<float>(g, ax, hp, 1, g->geo32, g->fdm32, g->cd32, g->fd32, g->half32);
   if (st == FV_OK && g->half_ready && (std::max({n[0], n[1], n[2]}) + 1) / 2 <= kDigitMaxH) st = upload_digits(g, half);
-  if (st == FV_OK && tc_eligible(g)) {
-    std::vector<double> idx[3] = {ax[0].idx, ax[1].idx, ax[2].idx}, idc[3] = {ax[0].idc, ax[1].idc, ax[2].idc};
-    if (tc_setup(g, idx, idc) != FV_OK) {  // keep the SIMT passes
-      g->tc.ready = false;
-      cudaGetLastError();
-    }
+  if (st == FV_OK && tc_setup(g) != FV_OK) {  // keep the other passes
+    g->tc_ready = false;
+    cudaGetLastError();
   }
   if (st == FV_OK) {
-    if (cudaMalloc(&g->ws.err, sizeof(int)) != cudaSuccess || cudaMemset(g->ws.err, 0, sizeof(int)) != cudaSuccess ||
+    if (cudaMalloc(&g->ws.smax, 8 * sizeof(unsigned)) != cudaSuccess ||
+        cudaMemset(g->ws.smax, 0, 8 * sizeof(unsigned)) != cudaSuccess ||
+        cudaMalloc(&g->ws.err, sizeof(int)) != cudaSuccess || cudaMemset(g->ws.err, 0, sizeof(int)) != cudaSuccess ||
         cudaMalloc(&g->ws.partials, sizeof(double) * kReduceBlocks * 256) != cudaSuccess ||
         cudaMalloc(&g->ws.scalars, sizeof(double) * kMaxScalars) != cudaSuccess ||
         cudaMallocHost(&g->ws.host_scalars, sizeof(double) * kMaxScalars) != cudaSuccess) {
@@ -668,7 +670,8 @@ int fv_grid_destroy(fv_grid g) {
   if (g->ws.scalars) cudaFree(g->ws.scalars);
   if (g->ws.host_scalars) cudaFreeHost(g->ws.host_scalars);
   for (cudaEvent_t e : g->prof.pool) cudaEventDestroy(e);
-  if (g->tc.buf) cudaFree(g->tc.buf);
+  if (g->ws.smax) cudaFree(g->ws.smax);
+  if (g->ws.bmax) cudaFree(g->ws.bmax);
   if (g->digit_buf) cudaFree(g->digit_buf);
   if (g->ws.err) cudaFree(g->ws.err);
   if (g->batch_exec) cudaGraphExecDestroy(g->batch_exec);
@@ -785,6 +788,16 @@ static int ensure_batch_ws(fv_grid_s* g, int nvec) {
       set_error("block workspace allocation failed");
       return FV_ENOMEM;
     }
+  if (p == 1) {  // FP32: the fields' maxima of the tensor-core solves
+    if (g->ws.bmax) cudaFree(g->ws.bmax);
+    g->ws.bmax = nullptr;
+    const size_t bytes = 8 * sizeof(unsigned) * (size_t)nvec;
+    if (cudaMalloc(&g->ws.bmax, bytes) != cudaSuccess || cudaMemsetAsync(g->ws.bmax, 0, bytes, g->stream) != cudaSuccess) {
+      cudaGetLastError();
+      set_error("block workspace allocation failed");
+      return FV_ENOMEM;
+    }
+  }
   g->ws.bcap[p] = nvec;
   return FV_OK;
 }

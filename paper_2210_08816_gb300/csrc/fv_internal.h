@@ -54,6 +54,8 @@ struct Workspace {
   void* Y[2] = {nullptr, nullptr};
   void* t0[2] = {nullptr, nullptr};
   void* t1[2] = {nullptr, nullptr};
+  unsigned* smax = nullptr;        // eight words of the FP32 solves' field maxima (fmax_slots)
+  unsigned* bmax = nullptr;        // the same for blocks, eight words per vector, grown with bY
   int* err = nullptr;              // device error word of bounded device-side waits (0 = none)
   double* partials = nullptr;      // reduction partials
   double* scalars = nullptr;       // device scalars (reduction results)
@@ -89,15 +91,6 @@ struct Profiler {
   std::vector<cudaEvent_t> pool;
   size_t used = 0;
 };
-// Operands of the tensor-core (tcgen05) pressure-solve passes.
-struct TcState {
-  bool ready = false;
-  void* buf = nullptr;
-  const float* lam[3] = {nullptr, nullptr, nullptr};  // eigenvalues in the tensor-core mode order
-  // per axis and direction (0 forward, 1 backward): the four B matrices of every K step laid out as the
-  // shared-memory stage holds them (64-byte swizzled rows), one contiguous block per step
-  const unsigned char* Bsw[3][2] = {{nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}};
-};
 }  // namespace fv
 
 struct fv_grid_s {
@@ -128,7 +121,7 @@ struct fv_grid_s {
   double sigma_default;
   double min_width[3];
   mutable fv::Profiler prof;
-  fv::TcState tc;
+  bool tc_ready = false;  // FP32 pressure solves on the tensor cores by kernels_tc.cu
   fv::Tune tune;
   mutable fv::FluxPlan flux[2];  // tiles of the flux stencil: single vectors, blocks
   // batched J.v + projection: the captured launch sequence of the last argument set, replayed while the
@@ -200,9 +193,10 @@ int launch_jvp(const fv_grid_s* g, double Gr, double sigma, const R* q, const R*
 // The one-cell J.v stencil over nvec states stored one after another in v and out (4N each), one launch.
 template <typename R>
 int launch_jvp_block(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out, int nvec);
-// nvec > 1: vel holds nvec states (4N each) and rhs nvec fields (N each), one after another.
+// nvec > 1: vel holds nvec states (4N each) and rhs nvec fields (N each), one after another.  for_solve: launch_poisson
+// on rhs follows directly (FP32 on tc_ready grids: the largest magnitude goes to the fields' slots).
 template <typename R>
-int launch_divergence(const fv_grid_s* g, const R* vel, R* rhs, int nvec = 1);
+int launch_divergence(const fv_grid_s* g, const R* vel, R* rhs, int nvec = 1, bool for_solve = true);
 // out = alpha (Y - G phi) + beta v + gamma w   (velocity; T without G phi).  v, w may be null.
 // norm_slot >= 0: also ||out||^2 into g->ws.scalars[norm_slot] (fused block partials).
 template <typename R>
@@ -287,12 +281,14 @@ int read_scalars(const fv_grid_s* g, int slot, int count, double* out);
 int encode_tensor_map(CUtensorMap* map, CUtensorMapDataType type, int rank, const void* ptr, const uint64_t* dims,
                       const uint64_t* strides, const uint32_t* box, CUtensorMapSwizzle swizzle);
 
-// Tensor-core pressure-solve passes (kernels_tc.cu), FP32 only.
-bool tc_eligible(const fv_grid_s* g);
-int tc_setup(fv_grid_s* g, const std::vector<double>* idx, const std::vector<double>* idc);
-// nvec fields stored one after another are transformed in one launch (persistent form only).
-int tc_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const float* in, float* out, bool scale,
-            int nvec = 1);
+// Tensor-core pressure-solve passes (kernels_tc.cu), FP32 only; slots: fmax_slots(g, nvec).
+int tc_setup(fv_grid_s* g);
+int tc_pass(const fv_grid_s* g, int pass, int na, int nb, const float* in, float* out, unsigned* slots, int nvec);
+// Eight words per field: the bits of the largest magnitude of a solve's right-hand side (word 0, written by
+// launch_divergence or launch_fieldmax directly before the solve) and of its passes' outputs.
+inline unsigned* fmax_slots(const fv_grid_s* g, int nvec) { return nvec > 1 ? g->ws.bmax : g->ws.smax; }
+// word 0 of the single field's slots from a field of N elements
+int launch_fieldmax(const fv_grid_s* g, const float* f);
 
 // ------------------------------------------------------------------ host linear algebra (host_linalg.cpp)
 // Symmetric tridiagonal eigen-decomposition (implicit QR with Wilkinson shifts).
@@ -313,6 +309,8 @@ void hessenberg_lstsq(int j, const double* H, int ld, double beta, std::vector<d
 
 // ------------------------------------------------------------------ tensor-core operands (host_tc.cpp)
 constexpr int kTcSlabCols = 16;  // FP32 K columns per slab of the tensor-core passes (one 64-byte row)
+// The half-size operators as TF32 heads and FP32 remainders.  The library's own passes take FP16 parts (build_halves);
+// this form is compiled by the host tests alone, which check its decompositions against the axis operators.
 // One float buffer: per axis [fwd_s_hi, fwd_s_lo, fwd_a_hi, fwd_a_lo, bwd_s_hi, bwd_s_lo, bwd_a_hi,
 // bwd_a_lo] (h x h each, at moff), the eigenvalues in the tensor-core mode order (n, at loff), and per
 // axis and direction the swizzled per-step B blocks of the persistent pass (4 h^2, at soff, 256-byte

@@ -396,14 +396,14 @@ int launch_poisson_block(const fv_grid_s* g, const R* rhs, R* phi, R* tmp, int n
     return FV_EINVAL;
   }
   if constexpr (sizeof(R) == 4) {
-    if (g->tc.ready) {  // the tensor-core passes over the stacked fields (3 x TF32 split, FP32 accuracy)
-      FV_TRY(tc_pass(g, 0, false, nz, ny, rhs, tmp, false, nvec));
-      FV_TRY(tc_pass(g, 1, false, nx, nz, tmp, phi, false, nvec));
-      FV_TRY(tc_pass(g, 2, false, ny, nx, phi, tmp, true, nvec));
-      FV_TRY(tc_pass(g, 0, true, nz, ny, tmp, phi, false, nvec));
-      FV_TRY(tc_pass(g, 1, true, nx, nz, phi, tmp, false, nvec));
-      FV_TRY(tc_pass(g, 2, true, ny, nx, tmp, phi, false, nvec));
-      return FV_OK;
+    if (g->tc_ready) {  // the tensor-core passes over the stacked fields
+      unsigned* slots = fmax_slots(g, nvec);
+      FV_TRY(tc_pass(g, 0, nz, ny, rhs, tmp, slots, nvec));
+      FV_TRY(tc_pass(g, 1, nx, nz, tmp, phi, slots, nvec));
+      FV_TRY(tc_pass(g, 2, ny, nx, phi, tmp, slots, nvec));
+      FV_TRY(tc_pass(g, 3, nz, ny, tmp, phi, slots, nvec));
+      FV_TRY(tc_pass(g, 4, nx, nz, phi, tmp, slots, nvec));
+      return tc_pass(g, 5, ny, nx, tmp, phi, slots, nvec);
     }
   }
   if (g->half_ready) {

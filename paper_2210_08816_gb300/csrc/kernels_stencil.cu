@@ -342,25 +342,45 @@ __global__ void __launch_bounds__(kTX * kTY, 3)
       bar_wait(smem_addr(&bar[(kk + kRing) % kRing]), (uint32_t)(((kk - k0 + 1) / kRing) & 1), err, 1LL << 22);
 }
 
-// rhs = D vel:  sum_d (vel_d(face p+1) - vel_d(face p)) / width, wall fluxes zero
+// The largest magnitude over a warp's threads (bits of nonnegative floats order like integers; a NaN's lie above all)
+// into *slot.  Every thread of the warp calls it.
+__device__ __forceinline__ void warp_max_to(unsigned* slot, unsigned bits) {
+  const unsigned m = __reduce_max_sync(0xffffffffu, bits);
+  if ((threadIdx.x & 31) == 0) atomicMax(slot, m);
+}
+
+__global__ void __launch_bounds__(256) k_fieldmax(size_t n, const float* __restrict__ f, unsigned* slot) {
+  pdl_begin();
+  const unsigned ready0 = pdl_wait();
+  f += ready0;
+  unsigned m = 0;
+  for (size_t t = (size_t)blockIdx.x * 256 + threadIdx.x; t < n; t += (size_t)gridDim.x * 256)
+    m = max(m, __float_as_uint(f[t]) & 0x7fffffffu);
+  warp_max_to(slot, m);
+}
+
+// rhs = D vel:  sum_d (vel_d(face p+1) - vel_d(face p)) / width, wall fluxes zero; slot (may be null): the largest
+// magnitude of rhs
 template <typename R>
 __global__ void __launch_bounds__(256) k_divergence(Geo<R> g, int N, const R* __restrict__ vel,
-                                                     R* __restrict__ rhs) {
+                                                     R* __restrict__ rhs, unsigned* slot) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
   vel += ready0;
   rhs += ready0;
   Cell<R> c;
-  if (!cell_of_thread(g, c)) return;
   R acc = R(0);
+  if (cell_of_thread(g, c)) {
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const R* f = vel + d * N;
-    const R lo = (c.p[d] >= 1) ? ld(f, c.o) : R(0);
-    const R hi = (c.p[d] + 1 < g.n[d]) ? ld(f, c.o + c.s[d]) : R(0);
-    acc += (hi - lo) * g.idx[d][c.p[d]];
+    for (int d = 0; d < 3; ++d) {
+      const R* f = vel + d * N;
+      const R lo = (c.p[d] >= 1) ? ld(f, c.o) : R(0);
+      const R hi = (c.p[d] + 1 < g.n[d]) ? ld(f, c.o + c.s[d]) : R(0);
+      acc += (hi - lo) * g.idx[d][c.p[d]];
+    }
+    rhs[c.o] = acc;
   }
-  rhs[c.o] = acc;
+  if (sizeof(R) == 4 && slot) warp_max_to(slot, __float_as_uint((float)acc) & 0x7fffffffu);
 }
 
 // out = alpha (Y - G phi) + beta v + gamma w, G phi = (phi(cell) - phi(cell - e_d)) / spacing on interior
@@ -458,7 +478,7 @@ __device__ __forceinline__ float4 zero4() { return make_float4(0.f, 0.f, 0.f, 0.
 
 // blockIdx.z = z-block + nzc * vector (states of 4N, rhs fields of N, one after another)
 __global__ void __launch_bounds__(256) k_divergence4(Geo<float> g, int N, const float* __restrict__ vel,
-                                                      float* __restrict__ rhs, int nzc) {
+                                                      float* __restrict__ rhs, int nzc, unsigned* slot) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
   vel += ready0;
@@ -483,6 +503,7 @@ __global__ void __launch_bounds__(256) k_divergence4(Geo<float> g, int N, const 
   }
   const int ob = act ? (k0 * ny + j) * nx + i0 : 0;
   float4 wlo = (act && k0 >= 1) ? ldg4(W, ob) : zero4();
+  unsigned top = 0;
 #pragma unroll
   for (int k = k0; k < k1; ++k) {
     const int o = ob + (k - k0) * pl;
@@ -502,8 +523,12 @@ __global__ void __launch_bounds__(256) k_divergence4(Geo<float> g, int N, const 
     r.z = (u.w - u.z) * rx.z + (vhi.z - vlo.z) * ry + (whi.z - wlo.z) * rz;
     r.w = (un - u.w) * rx.w + (vhi.w - vlo.w) * ry + (whi.w - wlo.w) * rz;
     *reinterpret_cast<float4*>(rhs + o) = r;
+    top = max(max(top, __float_as_uint(r.x) & 0x7fffffffu),
+              max(max(__float_as_uint(r.y) & 0x7fffffffu, __float_as_uint(r.z) & 0x7fffffffu),
+                  __float_as_uint(r.w) & 0x7fffffffu));
     wlo = whi;
   }
+  if (slot) warp_max_to(slot + 8 * vec, top);
 }
 
 __device__ __forceinline__ void acc_sq(float& hi, float& lo, float r) {
@@ -717,10 +742,18 @@ int launch_jvp(const fv_grid_s* g, double Gr, double sigma, const R* q, const R*
   return launch_jvp_block<R>(g, Gr, sigma, q, v, out, 1);
 }
 
+int launch_fieldmax(const fv_grid_s* g, const float* f) {
+  ProfScope ps(g, PROF_REDUCE);
+  launch(k_fieldmax, 2 * g->sms, 256, 0, g->stream, g->N, f, g->ws.smax);
+  FV_CUDA(cudaGetLastError());
+  return FV_OK;
+}
+
 template <typename R>
-int launch_divergence(const fv_grid_s* g, const R* vel, R* rhs, int nvec) {
+int launch_divergence(const fv_grid_s* g, const R* vel, R* rhs, int nvec, bool for_solve) {
   dim3 grid, block;
   cell_grid(g, grid, block);
+  unsigned* slot = (sizeof(R) == 4 && for_solve && g->tc_ready) ? fmax_slots(g, nvec) : nullptr;
   ProfScope ps(g, PROF_DIVERGENCE);
   if constexpr (sizeof(R) == 4) {
     if (quad_ok(g, {vel, rhs})) {
@@ -731,14 +764,14 @@ int launch_divergence(const fv_grid_s* g, const R* vel, R* rhs, int nvec) {
         return FV_EINVAL;
       }
       qg.z = nzc * nvec;
-      launch(k_divergence4, qg, dim3(32, 8), 0, g->stream, g->geo32, (int)g->N, vel, rhs, nzc);
+      launch(k_divergence4, qg, dim3(32, 8), 0, g->stream, g->geo32, (int)g->N, vel, rhs, nzc, slot);
       FV_CUDA(cudaGetLastError());
       return FV_OK;
     }
   }
   for (int i = 0; i < nvec; ++i) {
     launch(k_divergence<R>, grid, block, 0, g->stream, geo_of<R>(g), (int)g->N, vel + (size_t)i * 4 * g->N,
-                                                   rhs + (size_t)i * g->N);
+           rhs + (size_t)i * g->N, slot ? slot + 8 * i : nullptr);
     FV_CUDA(cudaGetLastError());
   }
   return FV_OK;
@@ -804,8 +837,8 @@ template int launch_jvp<double>(const fv_grid_s*, double, double, const double*,
 template int launch_jvp<float>(const fv_grid_s*, double, double, const float*, const float*, float*);
 template int launch_jvp_block<double>(const fv_grid_s*, double, double, const double*, const double*, double*, int);
 template int launch_jvp_block<float>(const fv_grid_s*, double, double, const float*, const float*, float*, int);
-template int launch_divergence<double>(const fv_grid_s*, const double*, double*, int);
-template int launch_divergence<float>(const fv_grid_s*, const float*, float*, int);
+template int launch_divergence<double>(const fv_grid_s*, const double*, double*, int, bool);
+template int launch_divergence<float>(const fv_grid_s*, const float*, float*, int, bool);
 template int launch_correct_block<double>(const fv_grid_s*, const double*, const double*, const double*, double,
                                           double*, int);
 template int launch_correct_block<float>(const fv_grid_s*, const float*, const float*, const float*, double, float*,

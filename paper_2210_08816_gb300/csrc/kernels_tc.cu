@@ -1,31 +1,41 @@
-// Tensor-core (tcgen05) version of the fast-diagonalisation passes for FP32 fields.
+// Fast-diagonalisation passes of the pressure solve for FP32 fields on the tensor cores (tcgen05), for grids whose axes
+// have 32 .. 256 cells, a multiple of 32, and mirror-symmetric faces.
 //
-// A pass is the GEMM  C[p][m] = sum_k A[p][k] B[m][k]  (A = field rows, k contiguous; B = a 1D eigenvector
-// matrix), stored transposed as out[m][p] (see kernels_fdm.cu).
+// A pass is the GEMM  C[p][m] = sum_k A[p][k] B[m][k]  (A = field rows, k contiguous; B = a 1D eigenvector matrix),
+// stored transposed as out[m][p] (see kernels_fdm.cu), in the half-size form of HalfOpHost: forward passes contract
+// the sums and differences of mirrored inputs with two h x h matrices (h = n / 2), backward passes write S +- A.
 //
-// Mirror symmetry.  The grid is symmetric about 1/2, so the 1D operators are centro-symmetric and every
-// eigenvector is either symmetric or antisymmetric.  With the modes ordered [symmetric | antisymmetric]
-// (the "tensor-core order"):
-//   forward  (cells -> modes):  phi_s = sum_{k<n/2} F_s[s][k] (r[k] + r[n-1-k]),
-//                               phi_a = sum_{k<n/2} F_a[a][k] (r[k] - r[n-1-k]);
-//   backward (modes -> cells):  S[i] = sum_s E_s[i][s] phi_s,  A[i] = sum_a E_a[i][a] phi_a  (i < n/2),
-//                               out[i] = S + A,  out[n-1-i] = S - A.
-// Each pass is then two GEMMs with K = n/2 and N = n/2: half the tensor work and half the B traffic of the
-// dense transform.  The forward sum / difference is formed in shared memory by the converter warps; the
-// backward S +- A in the epilogue.
+// FP32 accuracy on FP16 tensor cores: the field is scaled by one power of two into FP16's range (its largest
+// magnitude below 2^14, found by the kernel that wrote it), and every sum or difference x is split as hi = fp16(x),
+// lo = fp16(x - hi), 22 bits together; likewise the matrices (on the host, build_halves).  hi hi + hi lo + lo hi are
+// accumulated in FP32; the dropped lo lo is 2^-24 of a product.  Values below 2^-17 of the field's largest keep an
+// absolute error of 2^-39 of it.  Against the same three products of TF32 parts, which have the same mantissas: half
+// the bytes per input in shared memory, half the MMA time, and half as many truncated accumulations (the projection's
+// error against 64 bits falls from 0.83e-6 to 0.58e-6 at 64^3, from 2.0e-6 to 1.2e-6 at 256^3).
 //
-// FP32 accuracy on TF32 tensor cores by the three-product split: A = A_hi + A_lo, B = B_hi + B_lo with
-// A_hi, B_hi exactly representable in TF32, and  A B ~ A_hi B_hi + A_hi B_lo + A_lo B_hi  (the dropped
-// A_lo B_lo and the TF32 rounding of the lo parts are ~2^-22 relative).  B_hi / B_lo are prepared on the
-// host; A is split in shared memory by the converter warps.
+// One CTA per SM walks the 128-row tiles blockIdx.x, +gridDim.x, ... with all n outputs (rows and fields are whole
+// tiles: a field has at least 32 x 32 rows).  Per step 32 inputs of each half: two TMA boxes of A (slab j and its mirror
+// forward, slabs j and h + 32 j backward; 128-byte swizzle), the four B slabs (bulk copies of the pre-swizzled blocks;
+// kept where all of B fits), and per k-step of 16 inputs 2 halves x 3 products of tcgen05.mma (M = 128, N = h, K = 16).
+// Two TMEM accumulators (columns 0 and 256) let the epilogue of a tile run under the MMAs of the next.
+// Warps: 0 TMA of A, 1 MMA issue, then converters, epilogue (8), bulk copies of B (the last).
+// Barriers: afull / afree per raw stage (A landed / converted), bfull / bfree per B slab, conv / done per k-step
+// (converted / MMAs complete); accf / acce per tile.  Every wait is bounded; on expiry the kernel records a code, stops
+// issuing, lets its copies and MMAs complete and returns.
 //
+// What bounds it: memory.  256^3, six passes of 134 MB each: 198 us by themselves, 149 within a time step's launches
+// (TF32 parts: 222), 5.4 TB/s; a pass's reads alone run at 5.2 TB/s through two stages of 32 KB per SM.  More stages
+// are slower (three: 630 us for the whole chebyshev step against 600), and so are equal row ranges instead of
+// neighbouring tiles at a time (650): the writes are 512-byte pieces of n rows, and neighbours share DRAM pages.
 #include <cuda.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "fv_internal.h"
@@ -35,10 +45,15 @@
 namespace fv {
 namespace {
 
-constexpr int kTcBM = 128;                 // rows per tile
-constexpr int kTcBK = 16;                  // fp32 elements per K slab (64 bytes: one 64-byte swizzle row)
-constexpr int kTcRowBytes = kTcBK * 4;
-constexpr int kTcABytes = kTcBM * kTcRowBytes;  // one A slab tile (8 KB)
+constexpr int kTcBM = 128;                  // rows per tile
+constexpr int kTcBK = 32;                   // inputs of a half per step: one 128-byte FP32 row, one 64-byte FP16 row
+constexpr int kTcABytes = kTcBM * kTcBK * 4;  // one raw A slab (16 KB)
+constexpr int kTcCBytes = kTcBM * kTcBK * 2;  // one converted slab (8 KB)
+constexpr int kTcRing = 2;                    // raw stages
+constexpr int kTcSteps = 4;  // converted k-steps of 16 inputs in flight, two to a slot of four slabs
+constexpr int kTcEpi = 8;     // epilogue warps
+constexpr size_t kTcSmemMost = 229376 + 1024;
+constexpr int tc_threads(int conv) { return 64 + conv + 32 * kTcEpi + 32; }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
   asm volatile(
@@ -48,20 +63,14 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
-__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
           tmem_d),
       "l"(a), "l"(b), "r"(idesc), "r"(acc)
       : "memory");
 }
 
-// Converter helpers.  A 64-byte swizzled row r keeps its 16-byte chunk c at physical chunk c ^ ((r >> 1) & 3).
-__device__ __forceinline__ float tf32_hi(float x) {
-  uint32_t u;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(u) : "f"(x));
-  return __uint_as_float(u);
-}
 // approximate reciprocal (PTX rcp.approx, relative error about 2^-23): far below the 3 x TF32 error
 __device__ __forceinline__ float rcp_approx(float x) {
   float r;
@@ -69,71 +78,86 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return r;
 }
 
-__device__ __forceinline__ void split4(const float4 x, float4& h, float4& l) {
-  h.x = tf32_hi(x.x);
-  h.y = tf32_hi(x.y);
-  h.z = tf32_hi(x.z);
-  h.w = tf32_hi(x.w);
-  l.x = x.x - h.x;
-  l.y = x.y - h.y;
-  l.z = x.z - h.z;
-  l.w = x.w - h.w;
+// eight values as FP16 heads and remainders
+__device__ __forceinline__ void split8(const float (&x)[8], uint4& h, uint4& l) {
+  uint32_t hw[4], lw[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const __half2 hh = __floats2half2_rn(x[2 * i], x[2 * i + 1]);
+    const float2 f = __half22float2(hh);
+    const __half2 ll = __floats2half2_rn(x[2 * i] - f.x, x[2 * i + 1] - f.y);
+    hw[i] = *reinterpret_cast<const uint32_t*>(&hh);
+    lw[i] = *reinterpret_cast<const uint32_t*>(&ll);
+  }
+  h = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+  l = make_uint4(lw[0], lw[1], lw[2], lw[3]);
 }
 
-// One CTA per SM walks the 128-row tiles blockIdx.x, +gridDim.x, ... with all n outputs; per step two 16-wide K slabs
-// of A (slab j and its mirror n/16-1-j forward, slab j and j + n/32 backward) and the matching slabs of the two
-// half-size B matrices, 2 k-steps x 3 products x 2 halves of tcgen05.mma (M = 128, N = n/2, K = 8); the
-// shared-memory ring's phases run on across tiles (global stage counter), and two TMEM accumulators
-// (columns 0 and 256) let a separate epilogue warpgroup drain tile t while the MMAs of tile t + 1 run.
-// Warps: 0 TMA producer, 1 MMA issuer, 2-9 converters (half a row of the A tiles each), 10-13 epilogue.
-// Barriers per step gi: full (TMA landed) -> conv (hi in place, lo in slot gi % 2) -> MMAs, whose commits
-// free the TMA stage (empty) and the remainder slot (lofree) for step gi + 4 and gi + 2.
-constexpr int kTcpConv = 256;  // converter threads
-constexpr int kTcpThreads = 64 + kTcpConv + 128;
-// Ring depths of the persistent pass: the TMA ring (A slabs by tensor copies, the step's B slabs by one
-// bulk copy of their pre-swizzled image) runs four stages deep; the converters' TF32 remainders of A live
-// in a separate two-slot ring, so the bytes in flight from DRAM per SM grow by a third within the same
-// shared memory.
-constexpr int kTcpStages = 4;
-constexpr int kTcpLoSlots = 2;
+// The exponent field of a field's largest magnitude (its bits in a slot), at least 32 (zero and tiny fields).
+__device__ __forceinline__ int max_exponent(const unsigned* slot) { return max((int)(__ldcg(slot) >> 23), 32); }
 
-template <bool SCALE, bool BWD>
-__global__ void __launch_bounds__(kTcpThreads, 1)
-    k_transform_tcp(const __grid_constant__ CUtensorMap tmA, const unsigned char* __restrict__ bsw,
-                    float* __restrict__ out, int P, int Ptot, int n, const float* __restrict__ lx,
-                    const float* __restrict__ ly, const float* __restrict__ lz, int nb, int* err, long long spins) {
+// A warp's largest magnitude into a field's slot (fmaxf drops NaNs: one shows as a NaN in the next pass whatever the
+// scale).
+__device__ __forceinline__ void max_to(unsigned* slot, float top) {
+  const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(top));
+  if (threadIdx.x % 32 == 0) atomicMax(slot, m);
+}
+
+struct TcArgs {
+  const unsigned char* B;  // blocks [part][group of 64 outputs][slab]: 64 rows hi, 64 rows lo, of 64 bytes
+  const int* bexp;         // exponent of every output pair
+  float* out;
+  const float *lx, *ly, *lz;  // scaled pass: eigenvalues
+  const unsigned* max_in;     // slot of every vector: the bits of its largest input magnitude
+  unsigned *max_out, *max_reset;  // the same for the output; a consumed slot to clear (either may be null)
+  int P, Ptot, n, nb;
+  int bslots;   // B slabs in shared memory: all of them, or a ring of two
+  int* err;
+  long long spins;
+};
+
+// CONV: converter threads, 256 or 512
+template <bool SCALE, bool BWD, int CONV>
+__global__ void __launch_bounds__(tc_threads(CONV), 1)
+    k_pass_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ TcArgs t) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t bar_full[kTcpStages], bar_conv[kTcpStages], bar_empty[kTcpStages];
-  __shared__ __align__(8) uint64_t bar_lofree[kTcpLoSlots], bar_accf[2], bar_acce[2], bar_drain;
+  __shared__ __align__(8) uint64_t bar_afull[kTcRing], bar_afree[kTcRing], bar_bfull[4], bar_bfree[2],
+      bar_conv[kTcSteps], bar_done[kTcSteps],
+      bar_accf[2], bar_acce[2], bar_drain;
   __shared__ uint32_t tmem_slot;
-  __shared__ float lz_s[256];
-  const int h = n / 2;
-  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t b_bytes = (uint32_t)h * kTcRowBytes;
-  const uint32_t stage_bytes = 2u * kTcABytes + 4u * b_bytes;  // [A1 | A2 | B1hi | B1lo | B2hi | B2lo]
-  const uint32_t lo_base = base + kTcpStages * stage_bytes;  // slot s: [L1 | L2] at lo_base + s * 2 A slabs
+  __shared__ float lz_s[256], col_s[128];
+  const int n = t.n, h = n / 2, P = t.P;
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const uint32_t base = smem_u32(smem);
+  const int bslots = t.bslots;
+  constexpr uint32_t conv0 = kTcRing * 2u * kTcABytes, b0 = conv0 + (kTcSteps / 2) * 4u * kTcCBytes;
+  const uint32_t b_bytes = (uint32_t)h * 64u;  // one B slab
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int nst = n / (2 * kTcBK);
-  const int ntiles = (Ptot + kTcBM - 1) / kTcBM;
-  pdl_begin();
+  const int nst = (h + kTcBK - 1) / kTcBK;
+  const int ntiles = t.Ptot / kTcBM;
   const int my_tiles = (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-
+  pdl_begin();
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kTcpStages; ++s) {
-      mbar_init(smem_u32(&bar_full[s]), 1);
-      mbar_init(smem_u32(&bar_conv[s]), kTcpConv);
-      mbar_init(smem_u32(&bar_empty[s]), 1);
+    for (int s = 0; s < kTcRing; ++s) {
+      mbar_init(smem_u32(&bar_afull[s]), 1);
+      mbar_init(smem_u32(&bar_afree[s]), 16);
     }
-    for (int s = 0; s < kTcpLoSlots; ++s) mbar_init(smem_u32(&bar_lofree[s]), 1);
+    for (int s = 0; s < 4; ++s) mbar_init(smem_u32(&bar_bfull[s]), 1);
+    for (int s = 0; s < kTcSteps; ++s) {
+      mbar_init(smem_u32(&bar_conv[s]), 8);
+      mbar_init(smem_u32(&bar_done[s]), 1);
+    }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&bar_accf[b]), 1);
-      mbar_init(smem_u32(&bar_acce[b]), 4);  // one arrival per epilogue warp
+      mbar_init(smem_u32(&bar_acce[b]), kTcEpi);
     }
+    for (int b = 0; b < 2; ++b) mbar_init(smem_u32(&bar_bfree[b]), 1);
     mbar_init(smem_u32(&bar_drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (SCALE)
-    for (int m = threadIdx.x; m < n; m += kTcpThreads) lz_s[m] = lz[m];
+    for (int m = threadIdx.x; m < n; m += tc_threads(CONV)) lz_s[m] = t.lz[m];
+  for (int m = threadIdx.x; m < h; m += tc_threads(CONV)) col_s[m] = __int_as_float((t.bexp[m] + 127) << 23);
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                  "r"(512)
@@ -143,184 +167,235 @@ __global__ void __launch_bounds__(kTcpThreads, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
-  const unsigned ready0 = pdl_wait();
-  out += ready0;
-
+  if (warp == 2 + CONV / 32 + kTcEpi) {
+    // B, slab by slab as [half][hi | lo] of b_bytes each: kept for the CTA's lifetime where it fits, else around a ring
+    // of two.  It is the grid's own, so the copies start before the kernel before this one has ended.
+    if (lane == 0) {
+      const int groups = (h + 63) / 64, loads = bslots == nst ? nst : my_tiles * nst;
+      int issued = 0;
+      for (; issued < loads; ++issued) {
+        const int st = issued % bslots, j = issued % nst;
+        if (issued >= bslots &&
+            !mbar_wait(smem_u32(&bar_bfree[st]), ((issued / bslots) - 1) & 1, t.err, 13, t.spins))
+          break;
+        const uint32_t sb = base + b0 + st * 4u * b_bytes, fb = smem_u32(&bar_bfull[st]);
+        mbar_expect_tx(fb, 4u * b_bytes);
+        for (int part = 0; part < 2; ++part)
+          for (int gr = 0; gr < groups; ++gr) {
+            const uint32_t bytes = (uint32_t)std::min(64, h - 64 * gr) * 64u;
+            const unsigned char* src = t.B + ((size_t)(part * groups + gr) * nst + j) * 8192;
+            bulk_load(sb + (2 * part) * b_bytes + gr * 4096u, src, bytes, fb);
+            bulk_load(sb + (2 * part + 1) * b_bytes + gr * 4096u, src + 4096, bytes, fb);
+          }
+      }
+      // every issued copy has landed before the block may exit
+      for (int i = std::max(issued - bslots, 0); i < issued; ++i)
+        mbar_wait(smem_u32(&bar_bfull[i % bslots]), (i / bslots) & 1, t.err, 12, kWaitLimit);
+    }
+    __syncwarp();
+  }
+  // every role waits for the kernel before this one by itself, right where it first needs its results (the code up to
+  // there has then been fetched; a wait of the whole block here cost 1 us of a pass in instruction misses)
   if (warp == 0) {
     if (lane == 0) {
-      int issued = 0;
+      int gi = 0, issued = 0;
       bool ok = true;
       for (int ti = 0; ti < my_tiles && ok; ++ti) {
         const int p0 = ((int)blockIdx.x + ti * (int)gridDim.x) * kTcBM;
-        for (int j = 0; j < nst; ++j) {
-          const int gi = ti * nst + j, st = gi % kTcpStages;
-          if (gi >= kTcpStages && !mbar_wait(smem_u32(&bar_empty[st]), ((gi / kTcpStages) - 1) & 1, err, 11, spins)) {
+        for (int j = 0; j < nst; ++j, ++gi) {
+          const int st = gi % kTcRing;
+          if (gi >= kTcRing && !mbar_wait(smem_u32(&bar_afree[st]), ((gi / kTcRing) - 1) & 1, t.err, 11, t.spins)) {
             ok = false;
             break;
           }
-          const uint32_t sb = base + st * stage_bytes;
-          const uint32_t fb = smem_u32(&bar_full[st]);
-          const int k1 = j * kTcBK;
-          const int k2 = BWD ? h + j * kTcBK : n - kTcBK - j * kTcBK;
-          mbar_expect_tx(fb, 2u * kTcABytes + 4u * b_bytes);
-          tma_load_2d(sb, &tmA, fb, k1, p0);
-          tma_load_2d(sb + kTcABytes, &tmA, fb, k2, p0);
-          // the four B slabs of step j, already in the stage's swizzled layout: one contiguous copy
-          bulk_load(sb + 2u * kTcABytes, bsw + (size_t)j * 4u * b_bytes, 4u * b_bytes, fb);
+          const uint32_t sa = base + st * 2u * kTcABytes, fb = smem_u32(&bar_afull[st]);
+          const int x1 = j * kTcBK, x2 = BWD ? h + j * kTcBK : n - kTcBK - j * kTcBK;
+          mbar_expect_tx(fb, 2u * kTcABytes);
+          if (gi == 0) pdl_wait();
+          tma_load_2d(sa, &tmA, fb, x1, p0);
+          tma_load_2d(sa + kTcABytes, &tmA, fb, x2, p0);
           ++issued;
         }
       }
-      // drain: every issued copy has landed before the block may exit
-      for (int gi = (issued > kTcpStages ? issued - kTcpStages : 0); gi < issued; ++gi)
-        mbar_wait(smem_u32(&bar_full[gi % kTcpStages]), (gi / kTcpStages) & 1, err, 12, kWaitLimit);
+      // every issued copy has landed before the block may exit
+      for (int g2 = std::max(issued - kTcRing, 0); g2 < issued; ++g2)
+        mbar_wait(smem_u32(&bar_afull[g2 % kTcRing]), (g2 / kTcRing) & 1, t.err, 12, kWaitLimit);
     }
   } else if (warp == 1) {
-    // descriptors differ from the first stage's by multiples of 16 bytes: additions only (building each from its
+    // descriptors differ from the first slab's by multiples of 16 bytes: additions only (building each from its
     // address in one lane cost 140 clocks per MMA, more than the MMA's own 64)
     const uint64_t desc0 = smem_desc(base);
-    const uint32_t idesc =
-        (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(h >> 3) << 17) | ((uint32_t)(kTcBM >> 4) << 24);
+    const uint32_t idesc = (1u << 4) | ((uint32_t)(h >> 3) << 17) | ((uint32_t)(kTcBM >> 4) << 24);
+    int g2 = 0, gi = 0;  // k-steps of 16 inputs, steps of 32
     bool ok = true;
     for (int ti = 0; ti < my_tiles && ok; ++ti) {
       const int b = ti & 1;
       if (ti >= 2 &&
-          !__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_acce[b]), ((ti / 2) - 1) & 1, err, 13, spins))) {
+          !__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_acce[b]), ((ti / 2) - 1) & 1, t.err, 13, t.spins))) {
         ok = false;
         break;
       }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t dacc = tmem + (uint32_t)(b * 256);
-      for (int j = 0; j < nst; ++j) {
-        const int gi = ti * nst + j, st = gi % kTcpStages;
-        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_conv[st]), (gi / kTcpStages) & 1, err, 14, spins))) {
+      for (int j = 0; j < nst && ok; ++j, ++gi) {
+        const int bs = gi % bslots;
+        if ((ti == 0 || bslots < nst) &&
+            !__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_bfull[bs]), (gi / bslots) & 1, t.err, 14, t.spins))) {
           ok = false;
           break;
         }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint64_t ds = desc0 + (uint64_t)((st * stage_bytes) >> 4);
-        const uint64_t dl = desc0 + (uint64_t)((kTcpStages * stage_bytes + (gi % kTcpLoSlots) * (2u * kTcABytes)) >> 4);
-        if (elect_one()) {
-#pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            const uint64_t a_hi = ds + (half * kTcABytes >> 4), a_lo = dl + (half * kTcABytes >> 4);
-            const uint64_t b_hi = ds + ((2u * kTcABytes) >> 4) + (uint64_t)(2 * half) * (b_bytes >> 4);
-            const uint64_t b_lo = b_hi + (b_bytes >> 4);
-            const uint32_t d = dacc + (uint32_t)(half * h);
-#pragma unroll
-            for (int kk = 0; kk < kTcBK / 8; ++kk) {
-              mma_tf32(d, a_hi + 2 * kk, b_hi + 2 * kk, idesc, kk > 0 ? 1u : (uint32_t)(j > 0));
-              mma_tf32(d, a_hi + 2 * kk, b_lo + 2 * kk, idesc, 1u);
-              mma_tf32(d, a_lo + 2 * kk, b_hi + 2 * kk, idesc, 1u);
-            }
+        const uint64_t db = desc0 + ((b0 + bs * 4u * b_bytes) >> 4);
+        for (int kk = 0; kk < 2; ++kk, ++g2) {
+          const int st = g2 % kTcSteps;
+          if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_conv[st]), (g2 / kTcSteps) & 1, t.err, 15, t.spins))) {
+            ok = false;
+            break;
           }
-          mma_commit(smem_u32(&bar_empty[st]));
-          mma_commit(smem_u32(&bar_lofree[gi % kTcpLoSlots]));  // the remainder slot is free again
-          if (j == nst - 1) mma_commit(smem_u32(&bar_accf[b]));  // arrives once every MMA issued so far has completed
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t dc = desc0 + ((conv0 + (st >> 1) * 4u * kTcCBytes + 32u * kk) >> 4);
+          if (elect_one()) {
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+              const uint64_t a_hi = dc + ((2u * half * kTcCBytes) >> 4), a_lo = a_hi + (kTcCBytes >> 4);
+              const uint64_t b_hi = db + 2u * half * (uint64_t)(b_bytes >> 4) + 2 * kk, b_lo = b_hi + (b_bytes >> 4);
+              const uint32_t d = dacc + (uint32_t)(half * h);
+              mma_f16(d, a_hi, b_hi, idesc, (uint32_t)(j + kk > 0));
+              mma_f16(d, a_hi, b_lo, idesc, 1u);
+              mma_f16(d, a_lo, b_hi, idesc, 1u);
+            }
+            mma_commit(smem_u32(&bar_done[st]));
+            if (kk == 1 && bslots < nst) mma_commit(smem_u32(&bar_bfree[bs]));
+            if (kk == 1 && j == nst - 1) mma_commit(smem_u32(&bar_accf[b]));  // once every MMA so far has completed
+          }
+          __syncwarp();
         }
-        __syncwarp();
       }
     }
-    // give-up path: a commit after every MMA issued so far (including those of a tile left half done) arrives once
-    // they have all completed; wait for it (full limit) before the accumulators are freed
+    // give-up path: a commit after every MMA issued so far arrives once they have all completed; wait for it (full
+    // limit) before the accumulators are freed
     if (!ok) {
       if (elect_one()) mma_commit(smem_u32(&bar_drain));
-      mbar_wait(smem_u32(&bar_drain), 0, err, 16, kWaitLimit);
+      mbar_wait(smem_u32(&bar_drain), 0, t.err, 16, kWaitLimit);
     }
-  } else if (warp < 2 + kTcpConv / 32) {
-    // converters: threads t and t + 128 own row t of every stage's A tiles and of every remainder slot, one the
-    // 16-byte chunks 0 and 3, the other 1 and 2 (chunk c of a slab meets chunk 3 - c of its mirror, so neither reads
-    // what the other writes)
-    const int tt = threadIdx.x - 64, t = tt & 127, c0 = tt >> 7;
-    const int x = (t >> 1) & 3;  // swizzle pattern of this row
+  } else if (warp < 2 + CONV / 32) {
+    // converters: four threads to a row of every slab; those of one half of the warps take the first k-step of each
+    // raw stage, the others the second, a thread inputs 8 hf .. 8 hf + 7 of it
+    const int tt = threadIdx.x - 64, r = tt & 127, hf = (tt >> 7) & 1;
+    const unsigned* __restrict__ max_in = t.max_in + pdl_wait();
+    int gi = 0;
     bool ok = true;
     for (int ti = 0; ti < my_tiles && ok; ++ti) {
-      for (int j = 0; j < nst; ++j) {
-        const int gi = ti * nst + j, st = gi % kTcpStages, ls = gi % kTcpLoSlots;
-        if (!mbar_wait(smem_u32(&bar_full[st]), (gi / kTcpStages) & 1, err, 17, spins)) {
+      const int vec = ((int)blockIdx.x + ti * (int)gridDim.x) * kTcBM / P;
+      const float scale = __uint_as_float((unsigned)(267 - max_exponent(max_in + 8 * vec)) << 23);  // 2^(140 - E)
+      for (int j = 0; j < nst && ok; ++j, ++gi) {
+        const int st = gi % kTcRing;
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_afull[st]), (gi / kTcRing) & 1, t.err, 17, t.spins))) {
           ok = false;
           break;
         }
-        // the remainder slot was last read by the MMAs of step gi - kTcpLoSlots
-        if (gi >= kTcpLoSlots &&
-            !mbar_wait(smem_u32(&bar_lofree[ls]), ((gi / kTcpLoSlots) - 1) & 1, err, 19, spins)) {
-          ok = false;
-          break;
-        }
-        unsigned char* sp = smem_raw + ((base + st * stage_bytes) - smem_u32(smem_raw)) + t * kTcRowBytes;
-        unsigned char* lp =
-            smem_raw + ((lo_base + ls * 2u * kTcABytes) - smem_u32(smem_raw)) + t * kTcRowBytes;
-        float4* a1 = reinterpret_cast<float4*>(sp);
-        float4* a2 = reinterpret_cast<float4*>(sp + kTcABytes);
-        float4* l1 = reinterpret_cast<float4*>(lp);
-        float4* l2 = reinterpret_cast<float4*>(lp + kTcABytes);
-        const int pc[2] = {c0 ^ x, (3 - c0) ^ x};
-        const float4 av[2] = {a1[pc[0]], a1[pc[1]]}, mv[2] = {a2[pc[0]], a2[pc[1]]};
+        for (int kk = tt >> 8; kk < 2 && ok; kk += CONV / 256) {
+          const int g2 = 2 * gi + kk, sk = g2 % kTcSteps;
+          uint4 sh, sl, dh, dl;
+          const unsigned char* raw = smem + st * 2u * kTcABytes + r * 128;
+          float s[8], d[8];
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          float4 hh, ll;
-          if (BWD) {
-            split4(av[c], hh, ll);
-            a1[pc[c]] = hh;
-            l1[pc[c]] = ll;
-            split4(mv[c], hh, ll);
-          } else {
-            const float4 a = av[c], m = mv[1 - c];
-            split4(make_float4(a.x + m.w, a.y + m.z, a.z + m.y, a.w + m.x), hh, ll);
-            a1[pc[c]] = hh;
-            l1[pc[c]] = ll;
-            split4(make_float4(a.x - m.w, a.y - m.z, a.z - m.y, a.w - m.x), hh, ll);
+          for (int c = 0; c < 2; ++c) {
+            const int ca = 4 * kk + 2 * hf + c, cm = BWD ? ca : 7 - ca;  // forward: the mirrors in reverse order
+            const float4 x = *reinterpret_cast<const float4*>(raw + ((ca ^ (r & 7)) << 4));
+            const float4 y = *reinterpret_cast<const float4*>(raw + kTcABytes + ((cm ^ (r & 7)) << 4));
+            const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const float m = BWD ? ys[e] : ys[3 - e];
+              s[4 * c + e] = (BWD ? xs[e] : xs[e] + m) * scale;
+              d[4 * c + e] = (BWD ? m : xs[e] - m) * scale;
+            }
           }
-          a2[pc[c]] = hh;
-          l2[pc[c]] = ll;
+          split8(s, sh, sl);
+          split8(d, dh, dl);
+          // the k-step's part of the slot was last read by the MMAs of k-step g2 - kTcSteps
+          if (g2 >= kTcSteps &&
+              !__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_done[sk]), ((g2 / kTcSteps) - 1) & 1, t.err, 19, t.spins))) {
+            ok = false;
+            break;
+          }
+          unsigned char* dst =
+              smem + conv0 + (sk >> 1) * 4u * kTcCBytes + r * 64 + (((2 * kk + hf) ^ ((r >> 1) & 3)) << 4);
+          *reinterpret_cast<uint4*>(dst) = sh;
+          *reinterpret_cast<uint4*>(dst + kTcCBytes) = sl;
+          *reinterpret_cast<uint4*>(dst + 2 * kTcCBytes) = dh;
+          *reinterpret_cast<uint4*>(dst + 3 * kTcCBytes) = dl;
+          // the fence also stands between this thread's reads of the raw stage and its release: an arrival directly
+          // after the loads let the next copy overtake them
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) {
+            mbar_arrive(smem_u32(&bar_conv[sk]));
+            mbar_arrive(smem_u32(&bar_afree[st]));
+          }
         }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_arrive(smem_u32(&bar_conv[st]));
       }
     }
-  } else {
-    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31, one row of the tile per thread
-    const int q = warp % 4;
-    const int row = q * 32 + lane;
+  } else if (warp < 2 + CONV / 32 + kTcEpi) {
+    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31, one row of the tile per thread; the two warps of a quadrant
+    // take alternate chunks of 16 outputs
+    const int row = (warp % 4) * 32 + lane, half = (warp - 2 - CONV / 32) / 4;
+    const unsigned ready0 = pdl_wait();
+    const unsigned* __restrict__ max_in = t.max_in + ready0;
+    if (blockIdx.x == 0)  // a slot that the kernel before this one has read
+      for (int v = threadIdx.x - 64 - CONV; v * P < t.Ptot; v += 32 * kTcEpi) t.max_reset[8 * v] = 0;
+    float top = 0.f;  // the largest output of field top_vec so far
+    int top_vec = 0;
     for (int ti = 0; ti < my_tiles; ++ti) {
       const int b = ti & 1;
-      const bool ok = mbar_wait(smem_u32(&bar_accf[b]), (ti / 2) & 1, err, 18, spins);
+      // row p of field vec (fields of P x n, one after another)
+      const int p0 = ((int)blockIdx.x + ti * (int)gridDim.x) * kTcBM, vec = p0 / P, p = p0 + row - vec * P;
+      float* __restrict__ o = t.out + ready0 + (size_t)vec * P * n + p;
+      float sa = 0.f, sb = 0.f;
+      bool null_row = false;
+      if (SCALE) {
+        const int pa = p / t.nb;
+        sa = t.ly[pa];
+        sb = t.lx[p - pa * t.nb];
+        null_row = p == 0;
+      }
+      // 2^(E - 140); a field with an Inf or NaN keeps them through the splits
+      const float row_scale = __uint_as_float((unsigned)(std::min(max_exponent(max_in + 8 * vec), 254) - 13) << 23);
+      const bool ok = mbar_wait(smem_u32(&bar_accf[b]), (ti / 2) & 1, t.err, 18, t.spins);
       if (!__all_sync(0xffffffffu, ok)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      // row pg of the stacked block: row p of field vec (fields of P x n, one after another)
-      const int pg = ((int)blockIdx.x + ti * (int)gridDim.x) * kTcBM + row;
-      const int vec = pg / P, p = pg - vec * P;
-      const bool live = pg < Ptot;
-      float* __restrict__ o = out + (long long)vec * P * n;
-      float sa = 0.f, sb2 = 0.f;
-      int pa = 0, pb = 0;
-      if (SCALE && live) {
-        pa = p / nb;
-        pb = p - pa * nb;
-        sa = ly[pa];
-        sb2 = lx[pb];
+      const uint32_t lane_base = tmem + ((uint32_t)((warp % 4) * 32) << 16) + (uint32_t)(b * 256);
+      if (t.max_out && vec != top_vec) {
+        if (ti > 0) max_to(t.max_out + 8 * top_vec, top);
+        top = 0.f;
+        top_vec = vec;
       }
-      const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * 256);
-      for (int c0 = 0; c0 < h; c0 += 16) {
+      for (int c0 = 16 * half; c0 < h; c0 += 32) {
         uint32_t r1[16], r2[16];
         tmem_ld16(lane_base + (uint32_t)c0, r1);
         tmem_ld16(lane_base + (uint32_t)(h + c0), r2);
-        if (live) {
+        float* __restrict__ o1 = o + (size_t)c0 * P;
+        float* __restrict__ o2 = o + (size_t)(BWD ? n - 1 - c0 : h + c0) * P;
 #pragma unroll
-          for (int jj = 0; jj < 16; ++jj) {
-            const int m = c0 + jj;
-            const float v1 = __uint_as_float(r1[jj]), v2 = __uint_as_float(r2[jj]);
-            if (BWD) {  // cells m and n-1-m
-              o[(long long)m * P + p] = v1 + v2;
-              o[(long long)(n - 1 - m) * P + p] = v1 - v2;
-            } else if (SCALE) {  // symmetric mode m, antisymmetric mode h + m
-              const float s1 = (m == 0 && pa == 0 && pb == 0) ? 0.f : v1 * rcp_approx(lz_s[m] + sa + sb2);
-              o[(long long)m * P + p] = s1;
-              o[(long long)(h + m) * P + p] = v2 * rcp_approx(lz_s[h + m] + sa + sb2);
-            } else {
-              o[(long long)m * P + p] = v1;
-              o[(long long)(h + m) * P + p] = v2;
-            }
+        for (int jj = 0; jj < 16; ++jj) {
+          const float cs = col_s[c0 + jj];
+          float v1 = __uint_as_float(r1[jj]) * cs, v2 = __uint_as_float(r2[jj]) * cs;
+          if (BWD) {  // cells m and n-1-m
+            const float s = v1 + v2;
+            v2 = v1 - v2;
+            v1 = s;
           }
+          v1 *= row_scale;
+          v2 *= row_scale;
+          if (SCALE) {  // symmetric mode m, antisymmetric mode h + m
+            const int m = c0 + jj;
+            v1 = (m == 0 && null_row) ? 0.f : v1 * rcp_approx(lz_s[m] + sa + sb);
+            v2 *= rcp_approx(lz_s[h + m] + sa + sb);
+          }
+          top = fmaxf(top, fmaxf(fabsf(v1), fabsf(v2)));
+          *o1 = v1;
+          *o2 = v2;
+          o1 += P;
+          o2 += BWD ? -P : P;
         }
       }
       // the accumulator's values are in registers (tcgen05.wait::ld): the MMAs may reuse it
@@ -328,13 +403,12 @@ __global__ void __launch_bounds__(kTcpThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bar_acce[b]));
     }
+    if (t.max_out) max_to(t.max_out + 8 * top_vec, top);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 1) {
-    __syncwarp();
+  if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
-  }
 }
 
 using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -355,12 +429,21 @@ EncodeFn encoder() {
   return fn;
 }
 
-// rows x cols fp32 row-major matrix (cols contiguous), boxes of 16 columns x box_rows rows, 64-byte swizzle
-int encode(CUtensorMap* m, const float* ptr, long long rows, int cols, int box_rows) {
+// rows x cols FP32 row-major matrix (cols contiguous), boxes of 32 columns x 128 rows, 128-byte swizzle
+int encode(CUtensorMap* m, const float* ptr, long long rows, int cols) {
   const uint64_t dims[2] = {(uint64_t)cols, (uint64_t)rows};
   const uint64_t strides[1] = {(uint64_t)cols * 4};
-  const uint32_t box[2] = {(uint32_t)kTcBK, (uint32_t)box_rows};
-  return encode_tensor_map(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, ptr, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B);
+  const uint32_t box[2] = {(uint32_t)kTcBK, (uint32_t)kTcBM};
+  return encode_tensor_map(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, ptr, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
+// Shared memory of a pass of n outputs: the raw stages, the converted slots and B, all of it where it fits, else a ring
+// of two slabs.
+size_t tc_layout(int n, int& bslots) {
+  const int h = n / 2, nst = (h + kTcBK - 1) / kTcBK;
+  const size_t fixed = kTcRing * 2 * kTcABytes + (kTcSteps / 2) * 4 * kTcCBytes + 1024, slab = (size_t)4 * h * 64;
+  bslots = fixed + nst * slab <= kTcSmemMost ? nst : 2;
+  return fixed + bslots * slab;
 }
 
 }  // namespace
@@ -389,89 +472,69 @@ int encode_tensor_map(CUtensorMap* map, CUtensorMapDataType type, int rank, cons
   return FV_OK;
 }
 
-namespace {
-
-size_t tcp_smem_bytes(int n) {
-  return (size_t)kTcpStages * (2 * kTcABytes + 4 * (size_t)(n / 2) * kTcRowBytes) +
-         (size_t)kTcpLoSlots * 2 * kTcABytes + 1024;
-}
-
-}  // namespace
-
-bool tc_eligible(const fv_grid_s* g) {
-  const int ns[3] = {g->nx, g->ny, g->nz};
-  for (int d = 0; d < 3; ++d) {
-    if (ns[d] < 32 || ns[d] > 256 || ns[d] % 32 != 0) return false;
-    if (!mirror_symmetric(g->xf[d])) return false;  // the half-size eigenproblems need a symmetric axis
-  }
-  return encoder() != nullptr;
-}
-
-// Builds the passes' operands on the host (tc_host_operands), uploads them into one device buffer,
-// encodes the tensor maps of the B matrices and sets the kernels' shared-memory limits.
-int tc_setup(fv_grid_s* g, const std::vector<double>* idx, const std::vector<double>* idc) {
-  static_assert(kTcBK == kTcSlabCols, "the host operand layout and the kernels share the K slab width");
-  const int ns[3] = {g->nx, g->ny, g->nz};
-  TcOperands op;
-  FV_TRY(tc_host_operands(ns, idx, idc, op));
-  const size_t total = op.buf.size();
-  const std::vector<float>& hbuf = op.buf;
-  const auto& loff = op.loff;
-  const auto& soff = op.soff;
-  void* buf = nullptr;
-  if (cudaMalloc(&buf, total * sizeof(float)) != cudaSuccess) {
-    cudaGetLastError();
-    set_error("tensor-core operand allocation failed");
-    return FV_ENOMEM;
-  }
-  g->tc.buf = buf;
-  FV_CUDA(cudaMemcpy(buf, hbuf.data(), total * sizeof(float), cudaMemcpyHostToDevice));
-  for (int d = 0; d < 3; ++d) {
-    g->tc.lam[d] = (const float*)buf + loff[d];
-    for (int dir = 0; dir < 2; ++dir) g->tc.Bsw[d][dir] = (const unsigned char*)((const float*)buf + soff[d][dir]);
-  }
-  const int smemp_max = (int)tcp_smem_bytes(256);
-  FV_CUDA(cudaFuncSetAttribute(k_transform_tcp<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemp_max));
-  FV_CUDA(cudaFuncSetAttribute(k_transform_tcp<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemp_max));
-  FV_CUDA(cudaFuncSetAttribute(k_transform_tcp<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemp_max));
-  g->tc.ready = true;
+// The grid's FP32 pressure solves take these passes (half-size operators and their FP16 parts are ready).
+int tc_setup(fv_grid_s* g) {
+  static_assert(kDigitCols32 == 64 && kDigits32 == 2, "the B blocks hold 64 outputs, two parts");
+  for (int n : {g->nx, g->ny, g->nz})
+    if (n < 32 || n > 256 || n % 32 != 0) return FV_OK;
+  if (!g->digit_ready || !encoder()) return FV_OK;
+  for (auto k : {k_pass_tc<false, false, 256>, k_pass_tc<true, false, 256>, k_pass_tc<false, true, 256>,
+                 k_pass_tc<false, false, 512>, k_pass_tc<true, false, 512>, k_pass_tc<false, true, 512>})
+    FV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMost));
+  g->tc_ready = true;
   return FV_OK;
 }
 
-// one pass: in[a][b][k] (na*nb rows of n) -> out[m][a][b] with the matrices of `axis`; bwd selects the
-// backward (modes -> cells) matrices.  Mode indices are in the tensor-core order throughout.  nvec > 1:
-// that many fields of na*nb*n elements one after another in `in` and in `out`, each transformed alone,
-// all in one persistent launch.
-int tc_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const float* in, float* out, bool scale,
-            int nvec) {
+// Pass 0 .. 5 of a solve (forward x, y, z, backward x, y, z): in[a][b][k] (na*nb rows of n) -> out[m][a][b].  Mode
+// indices are in the half order throughout.  nvec > 1: that many fields of na*nb*n elements one after another in `in`
+// and in `out`, each transformed alone, all in one launch.  slots: 8 words per field; pass i reads the field's largest
+// magnitude in word i, leaves its output's in word i + 1 (not the last pass) and clears word i - 1 (the first pass:
+// word 5), so that every word is zero again before the next solve writes it.
+int tc_pass(const fv_grid_s* g, int pass, int na, int nb, const float* in, float* out, unsigned* slots, int nvec) {
+  const int axis = pass % 3;
+  const bool bwd = pass >= 3;
   const int n = (axis == 0) ? g->nx : (axis == 1) ? g->ny : g->nz;
-  const long long P = (long long)na * nb;
-  if (nvec < 1 || P * nvec > (1LL << 30)) {
+  const long long P = (long long)na * nb, Ptot = P * nvec;
+  if (nvec < 1 || Ptot > (1LL << 30)) {
     set_error("tc_pass: batch of fields not supported here");
     return FV_EINVAL;
   }
-  const long long Ptot = P * nvec;
   CUtensorMap tmA;
-  FV_TRY(encode(&tmA, in, Ptot, n, kTcBM));
-  const long long ntiles = (Ptot + kTcBM - 1) / kTcBM;
+  FV_TRY(encode(&tmA, in, Ptot, n));
+  const HalfDev<float>& d = g->half32[axis][HALF_NEUMANN];
+  TcArgs t{};
+  t.B = d.dig[bwd ? 1 : 0];
+  t.bexp = d.dexp[bwd ? 1 : 0];
+  t.out = out;
+  t.lx = g->half32[0][HALF_NEUMANN].lam;
+  t.ly = g->half32[1][HALF_NEUMANN].lam;
+  t.lz = g->half32[2][HALF_NEUMANN].lam;
+  t.max_in = slots + pass;
+  t.max_out = pass < 5 ? slots + pass + 1 : nullptr;
+  t.max_reset = slots + (pass + 5) % 6;
+  t.P = (int)P;
+  t.Ptot = (int)Ptot;
+  t.n = n;
+  t.nb = nb;
+  const size_t smem = tc_layout(n, t.bslots);
+  t.err = g->ws.err;
+  t.spins = wait_spins(g);
+  const long long ntiles = Ptot / kTcBM;
+  const dim3 grid((unsigned)std::min<long long>(ntiles, g->sms));
   ProfScope ps(g, PROF_TRANSFORM_TC);
-  {
-    const size_t smemp = tcp_smem_bytes(n);
-    const unsigned char* bsw = g->tc.Bsw[axis][bwd ? 1 : 0];
-    const dim3 pgrid((unsigned)std::min<long long>(ntiles, g->sms));
-    if (bwd)
-      launch(k_transform_tcp<false, true>, pgrid, kTcpThreads, smemp, g->stream, 
-          tmA, bsw, out, (int)P, (int)Ptot, n, nullptr, nullptr, nullptr, nb, g->ws.err, wait_spins(g));
-    else if (scale)
-      launch(k_transform_tcp<true, false>, pgrid, kTcpThreads, smemp, g->stream, 
-          tmA, bsw, out, (int)P, (int)Ptot, n, g->tc.lam[0], g->tc.lam[1], g->tc.lam[2], nb, g->ws.err,
-          wait_spins(g));
-    else
-      launch(k_transform_tcp<false, false>, pgrid, kTcpThreads, smemp, g->stream, 
-          tmA, bsw, out, (int)P, (int)Ptot, n, nullptr, nullptr, nullptr, nb, g->ws.err, wait_spins(g));
-    FV_CUDA(cudaGetLastError());
-    return FV_OK;
-  }
+  // twice the converters from five steps a tile on (256^3 chebyshev step 613 -> 602 us); with fewer steps the larger
+  // block's start costs more than they save (64^3 product 47 -> 49 us)
+  auto go = [&](auto conv) {
+    constexpr int C = decltype(conv)::value;
+    auto k = bwd ? k_pass_tc<false, true, C> : pass == 2 ? k_pass_tc<true, false, C> : k_pass_tc<false, false, C>;
+    launch(k, grid, tc_threads(C), smem, g->stream, tmA, t);
+  };
+  if (n > 128)
+    go(std::integral_constant<int, 512>());
+  else
+    go(std::integral_constant<int, 256>());
+  FV_CUDA(cudaGetLastError());
+  return FV_OK;
 }
 
 }  // namespace fv
