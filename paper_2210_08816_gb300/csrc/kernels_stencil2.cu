@@ -134,53 +134,81 @@ struct Ring2 {
 };
 
 
-// Transverse (D != C) fluxes of momentum component C through the D-faces of its control volume:
-// the D-velocity interpolated along C to the C-face times the C-velocity interpolated along D.
-template <int C, int D, typename BC, typename BD>
-__device__ __forceinline__ void transverse(const Ring2& S, const BC& MC, const BD& MD, float2 aH, float2 bH,
-                                           float2& conv, float2& lap) {
+// The convective flux of momentum component C through the low or high D-face of its control volume (D != C): the
+// D-velocity interpolated along C to the edge times the C-velocity interpolated along D.  Exchanging C and D exchanges
+// the two factors: components C and D share the flux of every edge.  n: the C-pair across the face.
+template <int C, int D>
+__device__ __forceinline__ float2 edge_lo(const Ring2& S, const Bundle<float2>& MC, const Bundle<float2>& MD, float2 aH,
+                                          float2 bH, float2 bCm) {
   constexpr int cx = unit_(C, 0), cy = unit_(C, 1), cz = unit_(C, 2);
   constexpr int dx = unit_(D, 0), dy = unit_(D, 1), dz = unit_(D, 2);
   constexpr int AB = 4;
-  // low face
-  const float2 aDcL = fma2(MC.wl, S.ld<D, -cx, -cy, -cz>(), MC.wr * S.ld<D, 0, 0, 0>());
-  const float2 bDcL = fma2(MC.wl, S.ld<AB + D, -cx, -cy, -cz>(), MC.wr * S.ld<AB + D, 0, 0, 0>());
-  const float2 bCm = S.ld<AB + C, -dx, -dy, -dz>(), aCm = S.ld<C, -dx, -dy, -dz>();
-  const float2 aCdL = fma2(MD.wl, aCm, MD.wr * aH);
-  const float2 bCdL = fma2(MD.wl, bCm, MD.wr * bH);
-  const float2 fLo = fma2(aDcL, bCdL, bDcL * aCdL);
-  const float2 gLo = (bH - bCm) * MD.ic;
-  // high face
-  const float2 aDcH = fma2(MC.wl, S.ld<D, dx - cx, dy - cy, dz - cz>(), MC.wr * S.ld<D, dx, dy, dz>());
-  const float2 bDcH = fma2(MC.wl, S.ld<AB + D, dx - cx, dy - cy, dz - cz>(), MC.wr * S.ld<AB + D, dx, dy, dz>());
-  const float2 bCp = S.ld<AB + C, dx, dy, dz>(), aCp = S.ld<C, dx, dy, dz>();
-  const float2 aCdH = fma2(MD.wlp, aH, MD.wrp * aCp);
-  const float2 bCdH = fma2(MD.wlp, bH, MD.wrp * bCp);
-  const float2 fHi = fma2(aDcH, bCdH, bDcH * aCdH);
-  const float2 gHi = (bCp - bH) * MD.icp;
+  const float2 aDc = fma2(MC.wl, S.ld<D, -cx, -cy, -cz>(), MC.wr * S.ld<D, 0, 0, 0>());
+  const float2 bDc = fma2(MC.wl, S.ld<AB + D, -cx, -cy, -cz>(), MC.wr * S.ld<AB + D, 0, 0, 0>());
+  const float2 aCd = fma2(MD.wl, S.ld<C, -dx, -dy, -dz>(), MD.wr * aH);
+  const float2 bCd = fma2(MD.wl, bCm, MD.wr * bH);
+  return fma2(aDc, bCd, bDc * aCd);
+}
+template <int C, int D>
+__device__ __forceinline__ float2 edge_hi(const Ring2& S, const Bundle<float2>& MC, const Bundle<float2>& MD, float2 aH,
+                                          float2 bH, float2 bCp) {
+  constexpr int cx = unit_(C, 0), cy = unit_(C, 1), cz = unit_(C, 2);
+  constexpr int dx = unit_(D, 0), dy = unit_(D, 1), dz = unit_(D, 2);
+  constexpr int AB = 4;
+  const float2 aDc = fma2(MC.wl, S.ld<D, dx - cx, dy - cy, dz - cz>(), MC.wr * S.ld<D, dx, dy, dz>());
+  const float2 bDc = fma2(MC.wl, S.ld<AB + D, dx - cx, dy - cy, dz - cz>(), MC.wr * S.ld<AB + D, dx, dy, dz>());
+  const float2 aCd = fma2(MD.wlp, aH, MD.wrp * S.ld<C, dx, dy, dz>());
+  const float2 bCd = fma2(MD.wlp, bH, MD.wrp * bCp);
+  return fma2(aDc, bCd, bDc * aCd);
+}
+
+// conv, lap += the share of the D-faces of component C, whose low edge's convective flux is fLo
+template <int C, int D>
+__device__ __forceinline__ void across(const Ring2& S, const Bundle<float2>& MC, const Bundle<float2>& MD, float2 aH,
+                                       float2 bH, float2 fLo, float2& conv, float2& lap) {
+  constexpr int dx = unit_(D, 0), dy = unit_(D, 1), dz = unit_(D, 2);
+  constexpr int AB = 4;
+  const float2 bCm = S.ld<AB + C, -dx, -dy, -dz>(), bCp = S.ld<AB + C, dx, dy, dz>();
+  const float2 fHi = edge_hi<C, D>(S, MC, MD, aH, bH, bCp);
+  const float2 gLo = (bH - bCm) * MD.ic, gHi = (bCp - bH) * MD.icp;
   conv = fma2(fHi - fLo, MD.ix, conv);
   lap = fma2(gHi - gLo, MD.ix, lap);
 }
 
-// Momentum component C: conv = S(q, v) (symmetrised convective form), lap = Lap v
+// the same through the z-faces of u and v: both fluxes of the low face are the plane below's high ones (f, g), which
+// become this plane's
 template <int C>
-__device__ __forceinline__ void momentum_pair(const Ring2& S, const Bundle<float2>& mx, const Bundle<float2>& my,
-                                              const Bundle<float2>& mz, float2& conv, float2& lap) {
-  constexpr int cx = unit_(C, 0), cy = unit_(C, 1), cz = unit_(C, 2);
-  constexpr int AB = 4;
-  const auto& MC = pick<C>(mx, my, mz);
-  const float2 aH = S.ld<C, 0, 0, 0>(), bH = S.ld<AB + C, 0, 0, 0>();
-  const float2 aM = S.ld<C, -cx, -cy, -cz>(), bM = S.ld<AB + C, -cx, -cy, -cz>();
-  const float2 aP = S.ld<C, cx, cy, cz>(), bP = S.ld<AB + C, cx, cy, cz>();
+__device__ __forceinline__ void across_z(const Ring2& S, const Bundle<float2>& MC, const Bundle<float2>& mz, float2 aH,
+                                         float2 bH, float2& f, float2& g, float2& conv, float2& lap) {
+  const float2 bCp = S.ld<4 + C, 0, 0, 1>();
+  const float2 fHi = edge_hi<C, 2>(S, MC, mz, aH, bH, bCp);
+  const float2 gHi = (bCp - bH) * mz.icp;
+  conv = fma2(fHi - f, mz.ix, conv);
+  lap = fma2(gHi - g, mz.ix, lap);
+  f = fHi;
+  g = gHi;
+}
+
+// conv, lap of component C (x or y) through the faces across its own axis
+template <int C>
+__device__ __forceinline__ void along(const Ring2& S, const Bundle<float2>& MC, float2 aH, float2 bH, float2& conv,
+                                      float2& lap) {
+  constexpr int cx = unit_(C, 0), cy = unit_(C, 1);
+  const float2 aM = S.ld<C, -cx, -cy, 0>(), bM = S.ld<4 + C, -cx, -cy, 0>();
+  const float2 aP = S.ld<C, cx, cy, 0>(), bP = S.ld<4 + C, cx, cy, 0>();
   const float2 half = bc(0.5f), two = bc(2.f);
   const float2 aE = half * (aH + aP), bE = half * (bH + bP);
   const float2 aW = half * (aM + aH), bW = half * (bM + bH);
   conv = two * (aE * bE - aW * bW) * MC.ic;
   lap = ((bP - bH) * MC.ix - (bH - bM) * MC.ixm) * MC.ic;
-  constexpr int D1 = (C + 1) % 3, D2 = (C + 2) % 3;
-  transverse<C, D1>(S, MC, pick<D1>(mx, my, mz), aH, bH, conv, lap);
-  transverse<C, D2>(S, MC, pick<D2>(mx, my, mz), aH, bH, conv, lap);
 }
+
+// Fluxes through the low z-faces of a pair's four control volumes (convective f, diffusive g); across the w-face's own
+// axis the product of the halved sums and the scaled difference.  A thread marches along z: the next plane's low
+// fluxes are this plane's high ones, and w's low x- and y-edges are u's and v's low z-edges.
+struct LowZ {
+  float2 f[4], g[4];
+};
 
 // Temperature fluxes through the D-faces of the cell; y, z walls: zero flux (select), x: Dirichlet 0
 template <int D, typename BD>
@@ -203,14 +231,39 @@ __device__ __forceinline__ void temperature_dir(const Ring2& S, const BD& MD, fl
 }
 
 __device__ __forceinline__ void temperature_pair(const Ring2& S, const Bundle<float2>& mx, const Bundle<float2>& my,
-                                                 const Bundle<float2>& mz, int j, int ny, int k, int nz, float2& conv,
-                                                 float2& lap) {
+                                                 const Bundle<float2>& mz, int j, int ny, int k, int nz, float2& f,
+                                                 float2& g, float2& conv, float2& lap) {
   const float2 TaH = S.ld<3, 0, 0, 0>(), TbH = S.ld<4 + 3, 0, 0, 0>();
   conv = make_float2(0.f, 0.f);
   lap = make_float2(0.f, 0.f);
   temperature_dir<0>(S, mx, TaH, TbH, true, true, conv, lap);
   temperature_dir<1>(S, my, TaH, TbH, j >= 1, j + 1 <= ny - 1, conv, lap);
-  temperature_dir<2>(S, mz, TaH, TbH, k >= 1, k + 1 <= nz - 1, conv, lap);
+  const float2 Tap = S.ld<3, 0, 0, 1>(), Tbp = S.ld<4 + 3, 0, 0, 1>();
+  const float2 fHi = fma2(S.ld<2, 0, 0, 1>(), fma2(mz.wlp, TbH, mz.wrp * Tbp),
+                          S.ld<4 + 2, 0, 0, 1>() * fma2(mz.wlp, TaH, mz.wrp * Tap));
+  float2 gHi = (Tbp - TbH) * mz.icp;
+  if (k + 1 > nz - 1) gHi = make_float2(0.f, 0.f);
+  conv = fma2(fHi - f, mz.ix, conv);
+  lap = fma2(gHi - g, mz.ix, lap);
+  f = fHi;
+  g = gHi;
+}
+
+__device__ __forceinline__ void low_z(const Ring2& S, const Bundle<float2>& mx, const Bundle<float2>& my,
+                                      const Bundle<float2>& mz, int k, LowZ& z) {
+  const float2 half = bc(0.5f);
+  const float2 bu = S.ld<4, 0, 0, -1>(), bv = S.ld<5, 0, 0, -1>(), bH0 = S.ld<4, 0, 0, 0>(), bH1 = S.ld<5, 0, 0, 0>();
+  z.f[0] = edge_lo<0, 2>(S, mx, mz, S.ld<0, 0, 0, 0>(), bH0, bu);
+  z.g[0] = (bH0 - bu) * mz.ic;
+  z.f[1] = edge_lo<1, 2>(S, my, mz, S.ld<1, 0, 0, 0>(), bH1, bv);
+  z.g[1] = (bH1 - bv) * mz.ic;
+  const float2 bM = S.ld<6, 0, 0, -1>(), bH2 = S.ld<6, 0, 0, 0>();
+  z.f[2] = half * (S.ld<2, 0, 0, -1>() + S.ld<2, 0, 0, 0>()) * (half * (bM + bH2));
+  z.g[2] = (bH2 - bM) * mz.ixm;
+  const float2 Tam = S.ld<3, 0, 0, -1>(), Tbm = S.ld<7, 0, 0, -1>();
+  const float2 TaH = S.ld<3, 0, 0, 0>(), TbH = S.ld<7, 0, 0, 0>();
+  z.f[3] = fma2(S.ld<2, 0, 0, 0>(), fma2(mz.wl, Tbm, mz.wr * TbH), bH2 * fma2(mz.wl, Tam, mz.wr * TaH));
+  z.g[3] = k >= 1 ? (TbH - Tbm) * mz.ic : make_float2(0.f, 0.f);
 }
 
 __device__ __forceinline__ uint32_t smem_addr2(const void* p) {
@@ -242,7 +295,7 @@ __global__ void __launch_bounds__(kPX / 2 * kPY, 2)
                    int nch) {
   constexpr uint32_t kBox = 4u * kPL2 * sizeof(float);  // one state's box: 4 fields x kPHY x kPW2
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t bar[kPRing];
+  __shared__ __align__(8) uint64_t bar[kPRing], bar_done[2];
   float* sm = reinterpret_cast<float*>(smem_raw);  // [kPRing][kPNA][kPL2]
   const int tid = threadIdx.x;
   const int tx = tid % (kPX / 2), ty = tid / (kPX / 2);
@@ -258,87 +311,121 @@ __global__ void __launch_bounds__(kPX / 2 * kPY, 2)
   if (tid == 0) {
     for (int s2 = 0; s2 < kPRing; ++s2)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr2(&bar[s2])) : "memory");
+    for (int s2 = 0; s2 < 2; ++s2)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr2(&bar_done[s2])), "r"(kPX / 2 * kPY / 32)
+                   : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   const unsigned ready0 = pdl_wait();
   out += ready0;
+  // thread 0: plane kk of both states (zeros outside the domain)
   auto issue_plane = [&](int kk) {
     float* slot = sm + ((kk + kPRing) % kPRing) * kPNA * kPL2;
     const uint32_t b = smem_addr2(&bar[(kk + kPRing) % kPRing]);
-    if (kk >= 0 && kk < nz) {
-      if (tid == 0) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(2u * kBox) : "memory");
-        asm volatile(
-            "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, "
-            "%5, %6}], [%2];" ::"r"(smem_addr2(slot)),
-            "l"(reinterpret_cast<uint64_t>(&tmq)), "r"(b), "r"(i0 - kPX0), "r"(j0 - 1), "r"(kk), "r"(0)
-            : "memory");
-        asm volatile(
-            "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, "
-            "%5, %6}], [%2];" ::"r"(smem_addr2(slot + 4 * kPL2)),
-            "l"(reinterpret_cast<uint64_t>(&tmv)), "r"(b), "r"(i0 - kPX0), "r"(j0 - 1), "r"(kk), "r"(4 * vec)
-            : "memory");
-      }
-    } else {  // a plane outside the domain: zeros, and a plain arrival completes the barrier phase
-      for (int e = tid; e < kPNA * kPL2; e += kPX / 2 * kPY) slot[e] = 0.f;
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      if (tid == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
-    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(2u * kBox) : "memory");
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, "
+        "%5, %6}], [%2];" ::"r"(smem_addr2(slot)),
+        "l"(reinterpret_cast<uint64_t>(&tmq)), "r"(b), "r"(i0 - kPX0), "r"(j0 - 1), "r"(kk), "r"(0)
+        : "memory");
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, "
+        "%5, %6}], [%2];" ::"r"(smem_addr2(slot + 4 * kPL2)),
+        "l"(reinterpret_cast<uint64_t>(&tmv)), "r"(b), "r"(i0 - kPX0), "r"(j0 - 1), "r"(kk), "r"(4 * vec)
+        : "memory");
   };
   // plane kk lives in slot kk mod kPRing; it is that slot's use number (kk - k0 + 1) / kPRing
   auto wait_plane = [&](int kk) -> bool {
     return bar_wait2(smem_addr2(&bar[(kk + kPRing) % kPRing]), (uint32_t)(((kk - k0 + 1) / kPRing) & 1), err,
                      spins);
   };
-  issue_plane(k0 - 1);
-  issue_plane(k0);
-  issue_plane(k0 + 1);
-  int issued = k0 + 1;  // last plane whose copy was started (the same value in every thread)
-  __syncthreads();
+  if (tid == 0)
+    for (int kk = k0 - 1; kk <= k0 + 1; ++kk) issue_plane(kk);
+  int issued = k0 + 1;  // (thread 0) last plane whose copy was started
   bool ok = wait_plane(k0 - 1);
   ok = wait_plane(k0) && ok;
-  ok = __syncthreads_and(ok);  // one decision for the whole CTA
+  ok = __all_sync(0xffffffffu, ok);
   const int x = i0 + 2 * tx, j = j0 + ty;
   const bool active = (x < nx && j < ny);  // nx is a multiple of kPX: both cells are in the domain
   const Bundle<float2> mx = load_bundle_pair(g, active ? x : 0);
   const Bundle<float2> my = broadcast(load_bundle(g, 1, active ? j : 0));
+  LowZ z;
+  if (active && ok) {
+    Ring2 S;
+#pragma unroll
+    for (int dz = -1; dz <= 1; ++dz)
+      S.p[dz + 1] = sm + ((k0 + dz + kPRing) % kPRing) * kPNA * kPL2 + (ty + 1) * kPW2 + (2 * tx + kPX0);
+    low_z(S, mx, my, broadcast(load_bundle(g, 2, k0)), k0, z);
+  }
   for (int k = k0; k < kend && ok; ++k) {
-    if (k + 2 <= kend) {  // plane k+2 feeds the output plane k+1
-      issue_plane(k + 2);
-      issued = k + 2;
+    const Bundle<float2> mz = broadcast(load_bundle(g, 2, k));
+    // Plane k + 2 takes the slot of plane k - 2, which every warp has read once it has done plane k - 1.  The first warp
+    // alone waits for the others; they run on to the next plane by themselves.
+    if (tid < 32 && k + 2 <= kend) {
+      const int i = k - 1 - k0;
+      if (i >= 0 && !__all_sync(0xffffffffu, bar_wait2(smem_addr2(&bar_done[i & 1]), (uint32_t)((i >> 1) & 1), err, spins)))
+        ok = false;
+      if (ok) {
+        if (tid == 0) issue_plane(k + 2);
+        issued = k + 2;
+      }
     }
-    const bool ready = wait_plane(k + 1);
-    if (active && ready) {
-      const Bundle<float2> mz = broadcast(load_bundle(g, 2, k));
+    ok = __all_sync(0xffffffffu, wait_plane(k + 1)) && ok;
+    if (active && ok) {
       Ring2 S;
 #pragma unroll
       for (int dz = -1; dz <= 1; ++dz)
         S.p[dz + 1] = sm + ((k + dz + kPRing) % kPRing) * kPNA * kPL2 + (ty + 1) * kPW2 + (2 * tx + kPX0);
       float2 conv, lap;
-      momentum_pair<0>(S, mx, my, mz, conv, lap);
       const float2 msig = bc(-sigma);
-      float2 r0 = fma2(msig, S.ld<4, 0, 0, 0>(), lap - conv);
-      momentum_pair<1>(S, mx, my, mz, conv, lap);
-      const float2 r1 = fma2(msig, S.ld<5, 0, 0, 0>(), lap - conv);
-      momentum_pair<2>(S, mx, my, mz, conv, lap);
-      const float2 Tf = fma2(mz.wl, S.ld<7, 0, 0, -1>(), mz.wr * S.ld<7, 0, 0, 0>());
-      const float2 r2 = fma2(msig, S.ld<6, 0, 0, 0>(), fma2(bc(Gr), Tf, lap - conv));
-      temperature_pair(S, mx, my, mz, j, ny, k, nz, conv, lap);
-      const float2 r3 = fma2(msig, S.ld<7, 0, 0, 0>(), lap * bc(invPr) - conv);
       const int o = (k * ny + j) * nx + x;
-      if (x == 0) r0.x = 0.f;  // the x = 0 wall slot of u
       const float2 zero = make_float2(0.f, 0.f);
-      *reinterpret_cast<float2*>(out + o) = r0;
-      *reinterpret_cast<float2*>(out + N + o) = (j >= 1) ? r1 : zero;
-      *reinterpret_cast<float2*>(out + 2 * N + o) = (k >= 1) ? r2 : zero;
+      {  // w: its low edges are u's and v's low z-edges
+        const float2 aH = S.ld<2, 0, 0, 0>(), bH = S.ld<6, 0, 0, 0>(), bP = S.ld<6, 0, 0, 1>();
+        const float2 half = bc(0.5f);
+        const float2 fE = half * (aH + S.ld<2, 0, 0, 1>()) * (half * (bH + bP)), gE = (bP - bH) * mz.ix;
+        conv = bc(2.f) * (fE - z.f[2]) * mz.ic;
+        lap = (gE - z.g[2]) * mz.ic;
+        z.f[2] = fE;
+        z.g[2] = gE;
+        across<2, 0>(S, mz, mx, aH, bH, z.f[0], conv, lap);
+        across<2, 1>(S, mz, my, aH, bH, z.f[1], conv, lap);
+        const float2 Tf = fma2(mz.wl, S.ld<7, 0, 0, -1>(), mz.wr * S.ld<7, 0, 0, 0>());
+        const float2 r2 = fma2(msig, bH, fma2(bc(Gr), Tf, lap - conv));
+        *reinterpret_cast<float2*>(out + 2 * N + o) = (k >= 1) ? r2 : zero;
+      }
+      float2 exy;  // the flux of the low x-y edge, u's and v's
+      {
+        const float2 aH = S.ld<0, 0, 0, 0>(), bH = S.ld<4, 0, 0, 0>();
+        exy = edge_lo<0, 1>(S, mx, my, aH, bH, S.ld<4, 0, -1, 0>());
+        along<0>(S, mx, aH, bH, conv, lap);
+        across<0, 1>(S, mx, my, aH, bH, exy, conv, lap);
+        across_z<0>(S, mx, mz, aH, bH, z.f[0], z.g[0], conv, lap);
+        float2 r0 = fma2(msig, bH, lap - conv);
+        if (x == 0) r0.x = 0.f;  // the x = 0 wall slot of u
+        *reinterpret_cast<float2*>(out + o) = r0;
+      }
+      {
+        const float2 aH = S.ld<1, 0, 0, 0>(), bH = S.ld<5, 0, 0, 0>();
+        along<1>(S, my, aH, bH, conv, lap);
+        across_z<1>(S, my, mz, aH, bH, z.f[1], z.g[1], conv, lap);
+        across<1, 0>(S, my, mx, aH, bH, exy, conv, lap);
+        const float2 r1 = fma2(msig, bH, lap - conv);
+        *reinterpret_cast<float2*>(out + N + o) = (j >= 1) ? r1 : zero;
+      }
+      temperature_pair(S, mx, my, mz, j, ny, k, nz, z.f[3], z.g[3], conv, lap);
+      const float2 r3 = fma2(msig, S.ld<7, 0, 0, 0>(), lap * bc(invPr) - conv);
       *reinterpret_cast<float2*>(out + 3 * N + o) = r3;
     }
-    ok = __syncthreads_and(ready);  // nobody reads the slot of plane k-1 any more; stop together on a give-up
+    __syncwarp();
+    if ((tid & 31) == 0)
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr2(&bar_done[(k - k0) & 1])) : "memory");
   }
-  // give-up path: every plane copy still in flight lands (waited for with the full limit) before the CTA
-  // exits, so that no bulk copy writes into shared memory the CTA no longer owns
+  // give-up path (a warp that stops arrives no more, so the first one runs into its limit too): every plane copy still in
+  // flight lands (waited for with the full limit) before the CTA exits, so that no bulk copy writes into shared memory
+  // the CTA no longer owns
   if (!ok && tid == 0)
     for (int kk = max(k0 - 1, issued - kPRing + 1); kk <= issued; ++kk)
       bar_wait2(smem_addr2(&bar[(kk + kPRing) % kPRing]), (uint32_t)(((kk - k0 + 1) / kPRing) & 1), err,
