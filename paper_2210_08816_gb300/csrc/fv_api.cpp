@@ -224,6 +224,29 @@ static int ensure_ws(fv_grid_s* g) {
 }
 
 // ------------------------------------------------------------------ the hot path
+// Whether the stencil writes T of out = alpha (..) + beta v + gamma w (nvec states from v on and from out on, FP32), and
+// with what: not where another thread block may still read what it would overwrite (out within q or v), nor where w and
+// out overlap other than element by element, nor (t.out null) from unaligned states, which the stencil's pairs of cells
+// cannot take.
+template <typename R>
+static TempOut temp_out(const fv_grid_s* g, const R* q, const R* v, bool add_v, double alpha, double beta, const R* w,
+                        double gamma, R* out, int nvec) {
+  TempOut t;
+  if constexpr (sizeof(R) == 4) {
+    const uintptr_t one = 4 * g->N * sizeof(R), o = (uintptr_t)out, end = o + one * nvec;
+    auto apart = [&](const R* p, int n) { return (uintptr_t)p >= end || (uintptr_t)p + one * n <= o; };
+    if (!apart(q, 1) || !apart(v, nvec) || (w && w != out && !apart(w, nvec))) return t;
+    if (o % 16 != 0 || (uintptr_t)w % 16 != 0) return t;
+    t.alpha = (float)alpha;
+    t.beta = (float)beta;
+    t.gamma = (float)gamma;
+    t.add_v = add_v;
+    t.w = w;
+    t.out = out;
+  }
+  return t;
+}
+
 template <typename R>
 int jvp_project(fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out) {
   FV_TRY(ensure_ws<R>(g));
@@ -231,10 +254,11 @@ int jvp_project(fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R
   R* Y = (R*)g->ws.Y[p];
   R* phi = (R*)g->ws.t1[p];
   R* tmp = (R*)g->ws.t0[p];
-  FV_TRY(launch_jvp<R>(g, Gr, sigma, q, v, Y));
+  const TempOut t = temp_out<R>(g, q, v, sigma != 0.0, 1.0, sigma, nullptr, 0.0, out, 1);
+  FV_TRY(launch_jvp<R>(g, Gr, sigma, q, v, Y, t));
   FV_TRY(launch_divergence<R>(g, Y, phi));
   FV_TRY(launch_poisson<R>(g, phi, phi, tmp));
-  FV_TRY(launch_correct<R>(g, Y, phi, 1.0, sigma != 0.0 ? v : nullptr, sigma, nullptr, 0.0, out));
+  FV_TRY(launch_correct<R>(g, Y, phi, 1.0, sigma != 0.0 ? v : nullptr, sigma, nullptr, 0.0, out, -1, t.out != nullptr));
   return FV_OK;
 }
 
@@ -247,10 +271,11 @@ int chebyshev_step(fv_grid_s* g, double Gr, double sigma, const R* q, const R* y
   R* Y = (R*)g->ws.Y[p];
   R* phi = (R*)g->ws.t1[p];
   R* tmp = (R*)g->ws.t0[p];
-  FV_TRY(launch_jvp<R>(g, Gr, sigma, q, y, Y));
+  const TempOut t = temp_out<R>(g, q, y, true, alpha, beta, yprev, gamma, out, 1);
+  FV_TRY(launch_jvp<R>(g, Gr, sigma, q, y, Y, t));
   FV_TRY(launch_divergence<R>(g, Y, phi));
   FV_TRY(launch_poisson<R>(g, phi, phi, tmp));
-  FV_TRY(launch_correct<R>(g, Y, phi, alpha, y, beta, yprev, gamma, out, norm_slot));
+  FV_TRY(launch_correct<R>(g, Y, phi, alpha, y, beta, yprev, gamma, out, norm_slot, t.out != nullptr));
   return FV_OK;
 }
 
@@ -814,16 +839,17 @@ static int jvp_project_block(fv_grid_s* g, double Gr, double sigma, const R* q, 
   R* phi = (R*)g->ws.bt1[p];
   R* tmp = (R*)g->ws.bt0[p];
   const size_t n4 = 4 * g->N;
+  const TempOut t = temp_out<R>(g, q, V, sigma != 0.0, 1.0, sigma, nullptr, 0.0, W, nvec);
   bool pair = false;
   if constexpr (sizeof(R) == 4) pair = stencil_pair_eligible(g, q, V);
   if constexpr (sizeof(R) == 4) {
-    if (pair) FV_TRY(launch_stencil_pair(g, Gr, sigma, q, V, Y, nvec));
+    if (pair) FV_TRY(launch_stencil_pair(g, Gr, sigma, q, V, Y, nvec, t));
   }
   (void)n4;
-  if (!pair) FV_TRY(launch_jvp_block<R>(g, Gr, sigma, q, V, Y, nvec));
+  if (!pair) FV_TRY(launch_jvp_block<R>(g, Gr, sigma, q, V, Y, nvec, t));
   FV_TRY(launch_divergence<R>(g, Y, phi, nvec));
   FV_TRY(launch_poisson_block<R>(g, phi, phi, tmp, nvec));
-  FV_TRY(launch_correct_block<R>(g, Y, phi, sigma != 0.0 ? V : nullptr, sigma, W, nvec));
+  FV_TRY(launch_correct_block<R>(g, Y, phi, sigma != 0.0 ? V : nullptr, sigma, W, nvec, t.out != nullptr));
   return FV_OK;
 }
 

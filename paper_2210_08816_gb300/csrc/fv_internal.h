@@ -188,25 +188,40 @@ struct ProfScope {
 // Stencils (kernels_stencil.cu)
 template <typename R>
 int launch_residual(const fv_grid_s* g, double Gr, const R* q, R* F);
+// T takes no pressure correction, so a step's T = alpha Y_T + beta v_T + gamma w_T needs no more than the stencil has at
+// hand (and w): FP32 stencils write it straight to `out` (the step's states, 4N each) instead of Y_T to the workspace, and
+// the correction, which memory bounds, leaves T alone (t_done): 13 or 14 array passes instead of 17 (10 of 13 without w)
+// for one read of w_T in the stencil.  256^3 chebyshev step: correction 183 -> 159 us, stencil 191 -> 202, the step 590 ->
+// 576; 16 x 64^3: correction 59.7 -> 41.3, stencil 57.7 -> 62.8, 182 -> 168.  FP64 stays: there both kernels are bound by
+// the FP64 pipe, which the move does not relieve.  out null: Y_T as any other component.
+struct TempOut {
+  float alpha = 1.f, beta = 0.f, gamma = 0.f;
+  int add_v = 0;
+  const float* w = nullptr;
+  float* out = nullptr;
+};
 template <typename R>
-int launch_jvp(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out);
+int launch_jvp(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out,
+               const TempOut& t = TempOut());
 // The one-cell J.v stencil over nvec states stored one after another in v and out (4N each), one launch.
 template <typename R>
-int launch_jvp_block(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out, int nvec);
+int launch_jvp_block(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out, int nvec,
+                     const TempOut& t = TempOut());
 // nvec > 1: vel holds nvec states (4N each) and rhs nvec fields (N each), one after another.  for_solve: launch_poisson
 // on rhs follows directly (FP32 on tc_ready grids: the largest magnitude goes to the fields' slots).
 template <typename R>
 int launch_divergence(const fv_grid_s* g, const R* vel, R* rhs, int nvec = 1, bool for_solve = true);
 // out = alpha (Y - G phi) + beta v + gamma w   (velocity; T without G phi).  v, w may be null.
-// norm_slot >= 0: also ||out||^2 into g->ws.scalars[norm_slot] (fused block partials).
+// norm_slot >= 0: also ||out||^2 into g->ws.scalars[norm_slot] (fused block partials).  t_done: out's T is there already.
 template <typename R>
 int launch_correct(const fv_grid_s* g, const R* Y, const R* phi, double alpha, const R* v, double beta,
-                   const R* w, double gamma, R* out, int norm_slot = -1);
+                   const R* w, double gamma, R* out, int norm_slot = -1, bool t_done = false);
 
 // out_i = (Y_i - G phi_i) + beta v_i for nvec states one after another (Y, v, out: 4N each; phi: N each);
 // v may be null.  No norm.
 template <typename R>
-int launch_correct_block(const fv_grid_s* g, const R* Y, const R* phi, const R* v, double beta, R* out, int nvec);
+int launch_correct_block(const fv_grid_s* g, const R* Y, const R* phi, const R* v, double beta, R* out, int nvec,
+                         bool t_done = false);
 
 // FP64 F (MODE 0) and J.v (MODE 1) with every flux computed once (kernels_flux.cu), nvec states one after another in
 // v and out.
@@ -219,7 +234,7 @@ int launch_flux(const fv_grid_s* g, double Gr, double sigma, const double* q, co
 bool stencil_pair_eligible(const fv_grid_s* g, const float* q, const float* v);
 // nvec > 1: v and out hold nvec states one after another (4N elements each), all in one launch.
 int launch_stencil_pair(const fv_grid_s* g, double Gr, double sigma, const float* q, const float* v, float* out,
-                        int nvec = 1);
+                        int nvec = 1, const TempOut& t = TempOut());
 
 // Trilinear transfer of an FP64 state from grid gc to grid gf in physical coordinates, with the wall values
 // of Eqs. 4-6 (kernels_prolong.cu); runs on gf's stream.  Not projected.

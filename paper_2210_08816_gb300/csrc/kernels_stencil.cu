@@ -211,7 +211,7 @@ template <typename R>
 __global__ void __launch_bounds__(kTX * kTY, 3)
     k_stencil_z(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmv, int use_tma,
                 int* err, long long spins, Geo<R> g, int N, R Gr, R invPr, R sigma, const R* __restrict__ q, const R* __restrict__ v,
-                R* __restrict__ out, int zc, int nch) {
+                R* __restrict__ out, int zc, int nch, const TempOut t) {
   constexpr int NA = 8, AB = 4;
   constexpr int NWARP = kTX * kTY / 32;
   constexpr uint32_t kBox = 4u * kPL * sizeof(R);  // one state's box: 4 fields x kHY x kPW
@@ -330,7 +330,15 @@ __global__ void __launch_bounds__(kTX * kTY, 3)
       out[o] = (i >= 1) ? r0 : R(0);
       out[N + o] = (j >= 1) ? r1 : R(0);
       out[2 * N + o] = (k >= 1) ? r2 : R(0);
-      out[3 * N + o] = r3;
+      if (t.out) {
+        const size_t oT = (size_t)(4 * vec + 3) * N + o;
+        R r = t.alpha * r3;
+        if (t.add_v) r += t.beta * S.at(AB + 3, 0, 0, 0);
+        if (t.w) r += t.gamma * (t.w + ready0)[oT];
+        (t.out + ready0)[oT] = r;
+      } else {
+        out[3 * N + o] = r3;
+      }
     }
     if (!use_tma) cp_async_wait_all();  // plane k+2 has landed
     ok = __syncthreads_and(ready);      // nobody reads the slot of plane k-1 any more; stop together
@@ -396,7 +404,7 @@ __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
 template <typename R>
 __global__ void __launch_bounds__(256) k_correct(Geo<R> g, int N, const R* Y, const R* __restrict__ phi,
                                                   R alpha, const R* v, R beta, const R* w, R gamma, R* out,
-                                                  double* __restrict__ part) {
+                                                  double* __restrict__ part, bool t_done) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
   Y += ready0;
@@ -421,12 +429,17 @@ __global__ void __launch_bounds__(256) k_correct(Geo<R> g, int N, const R* Y, co
         }
         const R G = (ph - ld(phi, c.o - c.s[d])) * g.idc[d][c.p[d]];
         r = alpha * (Y[o] - G);
+      } else if (t_done) {
+        if (!part) continue;
+        r = out[o];
       } else {
         r = alpha * Y[o];
       }
-      if (v) r += beta * v[o];
-      if (w) r += gamma * w[o];
-      out[o] = r;
+      if (d < 3 || !t_done) {
+        if (v) r += beta * v[o];
+        if (w) r += gamma * w[o];
+        out[o] = r;
+      }
       if (part) {
         if (sizeof(R) == 4) {
           const float rf = (float)r, p2 = rf * rf;
@@ -539,6 +552,7 @@ __device__ __forceinline__ void acc_sq(float& hi, float& lo, float r) {
 
 // out = alpha (Y - G phi) + beta v + gamma w on four cells; out may alias Y or w (read, then written,
 // by the same thread)
+template <bool T_DONE>
 __global__ void __launch_bounds__(256) k_correct4(Geo<float> g, int N, const float* Y, const float* __restrict__ phi,
                                                    float alpha, const float* v, float beta, const float* w,
                                                    float gamma, float* out, double* __restrict__ part, int nzc) {
@@ -596,7 +610,10 @@ __global__ void __launch_bounds__(256) k_correct4(Geo<float> g, int N, const flo
     for (int d = 0; d < 4; ++d) {
       const int od = d * N + o;
       float4 r;
-      if (d < 3 && wall[d]) {
+      if (d == 3 && T_DONE) {
+        if (!part) continue;
+        r = ld4(out, od);
+      } else if (d < 3 && wall[d]) {
         r = zero4();
       } else {
         const float4 y = ld4(Y, od);
@@ -612,7 +629,7 @@ __global__ void __launch_bounds__(256) k_correct4(Geo<float> g, int N, const flo
         }
         if (d == 0 && i0 == 0) r.x = 0.f;  // the x = 0 wall slot
       }
-      *reinterpret_cast<float4*>(out + od) = r;
+      if (d < 3 || !T_DONE) *reinterpret_cast<float4*>(out + od) = r;
       if (part) {
         acc_sq(shi, slo, r.x);
         acc_sq(shi, slo, r.y);
@@ -690,7 +707,8 @@ int state_map(const fv_grid_s* g, const R* ptr, CUtensorMap* m, int nvec = 1) {
 }
 
 template <typename R>
-int launch_stencil_z(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out, int nvec = 1) {
+int launch_stencil_z(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out, int nvec,
+                     const TempOut& t) {
   constexpr int NA = 8;
   const size_t smem = (size_t)NA * kRing * kPL * sizeof(R);
   static bool attr_set = false;
@@ -714,7 +732,7 @@ int launch_stencil_z(const fv_grid_s* g, double Gr, double sigma, const R* q, co
   dim3 grid(gx, gy, nch * nvec);
   ProfScope ps(g, PROF_STENCIL);
   launch(k_stencil_z<R>, grid, kTX * kTY, smem, g->stream, tq, tv, use_tma, g->ws.err, wait_spins(g), geo_of<R>(g), (int)g->N,
-                                                             (R)Gr, (R)(1.0 / g->Pr), (R)sigma, q, v, out, zc, nch);
+                                                             (R)Gr, (R)(1.0 / g->Pr), (R)sigma, q, v, out, zc, nch, t);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }
@@ -727,19 +745,20 @@ int launch_residual(const fv_grid_s* g, double Gr, const R* q, R* F) {
 }
 
 template <typename R>
-int launch_jvp_block(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out, int nvec) {
+int launch_jvp_block(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out, int nvec,
+                     const TempOut& t) {
   if constexpr (sizeof(R) == 8)
     return launch_flux<1>(g, Gr, sigma, q, v, out, nvec);
   else
-    return launch_stencil_z<R>(g, Gr, sigma, q, v, out, nvec);
+    return launch_stencil_z<R>(g, Gr, sigma, q, v, out, nvec, t);
 }
 
 template <typename R>
-int launch_jvp(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out) {
+int launch_jvp(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out, const TempOut& t) {
   if constexpr (sizeof(R) == 4) {  // two cells per thread (kernels_stencil2.cu) where its tiles fit
-    if (stencil_pair_eligible(g, q, v)) return launch_stencil_pair(g, Gr, sigma, q, v, out);
+    if (stencil_pair_eligible(g, q, v)) return launch_stencil_pair(g, Gr, sigma, q, v, out, 1, t);
   }
-  return launch_jvp_block<R>(g, Gr, sigma, q, v, out, 1);
+  return launch_jvp_block<R>(g, Gr, sigma, q, v, out, 1, t);
 }
 
 int launch_fieldmax(const fv_grid_s* g, const float* f) {
@@ -778,14 +797,15 @@ int launch_divergence(const fv_grid_s* g, const R* vel, R* rhs, int nvec, bool f
 }
 
 template <typename R>
-int launch_correct_block(const fv_grid_s* g, const R* Y, const R* phi, const R* v, double beta, R* out, int nvec) {
+int launch_correct_block(const fv_grid_s* g, const R* Y, const R* phi, const R* v, double beta, R* out, int nvec,
+                         bool t_done) {
   bool quad = false;
   if constexpr (sizeof(R) == 4) quad = quad_ok(g, {Y, phi, v, out});
   if (!quad) {
     for (int i = 0; i < nvec; ++i)
       FV_TRY(launch_correct<R>(g, Y + (size_t)i * 4 * g->N, phi + (size_t)i * g->N, 1.0,
                                v ? v + (size_t)i * 4 * g->N : nullptr, beta, nullptr, 0.0,
-                               out + (size_t)i * 4 * g->N, -1));
+                               out + (size_t)i * 4 * g->N, -1, t_done));
     return FV_OK;
   }
   if constexpr (sizeof(R) == 4) {
@@ -797,7 +817,7 @@ int launch_correct_block(const fv_grid_s* g, const R* Y, const R* phi, const R* 
     }
     qg.z = nzc * nvec;
     ProfScope ps(g, PROF_CORRECT);
-    launch(k_correct4, qg, dim3(32, 8), 0, g->stream, g->geo32, (int)g->N, Y, phi, 1.0f, v, (float)beta, nullptr, 0.0f,
+    launch(t_done ? k_correct4<true> : k_correct4<false>, qg, dim3(32, 8), 0, g->stream, g->geo32, (int)g->N, Y, phi, 1.0f, v, (float)beta, nullptr, 0.0f,
                                                   out, nullptr, nzc);
     FV_CUDA(cudaGetLastError());
   }
@@ -806,7 +826,7 @@ int launch_correct_block(const fv_grid_s* g, const R* Y, const R* phi, const R* 
 
 template <typename R>
 int launch_correct(const fv_grid_s* g, const R* Y, const R* phi, double alpha, const R* v, double beta,
-                   const R* w, double gamma, R* out, int norm_slot) {
+                   const R* w, double gamma, R* out, int norm_slot, bool t_done) {
   dim3 grid, block;
   cell_grid(g, grid, block);
   bool quad = false;
@@ -818,13 +838,13 @@ int launch_correct(const fv_grid_s* g, const R* Y, const R* phi, double alpha, c
     ProfScope ps(g, PROF_CORRECT);
     if constexpr (sizeof(R) == 4) {
       if (quad)
-        launch(k_correct4, grid, dim3(32, 8), 0, g->stream, g->geo32, (int)g->N, Y, phi, (float)alpha, v, (float)beta, w,
+        launch(t_done ? k_correct4<true> : k_correct4<false>, grid, dim3(32, 8), 0, g->stream, g->geo32, (int)g->N, Y, phi, (float)alpha, v, (float)beta, w,
                                                         (float)gamma, out, want ? g->ws.partials : nullptr,
                                                         (int)grid.z);
     }
     if (!quad)
       launch(k_correct<R>, grid, block, 0, g->stream, geo_of<R>(g), (int)g->N, Y, phi, (R)alpha, v, (R)beta, w,
-                                                  (R)gamma, out, want ? g->ws.partials : nullptr);
+                                                  (R)gamma, out, want ? g->ws.partials : nullptr, t_done);
     FV_CUDA(cudaGetLastError());
   }
   if (want) return launch_sum_partials(g, nblocks, norm_slot);
@@ -833,19 +853,22 @@ int launch_correct(const fv_grid_s* g, const R* Y, const R* phi, double alpha, c
 }
 
 template int launch_residual<double>(const fv_grid_s*, double, const double*, double*);
-template int launch_jvp<double>(const fv_grid_s*, double, double, const double*, const double*, double*);
-template int launch_jvp<float>(const fv_grid_s*, double, double, const float*, const float*, float*);
-template int launch_jvp_block<double>(const fv_grid_s*, double, double, const double*, const double*, double*, int);
-template int launch_jvp_block<float>(const fv_grid_s*, double, double, const float*, const float*, float*, int);
+template int launch_jvp<double>(const fv_grid_s*, double, double, const double*, const double*, double*,
+                                const TempOut&);
+template int launch_jvp<float>(const fv_grid_s*, double, double, const float*, const float*, float*, const TempOut&);
+template int launch_jvp_block<double>(const fv_grid_s*, double, double, const double*, const double*, double*, int,
+                                      const TempOut&);
+template int launch_jvp_block<float>(const fv_grid_s*, double, double, const float*, const float*, float*, int,
+                                     const TempOut&);
 template int launch_divergence<double>(const fv_grid_s*, const double*, double*, int, bool);
 template int launch_divergence<float>(const fv_grid_s*, const float*, float*, int, bool);
 template int launch_correct_block<double>(const fv_grid_s*, const double*, const double*, const double*, double,
-                                          double*, int);
+                                          double*, int, bool);
 template int launch_correct_block<float>(const fv_grid_s*, const float*, const float*, const float*, double, float*,
-                                         int);
+                                         int, bool);
 template int launch_correct<double>(const fv_grid_s*, const double*, const double*, double, const double*, double,
-                                    const double*, double, double*, int);
+                                    const double*, double, double*, int, bool);
 template int launch_correct<float>(const fv_grid_s*, const float*, const float*, double, const float*, double,
-                                   const float*, double, float*, int);
+                                   const float*, double, float*, int, bool);
 
 }  // namespace fv

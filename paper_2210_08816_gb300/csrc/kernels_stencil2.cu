@@ -292,7 +292,7 @@ template <bool BLOCK>
 __global__ void __launch_bounds__(kPX / 2 * kPY, 2)
     k_stencil_pair(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmv, int* err,
                    long long spins, Geo<float> g, int N, float Gr, float invPr, float sigma, float* __restrict__ out, int zc,
-                   int nch) {
+                   int nch, const TempOut t) {
   constexpr uint32_t kBox = 4u * kPL2 * sizeof(float);  // one state's box: 4 fields x kPHY x kPW2
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar[kPRing], bar_done[2];
@@ -361,6 +361,9 @@ __global__ void __launch_bounds__(kPX / 2 * kPY, 2)
   }
   for (int k = k0; k < kend && ok; ++k) {
     const Bundle<float2> mz = broadcast(load_bundle(g, 2, k));
+    const size_t oT = (size_t)(4 * vec + 3) * N + (active ? (k * ny + j) * nx + x : 0);
+    float2 wT = make_float2(0.f, 0.f);  // read ahead of its use: at its use it cost 30 us at 256^3
+    if (t.w) wT = *reinterpret_cast<const float2*>(t.w + ready0 + oT);
     // Plane k + 2 takes the slot of plane k - 2, which every warp has read once it has done plane k - 1.  The first warp
     // alone waits for the others; they run on to the next plane by themselves.
     if (tid < 32 && k + 2 <= kend) {
@@ -417,7 +420,14 @@ __global__ void __launch_bounds__(kPX / 2 * kPY, 2)
       }
       temperature_pair(S, mx, my, mz, j, ny, k, nz, z.f[3], z.g[3], conv, lap);
       const float2 r3 = fma2(msig, S.ld<7, 0, 0, 0>(), lap * bc(invPr) - conv);
-      *reinterpret_cast<float2*>(out + 3 * N + o) = r3;
+      if (t.out) {
+        float2 r = bc(t.alpha) * r3;
+        if (t.add_v) r = fma2(bc(t.beta), S.ld<7, 0, 0, 0>(), r);
+        if (t.w) r = fma2(bc(t.gamma), wT, r);
+        *reinterpret_cast<float2*>(t.out + ready0 + oT) = r;
+      } else {
+        *reinterpret_cast<float2*>(out + 3 * N + o) = r3;
+      }
     }
     __syncwarp();
     if ((tid & 31) == 0)
@@ -448,7 +458,7 @@ bool stencil_pair_eligible(const fv_grid_s* g, const float* q, const float* v) {
 }
 
 int launch_stencil_pair(const fv_grid_s* g, double Gr, double sigma, const float* q, const float* v, float* out,
-                        int nvec) {
+                        int nvec, const TempOut& t) {
   const size_t smem = (size_t)kPRing * kPNA * kPL2 * sizeof(float);
   static bool attr_set = false;
   if (!attr_set) {
@@ -473,10 +483,10 @@ int launch_stencil_pair(const fv_grid_s* g, double Gr, double sigma, const float
   ProfScope ps(g, PROF_STENCIL);
   if (nvec > 1)
     launch(k_stencil_pair<true>, grid, kPX / 2 * kPY, smem, g->stream, tq, tv, g->ws.err, wait_spins(g), g->geo32, (int)g->N, (float)Gr,
-                                                                 (float)(1.0 / g->Pr), (float)sigma, out, zc, nch);
+                                                                 (float)(1.0 / g->Pr), (float)sigma, out, zc, nch, t);
   else
     launch(k_stencil_pair<false>, grid, kPX / 2 * kPY, smem, g->stream, tq, tv, g->ws.err, wait_spins(g), g->geo32, (int)g->N, (float)Gr,
-                                                                  (float)(1.0 / g->Pr), (float)sigma, out, zc, nch);
+                                                                  (float)(1.0 / g->Pr), (float)sigma, out, zc, nch, t);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }
