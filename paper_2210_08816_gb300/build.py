@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIBDIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(LIBDIR, "libcubefv.so")
-SOURCES = ["kernels_stencil.cu", "kernels_stencil2.cu", "kernels_flux.cu", "kernels_fdm.cu", "kernels_tc.cu", "kernels_digit.cu", "kernels_blas.cu", "host_linalg.cpp",
+SOURCES = ["kernels_stencil.cu", "kernels_stencil2.cu", "kernels_flux.cu", "kernels_fdm.cu", "kernels_tc.cu", "kernels_plane.cu", "kernels_digit.cu", "kernels_blas.cu", "host_linalg.cpp",
            "host_cheb.cpp", "host_grid.cpp", "host_digits.cpp", "fv_api.cpp", "noalloc.cu", "kernels_prolong.cu", "kernels_diag.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -296,6 +296,11 @@ int read_scalars(const fv_grid_s* g, int slot, int count, double* out);
 int encode_tensor_map(CUtensorMap* map, CUtensorMapDataType type, int rank, const void* ptr, const uint64_t* dims,
                       const uint64_t* strides, const uint32_t* box, CUtensorMapSwizzle swizzle);
 
+// The six FP64 passes of nf fields as three launches (kernels_plane.cu), in -> out (which may be in).
+bool plane_wins(const fv_grid_s* g, int nf);
+int plane_solve(const fv_grid_s* g, const int (*kinds)[3], bool per_field, const double* sfac, const double* shift,
+                bool zero_mode, const double* in, double* out, int nf);
+
 // Tensor-core pressure-solve passes (kernels_tc.cu), FP32 only; slots: fmax_slots(g, nvec).
 int tc_setup(fv_grid_s* g);
 int tc_pass(const fv_grid_s* g, int pass, int na, int nb, const float* in, float* out, unsigned* slots, int nvec);

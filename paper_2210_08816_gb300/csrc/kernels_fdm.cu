@@ -323,6 +323,9 @@ int half_solve(const fv_grid_s* g, const int (*kinds)[3], bool per_field, const 
     set_error("half_solve: number of fields out of range");
     return FV_EINVAL;
   }
+  if constexpr (sizeof(R) == 8) {
+    if (plane_wins(g, nf)) return plane_solve(g, kinds, per_field, sfac, shift, zero_mode, in, out, nf);
+  }
   // forward: (z,y,x) -> (mx,z,y) -> (my,mx,z) -> (mz,my,mx) / Lambda; backward the same way round
   FV_TRY(half_pass<R>(g, 0, false, nz, ny, kinds, per_field, sfac, shift, in, tmp, false, zero_mode, nf));
   FV_TRY(half_pass<R>(g, 1, false, nx, nz, kinds, per_field, sfac, shift, tmp, out, false, zero_mode, nf));

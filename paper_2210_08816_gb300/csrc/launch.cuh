@@ -45,6 +45,25 @@ inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cud
                    typename same_type<P>::type... args) {
   launch(true, kernel, grid, block, smem, stream, args...);
 }
+// With the overlap, in clusters of C blocks along x.
+template <typename... P>
+inline void launch_cluster(int C, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                           typename same_type<P>::type... args) {
+  cudaLaunchAttribute at[2] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)C;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = stream;
+  c.attrs = at;
+  c.numAttrs = 2;
+  cudaLaunchKernelEx(&c, kernel, args...);
+}
 // Without the overlap, for kernels bound by the FP64 pipe (two operations per clock and SM): blocks placed while the
 // predecessor still occupies most SMs pile up on the others, and the busiest SM sets the time (32^3 FP64 J.v +
 // projection 101 us with the overlap, 71 without).  A kernel whose registers or shared memory let one block on an SM
