@@ -47,7 +47,6 @@ namespace {
 
 constexpr int kDgRows = 128;
 constexpr int kDgWarps = 16;  // workers
-constexpr int kDgIts = kDgRows / (2 * kDgWarps);  // row pairs of a worker warp per slab
 constexpr int kDgThreads = 32 * (2 + kDgWarps);
 constexpr int kDgDigitBytes = kDgRows * 64;  // one digit of a 128 x 32 slab (64-byte swizzled rows)
 
@@ -210,9 +209,12 @@ struct DgUnit {
   }
 };
 
-template <typename R, bool BWD>
+// ITS: row pairs of a worker warp per slab; tiles of kRowsT = 32 ITS rows (the MMAs take 128, what the others hold is
+// not read)
+template <typename R, bool BWD, int ITS>
 __global__ void __launch_bounds__(kDgThreads, 1)
     k_digit_pass(const __grid_constant__ DgArgs<R> t, const R* __restrict__ in, R* __restrict__ out) {
+  constexpr int kRowsT = 2 * kDgWarps * ITS;
   constexpr int D = Dg<R>::D, NC = Dg<R>::NC, ACC = Dg<R>::ACC, E_ = Dg<R>::E, kSlots = Dg<R>::kSlots;
   constexpr bool F64 = sizeof(R) == 8;
   constexpr int kExpShift = F64 ? 20 : 23, kExpMax = F64 ? 2047 : 255, kExpMin = F64 ? 64 : 32;
@@ -272,8 +274,8 @@ __global__ void __launch_bounds__(kDgThreads, 1)
           do nx.step(t), ++v;
           while (nx.group != 0);
           if (v < u1) {
-            const R* src = in + ((size_t)nx.field * P + (size_t)nx.tile * kDgRows) * n;
-            const uint32_t bytes = (uint32_t)(min(kDgRows, P - nx.tile * kDgRows) * n * sizeof(R)) & ~15u;
+            const R* src = in + ((size_t)nx.field * P + (size_t)nx.tile * kRowsT) * n;
+            const uint32_t bytes = (uint32_t)(min(kRowsT, P - nx.tile * kRowsT) * n * sizeof(R)) & ~15u;
             if ((uintptr_t)src % 16 == 0 && bytes)
               asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
           }
@@ -371,7 +373,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
     DgUnit<R> un(t, u0), nx = un, pv = un;  // this unit, the next slab's, the one before
     // inputs of row pair `it` for the slab of an item; those of the next slab are requested as soon as this one's
     // are converted
-    R x0[kDgIts], x1[kDgIts], y0[kDgIts], y1[kDgIts];
+    R x0[ITS], x1[ITS], y0[ITS], y1[ITS];
     auto load_row = [&](int it, const R* __restrict__ src, int rows, int k, int k0, int S) {
       const int row = 2 * (kDgWarps * it + cw) + rh;
       const bool two = k + 1 < h;
@@ -396,16 +398,16 @@ __global__ void __launch_bounds__(kDgThreads, 1)
       if (item < total) {
         const int op = un.field & t.op_mask;
         const int k0 = t.k0[op], S = t.S[op];
-        const R* __restrict__ src = in + ((size_t)un.field * P + (size_t)un.tile * kDgRows) * n;
-        const int rows = min(kDgRows, P - un.tile * kDgRows);
+        const R* __restrict__ src = in + ((size_t)un.field * P + (size_t)un.tile * kRowsT) * n;
+        const int rows = min(kRowsT, P - un.tile * kRowsT);
         if (item == 0) {
 #pragma unroll
-          for (int it = 0; it < kDgIts; ++it) load_row(it, src, rows, kl, k0, S);
+          for (int it = 0; it < ITS; ++it) load_row(it, src, rows, kl, k0, S);
         }
         if (j == 0 && (du == 0 || un.group == 0)) ++tc;
         if (j == 0 && (du == 0 || un.group == 0) && t.nslab == 1) {  // the rows are in the registers
 #pragma unroll
-          for (int it = 0; it < kDgIts; ++it) {
+          for (int it = 0; it < ITS; ++it) {
             unsigned m = max(max(magnitude_bits(x0[it]), magnitude_bits(x1[it])),
                              max(magnitude_bits(y0[it]), magnitude_bits(y1[it])));
 #pragma unroll
@@ -416,7 +418,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
         } else if (j == 0 && (du == 0 || un.group == 0)) {
           // largest magnitude of each of the warp's rows (FP64: by the high words), 32 loads in flight; a face
           // axis' wall slot holds no input
-          constexpr int kRows = 2 * kDgIts, kStep = sizeof(R) / 4;
+          constexpr int kRows = 2 * ITS, kStep = sizeof(R) / 4;
           unsigned m[kRows];
 #pragma unroll
           for (int r = 0; r < kRows; ++r) m[r] = 0;
@@ -448,14 +450,14 @@ __global__ void __launch_bounds__(kDgThreads, 1)
         const int gi = 2 * item, s0 = gi % kSlots, s1 = (gi + 1) % kSlots;
         // the next item: this unit's next slab, or the first of the next unit
         if (j + 1 == t.nslab) nx.step(t);
-        const R* __restrict__ nsrc = in + ((size_t)nx.field * P + (size_t)nx.tile * kDgRows) * n;
-        const int nrows = item + 1 < total ? min(kDgRows, P - nx.tile * kDgRows) : 0;
+        const R* __restrict__ nsrc = in + ((size_t)nx.field * P + (size_t)nx.tile * kRowsT) * n;
+        const int nrows = item + 1 < total ? min(kRowsT, P - nx.tile * kRowsT) : 0;
         const int nk = (j + 1 == t.nslab ? 0 : (j + 1) * 32) + kl;
         const int nk0 = t.k0[nx.field & t.op_mask], nS = t.S[nx.field & t.op_mask];
         using Val = typename Dg<R>::Val;
-        Val i0[kDgIts], i1[kDgIts], j0[kDgIts], j1[kDgIts];
+        Val i0[ITS], i1[ITS], j0[ITS], j1[ITS];
 #pragma unroll
-        for (int it = 0; it < kDgIts; ++it) {
+        for (int it = 0; it < ITS; ++it) {
           const int E = re[2 * (kDgWarps * it + cw) + rh];
           i0[it] = scaled(x0[it], E);
           i1[it] = scaled(x1[it], E);
@@ -472,7 +474,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
         }
         unsigned char* dst = smem + s0 * kSlotBytes + off;
 #pragma unroll
-        for (int it = 0; it < kDgIts; ++it)
+        for (int it = 0; it < ITS; ++it)
           put_digits(dst + it * kRow, BWD ? i0[it] : i0[it] + j0[it], BWD ? i1[it] : i1[it] + j1[it]);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive(smem_u32(&bar_conv[s0]));
@@ -483,15 +485,15 @@ __global__ void __launch_bounds__(kDgThreads, 1)
         }
         dst = smem + s1 * kSlotBytes + off;
 #pragma unroll
-        for (int it = 0; it < kDgIts; ++it)
+        for (int it = 0; it < ITS; ++it)
           put_digits(dst + it * kRow, BWD ? j0[it] : i0[it] - j0[it], BWD ? j1[it] : i1[it] - j1[it]);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive(smem_u32(&bar_conv[s1]));
       }
       if (j == 0 && du > 0) {  // epilogue of the previous unit
-        const int group = pv.group, op = pv.field & t.op_mask, p = pv.tile * kDgRows + erow;
+        const int group = pv.group, op = pv.field & t.op_mask, p = pv.tile * kRowsT + erow;
         const bool newer = item < total && un.group == 0;  // tile tc is already the next one
-        const bool live = p < P;
+        const bool live = erow < kRowsT && p < P;
         const int k0 = t.k0[op], S = t.S[op];
         R* __restrict__ o = out + (size_t)pv.field * P * n + p;
         R l01 = R(0);
@@ -509,7 +511,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
         const bool bad = E == kExpMax;  // an Inf or NaN among the row's inputs
         // FP32: 2^(E - 140), E in 32 .. 254
         const float row_scale = __uint_as_float((unsigned)(min(E, 254) - 13) << 23);
-        const int c1 = min(NC, h - group * NC);
+        const int c1 = __any_sync(0xffffffffu, live) ? min(NC, h - group * NC) : 0;
 #pragma unroll 1
         for (int c0 = (cw >> 2) * E_; c0 < c1; c0 += (kDgWarps / 4) * E_) {
           typename Dg<R>::Val vs[E_], va[E_];
@@ -597,17 +599,21 @@ const HalfDev<float> (&half_of<float>(const fv_grid_s* g))[3][3] { return g->hal
 
 }  // namespace
 
+template <typename R, int ITS>
+static int digit_setup_its() {
+  for (auto k : {k_digit_pass<R, false, ITS>, k_digit_pass<R, true, ITS>})
+    FV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)digit_smem<R>()));
+  return FV_OK;
+}
+
 int digit_setup() {
   static_assert(digit_smem<double>() <= 227 * 1024 && digit_smem<float>() <= 227 * 1024, "ring fits shared memory");
-  FV_CUDA(cudaFuncSetAttribute(k_digit_pass<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)digit_smem<double>()));
-  FV_CUDA(cudaFuncSetAttribute(k_digit_pass<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)digit_smem<double>()));
-  FV_CUDA(cudaFuncSetAttribute(k_digit_pass<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)digit_smem<float>()));
-  FV_CUDA(cudaFuncSetAttribute(k_digit_pass<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)digit_smem<float>()));
-  return FV_OK;
+  FV_TRY((digit_setup_its<double, 1>()));
+  FV_TRY((digit_setup_its<double, 3>()));
+  FV_TRY((digit_setup_its<double, 4>()));
+  FV_TRY((digit_setup_its<float, 1>()));
+  FV_TRY((digit_setup_its<float, 3>()));
+  return digit_setup_its<float, 4>();
 }
 
 template <typename R>
@@ -636,9 +642,20 @@ int digit_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int
   }
   // pairs of neighbours by one load: rows of an even length from an aligned base, pairs at even offsets
   t.vec = t.n % 2 == 0 && (bwd ? h % 2 == 0 : cells) && (uintptr_t)in % (2 * sizeof(R)) == 0;
-  t.tiles = (t.P + kDgRows - 1) / kDgRows;
   t.groups = (h + Dg<R>::NC - 1) / Dg<R>::NC;
   t.nslab = (h + 31) / 32;
+  // Height of the tiles by the workers' time of the busiest SM's units: the conversions of their slabs (which go by the
+  // rows) and an epilogue worth about four slabs of 32 rows (which does not).  Fewer rows where a launch has few units.
+  int its = 4;
+  long long best = -1;
+  for (int i : {4, 3, 1}) {
+    const int rows = i * 2 * kDgWarps;
+    const long long units = (long long)((t.P + rows - 1) / rows) * t.groups * nf;
+    const long long cost = (units + g->sms - 1) / g->sms * (i * t.nslab + 4);
+    if (best < 0 || cost < best) best = cost, its = i;
+  }
+  const int rows = its * 2 * kDgWarps;
+  t.tiles = (t.P + rows - 1) / rows;
   const long long units = (long long)t.tiles * t.groups * nf;
   if (units > (1LL << 30)) {
     set_error("digit_pass: too many fields in one block");
@@ -649,10 +666,17 @@ int digit_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int
   t.spins = wait_spins(g);
   const unsigned grid = (unsigned)std::min<long long>(units, g->sms);
   ProfScope ps(g, PROF_TRANSFORM_TC);
-  if (bwd)
-    launch(k_digit_pass<R, true>, grid, kDgThreads, digit_smem<R>(), g->stream, t, in, out);
+  auto go = [&](auto i) {
+    constexpr int ITS = decltype(i)::value;
+    launch(bwd ? k_digit_pass<R, true, ITS> : k_digit_pass<R, false, ITS>, grid, kDgThreads, digit_smem<R>(), g->stream, t,
+           in, out);
+  };
+  if (its == 4)
+    go(std::integral_constant<int, 4>());
+  else if (its == 3)
+    go(std::integral_constant<int, 3>());
   else
-    launch(k_digit_pass<R, false>, grid, kDgThreads, digit_smem<R>(), g->stream, t, in, out);
+    go(std::integral_constant<int, 1>());
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }
