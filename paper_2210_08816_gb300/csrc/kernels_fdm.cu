@@ -247,13 +247,15 @@ template <>
 const HalfDev<float> (&half_of<float>(const fv_grid_s* g))[3][3] { return g->half32; }
 
 // Digit products on the tensor cores (kernels_digit.cu) instead of the CUDA-core form, by the multiplications of a
-// half-size pass: a digit pass has a floor of ~10 us (FP64 ~16) before its length shows.  Measured (us a pass, with
-// ~3 of event overhead, CUDA cores / digits): FP64 32^3 9.7 / 16, 56^3 19.2 / 19.4, 64^3 25.6 / 19.8, 100^3 130 / 36,
-// 160^3 589 / 78, four fields of 40^3 26 / 21; FP32 65^3 9.6 / 14, 100^3 16.1 / 12.7, 150^3 40.4 / 29.6, 200^3
-// 109 / 51, 250^3 227 / 75, four fields of 64^3 10.5 / 10.7, of 96^3 28.6 / 20.0, of 256^3 875 / 275.
+// half-size pass: a digit pass has a floor of ~6 us (FP64 ~11) before its length shows.  Measured (us a projection, CUDA
+// cores / digits): FP64 40^3 (1.3e6) 53 / 69, 44^3 67 / 70, 48^3 (2.7e6) 70 / 71, 52^3 (3.7e6) 108 / 77, 56^3 113 / 78;
+// FP32 50^3 32 / 35, 60^3 42.5 / 44, 70^3 (1.2e7) 49 / 54, 80^3 (2.0e7) 69 / 61, 90^3 68 / 60; the diffusion solve's
+// four fields in FP32 50^3 (1.3e7) 39 / 33, 60^3 (2.6e7) 43 / 34, 80^3 96 / 81.  Single passes at 160^3 FP64 589 / 78,
+// 250^3 FP32 227 / 75.  The number of vectors in a block does not count: a block's results are those of its vectors one
+// by one, bit for bit.
 template <typename R>
 bool digit_wins(int n, long long rows) {
-  return (double)rows * n * ((n + 1) / 2) >= (sizeof(R) == 8 ? 4.5e6 : 3.5e7);
+  return (double)rows * n * ((n + 1) / 2) >= (sizeof(R) == 8 ? 3.2e6 : 1.6e7);
 }
 
 // One pass along `axis` over nf fields of a (na x nb) x n block, kinds[op][axis] = the operators (one, or four
@@ -262,7 +264,7 @@ template <typename R>
 int half_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int (*kinds)[3], bool per_field,
               const double* sfac, const double* shift, const R* in, R* out, bool scale, bool zero_mode, int nf) {
   const int len = axis == 0 ? g->nx : axis == 1 ? g->ny : g->nz;
-  if (g->digit_ready && digit_wins<R>(len, (long long)na * nb * nf))
+  if (g->digit_ready && digit_wins<R>(len, (long long)na * nb * (per_field ? 4 : 1)))
     return digit_pass<R>(g, axis, bwd, na, nb, kinds, per_field, sfac, shift, in, out, scale, zero_mode, nf);
   const auto& H = half_of<R>(g);
   HalfArgs<R> t{};

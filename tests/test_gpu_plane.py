@@ -68,3 +68,18 @@ def test_diffusion_solve_in_place(fv, shape):
     assert torch.equal(out, y) and torch.isfinite(out).all()
     o = out.view(4, nz, ny, nx)
     assert not (o[0, :, :, 0].any() or o[1, :, 0, :].any() or o[2, 0].any())
+
+
+@pytest.mark.parametrize("prec,shape,nvec", [(64, (24, 20, 36), 12), (64, (40, 40, 40), 3), (64, (16, 16, 16), 9),
+                                             (64, (56, 30, 44), 4), (32, (80, 40, 30), 16), (32, (68, 60, 52), 5)])
+def test_block_of_vectors_is_its_vectors_one_by_one(fv, prec, shape, nvec):
+    g = fv.Grid(*shape, stretch=1.5, Pr=0.71)
+    p, dt = (fv.FV_FP64, torch.float64) if prec == 64 else (fv.FV_FP32, torch.float32)
+    gen = torch.Generator().manual_seed(4)
+    q = torch.randn(g.n, generator=gen, dtype=torch.float64).to(dt).cuda()
+    V = torch.randn(nvec * g.n, generator=gen, dtype=torch.float64).to(dt).cuda()
+    W, one = torch.empty_like(V), torch.empty_like(V)
+    fv.fv_jvp_project_batch(g, p, 1.0e4, -90.0, q, V, W, nvec)
+    for i in range(nvec):
+        fv.fv_jvp_project(g, p, 1.0e4, -90.0, q, V[i * g.n:(i + 1) * g.n], one[i * g.n:(i + 1) * g.n])
+    assert torch.equal(W, one)
