@@ -261,31 +261,30 @@ def gpu_arm(args, ws, rank, local):
         # One pass reads the N-cell field and writes it with the contracted axis rotated: 2 N FP32 values of
         # HBM traffic, which bounds it.  Its tensor work: the grid is mirror-symmetric, so a pass contracts
         # the sums and differences of mirrored inputs with two n/2 x n/2 matrices, N n flops (half of the
-        # dense 2 N n), executed three times as 3 x TF32.
+        # dense 2 N n), executed three times as products of FP16 heads and remainders.
         traffic_bytes = 2 * N * 4
         achieved = traffic_bytes / (per_launch_ms * 1e-3) / 1e9
         flops = 1.0 * N * n
         bf16 = float(peaks.get("bf16_tflops", 1900.0))
-        tf32_peak = bf16 * (1.1 / 2.25)   # TF32 dense = bf16 dense x nominal ratio 1.1 / 2.25 PFLOP/s
         executed = 3.0 * flops / (per_launch_ms * 1e-3) / 1e12
-        roof = {"kernel": "k_transform_tcp (tcgen05 fast-diagonalisation pass, 3 x TF32 split)", "bound": "hbm",
+        roof = {"kernel": "k_pass_tc (tcgen05 fast-diagonalisation pass, three products of FP16 parts)", "bound": "hbm",
                 "achieved": round(achieved, 1), "peak": hbm_peak, "unit": "GB/s",
                 "frac": round(achieved / hbm_peak, 4), "peak_source": hbm_src,
-                "tensor": {"executed_tflops": round(executed, 2), "peak": round(tf32_peak, 1),
-                           "frac": round(executed / tf32_peak, 4), "flops_per_pass": 3 * flops,
-                           "peak_source": ("measured bf16 burst x 1.1/2.25 (TF32)" if "bf16_tflops" in peaks
-                                           else "fallback 1.9 PF bf16 x 1.1/2.25")}}
+                "tensor": {"executed_tflops": round(executed, 2), "peak": round(bf16, 1),
+                           "frac": round(executed / bf16, 4), "flops_per_pass": 3 * flops,
+                           "peak_source": ("measured bf16 burst (FP16 runs at the same rate)" if "bf16_tflops" in peaks
+                                           else "fallback 1.9 PF bf16")}}
     elif dom == "transform":
         flops = 2.0 * N * n
         achieved = flops / (per_launch_ms * 1e-3) / 1e12
         peak = SM_COUNT * FP32_LANES * 2 * SM_MAX_MHZ * 1e6 / 1e12
-        roof = {"kernel": "k_transform (SIMT fast-diagonalisation pass)", "bound": "alu",
+        roof = {"kernel": "k_half / k_transform (CUDA-core fast-diagonalisation pass)", "bound": "alu",
                 "achieved": round(achieved, 3), "peak": round(peak, 2), "unit": "TFLOP/s",
                 "frac": round(achieved / peak, 4),
                 "peak_source": "FP32 FMA lanes x 2 x 152 SMs x 2070 MHz (unit counts and max clock)"}
         traffic_bytes = 2 * N * 4
     else:
-        bytes_per = {"stencil": 12 * N * 4, "correct": 17 * N * 4, "divergence": 4 * N * 4}.get(dom, 2 * 4 * N * 4)
+        bytes_per = {"stencil": 13 * N * 4, "correct": 14 * N * 4, "divergence": 4 * N * 4}.get(dom, 2 * 4 * N * 4)
         achieved = bytes_per / (per_launch_ms * 1e-3) / 1e9
         names = {"stencil": stencil_name(n), "correct": "k_correct4", "divergence": "k_divergence4"}
         roof = {"kernel": names.get(dom, dom), "bound": "hbm", "achieved": round(achieved, 1), "peak": hbm_peak,
@@ -295,13 +294,14 @@ def gpu_arm(args, ws, rank, local):
     roof["algorithmic_bytes"] = traffic_bytes
     roof["launch_ms"] = round(per_launch_ms, 4)
     st_ms, st_n = prof["stencil"]
-    st_gbs = 12 * N * 4 / (st_ms / st_n * 1e-3) / 1e9
+    st_gbs = 13 * N * 4 / (st_ms / st_n * 1e-3) / 1e9
     hbm_stencil = {"kernel": stencil_name(n), "achieved": round(st_gbs, 1), "peak": hbm_peak,
-                   "unit": "GB/s", "frac": round(st_gbs / hbm_peak, 4), "algorithmic_bytes": 12 * N * 4,
+                   "unit": "GB/s", "frac": round(st_gbs / hbm_peak, 4), "algorithmic_bytes": 13 * N * 4,
                    "launch_ms": round(st_ms / st_n, 4), "traffic": measured_traffic("stencil", n)}
-    # algorithmic bytes of one step: stencil 12 N, divergence 4 N, six passes 2 N each, correction 17 N
-    # (the norm is summed inside the correction pass)
-    step_bytes = (12 + 4 + 12 + 17) * N * 4
+    # algorithmic bytes of one step: stencil 13 N (q, v and w's T in; the velocity of J.v and the step's T out), divergence
+    # 4 N, six passes 2 N each, correction 14 N (the velocities of J.v, v, w and the result, the potential, and the result's
+    # T for the norm, which is summed there)
+    step_bytes = (13 + 4 + 12 + 14) * N * 4
     breakdown = {k: {"ms_per_step": round(v[0] / K, 4), "launches_per_step": v[1] / K} for k, v in prof.items()}
     # the pressure solve's share of the step: the most that any replacement of the direct solve (a learned
     # Poisson surrogate included) could remove, since the direct solve needs one pass (I_p = 1)

@@ -73,9 +73,11 @@ typedef struct {
 
 /* Create a grid handle: metric arrays, the 1D generalised eigen-decompositions
  * used by the pressure solve (computed on the host in FP64), and workspace.
- * The FP32 pressure solve runs on the tensor cores when every axis has 32 to 256
- * cells, a multiple of 32, and faces mirror-symmetric about 1/2 (as the built-in
- * grids are); other grids take the CUDA-core passes, with the same results.
+ * Faces mirror-symmetric about 1/2 (as the built-in grids' are) give half-size
+ * transforms in the direct solves; the FP32 pressure solve then runs on the tensor
+ * cores when every axis has 32 to 256 cells, a multiple of 32, and other large
+ * solves (FP64 too) run there as products of FP16 parts that keep their precision;
+ * other grids take the CUDA-core passes, with the same results to round-off.
  * `stream` is a cudaStream_t (NULL = legacy default stream).
  * Errors: FV_EINVAL (sizes, faces), FV_ENOMEM, FV_ECUDA. */
 int fv_grid_create(const fv_grid_desc* desc, void* stream, fv_grid* out);
@@ -457,7 +459,8 @@ int fv_richardson(int n, const double* h2, const double* value, double* limit, d
  * synchronises the stream and returns, per class (host arrays of FV_PROF_CLASSES), the summed
  * milliseconds and the launch counts.  Classes: 0 stencil (F, J.v), 1 divergence, 2 pressure-solve
  * transforms (CUDA cores), 3 gradient correction, 4 reductions, 5 other vector kernels,
- * 6 pressure-solve transforms on the tensor cores (FP32 data, tcgen05).
+ * 6 pressure-solve and diffusion-solve transforms on the tensor cores (tcgen05).  One launch may
+ * hold two transforms (FP64, small grids).
  * Errors: FV_EINVAL, FV_ECUDA, FV_ENOMEM. */
 enum { FV_PROF_CLASSES = 7 };
 int fv_profile(fv_grid g, int enable);

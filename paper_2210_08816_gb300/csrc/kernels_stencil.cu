@@ -738,7 +738,7 @@ int launch_stencil_z(const fv_grid_s* g, double Gr, double sigma, const R* q, co
 }
 
 // FP64 by the flux form (kernels_flux.cu), whose operation count bounds it; FP32 by the forms below it measured
-// against: 256^3 two cells per thread 206 us, flux form 334; 100^3 one cell 33, flux 46; 64^3 10.8 / 16.6
+// against: 256^3 two cells per thread 206 us (191 since), flux form 334; 100^3 one cell 33, flux 46; 64^3 10.8 / 16.6
 template <typename R>
 int launch_residual(const fv_grid_s* g, double Gr, const R* q, R* F) {
   return launch_flux<0>(g, Gr, 0.0, q, q, F);

@@ -23,10 +23,11 @@
 // (converted / MMAs complete); accf / acce per tile.  Every wait is bounded; on expiry the kernel records a code, stops
 // issuing, lets its copies and MMAs complete and returns.
 //
-// What bounds it: memory.  256^3, six passes of 134 MB each: 198 us by themselves, 149 within a time step's launches
-// (TF32 parts: 222), 5.4 TB/s; a pass's reads alone run at 5.2 TB/s through two stages of 32 KB per SM.  More stages
-// are slower (three: 630 us for the whole chebyshev step against 600), and so are equal row ranges instead of
-// neighbouring tiles at a time (650): the writes are 512-byte pieces of n rows, and neighbours share DRAM pages.
+// What bounds it: the copies' arrival and the hand-offs of a step, not a unit.  256^3, six passes of 134 MB each: 198 us by
+// themselves, ~150 within a time step's overlapping launches (TF32 parts: 222); DRAM 32 % (most of a field stays in L2
+// between passes), L2 24 %.  Two stages of 32 KB of A arrive every ~1750 clocks per step.  More stages are slower (three:
+// 630 us for the whole chebyshev step against 600), and so are equal row ranges instead of neighbouring tiles at a time
+// (650): the writes are 512-byte pieces of n rows, and neighbours share DRAM pages.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -71,7 +72,7 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t a, uint64_t b,
       : "memory");
 }
 
-// approximate reciprocal (PTX rcp.approx, relative error about 2^-23): far below the 3 x TF32 error
+// approximate reciprocal (PTX rcp.approx, relative error about 2^-23): far below the error of the parts
 __device__ __forceinline__ float rcp_approx(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
