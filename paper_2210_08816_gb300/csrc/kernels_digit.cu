@@ -17,15 +17,16 @@
 //
 // Why: GB300 issues two FP64 operations per clock and SM (1.23 TFLOP/s measured in k_half); the 28 FP16 products
 // cost 155 GFLOP per 256^3 pass where the FP16 tensor rate is 1.9 PFLOP/s.  Measured, six passes, CUDA cores / here:
-// FP64 256^3 21.9 / 1.94 ms, 100^3 794 / 217 us; FP32 100^3 98 / 76 us, 250^3 1360 / 450 us, four fields of 256^3
+// FP64 256^3 21.9 / 1.94 ms, 100^3 794 / 193 us; FP32 100^3 98 / 76 us, 250^3 1360 / 450 us, four fields of 256^3
 // 5.2 / 1.65 ms.  Errors against 64 bits are at or below those of the CUDA-core passes (FP32 100^3 product 3.9e-7 ->
 // 2.4e-7, FP64 256^3 3.4e-14 as before).  What bounds a unit is the workers' instruction issue (FP64: digits and the
 // joining of the accumulators, 56 % of the integer pipe), not the MMAs (19 % of the tensor pipe).
 //
 // Layout (FP64).  Stacking the matrix digits j = 0 .. D-1-i of NC outputs as rows of one B operand makes all products of
 // input digit i ONE instruction: N = (D - i) NC columns, accumulated at column i NC, where block d of NC columns
-// holds order d.  (FP32: blocks hi hi twice, then the rest.)  A unit of work is 128 rows x NC pairs, both parts; TMEM columns 0 and 256 hold the symmetric and
-// the antisymmetric accumulators.  A CTA walks a contiguous range of units (the groups of NC pairs of a tile follow
+// holds order d.  (FP32: blocks hi hi twice, then the rest.)  A unit of work is 128, 96 or 32 rows x NC pairs, both
+// parts; TMEM columns 0 and 256 hold the symmetric and the antisymmetric accumulators.  A CTA walks a contiguous range
+// of units (the groups of NC pairs of a tile follow
 // each other, so its rows stay in L2 and their exponents are found once).  Warps:
 //   0      bulk copies of the B digits (pre-swizzled blocks) into the slots of a ring
 //   1      TMEM allocation, MMA issue
