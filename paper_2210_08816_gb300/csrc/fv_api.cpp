@@ -660,10 +660,10 @@ int fv_grid_create(const fv_grid_desc* desc, void* stream, fv_grid* out) {
   if (st == FV_OK) {
     if (cudaMalloc(&g->ws.smax, 8 * sizeof(unsigned)) != cudaSuccess ||
         cudaMemset(g->ws.smax, 0, 8 * sizeof(unsigned)) != cudaSuccess ||
-        cudaMalloc(&g->ws.err, sizeof(int)) != cudaSuccess || cudaMemset(g->ws.err, 0, sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&g->ws.err, sizeof(double) * (1 + kMaxScalars)) != cudaSuccess ||
+        cudaMemset(g->ws.err, 0, sizeof(double)) != cudaSuccess ||
         cudaMalloc(&g->ws.partials, sizeof(double) * kReduceBlocks * 256) != cudaSuccess ||
-        cudaMalloc(&g->ws.scalars, sizeof(double) * kMaxScalars) != cudaSuccess ||
-        cudaMallocHost(&g->ws.host_scalars, sizeof(double) * kMaxScalars) != cudaSuccess) {
+        cudaMallocHost(&g->ws.host_scalars, sizeof(double) * (1 + kMaxScalars)) != cudaSuccess) {
       cudaGetLastError();
       st = FV_ENOMEM;
       set_error("workspace allocation failed");
@@ -673,6 +673,7 @@ int fv_grid_create(const fv_grid_desc* desc, void* stream, fv_grid* out) {
     fv_grid_destroy(g);
     return st;
   }
+  g->ws.scalars = reinterpret_cast<double*>(g->ws.err) + 1;
   double s = 0.0;
   for (int d = 0; d < 3; ++d) s += 4.0 / (g->min_width[d] * g->min_width[d]);
   g->sigma_default = -0.5 * std::max(1.0, 1.0 / g->Pr) * s;
@@ -692,7 +693,6 @@ int fv_grid_destroy(fv_grid g) {
     if (g->ws.bt1[p]) cudaFree(g->ws.bt1[p]);
   }
   if (g->ws.partials) cudaFree(g->ws.partials);
-  if (g->ws.scalars) cudaFree(g->ws.scalars);
   if (g->ws.host_scalars) cudaFreeHost(g->ws.host_scalars);
   for (cudaEvent_t e : g->prof.pool) cudaEventDestroy(e);
   if (g->ws.smax) cudaFree(g->ws.smax);
@@ -721,9 +721,9 @@ int fv_set_wait_limit(fv_grid g, long long spins) {
 
 int fv_sync(fv_grid g) {
   if (!g) return invalid("null handle");
-  int dev_err = 0;
-  FV_CUDA(cudaMemcpyAsync(&dev_err, g->ws.err, sizeof(int), cudaMemcpyDeviceToHost, g->stream));
+  FV_CUDA(cudaMemcpyAsync(g->ws.host_scalars, g->ws.err, sizeof(int), cudaMemcpyDeviceToHost, g->stream));
   FV_CUDA(cudaStreamSynchronize(g->stream));
+  const int dev_err = *reinterpret_cast<const int*>(g->ws.host_scalars);
   if (dev_err != 0) {
     FV_CUDA(cudaMemsetAsync(g->ws.err, 0, sizeof(int), g->stream));
     FV_CUDA(cudaStreamSynchronize(g->stream));

@@ -58,8 +58,8 @@ struct Workspace {
   unsigned* bmax = nullptr;        // the same for blocks, eight words per vector, grown with bY
   int* err = nullptr;              // device error word of bounded device-side waits (0 = none)
   double* partials = nullptr;      // reduction partials
-  double* scalars = nullptr;       // device scalars (reduction results)
-  double* host_scalars = nullptr;  // pinned host mirror
+  double* scalars = nullptr;       // device scalars (reduction results), directly after the error word's eight bytes
+  double* host_scalars = nullptr;  // pinned host mirror of the error word and the scalars
   // block of vectors (fv_jvp_project_batch), per precision: J.v outputs (cap * 4N), two transform buffers
   // (cap * N each), grown on demand
   void* bY[2] = {nullptr, nullptr};
