@@ -469,7 +469,10 @@ __global__ void __launch_bounds__(kDgThreads, 1)
         // each slot is filled as soon as it is free: with three slots, the MMAs of the slab before run meanwhile
         constexpr int kRow = 2 * kDgWarps * 64;
         const int off = (2 * cw + rh) * 64 + (((kl >> 3) ^ (cw & 3)) << 4) + (kl & 7) * 2;  // row >> 1 = cw mod 4
-        if (gi >= kSlots && !mbar_wait(smem_u32(&bar_empty[s0]), ((gi / kSlots) - 1) & 1, t.err, 37, t.spins)) {
+        // (the warp gives up as one: the shuffles and votes further on take every lane)
+        if (gi >= kSlots &&
+            !__all_sync(0xffffffffu,
+                        mbar_wait(smem_u32(&bar_empty[s0]), ((gi / kSlots) - 1) & 1, t.err, 37, t.spins))) {
           ok = false;
           break;
         }
@@ -480,7 +483,8 @@ __global__ void __launch_bounds__(kDgThreads, 1)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive(smem_u32(&bar_conv[s0]));
         if (gi + 1 >= kSlots &&
-            !mbar_wait(smem_u32(&bar_empty[s1]), (((gi + 1) / kSlots) - 1) & 1, t.err, 38, t.spins)) {
+            !__all_sync(0xffffffffu,
+                        mbar_wait(smem_u32(&bar_empty[s1]), (((gi + 1) / kSlots) - 1) & 1, t.err, 38, t.spins))) {
           ok = false;
           break;
         }

@@ -1,0 +1,37 @@
+"""Rules of the device code that a GPU run cannot show without a hang or a race, checked on the sources."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2210_08816_gb300", "csrc")
+
+
+def _source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+# waits of one elected lane (the copies' warps): every lane of the other roles takes part
+ONE_LANE = {"kernels_digit.cu": {"31"}, "kernels_tc.cu": {"11", "13b"}}
+
+
+@pytest.mark.parametrize("name", sorted(ONE_LANE))
+def test_bounded_waits_of_whole_warps_are_decided_by_the_warp(name):
+    """A wait with the user's limit may run out for some lanes only; lanes that leave alone would miss the votes,
+    shuffles and aligned tensor-memory loads that the others go on to."""
+    src = _source(name)
+    seen = 0
+    for m in re.finditer(r"mbar_wait\(", src):
+        stmt = src[max(src.rfind(c, 0, m.start()) for c in ";{}") + 1:]
+        stmt = stmt[:re.search(r"[;{]", stmt).start()]
+        code = re.search(r"t\.err, (\d+), t\.spins", stmt)
+        if not code:
+            continue
+        seen += 1
+        tag = code.group(1) + ("b" if "bfree" in stmt else "")
+        after = src[m.start():]
+        after = after[after.index(";") + 1:]
+        voted = "__all_sync(0xffffffffu" in stmt or re.match(r"\s*if \(!__all_sync\(0xffffffffu, ok\)\)", after)
+        assert voted or tag in ONE_LANE[name], f"{name}: wait {tag} is decided lane by lane"
+    assert seen >= 7
