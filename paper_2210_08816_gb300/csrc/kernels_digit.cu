@@ -356,11 +356,10 @@ __global__ void __launch_bounds__(kDgThreads, 1)
           __syncwarp();
         }
     }
-    // give-up path: wait (full limit) for every MMA issued so far before the accumulators are freed
-    if (!ok) {
-      if (elect_one()) mma_commit(smem_u32(&bar_drain));
-      mbar_wait(smem_u32(&bar_drain), 0, t.err, 36, kWaitLimit);
-    }
+    // Whoever gives up (a worker's wait for the last unit can run out when this warp has issued everything): wait (full
+    // limit) for every MMA issued so far before the accumulators are freed and the block may exit
+    if (elect_one()) mma_commit(smem_u32(&bar_drain));
+    mbar_wait(smem_u32(&bar_drain), 0, t.err, 36, kWaitLimit);
   } else {
     // a worker warp converts rows 2 (kDgWarps it + cw), + 1 (half a warp each; a lane takes two neighbouring input
     // pairs) and reads TMEM lanes 32 (warp % 4) .. + 31 in the epilogue (one row per thread)

@@ -271,12 +271,11 @@ __global__ void __launch_bounds__(tc_threads(CONV), 1)
         }
       }
     }
-    // give-up path: a commit after every MMA issued so far arrives once they have all completed; wait for it (full
-    // limit) before the accumulators are freed
-    if (!ok) {
-      if (elect_one()) mma_commit(smem_u32(&bar_drain));
-      mbar_wait(smem_u32(&bar_drain), 0, t.err, 16, kWaitLimit);
-    }
+    // A commit after every MMA issued so far arrives once they have all completed; wait for it (full limit) before the
+    // accumulators are freed and the block may exit, whoever gave up: the epilogue's wait for the last tiles can run out
+    // when this warp has issued everything
+    if (elect_one()) mma_commit(smem_u32(&bar_drain));
+    mbar_wait(smem_u32(&bar_drain), 0, t.err, 16, kWaitLimit);
   } else if (warp < 2 + CONV / 32) {
     // converters: four threads to a row of every slab; those of one half of the warps take the first k-step of each
     // raw stage, the others the second, a thread inputs 8 hf .. 8 hf + 7 of it

@@ -35,3 +35,16 @@ def test_bounded_waits_of_whole_warps_are_decided_by_the_warp(name):
         voted = "__all_sync(0xffffffffu" in stmt or re.match(r"\s*if \(!__all_sync\(0xffffffffu, ok\)\)", after)
         assert voted or tag in ONE_LANE[name], f"{name}: wait {tag} is decided lane by lane"
     assert seen >= 7
+
+
+@pytest.mark.parametrize("name", sorted(ONE_LANE))
+def test_matrix_products_drain_before_tensor_memory_is_freed(name):
+    """The MMA warp waits for its products whether or not it gave up itself: another role's wait can run out after the
+    last product has been issued, and the block would free the accumulators and exit under it."""
+    src = _source(name)
+    drain = src.index("mma_commit(smem_u32(&bar_drain))")
+    assert "tcgen05.dealloc" in src[drain:]
+    before = src[:drain].rstrip()
+    assert before.endswith("if (elect_one())")
+    before = before[:-len("if (elect_one())")].rstrip()
+    assert before.endswith("}") and not re.search(r"if \(!ok\) \{$", before)
