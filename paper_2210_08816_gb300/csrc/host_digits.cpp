@@ -1,6 +1,7 @@
 // Host side of the digit passes (kernels_digit.cu): the half-size matrices of an axis operator as balanced base-256
 // digits in FP16, in the blocks and the shared-memory layout that the kernel copies.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -37,20 +38,40 @@ static int row_exponent(const std::vector<double> (&M)[2], int h, int j) {
 // Offset, in halves, of column k of row r of a block: 64-byte rows, 16-byte chunk c at c ^ ((r >> 1) & 3)
 static inline size_t swizzled(int r, int kk) { return (size_t)r * 32 + (((kk >> 3) ^ ((r >> 1) & 3)) << 3) + (kk & 7); }
 
-void build_digits(const std::vector<double> (&M)[2], int h, int D, int NC, std::vector<unsigned char>& blocks,
-                  std::vector<int>& exps) {
+void build_digits(const std::vector<double> (&M)[2], int h, int D, int NC, bool columns, std::vector<unsigned char>& blocks,
+                  std::vector<int>& exps, std::vector<unsigned char>& cexps) {
   static const HalfTable table;
   const int groups = (h + NC - 1) / NC, nslab = (h + 31) / 32;
   const size_t block = (size_t)D * NC * 32;  // halves
   blocks.assign(block * 2 * groups * nslab * 2, 0);
   uint16_t* out = reinterpret_cast<uint16_t*>(blocks.data());
   exps.assign(h, 0);
+  cexps.assign(2 * (size_t)h, 0);
+  if (columns) {
+    std::vector<int> q(2 * (size_t)h, INT_MIN);
+    int top = INT_MIN;
+    for (int part = 0; part < 2; ++part)
+      for (int k = 0; k < h; ++k) {
+        double most = 0.0;
+        for (int j = 0; j < h; ++j) most = std::max(most, std::fabs(M[part][(size_t)j * h + k]));
+        if (most > 0.0) std::frexp(most, &q[part * h + k]);
+        top = std::max(top, q[part * h + k]);
+      }
+    for (size_t i = 0; i < q.size(); ++i)
+      if (q[i] != INT_MIN) cexps[i] = (unsigned char)std::min(top - q[i], kDigitMaxColumn);
+  }
+  std::vector<double> S[2];
+  for (int part = 0; part < 2; ++part) {
+    S[part] = M[part];
+    for (int j = 0; j < h; ++j)
+      for (int k = 0; k < h; ++k) S[part][(size_t)j * h + k] = std::ldexp(S[part][(size_t)j * h + k], cexps[part * h + k]);
+  }
   for (int j = 0; j < h; ++j) {
-    exps[j] = row_exponent(M, h, j) - (8 * D - 1);  // integers of magnitude <= 2^(8 D - 1)
+    exps[j] = row_exponent(S, h, j) - (8 * D - 1);  // integers of magnitude <= 2^(8 D - 1)
     const double scale = std::ldexp(1.0, -exps[j]);
     for (int part = 0; part < 2; ++part)
       for (int k = 0; k < h; ++k) {
-        long long J = std::llrint(M[part][(size_t)j * h + k] * scale);
+        long long J = std::llrint(S[part][(size_t)j * h + k] * scale);
         uint16_t* b = out + ((size_t)(part * groups + j / NC) * nslab + k / 32) * block;
         for (int i = D - 1; i >= 0; --i) {
           const int dgt = i == 0 ? (int)J : (int)(((J + 128) & 255) - 128);

@@ -10,6 +10,10 @@
 // order i + j is an integer of at most 2^24: FP32 accumulators hold it exactly.  Orders 0 .. 6 are kept (28 products;
 // the first dropped one lies 2^-56 below the row's largest product) and joined in the epilogue as a 64-bit integer,
 // so the only roundings are the digits' quantisation, the dropped orders and the conversion of the result.
+// These are absolute in a row, so what a row spans must not be spanned by its inputs and its matrix separately.  The
+// backward matrices of a stretched axis do: the modes of the wall cells have entries larger than the others' by the square
+// root of the ratio of the widths, and coefficients as much smaller.  Every mode's column is therefore brought into the same
+// binade on the host and its inputs are lowered by as much (cexp: an integer addition to their exponents).
 //
 // FP32: rows scaled by a power of two into FP16's range, every value as the sum of two FP16 numbers (23 bits), all four
 // products, with the leading one spread over two accumulators.  (Fixed-point digits as in FP64 would need 32 bits: with
@@ -70,6 +74,7 @@ template <typename R>
 struct DgArgs {
   const unsigned char* B[4];  // per operator: digit blocks [part][group][slab] of this direction
   const int* eM[4];           // per operator: exponent of every output pair
+  const unsigned char* cM[4];  // FP64 backward, per operator: what the exponent of every input is lowered by
   const R* lam[3][4];         // scaled pass: eigenvalues of the three axes per operator
   R fac[4], shift[4];         // scaled pass: fac / (lam_z + lam_y + lam_x - shift)
   int k0[4], S[4];
@@ -101,8 +106,8 @@ __device__ __forceinline__ unsigned magnitude_bits(float x) { return __float_as_
 
 // x on the row's exponent E.  FP64: an integer, truncated, |I| < 2^54 with value I 2^(E - 1076); E >= 64 and shifts
 // clamp, so that zeros and subnormals shift out (the dropped bits lie below 2^-53 of the row's largest input, a
-// fraction of what the roundings of an FMA chain over its inputs add up to).  FP32: scaled below 2^14, value
-// y 2^(E - 140).
+// fraction of what the roundings of an FMA chain over its inputs add up to).  x 2^-c: E + c instead of E.  FP32: scaled
+// below 2^14, value y 2^(E - 140).
 __device__ __forceinline__ long long scaled(double x, int E) {
   const int hi = __double2hiint(x);
   const unsigned lo = (unsigned)__double2loint(x);
@@ -112,6 +117,11 @@ __device__ __forceinline__ long long scaled(double x, int E) {
   return ((long long)m ^ sg) - sg;
 }
 __device__ __forceinline__ float scaled(float x, int E) { return x * __uint_as_float((unsigned)(267 - E) << 23); }
+
+// The high word of |x| 2^-c (0 where it would fall below the smallest exponent; an Inf or NaN keeps its own)
+__device__ __forceinline__ unsigned lowered(unsigned high, int c) {
+  return high >= 0x7ff00000u ? high : (unsigned)max((int)high - (c << 20), 0);
+}
 
 // The D digits of two neighbouring inputs as FP16 pairs, digit i at dst + i * kDgDigitBytes.  FP64: balanced base-256
 // digits; adding 128 to each makes them the bytes of an unsigned integer; 0x6400 | byte is the FP16 number
@@ -227,6 +237,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
   // exponents of the rows, four tiles deep: a warp can find those of tile T + 1 while another still reads T - 1's in
   // an epilogue (tile T + 2 has to wait for that epilogue's MMAs)
   __shared__ int row_exp[4][kDgRows];
+  __shared__ unsigned char in_exp[4][2 * kDigitMaxH + 4];  // FP64 backward: cM
   __shared__ int out_exp[4][kDigitMaxH];  // exponents of the matrix rows per operator (FP32: 2^exponent, as bits)
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t base = smem_u32(smem);
@@ -249,6 +260,8 @@ __global__ void __launch_bounds__(kDgThreads, 1)
   }
   for (int i = threadIdx.x; i < (t.op_mask + 1) * h; i += kDgThreads) 
     out_exp[i / h][i % h] = F64 ? t.eM[i / h][i % h] : (t.eM[i / h][i % h] + 127) << 23;  // FP32: the power of two
+  if (F64 && BWD)
+    for (int i = threadIdx.x; i < (t.op_mask + 1) * n; i += kDgThreads) in_exp[i / n][i % n] = t.cM[i / n][i % n];
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                  "r"(512)
@@ -404,12 +417,20 @@ __global__ void __launch_bounds__(kDgThreads, 1)
 #pragma unroll
           for (int it = 0; it < ITS; ++it) load_row(it, src, rows, kl, k0, S);
         }
+        // what these inputs' exponents are lowered by
+        struct {
+          int x0 = 0, x1 = 0, y0 = 0, y1 = 0;
+        } c;
+        if constexpr (F64 && BWD) {
+          const unsigned char* e = in_exp[op] + min(j * 32 + kl, h);  // (beyond h the inputs are zero)
+          c.x0 = e[0], c.x1 = e[1], c.y0 = e[h], c.y1 = e[h + 1];
+        }
         if (j == 0 && (du == 0 || un.group == 0)) ++tc;
         if (j == 0 && (du == 0 || un.group == 0) && t.nslab == 1) {  // the rows are in the registers
 #pragma unroll
           for (int it = 0; it < ITS; ++it) {
-            unsigned m = max(max(magnitude_bits(x0[it]), magnitude_bits(x1[it])),
-                             max(magnitude_bits(y0[it]), magnitude_bits(y1[it])));
+            unsigned m = max(max(lowered(magnitude_bits(x0[it]), c.x0), lowered(magnitude_bits(x1[it]), c.x1)),
+                             max(lowered(magnitude_bits(y0[it]), c.y0), lowered(magnitude_bits(y1[it]), c.y1)));
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
             if ((lane & 15) == 0) row_exp[tc & 3][2 * (kDgWarps * it + cw) + rh] = max((int)(m >> kExpShift), kExpMin);
@@ -436,7 +457,9 @@ __global__ void __launch_bounds__(kDgThreads, 1)
 #pragma unroll
             for (int q = 0; q < 4; ++q)
 #pragma unroll
-              for (int r = 0; r < kRows; ++r) m[r] = max(m[r], v[q][r] & 0x7fffffffu);
+              for (int r = 0; r < kRows; ++r)
+                m[r] = max(m[r], F64 && BWD ? lowered(v[q][r] & 0x7fffffffu, in_exp[op][min(k + 32 * q, n - 1)])
+                                            : v[q][r] & 0x7fffffffu);
           }
 #pragma unroll
           for (int r = 0; r < kRows; ++r) {
@@ -459,10 +482,10 @@ __global__ void __launch_bounds__(kDgThreads, 1)
 #pragma unroll
         for (int it = 0; it < ITS; ++it) {
           const int E = re[2 * (kDgWarps * it + cw) + rh];
-          i0[it] = scaled(x0[it], E);
-          i1[it] = scaled(x1[it], E);
-          j0[it] = scaled(y0[it], E);
-          j1[it] = scaled(y1[it], E);
+          i0[it] = scaled(x0[it], E + c.x0);
+          i1[it] = scaled(x1[it], E + c.x1);
+          j0[it] = scaled(y0[it], E + c.y0);
+          j1[it] = scaled(y1[it], E + c.y1);
           load_row(it, nsrc, nrows, nk, nk0, nS);
         }
         // each slot is filled as soon as it is free: with three slots, the MMAs of the slab before run meanwhile
@@ -637,6 +660,7 @@ int digit_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int
     const HalfDev<R>& d = H[axis][kinds[op][axis]];
     t.B[op] = d.dig[bwd ? 1 : 0];
     t.eM[op] = d.dexp[bwd ? 1 : 0];
+    t.cM[op] = d.cexp;
     for (int x = 0; x < 3; ++x) t.lam[x][op] = H[x][kinds[op][x]].lam;
     t.fac[op] = (R)sfac[op];
     t.shift[op] = (R)shift[op];
