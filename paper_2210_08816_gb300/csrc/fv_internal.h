@@ -368,6 +368,8 @@ int build_axis(const std::vector<double>& xf, AxisHost& a, bool metrics_only = f
 // the tensor-core passes split each 1D eigenproblem into symmetric and antisymmetric halves, which holds
 // only on such axes.
 bool mirror_symmetric(const std::vector<double>& xf);
+// Widest over narrowest cell of an axis.
+double width_ratio(const std::vector<double>& xf);
 // The 1D operators of a mirror-symmetric axis as two half-size problems (symmetric and antisymmetric vectors).
 // Kinds: the Neumann operator of the pressure solve, the cell-centred and the face-centred Dirichlet diffusion
 // operators.  Unknown k0 + i pairs with S - k0 - i (i < h = ceil(n / 2)); the modes are in the order

@@ -22,6 +22,15 @@ int invalid(const std::string& msg) {
 
 }  // namespace
 
+double width_ratio(const std::vector<double>& xf) {
+  double least = 1.0, most = 0.0;
+  for (size_t i = 0; i + 1 < xf.size(); ++i) {
+    least = std::min(least, xf[i + 1] - xf[i]);
+    most = std::max(most, xf[i + 1] - xf[i]);
+  }
+  return most / least;
+}
+
 bool mirror_symmetric(const std::vector<double>& xf) {
   const int n = (int)xf.size() - 1;
   const double tol = 4.0 * std::numeric_limits<double>::epsilon();

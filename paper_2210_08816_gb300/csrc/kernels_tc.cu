@@ -1,5 +1,5 @@
 // Fast-diagonalisation passes of the pressure solve for FP32 fields on the tensor cores (tcgen05), for grids whose axes
-// have 32 .. 256 cells, a multiple of 32, and mirror-symmetric faces.
+// have 32 .. 256 cells, a multiple of 32, and mirror-symmetric faces, stretched to s = 4 or so at most (tc_setup).
 //
 // A pass is the GEMM  C[p][m] = sum_k A[p][k] B[m][k]  (A = field rows, k contiguous; B = a 1D eigenvector matrix),
 // stored transposed as out[m][p] (see kernels_fdm.cu), in the half-size form of HalfOpHost: forward passes contract
@@ -473,10 +473,18 @@ int encode_tensor_map(CUtensorMap* map, CUtensorMapDataType type, int rank, cons
 }
 
 // The grid's FP32 pressure solves take these passes (half-size operators and their FP16 parts are ready).
+// Not on strongly stretched grids: the parts keep 2^-39 of the field's largest value, and a corner cell's potential is put
+// together from coefficients smaller than that value by the square root of the product of the axes' width ratios.  Up to a
+// product of 2^29 what is lost stays below FP32's own rounding (2^-24); beyond it the passes with a scale per row
+// (kernels_digit.cu) or FP32 sums take over.  Projection's error, 128 x 64 x 32, s = 2, 3, 4, 6 (products 2^11, 2^20, 2^28,
+// 2^45): here 1.3e-6, 4.9e-6, 3.0e-5, 4.8e-2; FP32 sums of TF32 parts 1.7e-6, 5.4e-6, 3.5e-5, 1.3e-3; with a scale per row
+// 5e-7, 2e-6, 1.4e-5, 7e-4 (130 x 70 x 60).  Time of a 256^3 projection 337 us here, 593 with a scale per row.
+constexpr double kTcMostSpan = 536870912.0;
 int tc_setup(fv_grid_s* g) {
   static_assert(kDigitCols32 == 64 && kDigits32 == 2, "the B blocks hold 64 outputs, two parts");
   for (int n : {g->nx, g->ny, g->nz})
     if (n < 32 || n > 256 || n % 32 != 0) return FV_OK;
+  if (width_ratio(g->xf[0]) * width_ratio(g->xf[1]) * width_ratio(g->xf[2]) > kTcMostSpan) return FV_OK;
   if (!g->digit_ready || !encoder()) return FV_OK;
   for (auto k : {k_pass_tc<false, false, 256>, k_pass_tc<true, false, 256>, k_pass_tc<false, true, 256>,
                  k_pass_tc<false, false, 512>, k_pass_tc<true, false, 512>, k_pass_tc<false, true, 512>})

@@ -103,3 +103,10 @@ def _check_projection(fv, shape, stretch, prec, factor):
 @pytest.mark.parametrize("stretch", [4.0, 6.0])
 def test_fp64_projection_keeps_its_accuracy(fv, shape, stretch):
     _check_projection(fv, shape, stretch, 0, np.sqrt(6.0 * max(shape)))
+
+
+# multiples of 32: by FP16 parts under one scale per field while the widths allow it
+@pytest.mark.parametrize("shape", [(128, 64, 32), (64, 64, 64), (130, 70, 60), (30, 41, 36)])
+@pytest.mark.parametrize("stretch", [2.0, 4.0, 4.2, 6.0])
+def test_fp32_projection_keeps_its_accuracy(fv, shape, stretch):
+    _check_projection(fv, shape, stretch, 1, 2.0 * np.sqrt(6.0))
