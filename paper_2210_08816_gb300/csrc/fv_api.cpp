@@ -172,7 +172,7 @@ static int upload_digits(fv_grid_s* g, const HalfOpHost (*half)[3]) {
           if (prec)
             build_halves(dir ? o.E : o.F, (o.n + 1) / 2, kDigitCols32, blocks, exps);
           else
-            build_digits(dir ? o.E : o.F, (o.n + 1) / 2, kDigits64, kDigitCols64, dir == 1, blocks, exps, cexps);
+            build_digits(dir ? o.E : o.F, (o.n + 1) / 2, kDigits64, kDigitCols64, dir == 0, blocks, exps, cexps);
           it.cexp = put(cexps.data(), prec == 0 ? cexps.size() : 0);
           it.dig = put(blocks.data(), blocks.size());
           it.exp = put(exps.data(), exps.size() * sizeof(int));
@@ -191,7 +191,7 @@ static int upload_digits(fv_grid_s* g, const HalfOpHost (*half)[3]) {
       for (int dir = 0; dir < 2; ++dir) {
         g->half64[d][kind].dig[dir] = base + items[d][kind][0][dir].dig;
         g->half64[d][kind].dexp[dir] = (const int*)(base + items[d][kind][0][dir].exp);
-        if (dir) g->half64[d][kind].cexp = base + items[d][kind][0][dir].cexp;
+        g->half64[d][kind].cexp[dir] = base + items[d][kind][0][dir].cexp;
         g->half32[d][kind].dig[dir] = base + items[d][kind][1][dir].dig;
         g->half32[d][kind].dexp[dir] = (const int*)(base + items[d][kind][1][dir].exp);
       }

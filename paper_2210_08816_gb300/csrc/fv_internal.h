@@ -47,8 +47,8 @@ struct HalfDev {
   // the matrices as digits (build_digits) and their rows' exponents, forward and backward
   const unsigned char* dig[2] = {nullptr, nullptr};
   const int* dexp[2] = {nullptr, nullptr};
-  // FP64, backward: what a mode's inputs are scaled down by (2^-cexp), [h symmetric | floor(n / 2) antisymmetric]
-  const unsigned char* cexp = nullptr;
+  // FP64: what a column's inputs are scaled down by (2^-cexp), [h symmetric | h antisymmetric]
+  const unsigned char* cexp[2] = {nullptr, nullptr};
 };
 
 struct Workspace {
@@ -392,10 +392,10 @@ constexpr int kDigits64 = 7, kDigitCols64 = 32, kDigits32 = 2, kDigitCols32 = 64
 // The two h x h matrices as D balanced base-256 digits (FP16), row j on the common exponent exps[j] of both parts:
 // 2^cexps[part h + k] M[part][j][k] = 2^exps[j] sum_i digit_i 256^(D-1-i).  Blocks [part][group of NC rows][slab of 32
 // columns], each D NC rows (digit i, output j % NC at row i NC + j % NC) of 64 bytes, 64-byte swizzled.
-// columns: cexps (at most kDigitMaxColumn) bring every column's largest entry into the same binade, and the pass takes as
-// much off its inputs' exponents; else they are 0.
+// cexps (at most kDigitMaxColumn) bring every column's largest entry into the same binade, and the pass takes as much off
+// its inputs' exponents.  shared: column k of both parts gets the same (forward, where both take the same inputs).
 constexpr int kDigitMaxColumn = 48;
-void build_digits(const std::vector<double> (&M)[2], int h, int D, int NC, bool columns, std::vector<unsigned char>& blocks,
+void build_digits(const std::vector<double> (&M)[2], int h, int D, int NC, bool shared, std::vector<unsigned char>& blocks,
                   std::vector<int>& exps, std::vector<unsigned char>& cexps);
 // The same for FP32 fields: two FP16 parts of every entry, M[part][j][k] = 2^exps[j] (hi + lo), in the same blocks.
 void build_halves(const std::vector<double> (&M)[2], int h, int NC, std::vector<unsigned char>& blocks,

@@ -38,7 +38,7 @@ static int row_exponent(const std::vector<double> (&M)[2], int h, int j) {
 // Offset, in halves, of column k of row r of a block: 64-byte rows, 16-byte chunk c at c ^ ((r >> 1) & 3)
 static inline size_t swizzled(int r, int kk) { return (size_t)r * 32 + (((kk >> 3) ^ ((r >> 1) & 3)) << 3) + (kk & 7); }
 
-void build_digits(const std::vector<double> (&M)[2], int h, int D, int NC, bool columns, std::vector<unsigned char>& blocks,
+void build_digits(const std::vector<double> (&M)[2], int h, int D, int NC, bool shared, std::vector<unsigned char>& blocks,
                   std::vector<int>& exps, std::vector<unsigned char>& cexps) {
   static const HalfTable table;
   const int groups = (h + NC - 1) / NC, nslab = (h + 31) / 32;
@@ -47,19 +47,18 @@ void build_digits(const std::vector<double> (&M)[2], int h, int D, int NC, bool 
   uint16_t* out = reinterpret_cast<uint16_t*>(blocks.data());
   exps.assign(h, 0);
   cexps.assign(2 * (size_t)h, 0);
-  if (columns) {
-    std::vector<int> q(2 * (size_t)h, INT_MIN);
-    int top = INT_MIN;
-    for (int part = 0; part < 2; ++part)
-      for (int k = 0; k < h; ++k) {
-        double most = 0.0;
-        for (int j = 0; j < h; ++j) most = std::max(most, std::fabs(M[part][(size_t)j * h + k]));
-        if (most > 0.0) std::frexp(most, &q[part * h + k]);
-        top = std::max(top, q[part * h + k]);
-      }
-    for (size_t i = 0; i < q.size(); ++i)
-      if (q[i] != INT_MIN) cexps[i] = (unsigned char)std::min(top - q[i], kDigitMaxColumn);
-  }
+  std::vector<int> q(2 * (size_t)h, INT_MIN);  // largest magnitude of every column
+  int top = INT_MIN;
+  for (int part = 0; part < 2; ++part)
+    for (int k = 0; k < h; ++k) {
+      double most = 0.0;
+      for (int j = 0; j < h; ++j) most = std::max(most, std::fabs(M[part][(size_t)j * h + k]));
+      if (most > 0.0) std::frexp(most, &q[part * h + k]);
+      top = std::max(top, q[part * h + k]);
+    }
+  for (int k = 0; k < h && shared; ++k) q[k] = q[h + k] = std::max(q[k], q[h + k]);
+  for (size_t i = 0; i < q.size(); ++i)
+    if (q[i] != INT_MIN) cexps[i] = (unsigned char)std::min(top - q[i], kDigitMaxColumn);
   std::vector<double> S[2];
   for (int part = 0; part < 2; ++part) {
     S[part] = M[part];

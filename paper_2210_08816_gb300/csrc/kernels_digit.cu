@@ -11,9 +11,9 @@
 // the first dropped one lies 2^-56 below the row's largest product) and joined in the epilogue as a 64-bit integer,
 // so the only roundings are the digits' quantisation, the dropped orders and the conversion of the result.
 // These are absolute in a row, so what a row spans must not be spanned by its inputs and its matrix separately.  The
-// backward matrices of a stretched axis do: the modes of the wall cells have entries larger than the others' by the square
-// root of the ratio of the widths, and coefficients as much smaller.  Every mode's column is therefore brought into the same
-// binade on the host and its inputs are lowered by as much (cexp: an integer addition to their exponents).
+// matrices of a stretched axis do: the modes of the narrow cells have entries larger than the others' by the square root of
+// the ratio of the widths, and coefficients as much smaller.  Every column is therefore brought into the same binade on the
+// host and its inputs are lowered by as much (cexp: an integer addition to their exponents).
 //
 // FP32: rows scaled by a power of two into FP16's range, every value as the sum of two FP16 numbers (23 bits), all four
 // products, with the leading one spread over two accumulators.  (Fixed-point digits as in FP64 would need 32 bits: with
@@ -74,7 +74,7 @@ template <typename R>
 struct DgArgs {
   const unsigned char* B[4];  // per operator: digit blocks [part][group][slab] of this direction
   const int* eM[4];           // per operator: exponent of every output pair
-  const unsigned char* cM[4];  // FP64 backward, per operator: what the exponent of every input is lowered by
+  const unsigned char* cM[4];  // FP64, per operator: what the exponents of a column's inputs are lowered by
   const R* lam[3][4];         // scaled pass: eigenvalues of the three axes per operator
   R fac[4], shift[4];         // scaled pass: fac / (lam_z + lam_y + lam_x - shift)
   int k0[4], S[4];
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
   // exponents of the rows, four tiles deep: a warp can find those of tile T + 1 while another still reads T - 1's in
   // an epilogue (tile T + 2 has to wait for that epilogue's MMAs)
   __shared__ int row_exp[4][kDgRows];
-  __shared__ unsigned char in_exp[4][2 * kDigitMaxH + 4];  // FP64 backward: cM
+  __shared__ unsigned char in_exp[4][2 * kDigitMaxH + 4];  // FP64: cM of every input of a row
   __shared__ int out_exp[4][kDigitMaxH];  // exponents of the matrix rows per operator (FP32: 2^exponent, as bits)
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t base = smem_u32(smem);
@@ -260,8 +260,11 @@ __global__ void __launch_bounds__(kDgThreads, 1)
   }
   for (int i = threadIdx.x; i < (t.op_mask + 1) * h; i += kDgThreads) 
     out_exp[i / h][i % h] = F64 ? t.eM[i / h][i % h] : (t.eM[i / h][i % h] + 127) << 23;  // FP32: the power of two
-  if (F64 && BWD)
-    for (int i = threadIdx.x; i < (t.op_mask + 1) * n; i += kDgThreads) in_exp[i / n][i % n] = t.cM[i / n][i % n];
+  if (F64)
+    for (int i = threadIdx.x; i < (t.op_mask + 1) * n; i += kDgThreads) {
+      const int op = i / n, r = i - op * n, k = r - t.k0[op];  // (forward: the cell k0 + k or its mirror)
+      in_exp[op][r] = t.cM[op][BWD ? r : max(min(k, t.S[op] - t.k0[op] - r), 0)];
+    }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                  "r"(512)
@@ -421,9 +424,9 @@ __global__ void __launch_bounds__(kDgThreads, 1)
         struct {
           int x0 = 0, x1 = 0, y0 = 0, y1 = 0;
         } c;
-        if constexpr (F64 && BWD) {
-          const unsigned char* e = in_exp[op] + min(j * 32 + kl, h);  // (beyond h the inputs are zero)
-          c.x0 = e[0], c.x1 = e[1], c.y0 = e[h], c.y1 = e[h + 1];
+        if constexpr (F64) {
+          const unsigned char* e = in_exp[op] + (BWD ? 0 : k0) + min(j * 32 + kl, h);  // (beyond h the inputs are zero)
+          c.x0 = e[0], c.x1 = e[1], c.y0 = e[BWD ? h : 0], c.y1 = e[BWD ? h + 1 : 1];
         }
         if (j == 0 && (du == 0 || un.group == 0)) ++tc;
         if (j == 0 && (du == 0 || un.group == 0) && t.nslab == 1) {  // the rows are in the registers
@@ -458,8 +461,8 @@ __global__ void __launch_bounds__(kDgThreads, 1)
             for (int q = 0; q < 4; ++q)
 #pragma unroll
               for (int r = 0; r < kRows; ++r)
-                m[r] = max(m[r], F64 && BWD ? lowered(v[q][r] & 0x7fffffffu, in_exp[op][min(k + 32 * q, n - 1)])
-                                            : v[q][r] & 0x7fffffffu);
+                m[r] = max(m[r], F64 ? lowered(v[q][r] & 0x7fffffffu, in_exp[op][min(k + 32 * q, n - 1)])
+                                     : v[q][r] & 0x7fffffffu);
           }
 #pragma unroll
           for (int r = 0; r < kRows; ++r) {
@@ -660,7 +663,7 @@ int digit_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int
     const HalfDev<R>& d = H[axis][kinds[op][axis]];
     t.B[op] = d.dig[bwd ? 1 : 0];
     t.eM[op] = d.dexp[bwd ? 1 : 0];
-    t.cM[op] = d.cexp;
+    t.cM[op] = d.cexp[bwd ? 1 : 0];
     for (int x = 0; x < 3; ++x) t.lam[x][op] = H[x][kinds[op][x]].lam;
     t.fac[op] = (R)sfac[op];
     t.shift[op] = (R)shift[op];
