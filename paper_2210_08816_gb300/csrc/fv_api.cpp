@@ -655,6 +655,8 @@ int fv_grid_create(const fv_grid_desc* desc, void* stream, fv_grid* out) {
   if (st == FV_OK) st = upload_axes<double>(g, ax, hp, 0, g->geo64, g->fdm64, g->cd64, g->fd64, g->half64);
   if (st == FV_OK) st = upload_axes<float>(g, ax, hp, 1, g->geo32, g->fdm32, g->cd32, g->fd32, g->half32);
   if (st == FV_OK && g->half_ready && (std::max({n[0], n[1], n[2]}) + 1) / 2 <= kDigitMaxH) st = upload_digits(g, half);
+  for (auto setup : {half_setup, plane_setup, flux_setup, stencil_setup, stencil_pair_setup})
+    if (st == FV_OK) st = setup();
   if (st == FV_OK && tc_setup(g) != FV_OK) {  // keep the other passes
     g->tc_ready = false;
     cudaGetLastError();

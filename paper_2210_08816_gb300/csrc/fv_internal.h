@@ -264,7 +264,13 @@ int launch_diffusion_solve(const fv_grid_s* g, const R* in, R* out, R* tmp, doub
 template <typename R>
 int digit_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int (*kinds)[3], bool per_field,
                const double* sfac, const double* shift, const R* in, R* out, bool scale, bool zero_mode, int nf);
+// Shared-memory limits of the kernels.  They belong to a device, so every grid's creation sets them on its own.
 int digit_setup();
+int half_setup();
+int plane_setup();
+int flux_setup();
+int stencil_setup();
+int stencil_pair_setup();
 
 // BLAS-1 and reductions (kernels_blas.cu).  Results land in g->ws.scalars[slot...].
 template <typename R>

@@ -258,6 +258,18 @@ bool digit_wins(int n, long long rows) {
   return (double)rows * n * ((n + 1) / 2) >= (sizeof(R) == 8 ? 3.2e6 : 1.6e7);
 }
 
+// Unused shared memory that leaves room for `per` blocks of the FP64 form on an SM.
+constexpr int half_pad(int U, int per) {
+  return 222 * 1024 / per - (int)(sizeof(double) * (2 * kHalfK * 33 + 2 * 4 * U * kHalfK)) - 1024;
+}
+
+template <int U>
+int half_setup_u() {
+  for (auto k : {k_half<double, false, U>, k_half<double, true, U>})
+    FV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, half_pad(U, 1)));
+  return FV_OK;
+}
+
 // One pass along `axis` over nf fields of a (na x nb) x n block, kinds[op][axis] = the operators (one, or four
 // with per_field): in[a][b][k] -> out[m][a][b] with the modes in the half order.
 template <typename R>
@@ -298,14 +310,7 @@ int half_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int 
     // overlap its predecessor and still spread evenly (32^3 FP64 J.v + projection 73 us without the overlap, 58.5 so)
     const long long per = ((long long)grid.x * grid.y * grid.z + g->sms - 1) / g->sms;
     if (per <= 6) {
-      const int used = (int)(sizeof(double) * (2 * kHalfK * 33 + 2 * 4 * U * kHalfK)) + 1024;
-      const int pad = 222 * 1024 / (int)per - used;
-      static bool attr_set[2][5] = {};
-      if (!attr_set[bwd][U]) {
-        FV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 222 * 1024 - used));
-        attr_set[bwd][U] = true;
-      }
-      launch(k, grid, 128, pad, g->stream, t, in, out);
+      launch(k, grid, 128, half_pad(U, (int)per), g->stream, t, in, out);
     } else {
       launch_spread(k, grid, 128, 0, g->stream, t, in, out);
     }
@@ -392,6 +397,12 @@ template <>
 const FdmDev<float>& fd_of<float>(const fv_grid_s* g) { return g->fd32; }
 
 }  // namespace
+
+int half_setup() {
+  FV_TRY(half_setup_u<1>());
+  FV_TRY(half_setup_u<2>());
+  return half_setup_u<4>();
+}
 
 template <typename R>
 int launch_poisson_block(const fv_grid_s* g, const R* rhs, R* phi, R* tmp, int nvec) {

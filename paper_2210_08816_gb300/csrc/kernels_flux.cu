@@ -383,6 +383,13 @@ static FluxPlan flux_plan(const fv_grid_s* g, int nvec) {
   return best;
 }
 
+int flux_setup() {
+  auto most = [](int arrays) { return (int)((kFxRing * arrays * kFxTile + 8 * (2 * kFxCells + 64)) * sizeof(double)); };
+  FV_CUDA(cudaFuncSetAttribute(k_flux<double, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, most(4)));
+  FV_CUDA(cudaFuncSetAttribute(k_flux<double, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most(8)));
+  return FV_OK;
+}
+
 template <int MODE>
 int launch_flux(const fv_grid_s* g, double Gr, double sigma, const double* q, const double* v, double* out, int nvec) {
   using R = double;
@@ -426,12 +433,6 @@ int launch_flux(const fv_grid_s* g, double Gr, double sigma, const double* q, co
       t.use_tma = 0;
   }
   const size_t smem = ((size_t)kFxRing * NA * t.pl + 8 * ((size_t)pl.ty * (pl.tx + 1) + (size_t)(pl.ty + 1) * pl.tx)) * sizeof(R);
-  static bool attr_set = false;
-  if (!attr_set) {
-    const size_t most = ((size_t)kFxRing * NA * kFxTile + 8 * (size_t)(2 * kFxCells + 64)) * sizeof(R);
-    FV_CUDA(cudaFuncSetAttribute(k_flux<R, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
-    attr_set = true;
-  }
   const dim3 grid((g->nx + pl.tx - 1) / pl.tx, (g->ny + pl.ty - 1) / pl.ty, t.nch * nvec);
   ProfScope ps(g, PROF_STENCIL);
   launch(k_flux<R, MODE>, grid, kFxThreads, smem, g->stream, tq, tv, t);

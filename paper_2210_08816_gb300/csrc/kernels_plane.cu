@@ -199,6 +199,12 @@ bool plane_wins(const fv_grid_s* g, int nf) {
   return most <= 64 && (double)g->N * ((most + 1) / 2) * nf <= (enough ? 3.4e6 : 1.2e6);
 }
 
+int plane_setup() {
+  for (auto k : {k_plane<false, false>, k_plane<false, true>, k_plane<true, true>})
+    FV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+  return FV_OK;
+}
+
 int plane_solve(const fv_grid_s* g, const int (*kinds)[3], bool per_field, const double* sfac, const double* shift,
                 bool zero_mode, const double* in, double* out, int nf) {
   const int len[3] = {g->nx, g->ny, g->nz}, stride[3] = {1, g->nx, g->nx * g->ny};
@@ -240,11 +246,6 @@ int plane_solve(const fv_grid_s* g, const int (*kinds)[3], bool per_field, const
     if (planes * C <= g->sms) smem = std::max<size_t>(smem, 120 * 1024);
     void (*k)(PlaneArgs, const double*, double*) =
         pair == 0 ? k_plane<false, false> : pair == 1 ? k_plane<false, true> : k_plane<true, true>;
-    static bool attr_set[3] = {};
-    if (!attr_set[pair]) {
-      FV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-      attr_set[pair] = true;
-    }
     ProfScope ps(g, PROF_TRANSFORM);
     launch_cluster(C, k, dim3((unsigned)(len[axp] * C), nf), kPlThreads, smem, g->stream, t, pair == 0 ? in : out, out);
     FV_CUDA(cudaGetLastError());

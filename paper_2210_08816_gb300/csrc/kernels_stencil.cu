@@ -707,15 +707,19 @@ int state_map(const fv_grid_s* g, const R* ptr, CUtensorMap* m, int nvec = 1) {
 }
 
 template <typename R>
+constexpr size_t stencil_smem() {
+  return (size_t)8 * kRing * kPL * sizeof(R);
+}
+
+int stencil_setup() {
+  FV_CUDA(cudaFuncSetAttribute(k_stencil_z<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stencil_smem<float>()));
+  return FV_OK;
+}
+
+template <typename R>
 int launch_stencil_z(const fv_grid_s* g, double Gr, double sigma, const R* q, const R* v, R* out, int nvec,
                      const TempOut& t) {
-  constexpr int NA = 8;
-  const size_t smem = (size_t)NA * kRing * kPL * sizeof(R);
-  static bool attr_set = false;
-  if (!attr_set) {
-    FV_CUDA(cudaFuncSetAttribute(k_stencil_z<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr_set = true;
-  }
+  const size_t smem = stencil_smem<R>();
   // TMA needs 16-byte aligned rows and base addresses; small grids take the cp.async path
   CUtensorMap tq, tv;
   std::memset(&tq, 0, sizeof(tq));

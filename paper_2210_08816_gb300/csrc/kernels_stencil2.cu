@@ -22,6 +22,7 @@ constexpr int kPW2 = 72;            // ring row: x from i0 - 4 to i0 + 67 (TMA x
 constexpr int kPX0 = 4;             // column of the tile's first cell
 constexpr int kPL2 = kPHY * kPW2;   // one array's plane tile
 constexpr int kPRing = 4, kPNA = 8;
+constexpr size_t kPairSmem = (size_t)kPRing * kPNA * kPL2 * sizeof(float);
 constexpr long long kPWaitLimit = 1LL << 22;
 
 // ---------------------------------------------------------------- pair arithmetic
@@ -457,15 +458,15 @@ bool stencil_pair_eligible(const fv_grid_s* g, const float* q, const float* v) {
   return g->nx % kPX == 0 && g->ny >= 16 && ((uintptr_t)q % 16) == 0 && ((uintptr_t)v % 16) == 0;
 }
 
+int stencil_pair_setup() {
+  for (auto k : {k_stencil_pair<false>, k_stencil_pair<true>})
+    FV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem));
+  return FV_OK;
+}
+
 int launch_stencil_pair(const fv_grid_s* g, double Gr, double sigma, const float* q, const float* v, float* out,
                         int nvec, const TempOut& t) {
-  const size_t smem = (size_t)kPRing * kPNA * kPL2 * sizeof(float);
-  static bool attr_set = false;
-  if (!attr_set) {
-    FV_CUDA(cudaFuncSetAttribute(k_stencil_pair<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    FV_CUDA(cudaFuncSetAttribute(k_stencil_pair<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr_set = true;
-  }
+  const size_t smem = kPairSmem;
   // blocks of vectors march the z-chunk the autotuner picked, if it ran; otherwise stencil_chunk's
   const int zc = (nvec > 1 && g->tune.pair_zc > 0) ? g->tune.pair_zc
                                                    : stencil_chunk(g, g->nx / kPX * ((g->ny + kPY - 1) / kPY), nvec);

@@ -48,3 +48,23 @@ def test_matrix_products_drain_before_tensor_memory_is_freed(name):
     assert before.endswith("if (elect_one())")
     before = before[:-len("if (elect_one())")].rstrip()
     assert before.endswith("}") and not re.search(r"if \(!ok\) \{$", before)
+
+
+def test_kernel_attributes_are_set_for_every_grid():
+    """A kernel's shared-memory limit belongs to a device: a flag of the process would leave a second one without it."""
+    create = _source("fv_api.cpp")
+    create = create[create.index("int fv_grid_create("):create.index("int fv_grid_destroy(")]
+    setups = set()
+    for name in sorted(os.listdir(CSRC)):
+        if not name.endswith((".cu", ".cpp")):
+            continue
+        src = _source(name)
+        assert not re.search(r"static bool attr", src), name
+        for m in re.finditer(r"cudaFuncSetAttribute\(", src):
+            function = re.findall(r"^(?:static )?int (\w+)\(", src[:m.start()], re.M)[-1]
+            assert "_setup" in function, f"{name}: {function}"
+            setups.add(re.sub(r"_setup_\w+", "_setup", function))
+    assert len(setups) >= 7
+    for f in setups - {"digit_setup"}:
+        assert re.search(rf"\b{f}\b", create), f
+    assert "upload_digits" in create and "digit_setup()" in _source("fv_api.cpp")
