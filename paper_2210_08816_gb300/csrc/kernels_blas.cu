@@ -79,13 +79,13 @@ struct F2 {
 };
 
 template <typename R>
-__device__ __forceinline__ double dot_chunk(const R* __restrict__ a, const R* __restrict__ b, size_t s, size_t e) {
+__device__ __forceinline__ double dot_chunk(const R* a, const R* b, size_t s, size_t e) {
   double acc = 0.0;
   for (size_t t = s + threadIdx.x; t < e; t += kThreads) acc = fma((double)a[t], (double)b[t], acc);
   return acc;
 }
 template <>
-__device__ __forceinline__ double dot_chunk<float>(const float* __restrict__ a, const float* __restrict__ b, size_t s,
+__device__ __forceinline__ double dot_chunk<float>(const float* a, const float* b, size_t s,
                                                    size_t e) {
   F2 acc;
   for (size_t t = s + threadIdx.x; t < e; t += kThreads) acc.add_product(a[t], b[t]);
@@ -93,7 +93,7 @@ __device__ __forceinline__ double dot_chunk<float>(const float* __restrict__ a, 
 }
 
 template <typename R>
-__global__ void __launch_bounds__(kThreads) k_dot_partial(const R* __restrict__ a, const R* __restrict__ b, size_t n,
+__global__ void __launch_bounds__(kThreads) k_dot_partial(const R* a, const R* b, size_t n,
                                                            double* __restrict__ part) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(kThreads) k_dot_partial(const R* __restrict__ 
 }
 
 template <typename R>
-__global__ void __launch_bounds__(kThreads) k_maxabs_partial(const R* __restrict__ a, size_t n, double* __restrict__ part) {
+__global__ void __launch_bounds__(kThreads) k_maxabs_partial(const R* a, size_t n, double* __restrict__ part) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
   a += ready0;
@@ -132,8 +132,8 @@ __global__ void __launch_bounds__(kThreads) k_maxabs_partial(const R* __restrict
 
 // partial inner products of up to 8 basis vectors V[i] (leading dimension ldv) with w
 template <typename R>
-__global__ void __launch_bounds__(kThreads) k_multidot_partial(const R* __restrict__ V, size_t ldv, int m,
-                                                                const R* __restrict__ w, size_t n,
+__global__ void __launch_bounds__(kThreads) k_multidot_partial(const R* V, size_t ldv, int m,
+                                                                const R* w, size_t n,
                                                                 double* __restrict__ part) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kThreads) k_multidot_partial(const R* __restri
 
 // final pass: out[slot + blockIdx.x] = reduce(part[blockIdx.x * np .. + np])
 template <bool MAX>
-__global__ void __launch_bounds__(1024) k_finish(const double* __restrict__ part, int np, double* __restrict__ out) {
+__global__ void __launch_bounds__(1024) k_finish(const double* part, int np, double* __restrict__ out) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
   part += ready0;
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(1024) k_finish(const double* __restrict__ part
 
 // Vector updates run in the vectors' own precision (coefficients rounded to it once).
 // out[b] = sum of part[b * chunk .. min(np, (b + 1) * chunk)) in a fixed order
-__global__ void __launch_bounds__(1024) k_finish_chunks(const double* __restrict__ part, int np, int chunk,
+__global__ void __launch_bounds__(1024) k_finish_chunks(const double* part, int np, int chunk,
                                                          double* __restrict__ out) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
@@ -235,7 +235,7 @@ __global__ void k_lincomb(size_t n, int nvec, R c0, R c1, R c2, R c3, const R* x
 }
 
 template <typename R>
-__global__ void k_subtract_basis(const R* __restrict__ V, size_t ldv, int m, const double* __restrict__ h, R* w,
+__global__ void k_subtract_basis(const R* V, size_t ldv, int m, const double* h, R* w,
                                  size_t n) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
@@ -247,13 +247,13 @@ __global__ void k_subtract_basis(const R* __restrict__ V, size_t ldv, int m, con
   __syncthreads();
   for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
     R r = w[t];
-    for (int i = 0; i < m; ++i) r = fma(-hs[i], V[(size_t)i * ldv + t], r);
+    for (int i = 0; i < m; ++i) r = fma(-hs[i], load_global(V + (size_t)i * ldv + t), r);
     w[t] = r;
   }
 }
 
 template <typename S, typename D>
-__global__ void k_convert(size_t n, const S* __restrict__ src, D* __restrict__ dst) {
+__global__ void k_convert(size_t n, const S* src, D* __restrict__ dst) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
   src += ready0;

@@ -43,7 +43,7 @@ __device__ __forceinline__ double block_sum(double v) {
 // the factors across once per row, so that a face costs two FP64 operations; with a division and four products per
 // face the sum was bound by the FP64 pipe.  The other blocks: partial sums of the hot-wall flux over the ny * nz wall
 // cells.  (64^3, both diagnostics with their sums: four launches, 77 us of kernels; now two.)
-__global__ void __launch_bounds__(kThreads) k_diag_partial(Geo<double> g, const double* __restrict__ q, int be,
+__global__ void __launch_bounds__(kThreads) k_diag_partial(Geo<double> g, const double* q, int be,
                                                             double* __restrict__ part) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kThreads) k_diag_partial(Geo<double> g, const 
     const int lane = threadIdx.x & 31;
     for (int r = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); r < 3 * rows; r += be * (kThreads / 32)) {
       const int c = r / rows, jk = r - c * rows, k = jk / ny, j = jk - k * ny;
-      const double* __restrict__ f = q + (size_t)r * nx;
+      const double* f = q + (size_t)r * nx;
       const double* v = vol[c == 0 ? 0 : 1];
       double sum = 0.0;
       for (int x = lane; x < nx; x += 32) {
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kThreads) k_diag_partial(Geo<double> g, const 
 }
 
 // out[0] = sum of part[0 .. be), out[1] = sum of part[be .. be + bn), in a fixed order
-__global__ void __launch_bounds__(kThreads) k_diag_finish(const double* __restrict__ part, int be, int bn,
+__global__ void __launch_bounds__(kThreads) k_diag_finish(const double* part, int be, int bn,
                                                            double* __restrict__ out) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();

@@ -157,15 +157,15 @@ __device__ __forceinline__ void put_digits(unsigned char* dst, float y0, float y
 // Two neighbouring values: one vector load when `vec` (the pair is aligned), else two scalar ones; the second only
 // if `two`.
 template <typename R>
-__device__ __forceinline__ void load_two(const R* __restrict__ p, bool vec, bool two, R& a, R& b) {
+__device__ __forceinline__ void load_two(const R* p, bool vec, bool two, R& a, R& b) {
   if (vec) {
     using V2 = typename std::conditional<sizeof(R) == 8, double2, float2>::type;
-    const V2 v = __ldg(reinterpret_cast<const V2*>(p));
+    const V2 v = load_global(reinterpret_cast<const V2*>(p));
     a = v.x;
     b = v.y;
   } else {
-    a = __ldg(p);
-    b = two ? __ldg(p + 1) : R(0);
+    a = load_global(p);
+    b = two ? load_global(p + 1) : R(0);
   }
 }
 
@@ -224,7 +224,7 @@ struct DgUnit {
 // not read)
 template <typename R, bool BWD, int ITS>
 __global__ void __launch_bounds__(kDgThreads, 1)
-    k_digit_pass(const __grid_constant__ DgArgs<R> t, const R* __restrict__ in, R* __restrict__ out) {
+    k_digit_pass(const __grid_constant__ DgArgs<R> t, const R* in, R* __restrict__ out) {
   constexpr int kRowsT = 2 * kDgWarps * ITS;
   constexpr int D = Dg<R>::D, NC = Dg<R>::NC, ACC = Dg<R>::ACC, E_ = Dg<R>::E, kSlots = Dg<R>::kSlots;
   constexpr bool F64 = sizeof(R) == 8;
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
     // inputs of row pair `it` for the slab of an item; those of the next slab are requested as soon as this one's
     // are converted
     R x0[ITS], x1[ITS], y0[ITS], y1[ITS];
-    auto load_row = [&](int it, const R* __restrict__ src, int rows, int k, int k0, int S) {
+    auto load_row = [&](int it, const R* src, int rows, int k, int k0, int S) {
       const int row = 2 * (kDgWarps * it + cw) + rh;
       const bool two = k + 1 < h;
       x0[it] = x1[it] = y0[it] = y1[it] = R(0);
@@ -404,8 +404,8 @@ __global__ void __launch_bounds__(kDgThreads, 1)
           load_two<R>(p + S - k0 - k - 1, true, true, y1[it], y0[it]);
         } else {
           load_two<R>(p + k0 + k, false, two, x0[it], x1[it]);
-          y0[it] = __ldg(p + S - k0 - k);
-          y1[it] = two ? __ldg(p + S - k0 - k - 1) : R(0);
+          y0[it] = load_global(p + S - k0 - k);
+          y1[it] = two ? load_global(p + S - k0 - k - 1) : R(0);
         }
       }
     };
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
       if (item < total) {
         const int op = un.field & t.op_mask;
         const int k0 = t.k0[op], S = t.S[op];
-        const R* __restrict__ src = in + ((size_t)un.field * P + (size_t)un.tile * kRowsT) * n;
+        const R* src = in + ((size_t)un.field * P + (size_t)un.tile * kRowsT) * n;
         const int rows = min(kRowsT, P - un.tile * kRowsT);
         if (item == 0) {
 #pragma unroll
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
           unsigned m[kRows];
 #pragma unroll
           for (int r = 0; r < kRows; ++r) m[r] = 0;
-          const unsigned* __restrict__ w0 = reinterpret_cast<const unsigned*>(src) + (kStep - 1);
+          const unsigned* w0 = reinterpret_cast<const unsigned*>(src) + (kStep - 1);
 #pragma unroll 1
           for (int k = (BWD ? 0 : k0) + lane; k - lane < n; k += 128) {
             unsigned v[4][kRows];
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
 #pragma unroll
               for (int r = 0; r < kRows; ++r) {
                 const int row = min(2 * (kDgWarps * (r >> 1) + cw) + (r & 1), rows - 1);
-                v[q][r] = __ldg(w0 + ((size_t)row * n + min(k + 32 * q, n - 1)) * kStep);
+                v[q][r] = load_global(w0 + ((size_t)row * n + min(k + 32 * q, n - 1)) * kStep);
               }
 #pragma unroll
             for (int q = 0; q < 4; ++q)
@@ -472,11 +472,11 @@ __global__ void __launch_bounds__(kDgThreads, 1)
           }
           __syncwarp();
         }
-        const int* __restrict__ re = row_exp[tc & 3];
+        const int* re = row_exp[tc & 3];
         const int gi = 2 * item, s0 = gi % kSlots, s1 = (gi + 1) % kSlots;
         // the next item: this unit's next slab, or the first of the next unit
         if (j + 1 == t.nslab) nx.step(t);
-        const R* __restrict__ nsrc = in + ((size_t)nx.field * P + (size_t)nx.tile * kRowsT) * n;
+        const R* nsrc = in + ((size_t)nx.field * P + (size_t)nx.tile * kRowsT) * n;
         const int nrows = item + 1 < total ? min(kRowsT, P - nx.tile * kRowsT) : 0;
         const int nk = (j + 1 == t.nslab ? 0 : (j + 1) * 32) + kl;
         const int nk0 = t.k0[nx.field & t.op_mask], nS = t.S[nx.field & t.op_mask];

@@ -42,7 +42,7 @@ struct PassArgs {
 };
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_transform(PassArgs t, const R* __restrict__ in, const R* __restrict__ M,
+__global__ void __launch_bounds__(256) k_transform(PassArgs t, const R* in, const R* __restrict__ M,
                                                     R* __restrict__ out, const R* __restrict__ lx,
                                                     const R* __restrict__ ly, const R* __restrict__ lz) {
   using T = TileCfg<R>;
@@ -134,7 +134,7 @@ struct HalfArgs {
 };
 
 template <typename R, bool BWD, int U>
-__global__ void __launch_bounds__(128) k_half(const __grid_constant__ HalfArgs<R> t, const R* __restrict__ in,
+__global__ void __launch_bounds__(128) k_half(const __grid_constant__ HalfArgs<R> t, const R* in,
                                                R* __restrict__ out) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
@@ -149,8 +149,8 @@ __global__ void __launch_bounds__(128) k_half(const __grid_constant__ HalfArgs<R
   const int op = (int)blockIdx.z & t.op_mask;
   const int p0 = blockIdx.x * 32, j0 = blockIdx.y * UB;
   const int k0 = t.k0[op], S = t.S[op];
-  const R* __restrict__ Ms = t.M[0][op];
-  const R* __restrict__ Ma = t.M[1][op];
+  const R* Ms = t.M[0][op];
+  const R* Ma = t.M[1][op];
   in += (size_t)blockIdx.z * P * n;
   out += (size_t)blockIdx.z * P * n;
   R acc[2][U];

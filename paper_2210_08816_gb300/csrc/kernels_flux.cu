@@ -86,8 +86,8 @@ __global__ void __launch_bounds__(kFxThreads, 1)
   const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY, k0 = ((int)blockIdx.z - vec * t.nch) * t.zc;
   const int kend = min(k0 + t.zc, nz);
   const int pad = 1 + ((i0 - 1) & (A - 1)), xs = i0 - pad;  // the tile starts on a 16-byte boundary
-  const R* __restrict__ q = t.q;
-  const R* __restrict__ v = t.v + (size_t)vec * 4 * N;
+  const R* q = t.q;
+  const R* v = t.v + (size_t)vec * 4 * N;
   R* __restrict__ out = t.out + (size_t)vec * 4 * N;
   pdl_begin();
 

@@ -18,8 +18,8 @@ struct Cell {
 };
 
 template <typename R>
-__device__ __forceinline__ R ld(const R* __restrict__ a, int o) {
-  return __ldg(a + o);
+__device__ __forceinline__ R ld(const R* a, int o) {
+  return load_global(a + o);
 }
 
 template <typename R>
@@ -210,7 +210,7 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, int* err
 template <typename R>
 __global__ void __launch_bounds__(kTX * kTY, 3)
     k_stencil_z(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmv, int use_tma,
-                int* err, long long spins, Geo<R> g, int N, R Gr, R invPr, R sigma, const R* __restrict__ q, const R* __restrict__ v,
+                int* err, long long spins, Geo<R> g, int N, R Gr, R invPr, R sigma, const R* q, const R* v,
                 R* __restrict__ out, int zc, int nch, const TempOut t) {
   constexpr int NA = 8, AB = 4;
   constexpr int NWARP = kTX * kTY / 32;
@@ -357,7 +357,7 @@ __device__ __forceinline__ void warp_max_to(unsigned* slot, unsigned bits) {
   if ((threadIdx.x & 31) == 0) atomicMax(slot, m);
 }
 
-__global__ void __launch_bounds__(256) k_fieldmax(size_t n, const float* __restrict__ f, unsigned* slot) {
+__global__ void __launch_bounds__(256) k_fieldmax(size_t n, const float* f, unsigned* slot) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
   f += ready0;
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(256) k_fieldmax(size_t n, const float* __restr
 // rhs = D vel:  sum_d (vel_d(face p+1) - vel_d(face p)) / width, wall fluxes zero; slot (may be null): the largest
 // magnitude of rhs
 template <typename R>
-__global__ void __launch_bounds__(256) k_divergence(Geo<R> g, int N, const R* __restrict__ vel,
+__global__ void __launch_bounds__(256) k_divergence(Geo<R> g, int N, const R* vel,
                                                      R* __restrict__ rhs, unsigned* slot) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
@@ -402,7 +402,7 @@ __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_correct(Geo<R> g, int N, const R* Y, const R* __restrict__ phi,
+__global__ void __launch_bounds__(256) k_correct(Geo<R> g, int N, const R* Y, const R* phi,
                                                   R alpha, const R* v, R beta, const R* w, R gamma, R* out,
                                                   double* __restrict__ part, bool t_done) {
   pdl_begin();
@@ -436,8 +436,9 @@ __global__ void __launch_bounds__(256) k_correct(Geo<R> g, int N, const R* Y, co
         r = alpha * Y[o];
       }
       if (d < 3 || !t_done) {
-        if (v) r += beta * v[o];
-        if (w) r += gamma * w[o];
+        // (written out, so that every form of the loop rounds alike: with and without T, with and without v and w)
+        if (v) r = fma(beta, v[o], r);
+        if (w) r = fma(gamma, w[o], r);
         out[o] = r;
       }
       if (part) {
@@ -483,14 +484,14 @@ __global__ void __launch_bounds__(256) k_correct(Geo<R> g, int N, const R* Y, co
 // x-run of 128 cells).  Same arithmetic, element by element, as k_divergence / k_correct.
 constexpr int kVZ = 4;
 
-__device__ __forceinline__ float4 ldg4(const float* __restrict__ p, int o) {
-  return __ldg(reinterpret_cast<const float4*>(p + o));
+__device__ __forceinline__ float4 load4(const float* p, int o) {
+  return load_global(reinterpret_cast<const float4*>(p + o));
 }
 __device__ __forceinline__ float4 ld4(const float* p, int o) { return *reinterpret_cast<const float4*>(p + o); }
 __device__ __forceinline__ float4 zero4() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 
 // blockIdx.z = z-block + nzc * vector (states of 4N, rhs fields of N, one after another)
-__global__ void __launch_bounds__(256) k_divergence4(Geo<float> g, int N, const float* __restrict__ vel,
+__global__ void __launch_bounds__(256) k_divergence4(Geo<float> g, int N, const float* vel,
                                                       float* __restrict__ rhs, int nzc, unsigned* slot) {
   pdl_begin();
   const unsigned ready0 = pdl_wait();
@@ -515,20 +516,20 @@ __global__ void __launch_bounds__(256) k_divergence4(Geo<float> g, int N, const 
     ry = __ldg(g.idx[1] + j);
   }
   const int ob = act ? (k0 * ny + j) * nx + i0 : 0;
-  float4 wlo = (act && k0 >= 1) ? ldg4(W, ob) : zero4();
+  float4 wlo = (act && k0 >= 1) ? load4(W, ob) : zero4();
   unsigned top = 0;
 #pragma unroll
   for (int k = k0; k < k1; ++k) {
     const int o = ob + (k - k0) * pl;
-    const float4 u = act ? ldg4(U, o) : zero4();
+    const float4 u = act ? load4(U, o) : zero4();
     float un = __shfl_down_sync(0xffffffffu, u.x, 1);  // u on the face i0 + 4
-    if (lane == 31 && act && i0 + 4 < nx) un = __ldg(U + o + 4);
+    if (lane == 31 && act && i0 + 4 < nx) un = load_global(U + o + 4);
     if (i0 + 4 >= nx) un = 0.f;
     const float ux = (i0 == 0) ? 0.f : u.x;
     if (!act) continue;
-    const float4 vlo = (j >= 1) ? ldg4(V, o) : zero4();
-    const float4 vhi = (j + 1 < ny) ? ldg4(V, o + nx) : zero4();
-    const float4 whi = (k + 1 < nz) ? ldg4(W, o + pl) : zero4();
+    const float4 vlo = (j >= 1) ? load4(V, o) : zero4();
+    const float4 vhi = (j + 1 < ny) ? load4(V, o + nx) : zero4();
+    const float4 whi = (k + 1 < nz) ? load4(W, o + pl) : zero4();
     const float rz = __ldg(g.idx[2] + k);
     float4 r;
     r.x = (u.y - ux) * rx.x + (vhi.x - vlo.x) * ry + (whi.x - wlo.x) * rz;
@@ -553,7 +554,7 @@ __device__ __forceinline__ void acc_sq(float& hi, float& lo, float r) {
 // out = alpha (Y - G phi) + beta v + gamma w on four cells; out may alias Y or w (read, then written,
 // by the same thread)
 template <bool T_DONE>
-__global__ void __launch_bounds__(256) k_correct4(Geo<float> g, int N, const float* Y, const float* __restrict__ phi,
+__global__ void __launch_bounds__(256) k_correct4(Geo<float> g, int N, const float* Y, const float* phi,
                                                    float alpha, const float* v, float beta, const float* w,
                                                    float gamma, float* out, double* __restrict__ part, int nzc) {
   pdl_begin();
@@ -586,18 +587,18 @@ __global__ void __launch_bounds__(256) k_correct4(Geo<float> g, int N, const flo
     cy = __ldg(g.idc[1] + j);
   }
   const int ob = act ? (k0 * ny + j) * nx + i0 : 0;
-  float4 pzm = (act && k0 >= 1) ? ldg4(phi, ob - pl) : zero4();
+  float4 pzm = (act && k0 >= 1) ? load4(phi, ob - pl) : zero4();
   float shi = 0.f, slo = 0.f;
   for (int k = k0; k < k1; ++k) {
     const int o = ob + (k - k0) * pl;
-    const float4 ph = act ? ldg4(phi, o) : zero4();
+    const float4 ph = act ? load4(phi, o) : zero4();
     float pxm = __shfl_up_sync(0xffffffffu, ph.w, 1);  // phi in cell i0 - 1
-    if (lane == 0 && act && i0 > 0) pxm = __ldg(phi + o - 1);
+    if (lane == 0 && act && i0 > 0) pxm = load_global(phi + o - 1);
     if (!act) continue;
     float4 G[3];
     G[0] = make_float4((ph.x - pxm) * cx.x, (ph.y - ph.x) * cx.y, (ph.z - ph.y) * cx.z, (ph.w - ph.z) * cx.w);
     if (j >= 1) {
-      const float4 pym = ldg4(phi, o - nx);
+      const float4 pym = load4(phi, o - nx);
       G[1] = make_float4((ph.x - pym.x) * cy, (ph.y - pym.y) * cy, (ph.z - pym.z) * cy, (ph.w - pym.w) * cy);
     } else {
       G[1] = zero4();
@@ -621,11 +622,11 @@ __global__ void __launch_bounds__(256) k_correct4(Geo<float> g, int N, const flo
         r = make_float4(alpha * (y.x - gd.x), alpha * (y.y - gd.y), alpha * (y.z - gd.z), alpha * (y.w - gd.w));
         if (v) {
           const float4 a = ld4(v, od);
-          r.x += beta * a.x; r.y += beta * a.y; r.z += beta * a.z; r.w += beta * a.w;
+          r = make_float4(fmaf(beta, a.x, r.x), fmaf(beta, a.y, r.y), fmaf(beta, a.z, r.z), fmaf(beta, a.w, r.w));
         }
         if (w) {
           const float4 a = ld4(w, od);
-          r.x += gamma * a.x; r.y += gamma * a.y; r.z += gamma * a.z; r.w += gamma * a.w;
+          r = make_float4(fmaf(gamma, a.x, r.x), fmaf(gamma, a.y, r.y), fmaf(gamma, a.z, r.z), fmaf(gamma, a.w, r.w));
         }
         if (d == 0 && i0 == 0) r.x = 0.f;  // the x = 0 wall slot
       }

@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(tc_threads(CONV), 1)
     // converters: four threads to a row of every slab; those of one half of the warps take the first k-step of each
     // raw stage, the others the second, a thread inputs 8 hf .. 8 hf + 7 of it
     const int tt = threadIdx.x - 64, r = tt & 127, hf = (tt >> 7) & 1;
-    const unsigned* __restrict__ max_in = t.max_in + pdl_wait();
+    const unsigned* max_in = t.max_in + pdl_wait();
     int gi = 0;
     bool ok = true;
     for (int ti = 0; ti < my_tiles && ok; ++ti) {
@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(tc_threads(CONV), 1)
     // take alternate chunks of 16 outputs
     const int row = (warp % 4) * 32 + lane, half = (warp - 2 - CONV / 32) / 4;
     const unsigned ready0 = pdl_wait();
-    const unsigned* __restrict__ max_in = t.max_in + ready0;
+    const unsigned* max_in = t.max_in + ready0;
     if (blockIdx.x == 0)  // a slot that the kernel before this one has read
       for (int v = threadIdx.x - 64 - CONV; v * P < t.Ptot; v += 32 * kTcEpi) t.max_reset[8 * v] = 0;
     float top = 0.f;  // the largest output of field top_vec so far

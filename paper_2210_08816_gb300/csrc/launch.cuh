@@ -8,6 +8,10 @@
 // added to each pointer to such data: the addresses then depend on the wait.  (Passing the pointers themselves through
 // an asm statement loses their address space and __restrict__: 32^3 FP64 products 71 -> 101 us.)  Data written once at
 // grid creation (metrics, matrices) may be read before.
+//
+// What a predecessor wrote is read by ordinary loads: not by __ldg, nor through a kernel's `const __restrict__` pointer,
+// which the compiler may turn into the same.  The read-only path is defined for data that nobody writes while the kernel is
+// resident, and such a kernel is resident while its predecessor still writes.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -18,6 +22,41 @@ __device__ __forceinline__ unsigned pdl_wait() {
   unsigned zero;
   asm volatile("griddepcontrol.wait;\n mov.u32 %0, 0;" : "=r"(zero)::"memory");
   return zero;
+}
+
+// An ordinary load that the compiler may move past stores, as it could __ldg (the kernel does not write what it reads; the
+// address holds pdl_wait()'s zero).
+__device__ __forceinline__ float load_global(const float* p) {
+  float v;
+  asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ double load_global(const double* p) {
+  double v;
+  asm("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ unsigned load_global(const unsigned* p) {
+  unsigned v;
+  asm("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ float2 load_global(const float2* p) {
+  float2 v;
+  asm("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ double2 load_global(const double2* p) {
+  double2 v;
+  asm("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ float4 load_global(const float4* p) {
+  float4 v;
+  asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+      : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+      : "l"(__cvta_generic_to_global(p)));
+  return v;
 }
 
 template <typename T>

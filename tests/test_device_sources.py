@@ -68,3 +68,22 @@ def test_kernel_attributes_are_set_for_every_grid():
     for f in setups - {"digit_setup"}:
         assert re.search(rf"\b{f}\b", create), f
     assert "upload_digits" in create and "digit_setup()" in _source("fv_api.cpp")
+
+
+def test_overlapping_kernels_read_their_predecessors_results_by_ordinary_loads():
+    """A kernel that overlaps its predecessor is resident while that one still writes; the read-only load path (__ldg, or a
+    kernel's const __restrict__ pointer) is defined for data that nobody writes meanwhile.  Grid data, written once at
+    creation, may take it: metrics (g.*), matrices (M, t.M) and eigenvalues (lx, ly, lz)."""
+    seen = 0
+    for name in sorted(os.listdir(CSRC)):
+        if not name.endswith(".cu"):
+            continue
+        src = _source(name)
+        if "pdl_wait()" not in src:
+            continue
+        seen += 1
+        for m in re.finditer(r"__ldg\(\s*([\w.]+)", src):
+            assert re.match(r"(g\.|t\.M)", m.group(1)), f"{name}: __ldg({m.group(1)}"
+        for m in re.finditer(r"const \w+\* __restrict__ (\w+)", src):
+            assert m.group(1) in {"M", "lx", "ly", "lz"}, f"{name}: const __restrict__ {m.group(1)}"
+    assert seen >= 8
