@@ -22,6 +22,19 @@ int invalid(const std::string& msg) {
 
 }  // namespace
 
+int stencil_chunk(int nz, int sms, int tiles, int nvec) {
+  int best = nz;
+  long long best_cost = -1;
+  each_chunk(nz, [&](int zc, int n) {
+    const long long ctas = (long long)tiles * n * nvec;
+    if (ctas > 1LL << 20 || (long long)n * nvec > 65535) return false;
+    const long long cost = (ctas + sms - 1) / sms * (zc + 1);
+    if (best_cost < 0 || cost < best_cost) best = zc, best_cost = cost;
+    return true;
+  });
+  return best;
+}
+
 double width_ratio(const std::vector<double>& xf) {
   double least = 1.0, most = 0.0;
   for (size_t i = 0; i + 1 < xf.size(); ++i) {

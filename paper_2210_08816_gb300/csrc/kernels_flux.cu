@@ -366,10 +366,8 @@ static FluxPlan flux_plan(const fv_grid_s* g, int nvec) {
       if ((4 * pl * sizeof(double)) % 128 != 0) continue;  // a state's box of a TMA plane keeps the next one aligned
       const long long tiles = (long long)((g->nx + tx - 1) / tx) * ((g->ny + ty - 1) / ty) * nvec;
       const int warps = (tx * ty + 31) / 32;
-      for (int nch = 1; nch <= g->nz; ++nch) {
-        const int zc = (g->nz + nch - 1) / nch, n = (g->nz + zc - 1) / zc;
-        if (n != nch) continue;
-        if ((long long)n * nvec > 65535) break;
+      each_chunk(g->nz, [&](int zc, int n) {
+        if ((long long)n * nvec > 65535) return false;
         const int w = tiles * n <= g->sms ? (warps + 3) / 4 * 4 : warps;
         const double per = 400.0 + zc * (104.0 * w + 80.0) + 45.0 * w;
         const double c = per * (double)((tiles * n + g->sms - 1) / g->sms);
@@ -377,7 +375,8 @@ static FluxPlan flux_plan(const fv_grid_s* g, int nvec) {
           cost = c;
           best = FluxPlan{nvec, tx, ty, zc};
         }
-      }
+        return true;
+      });
     }
   }
   return best;

@@ -682,20 +682,6 @@ inline void cell_grid(const fv_grid_s* g, dim3& grid, dim3& block) {
 
 }  // namespace
 
-int stencil_chunk(const fv_grid_s* g, int tiles, int nvec) {
-  int best = 1;
-  long long best_cost = -1;
-  for (int nch = 1; nch <= g->nz; ++nch) {
-    const int zc = (g->nz + nch - 1) / nch;
-    const long long ctas = (long long)tiles * ((g->nz + zc - 1) / zc) * nvec;
-    if (ctas > 1LL << 20 || (long long)((g->nz + zc - 1) / zc) * nvec > 65535) break;
-    const long long cost = ((ctas + g->sms - 1) / g->sms) * (zc + 1);
-    if (best_cost < 0 || cost < best_cost) best = zc, best_cost = cost;
-  }
-  if (best_cost < 0) best = g->nz;
-  return best;
-}
-
 // 4D tensor map of one state (x, y, z, field) with boxes of kPW x kHY x 1 x 4 elements
 template <typename R>
 int state_map(const fv_grid_s* g, const R* ptr, CUtensorMap* m, int nvec = 1) {
@@ -729,7 +715,7 @@ int launch_stencil_z(const fv_grid_s* g, double Gr, double sigma, const R* q, co
                  ((uintptr_t)v % 16) == 0) ? 1 : 0;
   if (use_tma && (state_map<R>(g, q, &tq) != FV_OK || state_map<R>(g, v, &tv, nvec) != FV_OK)) use_tma = 0;
   const int gx = (g->nx + kTX - 1) / kTX, gy = (g->ny + kTY - 1) / kTY;
-  const int zc = stencil_chunk(g, gx * gy, nvec), nch = (g->nz + zc - 1) / zc;
+  const int zc = stencil_chunk(g->nz, g->sms, gx * gy, nvec), nch = (g->nz + zc - 1) / zc;
   if (nvec < 1 || (long long)nch * nvec > 65535) {
     set_error("launch_stencil_z: too many vectors in one block");
     return FV_EINVAL;

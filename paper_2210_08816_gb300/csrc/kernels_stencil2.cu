@@ -469,7 +469,7 @@ int launch_stencil_pair(const fv_grid_s* g, double Gr, double sigma, const float
   const size_t smem = kPairSmem;
   // blocks of vectors march the z-chunk the autotuner picked, if it ran; otherwise stencil_chunk's
   const int zc = (nvec > 1 && g->tune.pair_zc > 0) ? g->tune.pair_zc
-                                                   : stencil_chunk(g, g->nx / kPX * ((g->ny + kPY - 1) / kPY), nvec);
+                                                   : stencil_chunk(g->nz, g->sms, g->nx / kPX * ((g->ny + kPY - 1) / kPY), nvec);
   const int nch = (g->nz + zc - 1) / zc;
   if (nvec < 1 || (long long)nch * nvec > 65535) {
     set_error("launch_stencil_pair: too many vectors in one block for this z-chunk");
