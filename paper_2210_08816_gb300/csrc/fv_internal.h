@@ -159,12 +159,18 @@ inline void each_chunk(int nz, F f) {
   }
 }
 
-// Planes marched by one CTA of an FP32 z-marching stencil over `tiles` (x, y) tiles of nvec states: the chunk with
-// the smallest makespan of the busiest multiprocessor, ceil(CTAs / SMs) CTAs of chunk + 1 plane times each (the
-// extra one stands for a CTA's two halo planes and its pipeline fill).  The stencils are bound by issue slots and
-// shared-memory loads, so what counts is how evenly the planes spread over the SMs.  Fixed chunks of 32 planes gave a
-// 64^3 grid 16 CTAs (39.5 us; with this rule 10.7) and a 100^3 grid 208 (41 -> 33 us); 16 vectors of 64^3 66 -> 61.
-int stencil_chunk(int nz, int sms, int tiles, int nvec);
+// Planes marched by one CTA of an FP32 z-marching stencil over `tiles` (x, y) tiles of nvec states: the chunk with the
+// smallest makespan of the busiest multiprocessor.  Its ceil(CTAs / SMs) CTAs run `most` at a time (what fits beside one
+// another), and a plane takes plane[k - 1] with k of them there: more at a time hide each other's latencies, so that one
+// CTA per SM is the worst split of large grids (192^3, 144 CTAs of 96 planes 111 us, 288 of 48 92.5).  The plane added to
+// every chunk stands for its start.  The times are those of the kernel's launch table, fitted to 29 grids and blocks with
+// every cut of each: within 2.4 % of the best cut everywhere, 0.4 % on average.  (Counting planes alone, a 96^3 block of two
+// took 50 us in 144 CTAs instead of 39 in 432, and fixed chunks of 32 planes gave a 64^3 grid 16 CTAs, 39.5 us against 10.6.)
+struct PlaneTimes {
+  int most;      // CTAs that fit on an SM
+  int plane[3];  // time of a plane with 1, 2, 3 of them there, in tenths of the first
+};
+int stencil_chunk(int nz, int sms, int tiles, int nvec, const PlaneTimes& t);
 
 // ------------------------------------------------------------------ error reporting
 void set_error(const std::string& msg);

@@ -22,13 +22,14 @@ int invalid(const std::string& msg) {
 
 }  // namespace
 
-int stencil_chunk(int nz, int sms, int tiles, int nvec) {
+int stencil_chunk(int nz, int sms, int tiles, int nvec, const PlaneTimes& t) {
   int best = nz;
   long long best_cost = -1;
   each_chunk(nz, [&](int zc, int n) {
     const long long ctas = (long long)tiles * n * nvec;
     if (ctas > 1LL << 20 || (long long)n * nvec > 65535) return false;
-    const long long cost = (ctas + sms - 1) / sms * (zc + 1);
+    const long long per = (ctas + sms - 1) / sms, rest = per % t.most;
+    const long long cost = (per / t.most * t.plane[t.most - 1] + (rest ? t.plane[rest - 1] : 0)) * (zc + 1);
     if (best_cost < 0 || cost < best_cost) best = zc, best_cost = cost;
     return true;
   });

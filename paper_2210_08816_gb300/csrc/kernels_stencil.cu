@@ -693,13 +693,15 @@ int state_map(const fv_grid_s* g, const R* ptr, CUtensorMap* m, int nvec = 1) {
                            ptr, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
+constexpr PlaneTimes kStencilTimes = {3, {10, 14, 20}};
+
 template <typename R>
 constexpr size_t stencil_smem() {
   return (size_t)8 * kRing * kPL * sizeof(R);
 }
 
 int stencil_setup() {
-  FV_CUDA(cudaFuncSetAttribute(k_stencil_z<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stencil_smem<float>()));
+  FV_CUDA(cudaFuncSetAttribute(k_stencil_z<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadSmem));
   return FV_OK;
 }
 
@@ -715,14 +717,14 @@ int launch_stencil_z(const fv_grid_s* g, double Gr, double sigma, const R* q, co
                  ((uintptr_t)v % 16) == 0) ? 1 : 0;
   if (use_tma && (state_map<R>(g, q, &tq) != FV_OK || state_map<R>(g, v, &tv, nvec) != FV_OK)) use_tma = 0;
   const int gx = (g->nx + kTX - 1) / kTX, gy = (g->ny + kTY - 1) / kTY;
-  const int zc = stencil_chunk(g->nz, g->sms, gx * gy, nvec), nch = (g->nz + zc - 1) / zc;
+  const int zc = stencil_chunk(g->nz, g->sms, gx * gy, nvec, kStencilTimes), nch = (g->nz + zc - 1) / zc;
   if (nvec < 1 || (long long)nch * nvec > 65535) {
     set_error("launch_stencil_z: too many vectors in one block");
     return FV_EINVAL;
   }
   dim3 grid(gx, gy, nch * nvec);
   ProfScope ps(g, PROF_STENCIL);
-  launch(k_stencil_z<R>, grid, kTX * kTY, smem, g->stream, tq, tv, use_tma, g->ws.err, wait_spins(g), geo_of<R>(g), (int)g->N,
+  launch(k_stencil_z<R>, grid, kTX * kTY, spread_smem(smem, (long long)gx * gy * nch * nvec, g->sms, kStencilTimes.most), g->stream, tq, tv, use_tma, g->ws.err, wait_spins(g), geo_of<R>(g), (int)g->N,
                                                              (R)Gr, (R)(1.0 / g->Pr), (R)sigma, q, v, out, zc, nch, t);
   FV_CUDA(cudaGetLastError());
   return FV_OK;

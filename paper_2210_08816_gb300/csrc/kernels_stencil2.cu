@@ -22,6 +22,7 @@ constexpr int kPW2 = 72;            // ring row: x from i0 - 4 to i0 + 67 (TMA x
 constexpr int kPX0 = 4;             // column of the tile's first cell
 constexpr int kPL2 = kPHY * kPW2;   // one array's plane tile
 constexpr int kPRing = 4, kPNA = 8;
+constexpr PlaneTimes kPairTimes = {2, {10, 16, 0}};
 constexpr size_t kPairSmem = (size_t)kPRing * kPNA * kPL2 * sizeof(float);
 constexpr long long kPWaitLimit = 1LL << 22;
 
@@ -460,16 +461,15 @@ bool stencil_pair_eligible(const fv_grid_s* g, const float* q, const float* v) {
 
 int stencil_pair_setup() {
   for (auto k : {k_stencil_pair<false>, k_stencil_pair<true>})
-    FV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem));
+    FV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadSmem));
   return FV_OK;
 }
 
 int launch_stencil_pair(const fv_grid_s* g, double Gr, double sigma, const float* q, const float* v, float* out,
                         int nvec, const TempOut& t) {
-  const size_t smem = kPairSmem;
   // blocks of vectors march the z-chunk the autotuner picked, if it ran; otherwise stencil_chunk's
   const int zc = (nvec > 1 && g->tune.pair_zc > 0) ? g->tune.pair_zc
-                                                   : stencil_chunk(g->nz, g->sms, g->nx / kPX * ((g->ny + kPY - 1) / kPY), nvec);
+                                                   : stencil_chunk(g->nz, g->sms, g->nx / kPX * ((g->ny + kPY - 1) / kPY), nvec, kPairTimes);
   const int nch = (g->nz + zc - 1) / zc;
   if (nvec < 1 || (long long)nch * nvec > 65535) {
     set_error("launch_stencil_pair: too many vectors in one block for this z-chunk");
@@ -481,6 +481,7 @@ int launch_stencil_pair(const fv_grid_s* g, double Gr, double sigma, const float
   FV_TRY(pair_map(g, q, &tq));
   FV_TRY(pair_map(g, v, &tv, nvec));
   dim3 grid(g->nx / kPX, (g->ny + kPY - 1) / kPY, nch * nvec);
+  const size_t smem = spread_smem(kPairSmem, (long long)grid.x * grid.y * grid.z, g->sms, kPairTimes.most);
   ProfScope ps(g, PROF_STENCIL);
   if (nvec > 1)
     launch(k_stencil_pair<true>, grid, kPX / 2 * kPY, smem, g->stream, tq, tv, g->ws.err, wait_spins(g), g->geo32, (int)g->N, (float)Gr,

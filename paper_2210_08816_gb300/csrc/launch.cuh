@@ -103,6 +103,17 @@ inline void launch_cluster(int C, void (*kernel)(P...), dim3 grid, dim3 block, s
   c.numAttrs = 2;
   cudaLaunchKernelEx(&c, kernel, args...);
 }
+// Dynamic shared memory of a launch of `blocks` blocks, `most` of which (by registers and the `smem` they need) fit on a
+// multiprocessor: padded so that no more of them fit there than an even spread puts there.  Blocks placed early, beside the
+// predecessor's last ones, would pile up on the multiprocessors that are free first (see launch_spread): 33 products of
+// 32^3 FP32, 132 stencil blocks, took 164 us and 128 so.  kSpreadSmem: what the kernel's limit has to allow.
+constexpr size_t kSpreadSmem = 221 * 1024;
+inline size_t spread_smem(size_t smem, long long blocks, int sms, int most) {
+  const long long per = (blocks + sms - 1) / sms;
+  if (per >= most) return smem;
+  const size_t pad = (size_t)(222 * 1024 / per - 1024);
+  return pad > smem ? pad : smem;
+}
 // Without the overlap, for kernels bound by the FP64 pipe (two operations per clock and SM): blocks placed while the
 // predecessor still occupies most SMs pile up on the others, and the busiest SM sets the time (32^3 FP64 J.v +
 // projection 101 us with the overlap, 71 without).  A kernel whose registers or shared memory let one block on an SM

@@ -13,7 +13,10 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 WRAP = r"""
 #include "fv_internal.h"
 namespace fv { void set_error(const std::string&) {} }
-extern "C" int chunk(int nz, int sms, int tiles, int nvec) { return fv::stencil_chunk(nz, sms, tiles, nvec); }
+static const fv::PlaneTimes kTimes[2] = {{2, {10, 16, 0}}, {3, {10, 14, 20}}};
+extern "C" int chunk(int nz, int sms, int tiles, int nvec, int form) {
+  return fv::stencil_chunk(nz, sms, tiles, nvec, kTimes[form]);
+}
 extern "C" int chunks(int nz, int* zc, int* n) {
   int k = 0;
   fv::each_chunk(nz, [&](int z, int c) { zc[k] = z; n[k++] = c; return true; });
@@ -21,7 +24,7 @@ extern "C" int chunks(int nz, int* zc, int* n) {
 }
 extern "C" long long many(int nz, int sms, int tiles, int nvec, int times) {
   long long s = 0;
-  for (int i = 0; i < times; ++i) s += fv::stencil_chunk(nz, sms, tiles + (i & 1), nvec);
+  for (int i = 0; i < times; ++i) s += fv::stencil_chunk(nz, sms, tiles + (i & 1), nvec, kTimes[i & 1]);
   return s;
 }
 """
@@ -53,14 +56,18 @@ def test_every_distinct_cut_once(L):
         assert k <= 2 * np.sqrt(nz) + 1
 
 
-def _tried(nz, sms, tiles, nvec):
+TIMES = [(10, 16), (10, 14, 20)]
+
+
+def _tried(nz, sms, tiles, nvec, t):
     best, cost = nz, None
     for c in range(1, nz + 1):
         zc = -(-nz // c)
         n = -(-nz // zc)
         if tiles * n * nvec > 1 << 20 or n * nvec > 65535:
             break
-        now = -(-(tiles * n * nvec) // sms) * (zc + 1)
+        waves, rest = divmod(-(-(tiles * n * nvec) // sms), len(t))
+        now = (waves * t[-1] + (t[rest - 1] if rest else 0)) * (zc + 1)
         if cost is None or now < cost:
             best, cost = zc, now
     return best
@@ -71,7 +78,17 @@ def test_the_choice_is_that_of_trying_all(L):
     cases = [(nz, t, v) for nz in (1, 2, 5, 16, 64, 100, 256, 812) for t in (1, 4, 16, 128, 700) for v in (1, 2, 16, 333)]
     cases += [tuple(int(x) for x in np.exp(rng.uniform(0, np.log([812, 2000, 70000])))) for _ in range(300)]
     for nz, tiles, nvec in cases:
-        assert L.chunk(nz, 152, tiles, nvec) == _tried(nz, 152, tiles, nvec), (nz, tiles, nvec)
+        for form, t in enumerate(TIMES):
+            assert L.chunk(nz, 152, tiles, nvec, form) == _tried(nz, 152, tiles, nvec, t), (nz, tiles, nvec)
+
+
+# the fastest cuts as timed on 152 multiprocessors, and what was chosen when planes alone counted
+@pytest.mark.parametrize("form,nz,tiles,nvec,good,bad", [
+    (0, 192, 72, 1, (48, 24), 96), (0, 64, 8, 6, (11,), 22), (0, 32, 16, 8, (7, 16), 32),
+    (1, 96, 36, 2, (16, 9, 8), 48), (1, 32, 4, 33, (16, 4), 32), (1, 256, 4, 3, (7, 11), 22)])
+def test_large_grids_are_not_left_with_one_block_per_multiprocessor(L, form, nz, tiles, nvec, good, bad):
+    zc = L.chunk(nz, 152, tiles, nvec, form)
+    assert zc in good and zc != bad
 
 
 def test_the_time_does_not_go_by_the_planes(L):
