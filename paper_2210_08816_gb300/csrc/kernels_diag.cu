@@ -40,9 +40,10 @@ __device__ __forceinline__ double block_sum(double v) {
 
 // Blocks 0 .. be - 1: partial sums of u_f^2 V_f / 2 over the x-rows of the three velocity fields, a warp per row.  The
 // two x-factors of the control volumes (centre spacings and widths: one over the metrics) are formed once per block,
-// the factors across once per row, so that a face costs two FP64 operations; with a division and four products per
-// face the sum was bound by the FP64 pipe.  The other blocks: partial sums of the hot-wall flux over the ny * nz wall
-// cells.  (64^3, both diagnostics with their sums: four launches, 77 us of kernels; now two.)
+// the factors across once per row, a lane each for 32 of a warp's rows, so that a face costs two FP64 operations; with
+// a division and four products per face the sum was bound by the FP64 pipe, and with a division by the whole warp for every
+// row on grids of short rows (16 x 16 x 800: 72 us, now 25; 2 x 300 x 300 420, now 72).  The other blocks: partial sums of the hot-wall
+// flux over the ny * nz wall cells.  (64^3, both diagnostics with their sums: four launches, 70 us of kernels; now two, 18.)
 __global__ void __launch_bounds__(kThreads) k_diag_partial(Geo<double> g, const double* q, int be,
                                                             double* __restrict__ part) {
   pdl_begin();
@@ -58,17 +59,24 @@ __global__ void __launch_bounds__(kThreads) k_diag_partial(Geo<double> g, const 
       vol[1][x] = 1.0 / g.idx[0][x];
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    for (int r = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); r < 3 * rows; r += be * (kThreads / 32)) {
-      const int c = r / rows, jk = r - c * rows, k = jk / ny, j = jk - k * ny;
-      const double* f = q + (size_t)r * nx;
-      const double* v = vol[c == 0 ? 0 : 1];
-      double sum = 0.0;
-      for (int x = lane; x < nx; x += 32) {
-        const double u = f[x];
-        sum = fma(u * u, v[x], sum);
+    const int lane = threadIdx.x & 31, step = be * (kThreads / 32);
+    for (int r0 = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); r0 < 3 * rows; r0 += 32 * step) {
+      double across = 0.0;  // lane i: the factor across of the warp's i-th row from r0 on
+      const int mine = r0 + lane * step;
+      if (mine < 3 * rows) {
+        const int c = mine / rows, jk = mine - c * rows, k = jk / ny, j = jk - k * ny;
+        across = 0.5 / ((c == 1 ? g.idc[1][j] : g.idx[1][j]) * (c == 2 ? g.idc[2][k] : g.idx[2][k]));
       }
-      acc += 0.5 * sum / ((c == 1 ? g.idc[1][j] : g.idx[1][j]) * (c == 2 ? g.idc[2][k] : g.idx[2][k]));
+      for (int i = 0, r = r0; i < 32 && r < 3 * rows; ++i, r += step) {
+        const double* f = q + (size_t)r * nx;
+        const double* v = vol[r < rows ? 0 : 1];
+        double sum = 0.0;
+        for (int x = lane; x < nx; x += 32) {
+          const double u = f[x];
+          sum = fma(u * u, v[x], sum);
+        }
+        acc = fma(sum, __shfl_sync(0xffffffffu, across, i), acc);
+      }
     }
   } else {
     const double* T = q + 3 * (size_t)rows * nx;
