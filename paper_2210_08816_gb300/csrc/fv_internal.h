@@ -163,8 +163,8 @@ inline void each_chunk(int nz, F f) {
 // smallest makespan of the busiest multiprocessor.  Its ceil(CTAs / SMs) CTAs run `most` at a time (what fits beside one
 // another), and a plane takes plane[k - 1] with k of them there: more at a time hide each other's latencies, so that one
 // CTA per SM is the worst split of large grids (192^3, 144 CTAs of 96 planes 111 us, 288 of 48 92.5).  The plane added to
-// every chunk stands for its start.  The times are those of the kernel's launch table, fitted to 29 grids and blocks with
-// every cut of each: within 2.4 % of the best cut everywhere, 0.4 % on average.  (Counting planes alone, a 96^3 block of two
+// every chunk stands for its start.  The times are those of the kernel's launch table, fitted to 54 grids and blocks with
+// every cut of each: products within 3 % of the best cut's, 0.5 % on average.  (Counting planes alone, a 96^3 block of two
 // took 50 us in 144 CTAs instead of 39 in 432, and fixed chunks of 32 planes gave a 64^3 grid 16 CTAs, 39.5 us against 10.6.)
 struct PlaneTimes {
   int most;      // CTAs that fit on an SM

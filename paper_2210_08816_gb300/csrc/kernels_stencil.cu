@@ -693,7 +693,7 @@ int state_map(const fv_grid_s* g, const R* ptr, CUtensorMap* m, int nvec = 1) {
                            ptr, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
-constexpr PlaneTimes kStencilTimes = {3, {10, 14, 20}};
+constexpr PlaneTimes kStencilTimes = {3, {10, 16, 23}};
 
 template <typename R>
 constexpr size_t stencil_smem() {

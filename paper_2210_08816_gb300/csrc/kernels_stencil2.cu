@@ -22,7 +22,7 @@ constexpr int kPW2 = 72;            // ring row: x from i0 - 4 to i0 + 67 (TMA x
 constexpr int kPX0 = 4;             // column of the tile's first cell
 constexpr int kPL2 = kPHY * kPW2;   // one array's plane tile
 constexpr int kPRing = 4, kPNA = 8;
-constexpr PlaneTimes kPairTimes = {2, {10, 16, 0}};
+constexpr PlaneTimes kPairTimes = {2, {10, 17, 0}};
 constexpr size_t kPairSmem = (size_t)kPRing * kPNA * kPL2 * sizeof(float);
 constexpr long long kPWaitLimit = 1LL << 22;
 

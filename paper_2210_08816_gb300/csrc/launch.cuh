@@ -106,12 +106,14 @@ inline void launch_cluster(int C, void (*kernel)(P...), dim3 grid, dim3 block, s
 // Dynamic shared memory of a launch of `blocks` blocks, `most` of which (by registers and the `smem` they need) fit on a
 // multiprocessor: padded so that no more of them fit there than an even spread puts there.  Blocks placed early, beside the
 // predecessor's last ones, would pile up on the multiprocessors that are free first (see launch_spread): 33 products of
-// 32^3 FP32, 132 stencil blocks, took 164 us and 128 so.  kSpreadSmem: what the kernel's limit has to allow.
-constexpr size_t kSpreadSmem = 221 * 1024;
+// 32^3 FP32, 132 stencil blocks, took 164 us and 128 so.  No more than that takes, since a launch waits for what it asks
+// for (8^3, a block of eight: 41.4 us with all of an SM's memory for one block, 38.9 with half).  kSpreadSmem: what the
+// kernel's limit has to allow.
+constexpr size_t kSpreadSmem = 115 * 1024;
 inline size_t spread_smem(size_t smem, long long blocks, int sms, int most) {
   const long long per = (blocks + sms - 1) / sms;
   if (per >= most) return smem;
-  const size_t pad = (size_t)(222 * 1024 / per - 1024);
+  const size_t pad = (size_t)(228 * 1024 / (per + 1) + 1024);  // one block more does not fit
   return pad > smem ? pad : smem;
 }
 // Without the overlap, for kernels bound by the FP64 pipe (two operations per clock and SM): blocks placed while the

@@ -13,7 +13,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 WRAP = r"""
 #include "fv_internal.h"
 namespace fv { void set_error(const std::string&) {} }
-static const fv::PlaneTimes kTimes[2] = {{2, {10, 16, 0}}, {3, {10, 14, 20}}};
+static const fv::PlaneTimes kTimes[2] = {{2, {10, 17, 0}}, {3, {10, 16, 23}}};
 extern "C" int chunk(int nz, int sms, int tiles, int nvec, int form) {
   return fv::stencil_chunk(nz, sms, tiles, nvec, kTimes[form]);
 }
@@ -56,7 +56,7 @@ def test_every_distinct_cut_once(L):
         assert k <= 2 * np.sqrt(nz) + 1
 
 
-TIMES = [(10, 16), (10, 14, 20)]
+TIMES = [(10, 17), (10, 16, 23)]
 
 
 def _tried(nz, sms, tiles, nvec, t):
