@@ -258,15 +258,18 @@ bool digit_wins(int n, long long rows) {
   return (double)rows * n * ((n + 1) / 2) >= (sizeof(R) == 8 ? 3.2e6 : 1.6e7);
 }
 
-// Unused shared memory that leaves room for `per` blocks of the FP64 form on an SM.
+// Unused shared memory that leaves room for `per` blocks on an SM, all of it or (FP32, whose launches are short) no more than
+// that takes.
+template <typename R>
 constexpr int half_pad(int U, int per) {
-  return 222 * 1024 / per - (int)(sizeof(double) * (2 * kHalfK * 33 + 2 * 4 * U * kHalfK)) - 1024;
+  return (sizeof(R) == 8 ? 222 * 1024 / per : 228 * 1024 / (per + 1) + 1024) -
+         (int)(sizeof(R) * (2 * kHalfK * 33 + 2 * 4 * U * kHalfK)) - (sizeof(R) == 8 ? 1024 : 0);
 }
 
-template <int U>
+template <typename R, int U>
 int half_setup_u() {
-  for (auto k : {k_half<double, false, U>, k_half<double, true, U>})
-    FV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, half_pad(U, 1)));
+  for (auto k : {k_half<R, false, U>, k_half<R, true, U>})
+    FV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, half_pad<R>(U, 1)));
   return FV_OK;
 }
 
@@ -305,18 +308,15 @@ int half_pass(const fv_grid_s* g, int axis, bool bwd, int na, int nb, const int 
     k = U == 4 ? k_half<R, true, 4> : U == 2 ? k_half<R, true, 2> : k_half<R, true, 1>;
   else
     k = U == 4 ? k_half<R, false, 4> : U == 2 ? k_half<R, false, 2> : k_half<R, false, 1>;
-  if constexpr (sizeof(R) == 8) {
-    // one block per SM, or two, ...: unused shared memory keeps more from being placed there, so that the launch can
-    // overlap its predecessor and still spread evenly (32^3 FP64 J.v + projection 73 us without the overlap, 58.5 so)
-    const long long per = ((long long)grid.x * grid.y * grid.z + g->sms - 1) / g->sms;
-    if (per <= 6) {
-      launch(k, grid, 128, half_pad(U, (int)per), g->stream, t, in, out);
-    } else {
-      launch_spread(k, grid, 128, 0, g->stream, t, in, out);
-    }
-  } else {
-    launch(k, grid, 128, 0, g->stream, t, in, out);
-  }
+  // One block per SM, or two, ...: unused shared memory keeps more from being placed there, so that the launch can overlap
+  // its predecessor and still spread evenly: 32^3 FP64 J.v + projection 73 us without the overlap, 58.5 so; FP32 projection of
+  // 800 x 16 x 16 113 us with the overlap alone, 90 so, 60^3 41.3 and 36.5.  From seven blocks per SM on FP64 passes go
+  // without the overlap and FP32 ones, whose blocks leave each other room, without the padding.
+  const long long per = ((long long)grid.x * grid.y * grid.z + g->sms - 1) / g->sms;
+  if (per <= 6)
+    launch(k, grid, 128, half_pad<R>(U, (int)per), g->stream, t, in, out);
+  else
+    launch(sizeof(R) == 4, k, grid, 128, 0, g->stream, t, in, out);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }
@@ -399,9 +399,12 @@ const FdmDev<float>& fd_of<float>(const fv_grid_s* g) { return g->fd32; }
 }  // namespace
 
 int half_setup() {
-  FV_TRY(half_setup_u<1>());
-  FV_TRY(half_setup_u<2>());
-  return half_setup_u<4>();
+  FV_TRY((half_setup_u<double, 1>()));
+  FV_TRY((half_setup_u<double, 2>()));
+  FV_TRY((half_setup_u<double, 4>()));
+  FV_TRY((half_setup_u<float, 1>()));
+  FV_TRY((half_setup_u<float, 2>()));
+  return half_setup_u<float, 4>();
 }
 
 template <typename R>
