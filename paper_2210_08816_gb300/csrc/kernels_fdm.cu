@@ -41,8 +41,9 @@ struct PassArgs {
   double shift;          // scaled pass: sfac / (lam_z + lam_y + lam_x - shift)
 };
 
+// (launched without the overlap, so that its input is complete before it starts: the read-only path is open to it)
 template <typename R>
-__global__ void __launch_bounds__(256) k_transform(PassArgs t, const R* in, const R* __restrict__ M,
+__global__ void __launch_bounds__(256) k_transform(PassArgs t, const R* __restrict__ in, const R* __restrict__ M,
                                                     R* __restrict__ out, const R* __restrict__ lx,
                                                     const R* __restrict__ ly, const R* __restrict__ lz) {
   using T = TileCfg<R>;
