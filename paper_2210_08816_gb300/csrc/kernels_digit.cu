@@ -154,18 +154,28 @@ __device__ __forceinline__ void put_digits(unsigned char* dst, float y0, float y
   *reinterpret_cast<uint32_t*>(dst + kDgDigitBytes) = *reinterpret_cast<const uint32_t*>(&l);
 }
 
+// Inputs: FP32 passes by plain expressions, FP64 ones by loads that may pass stores (256^3 FP32 diffusion solve 1642 and
+// 1666 us, 100^3 FP64 513 and 507).
+template <typename R, typename T>
+__device__ __forceinline__ T load_in(const T* p) {
+  if constexpr (sizeof(R) == 8)
+    return load_global(p);
+  else
+    return *p;
+}
+
 // Two neighbouring values: one vector load when `vec` (the pair is aligned), else two scalar ones; the second only
 // if `two`.
 template <typename R>
 __device__ __forceinline__ void load_two(const R* p, bool vec, bool two, R& a, R& b) {
   if (vec) {
     using V2 = typename std::conditional<sizeof(R) == 8, double2, float2>::type;
-    const V2 v = load_global(reinterpret_cast<const V2*>(p));
+    const V2 v = load_in<R>(reinterpret_cast<const V2*>(p));
     a = v.x;
     b = v.y;
   } else {
-    a = load_global(p);
-    b = two ? load_global(p + 1) : R(0);
+    a = load_in<R>(p);
+    b = two ? load_in<R>(p + 1) : R(0);
   }
 }
 
@@ -404,8 +414,8 @@ __global__ void __launch_bounds__(kDgThreads, 1)
           load_two<R>(p + S - k0 - k - 1, true, true, y1[it], y0[it]);
         } else {
           load_two<R>(p + k0 + k, false, two, x0[it], x1[it]);
-          y0[it] = load_global(p + S - k0 - k);
-          y1[it] = two ? load_global(p + S - k0 - k - 1) : R(0);
+          y0[it] = load_in<R>(p + S - k0 - k);
+          y1[it] = two ? load_in<R>(p + S - k0 - k - 1) : R(0);
         }
       }
     };
@@ -443,9 +453,10 @@ __global__ void __launch_bounds__(kDgThreads, 1)
           // largest magnitude of each of the warp's rows (FP64: by the high words), 32 loads in flight; a face
           // axis' wall slot holds no input
           constexpr int kRows = 2 * ITS, kStep = sizeof(R) / 4;
-          unsigned m[kRows];
+          int m[kRows];
 #pragma unroll
           for (int r = 0; r < kRows; ++r) m[r] = 0;
+          unsigned raw = 0;  // of all rows, not lowered
           const unsigned* w0 = reinterpret_cast<const unsigned*>(src) + (kStep - 1);
 #pragma unroll 1
           for (int k = (BWD ? 0 : k0) + lane; k - lane < n; k += 128) {
@@ -455,18 +466,32 @@ __global__ void __launch_bounds__(kDgThreads, 1)
 #pragma unroll
               for (int r = 0; r < kRows; ++r) {
                 const int row = min(2 * (kDgWarps * (r >> 1) + cw) + (r & 1), rows - 1);
-                v[q][r] = load_global(w0 + ((size_t)row * n + min(k + 32 * q, n - 1)) * kStep);
+                v[q][r] = load_in<R>(w0 + ((size_t)row * n + min(k + 32 * q, n - 1)) * kStep);
               }
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
+            for (int q = 0; q < 4; ++q) {
+              const int c20 = F64 ? in_exp[op][min(k + 32 * q, n - 1)] << 20 : 0;
 #pragma unroll
-              for (int r = 0; r < kRows; ++r)
-                m[r] = max(m[r], F64 ? lowered(v[q][r] & 0x7fffffffu, in_exp[op][min(k + 32 * q, n - 1)])
-                                     : v[q][r] & 0x7fffffffu);
+              for (int r = 0; r < kRows; ++r) {
+                const unsigned high = v[q][r] & 0x7fffffffu;
+                m[r] = max(m[r], (int)high - c20);
+                if (F64) raw = max(raw, high);
+              }
+            }
+          }
+          if (F64 && __any_sync(0xffffffffu, raw >= 0x7ff00000u)) {  // an Inf or NaN keeps its exponent: which rows?
+#pragma unroll
+            for (int r = 0; r < kRows; ++r) {
+              const int row = min(2 * (kDgWarps * (r >> 1) + cw) + (r & 1), rows - 1);
+              unsigned top = 0;
+              for (int k = (BWD ? 0 : k0) + lane; k < n; k += 32)
+                top = max(top, load_in<R>(w0 + ((size_t)row * n + k) * kStep) & 0x7fffffffu);
+              if (top >= 0x7ff00000u) m[r] = (int)top;
+            }
           }
 #pragma unroll
           for (int r = 0; r < kRows; ++r) {
-            const unsigned top = __reduce_max_sync(0xffffffffu, m[r]);
+            const unsigned top = __reduce_max_sync(0xffffffffu, (unsigned)m[r]);
             if (lane == 0)
               row_exp[tc & 3][2 * (kDgWarps * (r >> 1) + cw) + (r & 1)] = max((int)(top >> kExpShift), kExpMin);
           }
