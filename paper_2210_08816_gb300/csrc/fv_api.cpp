@@ -141,15 +141,15 @@ static int upload_axes(fv_grid_s* g, const AxisHost* ax, const HalfOpHost (*half
   return FV_OK;
 }
 
-// The half-size operators as digits for the tensor-core passes, both precisions, in one device buffer; axes with
-// the same faces share theirs.
-static int upload_digits(fv_grid_s* g, const HalfOpHost (*half)[3]) {
+// The half-size operators as digits for the tensor-core passes, of the precisions that need them, in one device buffer;
+// axes with the same faces share theirs.
+static int upload_digits(fv_grid_s* g, const HalfOpHost (*half)[3], const bool (&need)[2]) {
   struct Item {
     size_t dig, exp, cexp;
   };
   std::vector<unsigned char> buf, blocks, cexps;
   std::vector<int> exps;
-  Item items[3][3][2][2];  // [axis][kind][precision][direction]
+  Item items[3][3][2][2] = {};  // [axis][kind][precision][direction]
   auto put = [&](const void* p, size_t bytes) {
     const size_t at = buf.size();
     buf.resize((at + bytes + 255) & ~(size_t)255, 0);
@@ -164,6 +164,7 @@ static int upload_digits(fv_grid_s* g, const HalfOpHost (*half)[3]) {
       for (int prec = 0; prec < 2; ++prec)
         for (int dir = 0; dir < 2; ++dir) {
           Item& it = items[d][kind][prec][dir];
+          if (!need[prec]) continue;
           if (same >= 0) {
             it = items[same][kind][prec][dir];
             continue;
@@ -654,7 +655,9 @@ int fv_grid_create(const fv_grid_desc* desc, void* stream, fv_grid* out) {
   const HalfOpHost(*hp)[3] = g->half_ready ? half : nullptr;
   if (st == FV_OK) st = upload_axes<double>(g, ax, hp, 0, g->geo64, g->fdm64, g->cd64, g->fd64, g->half64);
   if (st == FV_OK) st = upload_axes<float>(g, ax, hp, 1, g->geo32, g->fdm32, g->cd32, g->fd32, g->half32);
-  if (st == FV_OK && g->half_ready && (std::max({n[0], n[1], n[2]}) + 1) / 2 <= kDigitMaxH) st = upload_digits(g, half);
+  const bool digits[2] = {digits_reached(n, 0), digits_reached(n, 1)};
+  if (st == FV_OK && g->half_ready && (std::max({n[0], n[1], n[2]}) + 1) / 2 <= kDigitMaxH && (digits[0] || digits[1]))
+    st = upload_digits(g, half, digits);
   for (auto setup : {half_setup, plane_setup, flux_setup, stencil_setup, stencil_pair_setup})
     if (st == FV_OK) st = setup();
   if (st == FV_OK && tc_setup(g) != FV_OK) {  // keep the other passes

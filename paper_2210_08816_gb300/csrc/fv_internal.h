@@ -113,7 +113,7 @@ struct fv_grid_s {
   // the same operators as half-size problems, [axis][kind], when every axis is mirror-symmetric; the dense
   // matrices above are then not built
   bool half_ready = false;
-  bool digit_ready = false;  // ... and as digits for the tensor cores (h <= kDigitMaxH on every axis)
+  bool digit_ready = false;  // ... and as digits for the tensor cores, where a pass takes them (h <= kDigitMaxH on every axis)
   void* digit_buf = nullptr;
   fv::HalfDev<double> half64[3][3];
   fv::HalfDev<float> half32[3][3];
@@ -413,6 +413,12 @@ int build_half_op(const AxisHost& a, int kind, HalfOpHost& o);
 // Parts per value and outputs per unit of work of the digit passes, and their longest half axis (the FP64 order sums
 // stay within 2^24).
 constexpr int kDigits64 = 7, kDigitCols64 = 32, kDigits32 = 2, kDigitCols32 = 64, kDigitMaxH = 128;
+// Multiplications of a half-size pass (rows x n x h, four times that where four fields share it) from which the digit passes
+// win (kernels_fdm.cu), and whether any pass of a grid of n[0] x n[1] x n[2] cells gets there (prec 0: FP64, 1: FP32) or to
+// the FP32 pressure passes of kernels_tc.cu: smaller grids are created without the operands.
+constexpr double kDigitWork64 = 3.2e6, kDigitWork32 = 1.6e7;
+bool digits_reached(const int n[3], int prec);
+bool tc_sizes(const int n[3]);
 // The two h x h matrices as D balanced base-256 digits (FP16), row j on the common exponent exps[j] of both parts:
 // 2^cexps[part h + k] M[part][j][k] = 2^exps[j] sum_i digit_i 256^(D-1-i).  Blocks [part][group of NC rows][slab of 32
 // columns], each D NC rows (digit i, output j % NC at row i NC + j % NC) of 64 bytes, 64-byte swizzled.

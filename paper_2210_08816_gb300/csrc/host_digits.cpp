@@ -11,6 +11,17 @@
 
 namespace fv {
 
+bool tc_sizes(const int n[3]) {
+  for (int d = 0; d < 3; ++d)
+    if (n[d] < 32 || n[d] > 256 || n[d] % 32 != 0) return false;
+  return true;
+}
+
+bool digits_reached(const int n[3], int prec) {
+  const double work = 4.0 * n[0] * n[1] * n[2] * ((std::max({n[0], n[1], n[2]}) + 1) / 2);
+  return prec == 0 ? work >= kDigitWork64 : work >= kDigitWork32 || tc_sizes(n);
+}
+
 // FP16 bits of the integers -128 .. 128 (exact)
 struct HalfTable {
   uint16_t bits[257];
@@ -47,23 +58,28 @@ void build_digits(const std::vector<double> (&M)[2], int h, int D, int NC, bool 
   uint16_t* out = reinterpret_cast<uint16_t*>(blocks.data());
   exps.assign(h, 0);
   cexps.assign(2 * (size_t)h, 0);
-  std::vector<int> q(2 * (size_t)h, INT_MIN);  // largest magnitude of every column
+  std::vector<int> q(2 * (size_t)h, INT_MIN);  // exponent of every column's largest magnitude
+  std::vector<double> most(h);
   int top = INT_MIN;
-  for (int part = 0; part < 2; ++part)
+  for (int part = 0; part < 2; ++part) {
+    std::fill(most.begin(), most.end(), 0.0);
+    for (int j = 0; j < h; ++j)
+      for (int k = 0; k < h; ++k) most[k] = std::max(most[k], std::fabs(M[part][(size_t)j * h + k]));
     for (int k = 0; k < h; ++k) {
-      double most = 0.0;
-      for (int j = 0; j < h; ++j) most = std::max(most, std::fabs(M[part][(size_t)j * h + k]));
-      if (most > 0.0) std::frexp(most, &q[part * h + k]);
+      if (most[k] > 0.0) std::frexp(most[k], &q[part * h + k]);
       top = std::max(top, q[part * h + k]);
     }
+  }
   for (int k = 0; k < h && shared; ++k) q[k] = q[h + k] = std::max(q[k], q[h + k]);
   for (size_t i = 0; i < q.size(); ++i)
     if (q[i] != INT_MIN) cexps[i] = (unsigned char)std::min(top - q[i], kDigitMaxColumn);
-  std::vector<double> S[2];
+  std::vector<double> S[2];  // the columns scaled (powers of two: exact)
   for (int part = 0; part < 2; ++part) {
-    S[part] = M[part];
+    std::vector<double> scale(h);
+    for (int k = 0; k < h; ++k) scale[k] = std::ldexp(1.0, cexps[part * h + k]);
+    S[part].resize((size_t)h * h);
     for (int j = 0; j < h; ++j)
-      for (int k = 0; k < h; ++k) S[part][(size_t)j * h + k] = std::ldexp(S[part][(size_t)j * h + k], cexps[part * h + k]);
+      for (int k = 0; k < h; ++k) S[part][(size_t)j * h + k] = M[part][(size_t)j * h + k] * scale[k];
   }
   for (int j = 0; j < h; ++j) {
     exps[j] = row_exponent(S, h, j) - (8 * D - 1);  // integers of magnitude <= 2^(8 D - 1)

@@ -256,7 +256,7 @@ const HalfDev<float> (&half_of<float>(const fv_grid_s* g))[3][3] { return g->hal
 // by one, bit for bit.
 template <typename R>
 bool digit_wins(int n, long long rows) {
-  return (double)rows * n * ((n + 1) / 2) >= (sizeof(R) == 8 ? 3.2e6 : 1.6e7);
+  return (double)rows * n * ((n + 1) / 2) >= (sizeof(R) == 8 ? kDigitWork64 : kDigitWork32);
 }
 
 // Unused shared memory that leaves room for `per` blocks on an SM, all of it or (FP32, whose launches are short) no more than

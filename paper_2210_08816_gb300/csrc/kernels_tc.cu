@@ -482,8 +482,8 @@ int encode_tensor_map(CUtensorMap* map, CUtensorMapDataType type, int rank, cons
 constexpr double kTcMostSpan = 536870912.0;
 int tc_setup(fv_grid_s* g) {
   static_assert(kDigitCols32 == 64 && kDigits32 == 2, "the B blocks hold 64 outputs, two parts");
-  for (int n : {g->nx, g->ny, g->nz})
-    if (n < 32 || n > 256 || n % 32 != 0) return FV_OK;
+  const int n[3] = {g->nx, g->ny, g->nz};
+  if (!tc_sizes(n)) return FV_OK;
   if (width_ratio(g->xf[0]) * width_ratio(g->xf[1]) * width_ratio(g->xf[2]) > kTcMostSpan) return FV_OK;
   if (!g->digit_ready || !encoder()) return FV_OK;
   for (auto k : {k_pass_tc<false, false, 256>, k_pass_tc<true, false, 256>, k_pass_tc<false, true, 256>,
