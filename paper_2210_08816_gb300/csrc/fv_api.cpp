@@ -676,6 +676,8 @@ int fv_grid_create(const fv_grid_desc* desc, void* stream, fv_grid* out) {
       set_error("workspace allocation failed");
     }
   }
+  // the fills and copies above ran on the default stream, which a non-blocking stream of the handle does not wait for
+  if (st == FV_OK) st = cu_ok(cudaStreamSynchronize(nullptr), "fv_grid_create");
   if (st != FV_OK) {
     fv_grid_destroy(g);
     return st;

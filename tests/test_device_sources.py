@@ -90,3 +90,13 @@ def test_overlapping_kernels_read_their_predecessors_results_by_ordinary_loads()
             alone = f"launch_spread({kernel}<" in src and not re.search(rf"launch(_cluster)?\([^;]*\b{kernel}\b", src)
             assert alone or m.group(1) in {"M", "lx", "ly", "lz"}, f"{name}: const __restrict__ {m.group(1)}"
     assert seen >= 8
+
+
+def test_grid_creation_waits_for_its_own_fills():
+    """The field maxima, the error word, metrics and operands are filled on the default stream; a handle's non-blocking stream
+    does not wait for that one, and a solve would add its largest magnitude to what the memory held."""
+    create = _source("fv_api.cpp")
+    create = create[create.index("int fv_grid_create("):create.index("int fv_grid_destroy(")]
+    sync = create.index("cudaStreamSynchronize(nullptr)")
+    assert all(m.start() < sync for m in re.finditer(r"cudaMemset\(|upload_\w+[<(]|tc_setup\(", create))
+    assert sync < create.index("*out = g")
