@@ -259,26 +259,24 @@ def gpu_arm(args, ws, rank, local):
     hbm_src = "measured copy bandwidth" if "hbm_gbs" in peaks else "fallback 6.8 TB/s"
     if dom == "transform_tc":
         # One pass reads the N-cell field and writes it with the contracted axis rotated: 2 N FP32 values of
-        # HBM traffic, which bounds it.  Its tensor work: the grid is mirror-symmetric, so a pass contracts
-        # the sums and differences of mirrored inputs with two n/2 x n/2 matrices, N n flops (half of the
-        # dense 2 N n), executed three times as products of FP16 heads and remainders.
+        # HBM traffic, which bounds it.  Its tensor work: see pass_work.
         traffic_bytes = 2 * N * 4
         achieved = traffic_bytes / (per_launch_ms * 1e-3) / 1e9
-        flops = 1.0 * N * n
+        kernel, _, flops = pass_work(n, tensor=True)
         bf16 = float(peaks.get("bf16_tflops", 1900.0))
-        executed = 3.0 * flops / (per_launch_ms * 1e-3) / 1e12
-        roof = {"kernel": "k_pass_tc (tcgen05 fast-diagonalisation pass, three products of FP16 parts)", "bound": "hbm",
+        executed = flops / (per_launch_ms * 1e-3) / 1e12
+        roof = {"kernel": kernel, "bound": "hbm",
                 "achieved": round(achieved, 1), "peak": hbm_peak, "unit": "GB/s",
                 "frac": round(achieved / hbm_peak, 4), "peak_source": hbm_src,
                 "tensor": {"executed_tflops": round(executed, 2), "peak": round(bf16, 1),
-                           "frac": round(executed / bf16, 4), "flops_per_pass": 3 * flops,
+                           "frac": round(executed / bf16, 4), "flops_per_pass": flops,
                            "peak_source": ("measured bf16 burst (FP16 runs at the same rate)" if "bf16_tflops" in peaks
                                            else "fallback 1.9 PF bf16")}}
     elif dom == "transform":
-        flops = 2.0 * N * n
+        kernel, flops, _ = pass_work(n, tensor=False)
         achieved = flops / (per_launch_ms * 1e-3) / 1e12
         peak = SM_COUNT * FP32_LANES * 2 * SM_MAX_MHZ * 1e6 / 1e12
-        roof = {"kernel": "k_half / k_transform (CUDA-core fast-diagonalisation pass)", "bound": "alu",
+        roof = {"kernel": kernel, "bound": "alu",
                 "achieved": round(achieved, 3), "peak": round(peak, 2), "unit": "TFLOP/s",
                 "frac": round(achieved / peak, 4),
                 "peak_source": "FP32 FMA lanes x 2 x 152 SMs x 2070 MHz (unit counts and max clock)"}
@@ -317,6 +315,25 @@ def gpu_arm(args, ws, rank, local):
         fp64 = fp64_leg(fv, g, q64, y0_64, y1_64, sigma, K, ws, device, stream)
     return finish(args, ws, rank, n, value, K, W, ms_step, e2e, launches, roof, hbm_stencil, step_bytes, breakdown,
                   fp64, clocks, g, device)
+
+
+def pass_work(n, tensor):
+    """(kernel, algorithmic flops, executed flops) of one FP32 fast-diagonalisation pass of the n^3 bench grid.  The grid is
+    mirror-symmetric: a pass contracts the sums and differences of mirrored inputs with two h x h matrices, h = ceil(n / 2),
+    4 n^2 h^2 flops (half of the dense 2 n^4).  On the CUDA cores they are executed as they are.  On the tensor cores as
+    products of FP16 parts: three on axes of a multiple of 32 cells, 32 to 256, else four, with inputs padded to slabs of 32
+    and outputs to groups of 64."""
+    h = (n + 1) // 2
+    flops = 4.0 * n * n * h * h
+    if not tensor:
+        return "k_half (CUDA-core fast-diagonalisation pass of half-size operators)", flops, flops
+    if 32 <= n <= 256 and n % 32 == 0:
+        pad = -(-h // 32) * 32
+        return ("k_pass_tc (tcgen05 fast-diagonalisation pass, three products of FP16 parts)", flops,
+                3.0 * 4.0 * n * n * h * pad)
+    return ("k_digit_pass<float> (tcgen05 fast-diagonalisation pass, four products of FP16 parts)", flops,
+            4.0 * 4.0 * n * n * (-(-h // 32) * 32) * (-(-h // 64) * 64))
+
 
 
 def e2e_leg(fv, g, q, ya, yb, sigma, K, ws, device, stream):
