@@ -847,14 +847,12 @@ static int jvp_project_block(fv_grid_s* g, double Gr, double sigma, const R* q, 
   R* Y = (R*)g->ws.bY[p];
   R* phi = (R*)g->ws.bt1[p];
   R* tmp = (R*)g->ws.bt0[p];
-  const size_t n4 = 4 * g->N;
   const TempOut t = temp_out<R>(g, q, V, sigma != 0.0, 1.0, sigma, nullptr, 0.0, W, nvec);
   bool pair = false;
   if constexpr (sizeof(R) == 4) pair = stencil_pair_eligible(g, q, V);
   if constexpr (sizeof(R) == 4) {
     if (pair) FV_TRY(launch_stencil_pair(g, Gr, sigma, q, V, Y, nvec, t));
   }
-  (void)n4;
   if (!pair) FV_TRY(launch_jvp_block<R>(g, Gr, sigma, q, V, Y, nvec, t));
   FV_TRY(launch_divergence<R>(g, Y, phi, nvec));
   FV_TRY(launch_poisson_block<R>(g, phi, phi, tmp, nvec));

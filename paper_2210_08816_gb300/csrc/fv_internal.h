@@ -416,7 +416,7 @@ constexpr int kDigits64 = 7, kDigitCols64 = 32, kDigits32 = 2, kDigitCols32 = 64
 // Multiplications of a half-size pass (rows x n x h, four times that where four fields share it) from which the digit passes
 // win (kernels_fdm.cu), and whether any pass of a grid of n[0] x n[1] x n[2] cells gets there (prec 0: FP64, 1: FP32) or to
 // the FP32 pressure passes of kernels_tc.cu: smaller grids are created without the operands.
-constexpr double kDigitWork64 = 3.2e6, kDigitWork32 = 1.6e7;
+constexpr double kDigitWork64 = 3.2e6, kDigitWork32 = 2.0e7;
 bool digits_reached(const int n[3], int prec);
 bool tc_sizes(const int n[3]);
 // The two h x h matrices as D balanced base-256 digits (FP16), row j on the common exponent exps[j] of both parts:

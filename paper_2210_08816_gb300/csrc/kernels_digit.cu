@@ -21,8 +21,8 @@
 //
 // Why: GB300 issues two FP64 operations per clock and SM (1.23 TFLOP/s measured in k_half); the 28 FP16 products
 // cost 155 GFLOP per 256^3 pass where the FP16 tensor rate is 1.9 PFLOP/s.  Measured, six passes, CUDA cores / here:
-// FP64 256^3 21.9 / 1.94 ms, 100^3 794 / 193 us; FP32 100^3 98 / 76 us, 250^3 1360 / 450 us, four fields of 256^3
-// 5.2 / 1.65 ms.  Errors against 64 bits are at or below those of the CUDA-core passes (FP32 100^3 product 3.9e-7 ->
+// FP64 256^3 21.9 / 2.00 ms, 100^3 794 / 199 us; FP32 100^3 88 / 75 us, 250^3 1360 / 460 us, four fields of 256^3
+// 5.2 / 1.67 ms.  Errors against 64 bits are at or below those of the CUDA-core passes (FP32 100^3 product 3.9e-7 ->
 // 2.4e-7, FP64 256^3 3.4e-14 as before).  What bounds a unit is the workers' instruction issue (FP64: digits and the
 // joining of the accumulators, 56 % of the integer pipe), not the MMAs (19 % of the tensor pipe).
 //

@@ -249,10 +249,10 @@ const HalfDev<float> (&half_of<float>(const fv_grid_s* g))[3][3] { return g->hal
 
 // Digit products on the tensor cores (kernels_digit.cu) instead of the CUDA-core form, by the multiplications of a
 // half-size pass: a digit pass has a floor of ~6 us (FP64 ~11) before its length shows.  Measured (us a projection, CUDA
-// cores / digits): FP64 40^3 (1.3e6) 53 / 69, 44^3 67 / 70, 48^3 (2.7e6) 70 / 71, 52^3 (3.7e6) 108 / 77, 56^3 113 / 78;
-// FP32 50^3 32 / 35, 60^3 42.5 / 44, 70^3 (1.2e7) 49 / 54, 80^3 (2.0e7) 69 / 61, 90^3 68 / 60; the diffusion solve's
-// four fields in FP32 50^3 (1.3e7) 39 / 33, 60^3 (2.6e7) 43 / 34, 80^3 96 / 81.  Single passes at 160^3 FP64 589 / 78,
-// 250^3 FP32 227 / 75.  The number of vectors in a block does not count: a block's results are those of its vectors one
+// cores / digits): FP64 40^3 (1.4e6) 53 / 69, 44^3 65 / 70, 48^3 (2.8e6) 75 / 72, 52^3 (3.9e6) 104 / 77, 56^3 109 / 79;
+// FP32 50^3 29 / 33, 60^3 37.5 / 42, 70^3 (1.2e7) 45 / 51, 80^3 (2.1e7) 55 / 57, 86^3 (2.8e7) 56 / 55.5, 90^3 63 / 57; the
+// diffusion solve's four fields in FP32 50^3 (1.3e7) 31.8 / 32.9, 52^3 (1.5e7) 31.6 / 33.1, 56^3 (2.1e7) 34.7 / 33.2, 60^3
+// 42 / 36, 80^3 100 / 81.  The number of vectors in a block does not count: a block's results are those of its vectors one
 // by one, bit for bit.
 template <typename R>
 bool digit_wins(int n, long long rows) {

@@ -153,13 +153,13 @@ def test_halves_give_the_matrices_back(L, h, span):
 
 @pytest.mark.parametrize("n,want64,want32", [
     ((2, 2, 2), 0, 0), ((8, 8, 8), 0, 0), ((16, 16, 16), 0, 0), ((31, 31, 31), 0, 0), ((32, 32, 32), 0, 1), ((35, 35, 35), 0, 0),
-    ((36, 36, 36), 1, 0), ((40, 41, 42), 1, 0), ((17, 33, 65), 1, 0), ((16, 16, 256), 1, 1), ((12, 12, 255), 1, 1),
-    ((4, 4, 255), 0, 0), ((52, 52, 52), 1, 0), ((54, 54, 54), 1, 1), ((64, 64, 64), 1, 1)])
+    ((36, 36, 36), 1, 0), ((40, 41, 42), 1, 0), ((17, 33, 65), 1, 0), ((16, 16, 256), 1, 1), ((12, 12, 255), 1, 0),
+    ((4, 4, 255), 0, 0), ((55, 55, 55), 1, 0), ((57, 57, 57), 1, 1), ((64, 64, 64), 1, 1)])
 def test_operands_are_made_where_a_pass_takes_them(L, n, want64, want32):
     """A pass of four fields along the longest axis makes 4 N ceil(n / 2) multiplications and takes the digits from 3.2e6 on,
-    the FP32 parts from 1.6e7; axes of a multiple of 32 cells, 32 to 256, take the FP32 pressure passes."""
+    the FP32 parts from 2e7; axes of a multiple of 32 cells, 32 to 256, take the FP32 pressure passes."""
     work = 4.0 * n[0] * n[1] * n[2] * ((max(n) + 1) // 2)
     tc = all(32 <= k <= 256 and k % 32 == 0 for k in n)
     assert L.reached(*n, 0) == int(work >= 3.2e6)
-    assert L.reached(*n, 1) == int(work >= 1.6e7 or tc)
+    assert L.reached(*n, 1) == int(work >= 2.0e7 or tc)
     assert (L.reached(*n, 0), L.reached(*n, 1)) == (want64, want32)
