@@ -75,9 +75,10 @@ typedef struct {
  * used by the pressure solve (computed on the host in FP64), and workspace.
  * Faces mirror-symmetric about 1/2 (as the built-in grids' are) give half-size
  * transforms in the direct solves; the FP32 pressure solve then runs on the tensor
- * cores when every axis has 32 to 256 cells, a multiple of 32, and other large
- * solves (FP64 too) run there as products of FP16 parts that keep their precision;
- * other grids take the CUDA-core passes, with the same results to round-off.
+ * cores when every axis has 32 to 256 cells, a multiple of 32 (and the product of
+ * the axes' width ratios is at most 2^29), and other large solves (FP64 too) run
+ * there as products of FP16 parts that keep their precision; other grids take the
+ * CUDA-core passes, with the same results to round-off.
  * `stream` is a cudaStream_t (NULL = legacy default stream).
  * Errors: FV_EINVAL (sizes, faces), FV_ENOMEM, FV_ECUDA. */
 int fv_grid_create(const fv_grid_desc* desc, void* stream, fv_grid* out);
